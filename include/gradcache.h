@@ -15,7 +15,7 @@
  * dQ and dP together are the cache [u_1..u_B, v_1..v_N] of (B + N) d floats (Section 3.3).
  * The paper fixes tau = 1 and has no mask; for general tau these are the exact derivatives of
  * Eq. 1, and eps_j of Eq. 7 is the sum of f(s_k) over every k with r_k = j.  The B x N matrix
- * S is never written to memory.
+ * S is never held in memory: at most a strip of its rows is, in a workspace of bounded size.
  *
  * Conventions shared by all calls
  *   - Every pointer is a DEVICE pointer (including loss and dev_status) unless stated; the
@@ -72,24 +72,26 @@ typedef enum { GC_OP_FWD = 0, GC_OP_BWD = 1, GC_OP_BUILD = 2, GC_OP_BUILD_STORED
 enum { GC_DEV_POS_RANGE = 1, GC_DEV_POS_MASKED = 2, GC_DEV_WAIT_LIMIT = 4 };
 
 /* Bytes of workspace the given call needs for these sizes on the current device (a multiple
- * of 256).  O((B + N) d), never O(B N), for the three calls of the paper's path;
- * GC_OP_BUILD_STORED adds 2 B N bytes for its weight matrix.  Returns 0 for invalid arguments. */
+ * of 256).  O((B + N) d) plus, for the three calls of the paper's path, at most 1 GiB of softmax
+ * weights of a strip of query rows (bf16 rows of more than 2^16 passages: never fewer than 256
+ * queries); GC_OP_BUILD_STORED adds 2 B N bytes for its weight matrix.  Returns 0 for invalid arguments. */
 size_t gc_workspace_bytes(int op, int64_t B, int64_t N, int d, int dtype);
 
 /* Name of the kernel plan the library will use for these sizes:
  *   "tcgen05-one-tile"  one launch for a batch of one tile: B <= 128, N <= 256 (bf16) or N <= 128
  *                       (fp32, on the tensor cores as three bf16 terms), d a multiple of 8 up to 1024
- *   "tcgen05-tiles"     fp32 batches of tile pairs of 128 x 128 whose planes of partial sums,
- *                       4 d (B ceil(N/128) + N ceil(B/128)) bytes of workspace, stay within 2 GiB,
- *                       and bf16 batches of tile pairs of 128 x 256 that make at most two waves of
- *                       CTAs (d a multiple of 8 up to 4096): the same kernel per tile pair, then
- *                       combine and reduce kernels
- *   "tcgen05"           TMA + tcgen05 MMA sweeps with TMEM accumulators; bf16, d a multiple of 64
- *                       up to 4096; one CTA, a CTA pair or a cluster of four per tile, by shape
+ *   "tcgen05-tiles"     the strip plan (below) for fp32 batches whose tile pairs of 128 x 128 would
+ *                       need at most 2 GiB of partial sums, 4 d (B ceil(N/128) + N ceil(B/128)) bytes,
+ *                       and for bf16 batches of few tile pairs of 128 x 256 (d a multiple of 8 up to
+ *                       4096; at most two CTAs' worth of 64-column slices per SM)
+ *   "tcgen05"           bf16, d a multiple of 64 up to 4096, TMA + tcgen05 MMA.  The strip plan: three
+ *                       products over strips of query rows whose weights are held in the workspace;
+ *                       or, for rows of at most 384 values and many pairs, sweeps that keep every
+ *                       logit on the chip (one CTA, a CTA pair or a cluster of four per tile)
  *   "simt"              fp32 FMA tiles: every other case (other widths, fp32 batches beyond that)
  * "invalid" for an unknown op, non-positive sizes, or a problem GC_OP_BUILD_STORED refuses.
  * Static string.  With GRADCACHE_PLAN=sweeps in the environment (read at every call; a
- * diagnostic switch) the first two plans are not chosen. */
+ * diagnostic switch) the one-tile and strip plans are not chosen. */
 const char* gc_plan_name(int op, int64_t B, int64_t N, int d, int dtype);
 
 /* Number of kernels one call launches for these sizes (for launch accounting). */
@@ -116,10 +118,10 @@ int gc_loss_bwd(const void* Q, int64_t ldq, const void* P, int64_t ldp, const in
 
 /*
  * Step 2 of Section 3.3 in one call: loss, row_lse, (pos_logit) and the cache dQ, dP.  Nothing of
- * size B x N is written to global memory.  For bf16 rows (d a multiple of 64) the forward runs
+ * size B x N is held in global memory (see gc_workspace_bytes).  On the sweeps the forward runs
  * inside the dQ sweep; where each row's weights are scaled by its positive logit, the anchor
- * kernel that computes those logits and the sweep overlap (programmatic dependent launch).  Part of the work may be queued on a stream the library owns, between a fork from
- * and a join back into `cuda_stream`: the call is asynchronous on `cuda_stream` alone, but the
+ * kernel that computes those logits and the sweep overlap (programmatic dependent launch).  Part of
+ * that work may be queued on a stream the library owns, between a fork from and a join back into `cuda_stream`: the call is asynchronous on `cuda_stream` alone, but the
  * first such call on a device creates that stream and belongs outside any stream capture.
  */
 int gc_build_cache(const void* Q, int64_t ldq, const void* P, int64_t ldp, const int32_t* pos_idx,
@@ -131,7 +133,7 @@ int gc_build_cache(const void* Q, int64_t ldq, const void* P, int64_t ldp, const
 /*
  * The same results as gc_build_cache by a different route, kept as a measured comparison point:
  * Eq. 1 and Eq. 5-7 need every logit three times (loss, dQ, dP), and gc_build_cache recomputes
- * them so that nothing of size B x N ever leaves the chip.  This call trades memory for work: one
+ * them, or holds a bounded strip of them, so that nothing of size B x N is kept.  This call trades memory for work: one
  * forward sweep writes the un-normalised bf16 softmax weights 2^((S_ij - S_{i,r_i}) log2 e) of
  * all pairs to the workspace (2 B N bytes; 0 at masked pairs and at the positive column, whose
  * terms are added in fp32), and two plain GEMMs over that matrix form dQ and dP.  Rows whose
@@ -311,8 +313,9 @@ int gc_dist_dot_block(const void* Q, int64_t ldq, const void* P, int64_t ldp, in
 
 /*
  * Forward with library-owned scratch (no counterpart in the paper: it exists for the sake of
- * callers, not of the method).  Same inputs, outputs and results as gc_loss_fwd, but the caller
- * passes no workspace.  It is meant for callers that cannot obtain device memory at the point of
+ * callers, not of the method).  Same inputs and outputs as gc_loss_fwd, and the same results (within
+ * rounding where gc_loss_fwd uses more scratch than the array below has), but the caller passes no
+ * workspace.  It is meant for callers that cannot obtain device memory at the point of
  * the call: code running under a host framework that owns every byte of the device through its
  * own pool and offers no allocation hook to a C library, and loops on a hot path where an
  * allocator call is unwelcome because it may synchronise the whole device or fail late.  The

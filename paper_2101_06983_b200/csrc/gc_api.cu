@@ -108,6 +108,11 @@ Plan make_plan(int64_t B, int64_t N, int d, int dtype, bool stored) {
         // positive terms, then the gated fallback sequence
         pl.launches_build = 8 + (pl.g_mp > 1 ? 1 : 0) + pl.launches_build;
     }
+    pl.strips = strip_applicable(B, N, d, dtype) ? 1 : 0;
+    if (pl.strips) {
+        const size_t need = strip_workspace_bytes(B, N, d, dtype);
+        if (need > off) off = need;
+    }
     pl.total = off;
     return pl;
 }
@@ -202,6 +207,7 @@ Problem make_problem(const void* Q, int64_t ldq, const void* P, int64_t ldp,
     p.tau = tau; p.mask_mode = mask_mode; p.dtype = dtype;
     p.b_total = 0;
     p.mask_shift = 0;
+    p.pos_base = p.n_total = 0;
     return p;
 }
 
@@ -600,6 +606,14 @@ size_t forward_layout(Plan* pl, int64_t B, int64_t N) {
     return off;
 }
 
+// Scratch of the strip plan's forward where it serves this problem from the static array, else 0:
+// problems whose logits (fp32) or slots do not fit keep the plans that need less.
+size_t static_strip_need(int64_t B, int64_t N, int d, int dtype) {
+    if (!strip_applicable(B, N, d, dtype)) return 0;
+    const size_t need = strip_forward_bytes(B, N, d, dtype);
+    return need <= (size_t)GC_STATIC_SCRATCH_BYTES ? need : 0;
+}
+
 // Device address of g_static_scratch on the current device, or nullptr on failure.
 void* static_scratch_ptr() {
     static void* cached[64] = {nullptr};
@@ -635,13 +649,16 @@ const char* gc_plan_name(int op, int64_t B, int64_t N, int d, int dtype) {
     if (op < GC_OP_FWD || op > GC_OP_BUILD_STORED || B <= 0 || N <= 0 || d <= 0) return "invalid";
     if (op == GC_OP_BUILD_STORED && !make_plan(B, N, d, dtype, true).mat) return "invalid";
     if (op != GC_OP_BUILD_STORED && small_applicable(B, N, d, dtype)) return "tcgen05-one-tile";
-    if (op != GC_OP_BUILD_STORED && small_tiled_applicable(B, N, d, dtype)) return "tcgen05-tiles";
+    if (op != GC_OP_BUILD_STORED && strip_applicable(B, N, d, dtype))
+        return small_tiled_applicable(B, N, d, dtype) ? "tcgen05-tiles" : "tcgen05";
     return tc_supported(B, N, d, dtype) ? "tcgen05" : "simt";
 }
 
 int gc_kernel_launches(int op, int64_t B, int64_t N, int d, int dtype) {
     if (B <= 0 || N <= 0 || d <= 0) return 0;
     if (op >= GC_OP_FWD && op <= GC_OP_BUILD && small_applicable(B, N, d, dtype)) return 1;
+    if (op >= GC_OP_FWD && op <= GC_OP_BUILD && strip_applicable(B, N, d, dtype))
+        return strip_launches(op, B, N, d, dtype);
     if (op >= GC_OP_FWD && op <= GC_OP_BUILD && small_tiled_applicable(B, N, d, dtype)) {
         const int reduces = (small_tiles_y(N, dtype) > 1 ? 1 : 0) + (small_tiles_x(B) > 1 ? 1 : 0);
         if (op == GC_OP_FWD) return 2;                  // tile kernel, combine
@@ -671,6 +688,11 @@ int gc_loss_fwd(const void* Q, int64_t ldq, const void* P, int64_t ldp, const in
     if (small_applicable(B, N, d, dtype))
         return run_small(GC_OP_FWD, p, nullptr, loss, row_lse, pos_logit, nullptr, 0, nullptr, 0,
                          dev_status, static_cast<cudaStream_t>(cuda_stream));
+    if (pl.strips) {
+        KernelTimer t(0, static_cast<cudaStream_t>(cuda_stream));
+        return strip_forward(p, ws, loss, row_lse, pos_logit, dev_status,
+                             static_cast<cudaStream_t>(cuda_stream)) == cudaSuccess ? GC_OK : GC_ERR_CUDA;
+    }
     if (pl.tiles)
         return run_tiles_fwd(p, pl, static_cast<char*>(ws), loss, row_lse, pos_logit, dev_status,
                              static_cast<cudaStream_t>(cuda_stream));
@@ -680,6 +702,7 @@ int gc_loss_fwd(const void* Q, int64_t ldq, const void* P, int64_t ldp, const in
 
 size_t gc_static_scratch_need(int64_t B, int64_t N, int d, int dtype) {
     if (B <= 0 || N <= 0 || d <= 0 || (dtype != GC_F32 && dtype != GC_BF16)) return 0;
+    if (const size_t need = static_strip_need(B, N, d, dtype)) return need;
     Plan pl = make_plan(B, N, d, dtype);
     return forward_layout(&pl, B, N);
 }
@@ -692,7 +715,8 @@ int gc_loss_fwd_static(const void* Q, int64_t ldq, const void* P, int64_t ldp,
     if (rc) return rc;
     if (!loss || !row_lse) return GC_ERR_NULL;
     Plan pl = make_plan(B, N, d, dtype);
-    if (forward_layout(&pl, B, N) > (size_t)GC_STATIC_SCRATCH_BYTES) return GC_ERR_LIMIT;
+    const bool strips = static_strip_need(B, N, d, dtype) > 0;
+    if (!strips && forward_layout(&pl, B, N) > (size_t)GC_STATIC_SCRATCH_BYTES) return GC_ERR_LIMIT;
     if ((rc = check_device())) return rc;
     void* scratch = static_scratch_ptr();
     if (!scratch) return GC_ERR_CUDA;
@@ -701,6 +725,9 @@ int gc_loss_fwd_static(const void* Q, int64_t ldq, const void* P, int64_t ldp,
     if (small_applicable(B, N, d, dtype))      // one launch, no scratch at all
         return run_small(GC_OP_FWD, p, nullptr, loss, row_lse, pos_logit, nullptr, 0, nullptr, 0,
                          dev_status, static_cast<cudaStream_t>(cuda_stream));
+    if (strips)
+        return strip_forward(p, scratch, loss, row_lse, pos_logit, dev_status,
+                             static_cast<cudaStream_t>(cuda_stream)) == cudaSuccess ? GC_OK : GC_ERR_CUDA;
     if (pl.tiles)
         return run_tiles_fwd(p, pl, static_cast<char*>(scratch), loss, row_lse, pos_logit,
                              dev_status, static_cast<cudaStream_t>(cuda_stream));
@@ -726,6 +753,11 @@ int gc_loss_bwd(const void* Q, int64_t ldq, const void* P, int64_t ldp, const in
     if (small_applicable(B, N, d, dtype) && (dQ || dP))
         return run_small(GC_OP_BWD, p, row_lse, nullptr, nullptr, nullptr, dQ, lddq, dP, lddp,
                          dev_status, st);
+    if (pl.strips && (dQ || dP)) {
+        KernelTimer t(1, st);
+        return strip_backward(p, ws, row_lse, dQ, lddq, dP, lddp, dev_status, st) == cudaSuccess
+                   ? GC_OK : GC_ERR_CUDA;
+    }
     if (dev_status && launch_pos_check(pos_idx, B, N, mask_mode, dev_status, st) != cudaSuccess)
         return GC_ERR_CUDA;
     char* w = static_cast<char*>(ws);
@@ -755,6 +787,11 @@ int gc_build_cache(const void* Q, int64_t ldq, const void* P, int64_t ldp, const
     if (small_applicable(B, N, d, dtype))
         return run_small(GC_OP_BUILD, p, nullptr, loss, row_lse, pos_logit, dQ, lddq, dP, lddp,
                          dev_status, st);
+    if (pl.strips) {
+        KernelTimer t(1, st);
+        return strip_build(p, ws, loss, row_lse, pos_logit, dQ, lddq, dP, lddp, dev_status, st) ==
+                       cudaSuccess ? GC_OK : GC_ERR_CUDA;
+    }
     if (pl.tiles) {
         if ((rc = run_tiles_fwd(p, pl, w, loss, row_lse, pos_logit, dev_status, st))) return rc;
         return run_tiles_bwd(p, pl, w, row_lse, dQ, lddq, dP, lddp, dev_status, st);
@@ -810,6 +847,12 @@ int gc_shard_fwd_dq(const void* Q, int64_t ldq, const void* P, int64_t ldp, cons
     Problem p = make_problem(q_first, ldq, P, ldp, pos_idx + q0, q_count, N, d, tau, mask_mode, dtype);
     p.b_total = B;
     p.mask_shift = q0;             // local query i is query q0 + i of the batch
+    if (pl.strips) {
+        cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+        KernelTimer t(1, st);
+        return strip_build(p, ws, loss_part, row_lse + q0, pos_logit ? pos_logit + q0 : nullptr, dQ, lddq,
+                           nullptr, 0, dev_status, st) == cudaSuccess ? GC_OK : GC_ERR_CUDA;
+    }
     return run_build_sweeps(p, pl, static_cast<char*>(ws), loss_part, row_lse + q0,
                             pos_logit ? pos_logit + q0 : nullptr, dQ, lddq, nullptr, 0, dev_status,
                             static_cast<cudaStream_t>(cuda_stream), false);
@@ -831,12 +874,21 @@ int gc_shard_dp(const void* Q, int64_t ldq, const void* P, int64_t ldp, const in
     profile_begin_call();
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     char* w = static_cast<char*>(ws);
+    const char* p_first = static_cast<const char*>(P) + (size_t)p0 * (size_t)ldp * elem_size(dtype);
+    if (pl.strips) {
+        Problem p = make_problem(Q, ldq, p_first, ldp, pos_idx, B, p_count, d, tau, mask_mode, dtype);
+        p.mask_shift = -p0;
+        p.pos_base = p0;
+        p.n_total = N;
+        KernelTimer t(2, st);
+        return strip_backward(p, ws, row_lse, nullptr, 0, dP, lddp, dev_status, st) == cudaSuccess
+                   ? GC_OK : GC_ERR_CUDA;
+    }
     // positives counted from the slice's first passage; those outside the slice match no row
     int32_t* pos_local = reinterpret_cast<int32_t*>(w + pl.total);
     if (dev_status && launch_pos_check(pos_idx, B, N, mask_mode, dev_status, st) != cudaSuccess)
         return GC_ERR_CUDA;
     if (launch_shift_pos(pos_idx, B, p0, p_count, pos_local, st) != cudaSuccess) return GC_ERR_CUDA;
-    const char* p_first = static_cast<const char*>(P) + (size_t)p0 * (size_t)ldp * elem_size(dtype);
     Problem p = make_problem(Q, ldq, p_first, ldp, pos_local, B, p_count, d, tau, mask_mode, dtype);
     p.mask_shift = -p0;            // local passage j is passage p0 + j of the batch
     return run_sweep(p, pl, w, SWEEP_DP, row_lse, dP, lddp, dev_status, st);

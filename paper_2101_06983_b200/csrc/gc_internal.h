@@ -60,6 +60,8 @@ struct Problem {
     int64_t mask_shift;     // GC_MASK_SELF drops the pair (query i, passage j) with j == i +
                             // mask_shift: 0 for whole matrices, first query row minus first
                             // passage row (in the whole batch) when Q or P is a slice
+    int64_t pos_base, n_total;  // strip plan, P a slice: pos_idx counts the rows of the whole matrix of
+                            // n_total rows (0: N), of which P holds those from pos_base on
 };
 
 // The two tile sweeps share one shape: a stationary row tile X, a streamed row tile Y,
@@ -113,6 +115,7 @@ struct Plan {
     int tc;                 // 1: tcgen05 kernels, 0: SIMT kernels
     int tiles;              // 1: batch of a few tiles on the one-tile tcgen05 kernel
     int tiles_y;            // its passage tiles (slots per row of its forward)
+    int strips;             // 1: three products over strips of query rows (gc_strip.cu)
     int g_fwd, g_dq, g_dp;  // split factors of the streamed range
     size_t off_m, off_l, off_pos, off_red, off_accq, off_accp;
     size_t total;           // workspace bytes (multiple of 256)
@@ -210,6 +213,21 @@ cudaError_t launch_small_tiled_fwd(const Problem& pr, float* part_m, float* part
 cudaError_t launch_small_tiled_bwd(const Problem& pr, const float* row_lse, float* dQ, int64_t lddq,
                                    float* partial_q, float* dP, int64_t lddp, float* partial_p,
                                    int* dev_status, cudaStream_t st);
+
+// gc_strip.cu
+bool strip_applicable(int64_t B, int64_t N, int d, int dtype);
+size_t strip_workspace_bytes(int64_t B, int64_t N, int d, int dtype);
+size_t strip_forward_bytes(int64_t B, int64_t N, int d, int dtype);     // strip_forward's share of it
+int strip_launches(int op, int64_t B, int64_t N, int d, int dtype);
+cudaError_t strip_forward(const Problem& p, void* ws, float* loss, float* row_lse, float* pos_logit,
+                          int* dev_status, cudaStream_t st);
+cudaError_t strip_backward(const Problem& p, void* ws, const float* row_lse, float* dQ, int64_t lddq,
+                           float* dP, int64_t lddp, int* dev_status, cudaStream_t st,
+                           const float* col_neg = nullptr, float grad_scale = 1.f);
+// dP may be NULL
+cudaError_t strip_build(const Problem& p, void* ws, float* loss, float* row_lse, float* pos_logit,
+                        float* dQ, int64_t lddq, float* dP, int64_t lddp, int* dev_status,
+                        cudaStream_t st);
 
 // gc_gemm.cu
 int gemm_groups(int64_t m_rows, int64_t k_len, int d);

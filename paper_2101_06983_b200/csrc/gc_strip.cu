@@ -1,0 +1,1795 @@
+// Strip plan: Step 2 as three products over strips of query rows.
+//
+// The sweeps (gc_quad.cu, gc_tc.cu) form every logit twice, once per gradient, because nothing of
+// size B x N may leave the chip.  A strip of query rows may: the exponentials of `rows` queries
+// against all N passages fit the L2 for ordinary batches, and a bounded workspace for the rest.
+// Per strip:
+//
+//   logit kernel   S = Q P^T on tcgen05, 256 x 256 tiles; the epilogue leaves, per row and group of
+//                  64 columns, the raw maximum m and sum of e = 2^((s - m) log2e / tau) as a slot and
+//                  the e themselves as fp16 (each in [0, 1], its group's largest exactly 1, so the
+//                  error is 2^-12 of a value, whatever the range of the logits)
+//   row kernel     merges a row's slots into row_lse, its share of the loss, and turns the row, in
+//                  place, into the bf16 weights W_ij = p_ij - [j = r_i] (0 at the masked pair)
+//   grad kernel    dQ = W P and dP += W^T Q in one launch; tiles of both products are dealt out in
+//                  equal runs of 64-deep contraction blocks
+//
+// Six B N d multiply-adds for the six that count, against eight in the sweeps.  fp32 inputs take the
+// same route with every value as three bf16 terms (x = t1 + t2 + t3 exactly): six products for S,
+// the logits kept as fp32, weights as two terms, five products per gradient.  gc_loss_fwd runs the
+// logit kernel without its stores; gc_loss_bwd's logit kernel is given row_lse and writes W itself.
+//
+// All matrix work runs in CTA pairs (cta_group::2, M = 256): two producer warps, one issuing warp
+// (the leader's), eight epilogue warps; accumulators are double-buffered in tensor memory, so the
+// epilogue of a tile runs under the next tile's products.  Every wait is bounded.
+#include <cuda_fp16.h>
+#include <stdlib.h>
+#include <string.h>
+
+#include <utility>
+
+#include "tc_common.cuh"
+
+namespace gc {
+
+namespace {
+
+constexpr int ST_THREADS = 32 * (NPROD + 1 + NSOFT);
+constexpr int KB = 64;                               // contraction depth of a ring stage
+constexpr int MAX_ST = 6;
+constexpr uint32_t HALF_CHUNK = 8192;                // 64 rows x 128 bytes
+constexpr float LOG2E = 1.4426950408889634f;
+constexpr float LN2 = 0.6931471805599453f;
+
+enum LogitMode { LOGIT_FWD = 0, LOGIT_STASH = 1, LOGIT_W = 2, LOGIT_W2 = 3 };
+
+struct StripBars {
+    uint64_t full[MAX_ST];
+    uint64_t empty[MAX_ST];
+    uint64_t acc_full[2];
+    uint64_t acc_free[2];        // this CTA's epilogue warps have read the buffer
+    uint64_t acc_free_peer[2];   // leader: the same, forwarded from the second CTA
+};
+
+__device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap* map, int c0, int c1,
+                                                 int c2, uint32_t bar_cluster) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes "
+        "[%0], [%1, {%2, %3, %4}], [%5];"
+        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(bar_cluster)
+        : "memory");
+}
+__device__ __forceinline__ void tma_add_3d(const CUtensorMap* map, uint32_t src, int c0, int c1,
+                                           int c2) {
+    asm volatile(
+        "cp.reduce.async.bulk.tensor.3d.global.shared::cta.add.bulk_group [%0, {%2, %3, %4}], [%1];"
+        ::"l"(reinterpret_cast<uint64_t>(map)), "r"(src), "r"(c0), "r"(c1), "r"(c2)
+        : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+__device__ __forceinline__ void bulk_wait_read0() {
+    asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+}
+__device__ __forceinline__ void bulk_wait_all() {
+    asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+}
+__device__ __forceinline__ void sts_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};"
+                 ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+__device__ __forceinline__ uint32_t pack_h2(float lo, float hi) {
+    uint32_t r;
+    asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+    return r;
+}
+__device__ __forceinline__ uint32_t pack_b2(float lo, float hi) {
+    uint32_t r;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+    return r;
+}
+
+// p - 1 of a positive from its raw logit (roundings spelled out: two kernels form it, same bits).
+__device__ __forceinline__ float positive_weight(float raw, float inv_tau, float lse) {
+    return __fsub_rn(ex2(__fmul_rn(__fsub_rn(__fmul_rn(raw, inv_tau), lse), LOG2E)), 1.f);
+}
+
+// ---- what every matrix kernel of this file shares: setup, teardown, forwarding ---------------------
+struct PairCtx {
+    uint32_t tmem;
+    uint32_t rank;
+    uint32_t smem;           // 1024-byte aligned dynamic shared memory
+    int warp, lane;
+};
+
+__device__ __forceinline__ PairCtx pair_setup(uint8_t* raw, StripBars& bars, uint32_t* tmem_s,
+                                              int* abort_s) {
+    PairCtx c;
+    c.warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
+    c.lane = threadIdx.x & 31;
+    c.rank = cluster_ctarank();
+    c.smem = (smem_u32(raw) + 1023u) & ~1023u;
+    if (threadIdx.x == 0) {
+        *abort_s = 0;
+        for (int s = 0; s < MAX_ST; ++s) {
+            mbar_init(smem_u32(&bars.full[s]), 2);        // the leader's two producer warps
+            mbar_init(smem_u32(&bars.empty[s]), 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(smem_u32(&bars.acc_full[b]), 1);
+            mbar_init(smem_u32(&bars.acc_free[b]), NSOFT);
+            mbar_init(smem_u32(&bars.acc_free_peer[b]), 1);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (c.warp == MMA_WARP) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;"
+                     ::"r"(smem_u32(tmem_s)), "r"((uint32_t)TMEM_COLS) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();
+    tc_fence_after();
+    c.tmem = *tmem_s;
+    return c;
+}
+
+__device__ __forceinline__ void pair_teardown(const PairCtx& c, volatile int* abort_flag,
+                                              int* dev_status) {
+    tc_fence_before();
+    __syncthreads();
+    if (*abort_flag) {
+        // let bulk copies still in flight land before the shared memory is released
+        uint64_t t0 = global_ns();
+        while (global_ns() - t0 < 200000ull) __nanosleep(1000);
+        if (threadIdx.x == 0 && dev_status) atomicOr(dev_status, GC_DEV_WAIT_LIMIT);
+        __syncthreads();
+    }
+    cluster_sync_all();   // the peer's MMAs, loads and arrivals no longer touch this CTA
+    if (c.warp == MMA_WARP) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;"
+                     ::"r"(c.tmem), "r"((uint32_t)TMEM_COLS) : "memory");
+    }
+}
+
+// The second CTA's idle issuing warp passes "buffer read" on to the leader: one remote arrival per
+// use instead of eight (a remote arrival stalls the arriving warp for more than a thousand cycles).
+__device__ __forceinline__ void forward_acc_free(StripBars& bars, int uses, volatile int* abort_flag) {
+    for (int n = 0; n < uses; ++n) {
+        const int b = n & 1;
+        if (!mbar_wait(smem_u32(&bars.acc_free[b]), (uint32_t)(n >> 1) & 1u, abort_flag)) return;
+        if (elect_one()) mbar_arrive_cluster(mapa_u32(smem_u32(&bars.acc_free_peer[b]), 0));
+    }
+}
+__device__ __forceinline__ bool wait_acc_free(StripBars& bars, int n, volatile int* abort_flag) {
+    const int b = n & 1;
+    const uint32_t par = ((uint32_t)(n >> 1) & 1u) ^ 1u;
+    return mbar_wait(smem_u32(&bars.acc_free[b]), par, abort_flag) &&
+           mbar_wait(smem_u32(&bars.acc_free_peer[b]), par, abort_flag);
+}
+
+// ---------------------------------------------------------------------------------------------------
+// Logit kernel
+// ---------------------------------------------------------------------------------------------------
+struct LogitParams {
+    int rows, N;                 // rows of the strip, passages
+    int kblocks;                 // ceil(d / 64)
+    int tiles_m, tiles_n;
+    float c1;                    // log2(e) / tau
+    float inv_tau;
+    int mask_on, mask_shift;     // masked column of strip row i: i + mask_shift
+    const int32_t* pos_idx;      // of the strip's rows
+    int pos_base, pos_n;         // counted from passage pos_base of the pos_n a positive may point at
+    const float* row_lse;        // LOGIT_W, LOGIT_W2
+    const float* col_neg;        // LOGIT_W2: per passage, log2 of its multiplicity as a positive minus
+                                 // its own logsumexp over the queries (log2 units; -inf: none)
+    float2* slots;               // [rows][slot_pitch] (raw maximum, sum)
+    int slot_pitch;
+    float* pos_ws;               // positive's raw logit
+    float* res;                  // LOGIT_W: what the positive's weight lost to bf16
+    int* zero;                   // counters of the kernels that follow, cleared here
+    int zero_count;
+    int* dev_status;
+};
+
+// Tile order: groups of 8 row tiles, row tiles fastest, so that the tiles in flight share operands.
+__device__ __forceinline__ void logit_tile(int t, int tiles_m, int tiles_n, int* m, int* n) {
+    const int per = 8 * tiles_n;
+    const int g = t / per, r = t - g * per;
+    const int h = min(8, tiles_m - 8 * g);
+    *n = r / h;
+    *m = 8 * g + (r - *n * h);
+}
+
+// BN: passages per tile (a CTA loads BN / 2 of them).  What bounds it: tcgen05 at 256 x 256 tiles (a
+// stage of 64 is 512 cycles of products for 32 KB per CTA); the epilogue's two special-function
+// operations per 32 lanes and clock stay below that from d = 256 on.
+template <int MODE, int BN>
+__global__ void __launch_bounds__(ST_THREADS, 1)
+strip_logit_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapP,
+                   const __grid_constant__ CUtensorMap mapW, const LogitParams p) {
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(8) StripBars bars;
+    __shared__ uint32_t tmem_s;
+    __shared__ int abort_s;
+    volatile int* abort_flag = &abort_s;
+    const PairCtx c = pair_setup(smem_raw, bars, &tmem_s, &abort_s);
+    constexpr uint32_t A_BYTES = CHUNK_BYTES, B_BYTES = BN / 2 * 128, STAGE = A_BYTES + B_BYTES;
+    constexpr int NST = BN == 256 ? 5 : 6;
+    const int total = p.tiles_m * p.tiles_n;
+    const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
+    dep_release();
+    dep_wait();
+
+    if (c.warp < NPROD) {
+        // warp 0: query rows, warp 1: passage rows
+        const bool is_a = c.warp == 0;
+        int stage = 0;
+        uint32_t phase = 0;
+        bool ok = true;
+        for (int t = pair; t < total && ok; t += pairs) {
+            int m, n;
+            logit_tile(t, p.tiles_m, p.tiles_n, &m, &n);
+            const int row = is_a ? m * 256 + (int)c.rank * 128 : n * BN + (int)c.rank * (BN / 2);
+            for (int kb = 0; kb < p.kblocks; ++kb) {
+                ok = mbar_wait(smem_u32(&bars.empty[stage]), phase ^ 1u, abort_flag);
+                if (!ok) break;
+                const uint32_t full = smem_u32(&bars.full[stage]);
+                const uint32_t full_leader = mapa_u32(full, 0);
+                const uint32_t dst = c.smem + stage * STAGE + (is_a ? 0u : A_BYTES);
+                if (elect_one()) {
+                    if (c.rank == 0) mbar_expect_tx(full, 2 * (is_a ? A_BYTES : B_BYTES));
+                    tma_load_3d_pair(dst, is_a ? &mapQ : &mapP, kb * KB, row, 0, full_leader);
+                }
+                if (++stage == NST) { stage = 0; phase ^= 1u; }
+            }
+        }
+    } else if (c.warp == MMA_WARP) {
+        if (c.rank == 0) {
+            const uint32_t idesc = instr_desc(BN, false, 256, false);
+            int stage = 0, use = 0;
+            uint32_t phase = 0;
+            bool ok = true;
+            for (int t = pair; t < total && ok; t += pairs, ++use) {
+                ok = wait_acc_free(bars, use, abort_flag);
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t acc = c.tmem + (use & 1) * 256;
+                for (int kb = 0; kb < p.kblocks; ++kb) {
+                    ok = mbar_wait(smem_u32(&bars.full[stage]), phase, abort_flag);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t a = desc_lo(c.smem + stage * STAGE, 0);
+                    const uint32_t b = desc_lo(c.smem + stage * STAGE + A_BYTES, 0);
+                    if (elect_one()) {
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            if (k == 0 && kb == 0) mma_ss<false, true>(acc, a, b, idesc);
+                            else                   mma_ss<true, true>(acc, a + 2 * k, b + 2 * k, idesc);
+                        }
+                        tc_commit_pair(smem_u32(&bars.empty[stage]));
+                        if (kb == p.kblocks - 1) tc_commit_pair(smem_u32(&bars.acc_full[use & 1]));
+                    }
+                    if (++stage == NST) { stage = 0; phase ^= 1u; }
+                }
+            }
+        } else {
+            int uses = 0;
+            for (int t = pair; t < total; t += pairs) ++uses;
+            forward_acc_free(bars, uses, abort_flag);
+        }
+    } else {
+        const int ew = c.warp - (NPROD + 1);
+        const int q = c.warp & 3, half = ew >> 2, lane = c.lane;
+        constexpr int HC = BN / 2;                       // columns of this warp
+        if (p.zero && blockIdx.x < 8) {
+            for (int e = blockIdx.x * 256 + (ew * 32 + lane); e < p.zero_count; e += 8 * 256)
+                p.zero[e] = 0;
+        }
+        const uint32_t stage_buf = c.smem + NST * STAGE + (uint32_t)ew * (uint32_t)(HC * 64);
+        const uint64_t c1_2 = pack2(p.c1, p.c1);
+        int use = 0;
+        for (int t = pair; t < total; t += pairs, ++use) {
+            int m, n;
+            logit_tile(t, p.tiles_m, p.tiles_n, &m, &n);
+            const int row0 = m * 256 + (int)c.rank * 128 + 32 * q;
+            const int i = row0 + lane;
+            const int col0 = n * BN + half * HC;
+            // the row's special columns
+            int pos = -1, masked = -1;
+            float neg_lse = -INFINITY, lse_i = 0.f;
+            if (i < p.rows) {
+                pos = p.pos_idx[i];
+                int flag = pos < 0 || pos >= p.pos_n ? GC_DEV_POS_RANGE : 0;
+                pos -= p.pos_base;
+                if (p.mask_on) {
+                    masked = i + p.mask_shift;
+                    if (pos == masked && !flag) flag = GC_DEV_POS_MASKED;
+                }
+                if (flag || pos < 0 || pos >= p.N) pos = -1;
+                if (MODE == LOGIT_W || MODE == LOGIT_W2) {
+                    lse_i = p.row_lse[i];
+                    neg_lse = -(lse_i * LOG2E);
+                    if (n == 0 && half == 0) {
+                        if (pos < 0) p.res[i] = 0.f;     // no usable positive: nothing is lost to rounding
+                        if (flag && p.dev_status) atomicOr(p.dev_status, flag);
+                    }
+                }
+            }
+            if (!mbar_wait(smem_u32(&bars.acc_full[use & 1]), (uint32_t)(use >> 1) & 1u, abort_flag))
+                break;
+            tc_fence_after();
+            const uint32_t src = c.tmem + (use & 1) * 256 + ((uint32_t)(32 * q) << 16) + half * HC;
+            float run_m = -INFINITY, run_l = 0.f;
+#pragma unroll 1
+            for (int g = 0; g < HC / 64; ++g) {
+                const int jg = col0 + 64 * g;
+                float s[64];
+                {
+                    uint32_t v0[32], v1[32];
+                    tmem_ld32(src + 64 * g, v0);
+                    tmem_ld32(src + 64 * g + 32, v1);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) {
+                        s[e] = __uint_as_float(v0[e]);
+                        s[32 + e] = __uint_as_float(v1[e]);
+                    }
+                }
+                if (g == HC / 64 - 1) {                  // the buffer is free for the tile after next
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&bars.acc_free[use & 1]));
+                }
+                const int dp = pos - jg, dm = masked - jg;
+                const bool special = (unsigned)dp < 64u || (unsigned)dm < 64u;
+                const bool any_special = __any_sync(0xffffffffu, special) || jg + 64 > p.N;
+                float pos_raw = 0.f;
+                if (MODE != LOGIT_W2) {
+                    if (any_special) {
+#pragma unroll
+                        for (int e = 0; e < 64; ++e) {
+                            if (e == dp) {
+                                if (MODE == LOGIT_W) pos_raw = s[e];
+                                else p.pos_ws[i] = s[e];
+                            }
+                            if (e == dm || jg + e >= p.N) s[e] = -INFINITY;
+                        }
+                    }
+                    float mx[4] = {s[0], s[1], s[2], s[3]};
+#pragma unroll
+                    for (int e = 4; e < 64; ++e) mx[e & 3] = fmaxf(mx[e & 3], s[e]);
+                    const float gm = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+                    const float ref = gm == -INFINITY ? 0.f : gm;
+                    const float off = -ref * p.c1;
+                    const uint64_t off2 = pack2(off, off);
+                    uint64_t sum2 = pack2(0.f, 0.f), sum2b = sum2;
+#pragma unroll
+                    for (int e = 0; e < 64; e += 4) {
+                        float a, b, x, y;
+                        unpack2(fma2(pack2(s[e], s[e + 1]), c1_2, off2), a, b);
+                        unpack2(fma2(pack2(s[e + 2], s[e + 3]), c1_2, off2), x, y);
+                        s[e] = ex2(a); s[e + 1] = ex2(b); s[e + 2] = ex2(x); s[e + 3] = ex2(y);
+                        sum2 = add2(sum2, pack2(s[e], s[e + 1]));
+                        sum2b = add2(sum2b, pack2(s[e + 2], s[e + 3]));
+                    }
+                    float sa, sb;
+                    unpack2(add2(sum2, sum2b), sa, sb);
+                    const float sum = sa + sb;
+                    if (MODE == LOGIT_STASH) {
+                        if (i < p.rows) p.slots[(int64_t)i * p.slot_pitch + (jg >> 6)] = make_float2(gm, sum);
+                    } else if (MODE == LOGIT_W) {
+                        // what the row kernel makes of the stored exponentials, bit for bit
+                        const float f = gm > -INFINITY ? ex2(fmaf(gm, p.c1, neg_lse)) : 0.f;
+#pragma unroll
+                        for (int e = 0; e < 64; e += 2) {
+                            const uint32_t h = pack_h2(s[e], s[e + 1]);
+                            const float2 v = __half22float2(*reinterpret_cast<const __half2*>(&h));
+                            s[e] = v.x * f;
+                            s[e + 1] = v.y * f;
+                        }
+                        if ((unsigned)dp < 64u) {
+                            const float pw = positive_weight(pos_raw, p.inv_tau, lse_i);
+                            p.res[i] = pw - __bfloat162float(__float2bfloat16_rn(pw));
+#pragma unroll
+                            for (int e = 0; e < 64; ++e) if (e == dp) s[e] = pw;
+                        }
+                    } else {
+                        const float mn = fmaxf(run_m, gm), r = mn == -INFINITY ? 0.f : mn;
+                        run_l = run_l * ex2((run_m - r) * p.c1) + sum * ex2((gm - r) * p.c1);
+                        run_m = mn;
+                    }
+                } else {
+                    const float4* cn = reinterpret_cast<const float4*>(p.col_neg + jg);
+#pragma unroll
+                    for (int e = 0; e < 64; e += 4) {
+                        const float4 n4 = jg + e < p.N ? __ldg(cn + (e >> 2)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        const float nn[4] = {n4.x, n4.y, n4.z, n4.w};
+#pragma unroll
+                        for (int x = 0; x < 4; ++x)
+                            s[e + x] = ex2(fmaf(s[e + x], p.c1, neg_lse)) + ex2(fmaf(s[e + x], p.c1, nn[x]));
+                    }
+                    if (any_special) {
+#pragma unroll
+                        for (int e = 0; e < 64; ++e) {
+                            if (e == dp) {
+                                s[e] -= 2.f;
+                                p.res[i] = s[e] - __bfloat162float(__float2bfloat16_rn(s[e]));
+                            }
+                        }
+                    }
+                }
+                if (MODE != LOGIT_FWD) {
+                    // 32 rows x 64 columns of 16 bits, 128-byte swizzle, one bulk tensor store
+                    if (lane == 0) {
+                        if (HC == 128) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+                        else           bulk_wait_read0();
+                    }
+                    __syncwarp();
+                    const uint32_t buf = stage_buf + (uint32_t)g * 4096u + lane * 128;
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        uint32_t w[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+                            w[e] = MODE == LOGIT_STASH ? pack_h2(s[8 * j + 2 * e], s[8 * j + 2 * e + 1])
+                                                       : pack_b2(s[8 * j + 2 * e], s[8 * j + 2 * e + 1]);
+                        sts_v4(buf + (uint32_t)((j ^ (lane & 7)) << 4), w[0], w[1], w[2], w[3]);
+                    }
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) {                     // (an empty group when nothing is stored)
+                        if (row0 < p.rows && jg < p.N)
+                            tma_store_3d(&mapW, stage_buf + (uint32_t)g * 4096u, jg, row0, 0);
+                        else
+                            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                    }
+                }
+            }
+            if (MODE == LOGIT_FWD && i < p.rows)
+                p.slots[(int64_t)i * p.slot_pitch + 2 * n + half] = make_float2(run_m, run_l);
+        }
+        if (MODE != LOGIT_FWD) {
+            if (lane == 0) bulk_wait_all();
+            __syncwarp();
+        }
+    }
+    pair_teardown(c, abort_flag, p.dev_status);
+}
+
+// fp32 inputs as three bf16 terms each ([3][rows][d] planes): 256 x 128 tiles, six products per step.
+// The tensor core's additions truncate, so the leading product alternates between two accumulators
+// and the five small ones have a third; the epilogue adds the three in fp32 and writes the raw logits.
+// Bound by the products: 24 per stage of 72 KB per CTA.
+constexpr int F_BN = 128;
+constexpr uint32_t F_STAGE = 3 * CHUNK_BYTES + 3 * HALF_CHUNK;
+constexpr int F_NST = 2;
+
+__global__ void __launch_bounds__(ST_THREADS, 1)
+strip_logit_f32_kernel(const __grid_constant__ CUtensorMap mapQ,
+                       const __grid_constant__ CUtensorMap mapP,
+                       const __grid_constant__ CUtensorMap mapS, const LogitParams p) {
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(8) StripBars bars;
+    __shared__ uint32_t tmem_s;
+    __shared__ int abort_s;
+    volatile int* abort_flag = &abort_s;
+    const PairCtx c = pair_setup(smem_raw, bars, &tmem_s, &abort_s);
+    const int total = p.tiles_m * p.tiles_n;
+    const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
+    dep_release();
+    dep_wait();
+
+    if (c.warp < NPROD) {
+        const bool is_a = c.warp == 0;
+        const uint32_t bytes = is_a ? CHUNK_BYTES : HALF_CHUNK;
+        int stage = 0;
+        uint32_t phase = 0;
+        bool ok = true;
+        for (int t = pair; t < total && ok; t += pairs) {
+            int m, n;
+            logit_tile(t, p.tiles_m, p.tiles_n, &m, &n);
+            const int row = is_a ? m * 256 + (int)c.rank * 128 : n * F_BN + (int)c.rank * (F_BN / 2);
+            for (int kb = 0; kb < p.kblocks; ++kb) {
+                ok = mbar_wait(smem_u32(&bars.empty[stage]), phase ^ 1u, abort_flag);
+                if (!ok) break;
+                const uint32_t full = smem_u32(&bars.full[stage]);
+                const uint32_t full_leader = mapa_u32(full, 0);
+                const uint32_t dst = c.smem + stage * F_STAGE + (is_a ? 0u : 3 * CHUNK_BYTES);
+                if (elect_one()) {
+                    if (c.rank == 0) mbar_expect_tx(full, 6 * bytes);
+                    for (int term = 0; term < 3; ++term)
+                        tma_load_3d_pair(dst + term * bytes, is_a ? &mapQ : &mapP, kb * KB, row, term,
+                                         full_leader);
+                }
+                if (++stage == F_NST) { stage = 0; phase ^= 1u; }
+            }
+        }
+    } else if (c.warp == MMA_WARP) {
+        if (c.rank == 0) {
+            const uint32_t idesc = instr_desc(F_BN, false, 256, false);
+            int stage = 0, use = 0;
+            uint32_t phase = 0;
+            bool ok = true;
+            for (int t = pair; t < total && ok; t += pairs, ++use) {
+                // one set of accumulators: every use waits for the one before it
+                ok = mbar_wait(smem_u32(&bars.acc_free[0]), ((uint32_t)use & 1u) ^ 1u, abort_flag) &&
+                     mbar_wait(smem_u32(&bars.acc_free_peer[0]), ((uint32_t)use & 1u) ^ 1u, abort_flag);
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t rest = c.tmem + 256;
+                for (int kb = 0; kb < p.kblocks; ++kb) {
+                    ok = mbar_wait(smem_u32(&bars.full[stage]), phase, abort_flag);
+                    if (!ok) break;
+                    tc_fence_after();
+                    constexpr uint32_t TA = CHUNK_BYTES >> 4, TB = HALF_CHUNK >> 4;
+                    const uint32_t a0 = desc_lo(c.smem + stage * F_STAGE, 0);
+                    const uint32_t b0 = desc_lo(c.smem + stage * F_STAGE + 3 * CHUNK_BYTES, 0);
+                    if (elect_one()) {
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const uint32_t a = a0 + 2 * k, b = b0 + 2 * k;
+                            const uint32_t lead = c.tmem + 128 * (k & 1);
+                            if (kb == 0 && k < 2) mma_ss<false, true>(lead, a, b, idesc);
+                            else                  mma_ss<true, true>(lead, a, b, idesc);
+                            if (kb == 0 && k == 0) mma_ss<false, true>(rest, a, b + TB, idesc);
+                            else                   mma_ss<true, true>(rest, a, b + TB, idesc);
+                            mma_ss<true, true>(rest, a + TA, b, idesc);
+                            mma_ss<true, true>(rest, a + TA, b + TB, idesc);
+                            mma_ss<true, true>(rest, a, b + 2 * TB, idesc);
+                            mma_ss<true, true>(rest, a + 2 * TA, b, idesc);
+                        }
+                        tc_commit_pair(smem_u32(&bars.empty[stage]));
+                        if (kb == p.kblocks - 1) tc_commit_pair(smem_u32(&bars.acc_full[0]));
+                    }
+                    if (++stage == F_NST) { stage = 0; phase ^= 1u; }
+                }
+            }
+        } else {
+            int n = 0;
+            for (int t = pair; t < total; t += pairs, ++n) {
+                if (!mbar_wait(smem_u32(&bars.acc_free[0]), (uint32_t)n & 1u, abort_flag)) break;
+                if (elect_one()) mbar_arrive_cluster(mapa_u32(smem_u32(&bars.acc_free_peer[0]), 0));
+            }
+        }
+    } else {
+        const int ew = c.warp - (NPROD + 1);
+        const int q = c.warp & 3, half = ew >> 2, lane = c.lane;
+        if (p.zero && blockIdx.x < 8) {
+            for (int e = blockIdx.x * 256 + (ew * 32 + lane); e < p.zero_count; e += 8 * 256)
+                p.zero[e] = 0;
+        }
+        const uint32_t slot = c.smem + F_NST * F_STAGE + (uint32_t)ew * 8192u;
+        int use = 0;
+        for (int t = pair; t < total; t += pairs, ++use) {
+            int m, n;
+            logit_tile(t, p.tiles_m, p.tiles_n, &m, &n);
+            const int row0 = m * 256 + (int)c.rank * 128 + 32 * q;
+            const int col0 = n * F_BN + 64 * half;
+            if (!mbar_wait(smem_u32(&bars.acc_full[0]), (uint32_t)use & 1u, abort_flag)) break;
+            tc_fence_after();
+            const uint32_t src = c.tmem + ((uint32_t)(32 * q) << 16) + 64 * half;
+            uint32_t s[2][32];
+#pragma unroll
+            for (int g = 0; g < 2; ++g) {
+                uint32_t v[32], u[32];
+                tmem_ld32(src + 32 * g, s[g]);
+                tmem_ld32(src + 128 + 32 * g, v);
+                tmem_ld32(src + 256 + 32 * g, u);
+                tmem_ld_wait();
+#pragma unroll
+                for (int e = 0; e < 32; ++e)
+                    s[g][e] = __float_as_uint((__uint_as_float(s[g][e]) + __uint_as_float(v[e])) +
+                                              __uint_as_float(u[e]));
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) {
+                mbar_arrive(smem_u32(&bars.acc_free[0]));
+                bulk_wait_read0();
+            }
+            __syncwarp();
+#pragma unroll
+            for (int g = 0; g < 2; ++g) {
+                stage_block(slot + g * 4096, s[g], 1.f, lane);
+                __syncwarp();
+                if (lane == 0 && row0 < p.rows && col0 + 32 * g < p.N)
+                    tma_store_3d(&mapS, slot + g * 4096, col0 + 32 * g, row0, 0);
+            }
+        }
+        if (lane == 0) bulk_wait_all();
+        __syncwarp();
+    }
+    pair_teardown(c, abort_flag, p.dev_status);
+}
+
+// x = t1 + t2 + t3, each term the upper 16 bits of what the earlier ones left: planes [3][rows][ldt].
+__device__ __forceinline__ void split3(float x, uint32_t& t1, uint32_t& t2, uint32_t& t3) {
+    t1 = __float_as_uint(x) & 0xffff0000u;
+    const float r = x - __uint_as_float(t1);
+    t2 = __float_as_uint(r) & 0xffff0000u;
+    t3 = __float_as_uint(r - __uint_as_float(t2));
+}
+__global__ void __launch_bounds__(256)
+split_terms_kernel(const float* __restrict__ Q, int64_t ldq, int64_t B, uint2* __restrict__ tq,
+                   const float* __restrict__ P, int64_t ldp, int64_t N, uint2* __restrict__ tp,
+                   int d4) {
+    dep_release();
+    dep_wait();
+    const int64_t nq = B * d4, total = nq + N * d4;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
+         e += (int64_t)gridDim.x * blockDim.x) {
+        const bool is_q = e < nq;
+        const int64_t f = is_q ? e : e - nq;
+        const int64_t r = f / d4;
+        const int c = 4 * (int)(f - r * d4);
+        const float4 x = *reinterpret_cast<const float4*>(is_q ? Q + r * ldq + c : P + r * ldp + c);
+        const int64_t plane = is_q ? nq : N * d4;
+        uint2* dst = (is_q ? tq : tp) + f;
+        uint32_t a[4], b[4], t[4];
+        split3(x.x, a[0], b[0], t[0]); split3(x.y, a[1], b[1], t[1]);
+        split3(x.z, a[2], b[2], t[2]); split3(x.w, a[3], b[3], t[3]);
+        dst[0] = make_uint2(__byte_perm(a[0], a[1], 0x7632), __byte_perm(a[2], a[3], 0x7632));
+        dst[plane] = make_uint2(__byte_perm(b[0], b[1], 0x7632), __byte_perm(b[2], b[3], 0x7632));
+        dst[2 * plane] = make_uint2(__byte_perm(t[0], t[1], 0x7632), __byte_perm(t[2], t[3], 0x7632));
+    }
+}
+
+// ---------------------------------------------------------------------------------------------------
+// Row kernel
+// ---------------------------------------------------------------------------------------------------
+struct RowParams {
+    int rows, N;
+    int row0;                     // first row of the strip within the call
+    float c1, inv_tau;
+    int mask_on, mask_shift;      // masked column of strip row i: i + mask_shift
+    const int32_t* pos_idx;       // of the strip's rows
+    int pos_base, pos_n;          // as in LogitParams
+    const float2* slots;
+    int slot_pitch, nslots;
+    const float* pos_ws;
+    float* res;
+    float* row_lse;               // of the strip's rows: written, or read when lse_given
+    float* pos_logit;             // may be NULL
+    float* loss;
+    float* red;                   // with weights: one loss term per row of the call, summed by the
+                                  // gradient kernel; otherwise one share per block of the call
+    int* ticket;
+    int block0, blocks_total;     // this launch's first block and the blocks of all strips
+    float inv_mean;
+    int64_t ldw;                  // elements
+    int* dev_status;
+    // fp32 inputs
+    const float* S;
+    int64_t lds;
+    int lse_given, want_w;
+};
+
+// Shares of the loss are added in a fixed order: a block's rows in row order, then the blocks in a fixed
+// pattern by the block that draws the last ticket.
+__device__ __forceinline__ void loss_share(const RowParams& p, float mine) {
+    __shared__ int last_s;
+    __shared__ float warp_s[8];
+    if (threadIdx.x == 0) {
+        p.red[p.block0 + blockIdx.x] = mine;
+        __threadfence();
+        last_s = atomicAdd(p.ticket, 1) == p.blocks_total - 1;
+    }
+    __syncthreads();
+    if (!last_s) return;
+    __threadfence();
+    float v = 0.f;
+    for (int b = threadIdx.x; b < p.blocks_total; b += 256) v += __ldcg(p.red + b);
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) warp_s[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float s = 0.f;
+        for (int w = 0; w < 8; ++w) s += warp_s[w];
+        *p.loss = s * p.inv_mean;
+    }
+}
+
+// The positive of strip row i as a column of the strip (-1: none there), and what is wrong with it.
+__device__ __forceinline__ int row_pos(const RowParams& p, int i, int* flags) {
+    const int raw = p.pos_idx[i], pos = raw - p.pos_base;
+    *flags = raw < 0 || raw >= p.pos_n ? GC_DEV_POS_RANGE
+             : p.mask_on && pos == i + p.mask_shift ? GC_DEV_POS_MASKED : 0;
+    return *flags || pos < 0 || pos >= p.N ? -1 : pos;
+}
+
+// bf16 inputs, ROW_BATCH rows per block.  A warp per row merges the row's slots; then all threads turn
+// the rows' fp16 exponentials into bf16 weights in place (WRITE), the first of them requested before
+// the merge so that its chain of dependent loads and reductions is paid once per block.  Bound by the
+// L2: 4 bytes moved per pair.
+constexpr int ROW_BATCH = 4;
+template <bool WRITE>
+__global__ void __launch_bounds__(256)
+strip_row_kernel(uint4* __restrict__ W, const RowParams p) {
+    struct RowHead { float lse2, pw; int wpos; };
+    __shared__ RowHead heads[ROW_BATCH];
+    __shared__ float terms[ROW_BATCH];
+    dep_release();
+    dep_wait();
+    const int i0 = blockIdx.x * ROW_BATCH;
+    const int rows = min(ROW_BATCH, p.rows - i0);
+    const int n8 = (p.N + 7) / 8, pitch8 = (int)(p.ldw / 8);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    W += (int64_t)i0 * pitch8;
+    const float2* sl0 = p.slots + (int64_t)i0 * p.slot_pitch;
+    // pieces of 8 columns, row after row; each thread takes every 256th
+    constexpr int PIECES = 4;
+    int r = 0, k = threadIdx.x;
+    auto wrap = [&]() { while (k >= n8) { k -= n8; ++r; } };
+    wrap();
+    uint4 raw[PIECES];
+    float gm[PIECES];
+    int at[PIECES], of[PIECES];
+    auto fetch = [&]() {
+#pragma unroll
+        for (int x = 0; x < PIECES; ++x) {
+            of[x] = r;
+            at[x] = k;
+            if (r < rows) {
+                raw[x] = __ldcg(W + (int64_t)r * pitch8 + k);
+                gm[x] = __ldcg(&sl0[(int64_t)r * p.slot_pitch + (k >> 3)].x);
+            }
+            k += 256;
+            wrap();
+        }
+    };
+    if (WRITE) fetch();
+    if (warp < rows) {
+        const int i = i0 + warp;
+        const float2* sl = sl0 + (int64_t)warp * p.slot_pitch;
+        int flags;
+        const int pos = row_pos(p, i, &flags);
+        const float pos_raw = __ldcg(p.pos_ws + i);
+        constexpr int KEEP = 4;                     // slots held in registers (N <= 8192: all)
+        float2 kept[KEEP];
+#pragma unroll
+        for (int x = 0; x < KEEP; ++x)
+            kept[x] = lane + 32 * x < p.nslots ? __ldcg(sl + lane + 32 * x) : make_float2(-INFINITY, 0.f);
+        float m = -INFINITY, l = 0.f;
+#pragma unroll
+        for (int x = 0; x < KEEP; ++x) m = fmaxf(m, kept[x].x);
+        for (int s = lane + 32 * KEEP; s < p.nslots; s += 32) m = fmaxf(m, __ldcg(&sl[s].x));
+        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        const float ref = m == -INFINITY ? 0.f : m;
+#pragma unroll
+        for (int x = 0; x < KEEP; ++x) l = fmaf(kept[x].y, ex2((kept[x].x - ref) * p.c1), l);
+        for (int s = lane + 32 * KEEP; s < p.nslots; s += 32) {
+            const float2 v = __ldcg(sl + s);
+            l = fmaf(v.y, ex2((v.x - ref) * p.c1), l);
+        }
+        for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+        if (lane == 0) {
+            const float lse = m * p.inv_tau + log2f(l) * LN2;
+            const float pl = pos < 0 ? 0.f : pos_raw * p.inv_tau;
+            RowHead h;
+            h.lse2 = lse * LOG2E;
+            h.pw = positive_weight(pos_raw, p.inv_tau, lse);
+            h.wpos = pos;
+            heads[warp] = h;
+            terms[warp] = lse - pl;
+            p.row_lse[i] = lse;
+            if (p.pos_logit) p.pos_logit[i] = pl;
+            if (flags && p.dev_status) atomicOr(p.dev_status, flags);
+            if (WRITE) {
+                p.red[p.row0 + i] = lse - pl;
+                p.res[i] = pos < 0 ? 0.f : h.pw - __bfloat162float(__float2bfloat16_rn(h.pw));
+            }
+        }
+    }
+    __syncthreads();
+    if (!WRITE) {
+        float share = 0.f;
+        if (threadIdx.x == 0)
+            for (int w = 0; w < rows; ++w) share += terms[w];
+        loss_share(p, share);
+        return;
+    }
+    if constexpr (WRITE) {
+        while (of[0] < rows) {
+#pragma unroll
+            for (int x = 0; x < PIECES; ++x) {
+                if (of[x] >= rows) break;
+                const RowHead h = heads[of[x]];
+                // (a group with no allowed column holds zeros)
+                const float f = gm[x] > -INFINITY ? ex2(fmaf(gm[x], p.c1, -h.lse2)) : 0.f;
+                const __half2* e2 = reinterpret_cast<const __half2*>(&raw[x]);
+                float w[8];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float2 v = __half22float2(e2[e]);
+                    w[2 * e] = v.x * f;
+                    w[2 * e + 1] = v.y * f;
+                }
+                if ((h.wpos >> 3) == at[x]) {
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) if (e == (h.wpos & 7)) w[e] = h.pw;
+                }
+                W[(int64_t)of[x] * pitch8 + at[x]] =
+                    make_uint4(pack_b2(w[0], w[1]), pack_b2(w[2], w[3]), pack_b2(w[4], w[5]), pack_b2(w[6], w[7]));
+            }
+            fetch();
+        }
+    }
+}
+
+// fp32 inputs: one block per row of raw logits.  Maximum, sum and weights are three passes over the
+// row (from the first level cache after the first); the weights leave as two bf16 terms, planes
+// [2][rows][ldw].  With lse_given (gc_loss_bwd) only the last pass runs.
+__global__ void __launch_bounds__(256)
+strip_row_f32_kernel(uint2* __restrict__ W, const RowParams p) {
+    __shared__ float sm[8];
+    dep_release();
+    dep_wait();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int n4 = (p.N + 3) / 4;
+    float share = 0.f;
+    for (int i = blockIdx.x; i < p.rows; i += (int)gridDim.x) {
+        const float4* row = reinterpret_cast<const float4*>(p.S + (int64_t)i * p.lds);
+        const int masked = p.mask_on ? i + p.mask_shift : -1;
+        int flags;
+        const int pos = row_pos(p, i, &flags);
+        if (threadIdx.x == 0 && flags && p.dev_status) atomicOr(p.dev_status, flags);
+        auto load = [&](int k, float (&s)[4]) {
+            const float4 v = row[k];
+            s[0] = v.x; s[1] = v.y; s[2] = v.z; s[3] = v.w;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) if (4 * k + e == masked || 4 * k + e >= p.N) s[e] = -INFINITY;
+        };
+        auto block_max = [&](float v) {
+            for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+            if (lane == 0) sm[warp] = v;
+            __syncthreads();
+            v = sm[0];
+            for (int w = 1; w < 8; ++w) v = fmaxf(v, sm[w]);
+            __syncthreads();
+            return v;
+        };
+        auto block_sum = [&](float v) {
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (lane == 0) sm[warp] = v;
+            __syncthreads();
+            v = sm[0];
+            for (int w = 1; w < 8; ++w) v += sm[w];
+            __syncthreads();
+            return v;
+        };
+        float lse;
+        const float raw_pos = pos < 0 ? 0.f : p.S[(int64_t)i * p.lds + pos];
+        if (p.lse_given) {
+            lse = p.row_lse[i];
+        } else {
+            float m = -INFINITY;
+#pragma unroll 4
+            for (int k = threadIdx.x; k < n4; k += 256) {
+                float s[4];
+                load(k, s);
+                m = fmaxf(m, fmaxf(fmaxf(s[0], s[1]), fmaxf(s[2], s[3])));
+            }
+            m = block_max(m);
+            const float ref = m == -INFINITY ? 0.f : m;
+            float l = 0.f;
+#pragma unroll 4
+            for (int k = threadIdx.x; k < n4; k += 256) {
+                float s[4];
+                load(k, s);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) l += ex2((s[e] - ref) * p.c1);
+            }
+            l = block_sum(l);
+            // the row's logsumexp and its positive logit come out of the same product with 1/tau: their
+            // difference is exactly 0 when the positive is the only column
+            lse = m * p.inv_tau + log2f(l) * LN2;
+            const float pl = raw_pos * p.inv_tau;
+            if (threadIdx.x == 0) {
+                p.row_lse[i] = lse;
+                if (p.pos_logit) p.pos_logit[i] = pl;
+            }
+            share += lse - pl;
+            if (p.want_w && threadIdx.x == 0) p.red[p.row0 + i] = lse - pl;
+        }
+        if (p.want_w) {
+            const float lse2 = lse * LOG2E;
+            uint2* w1 = W + (int64_t)i * (p.ldw / 4);
+            uint2* w2 = w1 + (int64_t)p.rows * (p.ldw / 4);
+            const int wpos = pos;
+#pragma unroll 4
+            for (int k = threadIdx.x; k < n4; k += 256) {
+                float s[4];
+                load(k, s);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    s[e] = ex2(fmaf(s[e], p.c1, -lse2));
+                    if (4 * k + e == wpos) s[e] -= 1.f;
+                }
+                const uint32_t h0 = pack_b2(s[0], s[1]), h1 = pack_b2(s[2], s[3]);
+                w1[k] = make_uint2(h0, h1);
+                w2[k] = make_uint2(pack_b2(s[0] - __uint_as_float(h0 << 16), s[1] - __uint_as_float(h0 & 0xffff0000u)),
+                                   pack_b2(s[2] - __uint_as_float(h1 << 16), s[3] - __uint_as_float(h1 & 0xffff0000u)));
+            }
+        }
+    }
+    if (!p.lse_given && !p.want_w) loss_share(p, share);
+}
+
+// ---------------------------------------------------------------------------------------------------
+// Gradient kernel
+// ---------------------------------------------------------------------------------------------------
+struct GradSide {
+    int tiles;                    // output tiles: 256 rows x `width` columns, columns fastest
+    int tiles_n;
+    int kblocks;                  // contraction blocks of 64
+    int rows, cols;               // of the output
+    int add;                      // 1: add to the output (strips after the first)
+};
+
+struct GradParams {
+    GradSide side[2];             // 0: dQ = W P, 1: dP = W^T Q
+    // How the tiles are dealt out to the CTA pairs.  whole >= 0: as whole tiles, dQ's to the first
+    // `whole` pairs in turn, dP's to the others.  whole < 0: tiles_n neighbouring pairs form a group
+    // (one pair per column tile, in step, so that they share the rows of W they read); the row tiles
+    // of dQ, then of dP, are laid end to end and cut into `groups` equal runs of contraction blocks.
+    int whole;
+    int pairs;
+    int units;                    // contraction blocks of all row tiles
+    int groups;
+    float scale;                  // 1 / (B tau)
+    const float* res;             // dQ: what the positives' weights lost to bf16 (NULL: nothing)
+    const int32_t* pos_idx;
+    const __nv_bfloat16* P;       // passages, for the res terms
+    int64_t ldp;
+    const float* terms;           // loss terms of all rows of the call (NULL: no loss to form here)
+    int n_terms;
+    float inv_mean;
+    float* loss;
+    float* part;                  // [pairs][2 slots][2 CTAs][8 warps][32 x hw] partial tiles
+    int* count;                   // [tiles of both sides][2 CTAs][8 warps]
+    int* dev_status;
+};
+
+// A run of contraction blocks of one output tile.
+struct Segment {
+    int side, tile_m, tile_n, kb, n;
+    int t0;                       // whole < 0: first unit of the row tile
+};
+
+__device__ __forceinline__ int unit_start(const GradParams& p, int g) {
+    return (int)((int64_t)p.units * g / p.groups);
+}
+// Iterates over a pair's segments.
+struct SegmentWalk {
+    int u, end, group, tile_n;    // whole >= 0: u counts tiles
+    __device__ __forceinline__ SegmentWalk(const GradParams& p, int pair) {
+        if (p.whole >= 0) {
+            const bool q = pair < p.whole;
+            u = q ? pair : pair - p.whole;
+            end = p.side[q ? 0 : 1].tiles;
+            group = q ? p.whole : p.pairs - p.whole;        // stride
+            tile_n = q ? 0 : 1;                             // side
+        } else {
+            group = pair / p.side[0].tiles_n;
+            tile_n = pair - group * p.side[0].tiles_n;
+            u = unit_start(p, group);
+            end = unit_start(p, group + 1);
+        }
+    }
+    __device__ __forceinline__ bool next(const GradParams& p, Segment& s) {
+        if (u >= end) return false;
+        if (p.whole >= 0) {
+            s.side = tile_n;
+            s.tile_m = u / p.side[0].tiles_n;
+            s.tile_n = u - s.tile_m * p.side[0].tiles_n;
+            s.kb = 0;
+            s.n = s.side ? p.side[1].kblocks : p.side[0].kblocks;
+            s.t0 = 0;
+            u += group;
+        } else {
+            const int first_p = p.side[0].tiles / p.side[0].tiles_n * p.side[0].kblocks;
+            s.side = u >= first_p;
+            const int k = s.side ? p.side[1].kblocks : p.side[0].kblocks;
+            const int local = u - (s.side ? first_p : 0);
+            s.tile_m = local / k;
+            s.tile_n = tile_n;
+            s.kb = local - s.tile_m * k;
+            s.n = min(k - s.kb, end - u);
+            s.t0 = u - s.kb;
+            u += s.n;
+        }
+        return true;
+    }
+};
+
+// A tile cut between groups is summed from partial tiles in contraction order by whichever of its
+// warps finishes last (the order of the sum, not of the arrivals, decides the bits), so no pair ever
+// waits for another.
+//
+// F32: weights as two terms, rows of the other side as three; products w1 (t1 + t2 + t3) +
+// w2 (t1 + t2), 256 x 128 tiles.  The tensor core's additions truncate: every 128 of the contraction
+// the accumulator is read out and added in fp32 registers, the other buffer taking over meanwhile.
+template <bool F32, int WIDTH>
+__global__ void __launch_bounds__(ST_THREADS, 1)
+strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_constant__ CUtensorMap mapWm,
+                  const __grid_constant__ CUtensorMap mapP, const __grid_constant__ CUtensorMap mapQ,
+                  const __grid_constant__ CUtensorMap mapDQ, const __grid_constant__ CUtensorMap mapDP,
+                  const __grid_constant__ GradParams p) {
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(8) StripBars bars;
+    __shared__ uint32_t tmem_s;
+    __shared__ int abort_s;
+    volatile int* abort_flag = &abort_s;
+    const PairCtx c = pair_setup(smem_raw, bars, &tmem_s, &abort_s);
+    constexpr int TA = F32 ? 2 : 1, TB = F32 ? 3 : 1;     // operand terms
+    constexpr uint32_t B_TERM = WIDTH / 2 * 128;          // 64 contraction rows x WIDTH / 2 columns
+    constexpr uint32_t A_BYTES = TA * CHUNK_BYTES, STAGE = A_BYTES + TB * B_TERM;
+    constexpr int NST = F32 ? 3 : WIDTH == 128 ? 6 : 5;
+    constexpr int CHUNK_KB = 2;                           // F32: blocks per accumulator read-out
+    constexpr int HW = WIDTH / 2;                         // columns of an epilogue warp
+    const int pair = blockIdx.x >> 1;
+    dep_release();
+    dep_wait();
+    // columns of a tile that exist, in whole 128s: a last tile of at most 128 columns runs at half width
+    auto tile_width = [&](const GradSide& sd, int n0) { return WIDTH == 256 && sd.cols - n0 <= 128 ? 128 : WIDTH; };
+
+    if (c.warp < NPROD) {
+        const bool is_a = c.warp == 0;
+        int stage = 0;
+        uint32_t phase = 0;
+        bool ok = true;
+        SegmentWalk walk(p, pair);
+        Segment sg;
+        while (ok && walk.next(p, sg)) {
+            const GradSide& sd = p.side[sg.side];
+            const int m0 = sg.tile_m * 256 + (int)c.rank * 128;
+            const int n0t = sg.tile_n * WIDTH;
+            const int bw = tile_width(sd, n0t) / 2;       // columns this CTA loads
+            const int n0 = n0t + (int)c.rank * bw;
+            const uint32_t bytes = is_a ? A_BYTES : (uint32_t)TB * bw * 128u;
+            for (int k = 0; k < sg.n; ++k) {
+                ok = mbar_wait(smem_u32(&bars.empty[stage]), phase ^ 1u, abort_flag);
+                if (!ok) break;
+                const uint32_t full = smem_u32(&bars.full[stage]);
+                const uint32_t full_leader = mapa_u32(full, 0);
+                const uint32_t dst = c.smem + stage * STAGE + (is_a ? 0u : A_BYTES);
+                const int k0 = (sg.kb + k) * KB;
+                if (elect_one()) {
+                    if (c.rank == 0) mbar_expect_tx(full, 2 * bytes);
+                    if (is_a) {
+#pragma unroll
+                        for (int term = 0; term < TA; ++term) {
+                            const uint32_t d0 = dst + term * CHUNK_BYTES;
+                            if (sg.side == 0) {           // rows of W: K-major
+                                tma_load_3d_pair(d0, &mapWk, k0, m0, term, full_leader);
+                            } else {                      // columns of W: MN-major, two atoms
+                                tma_load_3d_pair(d0, &mapWm, m0, k0, term, full_leader);
+                                tma_load_3d_pair(d0 + HALF_CHUNK, &mapWm, m0 + 64, k0, term, full_leader);
+                            }
+                        }
+                    } else {
+                        const CUtensorMap* map = sg.side == 0 ? &mapP : &mapQ;
+#pragma unroll
+                        for (int term = 0; term < TB; ++term) {
+                            tma_load_3d_pair(dst + term * B_TERM, map, n0, k0, term, full_leader);
+                            if (WIDTH == 256 && bw == 128)
+                                tma_load_3d_pair(dst + HALF_CHUNK, map, n0 + 64, k0, term, full_leader);
+                        }
+                    }
+                }
+                if (++stage == NST) { stage = 0; phase ^= 1u; }
+            }
+        }
+    } else if (c.warp == MMA_WARP) {
+        if (c.rank == 0) {
+            int stage = 0, use = 0;
+            uint32_t phase = 0;
+            bool ok = true;
+            SegmentWalk walk(p, pair);
+            Segment sg;
+            while (ok && walk.next(p, sg)) {
+                const GradSide& sd = p.side[sg.side];
+                const int width = tile_width(sd, sg.tile_n * WIDTH);
+                const uint32_t idesc = instr_desc(width, true, 256, sg.side == 1);
+                const uint32_t a_lbo = sg.side ? HALF_CHUNK : 0, a_step = sg.side ? 128 : 2;
+                uint32_t acc = 0;
+                for (int k = 0; k < sg.n; ++k) {
+                    const bool fresh = F32 ? k % CHUNK_KB == 0 : k == 0;
+                    if (fresh) {
+                        ok = wait_acc_free(bars, use, abort_flag);
+                        if (!ok) break;
+                        tc_fence_after();
+                        acc = c.tmem + (use & 1) * 256;
+                    }
+                    ok = mbar_wait(smem_u32(&bars.full[stage]), phase, abort_flag);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t a = desc_lo(c.smem + stage * STAGE, a_lbo);
+                    const uint32_t b = desc_lo(c.smem + stage * STAGE + A_BYTES, HALF_CHUNK);
+                    const bool last = F32 ? (k % CHUNK_KB == CHUNK_KB - 1 || k == sg.n - 1) : k == sg.n - 1;
+                    if (elect_one()) {
+                        if (fresh) mma_ss<false, true>(acc, a, b, idesc);
+                        else       mma_ss<true, true>(acc, a, b, idesc);
+#pragma unroll
+                        for (int kk = 0; kk < 4; ++kk) {
+                            const uint32_t ak = a + kk * a_step, bk = b + kk * 128;
+                            if (kk) mma_ss<true, true>(acc, ak, bk, idesc);
+                            if (F32) {
+                                constexpr uint32_t A2 = CHUNK_BYTES >> 4, B1 = B_TERM >> 4;
+                                mma_ss<true, true>(acc, ak, bk + B1, idesc);
+                                mma_ss<true, true>(acc, ak, bk + 2 * B1, idesc);
+                                mma_ss<true, true>(acc, ak + A2, bk, idesc);
+                                mma_ss<true, true>(acc, ak + A2, bk + B1, idesc);
+                            }
+                        }
+                        tc_commit_pair(smem_u32(&bars.empty[stage]));
+                        if (last) tc_commit_pair(smem_u32(&bars.acc_full[use & 1]));
+                    }
+                    if (last) ++use;
+                    if (++stage == NST) { stage = 0; phase ^= 1u; }
+                }
+            }
+        } else {
+            int uses = 0;
+            SegmentWalk walk(p, pair);
+            Segment sg;
+            while (walk.next(p, sg)) uses += F32 ? (sg.n + CHUNK_KB - 1) / CHUNK_KB : 1;
+            forward_acc_free(bars, uses, abort_flag);
+        }
+    } else {
+        const int ew = c.warp - (NPROD + 1);
+        const int q = c.warp & 3, half = ew >> 2, lane = c.lane;
+                constexpr int SB = F32 ? 1 : 2;                   // staging buffers of 4 KB
+        const uint32_t stage_buf = c.smem + NST * STAGE + (uint32_t)ew * (SB * 4096u);
+        const int cw = (int)c.rank * 8 + ew;              // this warp among the 16 of a tile
+        constexpr size_t PART_FLOATS = 32 * HW;
+        int use = 0, nstore = 0;
+        bool ok = true;
+        if (p.terms && blockIdx.x == 0) {
+            // the loss: a fixed order of sums, under the first products
+            __shared__ float sums[NSOFT];
+            float v = 0.f;
+#pragma unroll 4
+            for (int e = ew * 32 + lane; e < p.n_terms; e += 32 * NSOFT) v += __ldcg(p.terms + e);
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (lane == 0) sums[ew] = v;
+            asm volatile("bar.sync 1, %0;" ::"n"(32 * NSOFT) : "memory");
+            if (ew == 0 && lane == 0) {
+                v = 0.f;
+                for (int w = 0; w < NSOFT; ++w) v += sums[w];
+                *p.loss = v * p.inv_mean;
+            }
+        }
+        SegmentWalk walk(p, pair);
+        Segment sg;
+        while (ok && walk.next(p, sg)) {
+            const GradSide& sd = p.side[sg.side];
+            const int row0 = sg.tile_m * 256 + (int)c.rank * 128 + 32 * q;
+            const int n0 = sg.tile_n * WIDTH;
+            const int hw = tile_width(sd, n0) / 2;        // columns of this warp
+            const int col0 = n0 + half * hw;
+            const bool whole = sg.n == sd.kblocks;
+            const uint32_t lanes = (uint32_t)(32 * q) << 16;
+            float r_i = 0.f;
+            const __nv_bfloat16* p_row = nullptr;
+            if (!F32 && sg.side == 0 && p.res && row0 + lane < sd.rows) {
+                r_i = p.res[row0 + lane];
+                if (r_i != 0.f) p_row = p.P + (int64_t)p.pos_idx[row0 + lane] * p.ldp;
+            }
+            float acc[F32 ? HW : 1];
+            if (F32) {
+                const int chunks = (sg.n + CHUNK_KB - 1) / CHUNK_KB;
+                for (int ch = 0; ch < chunks && ok; ++ch, ++use) {
+                    ok = mbar_wait(smem_u32(&bars.acc_full[use & 1]), (uint32_t)(use >> 1) & 1u, abort_flag);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t src = c.tmem + (use & 1) * 256 + lanes + half * HW;
+#pragma unroll
+                    for (int g = 0; g < HW / 32; ++g) {
+                        uint32_t v[32];
+                        tmem_ld32(src + 32 * g, v);
+                        tmem_ld_wait();
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) {
+                            const float x = __uint_as_float(v[e]);
+                            acc[32 * g + e] = ch == 0 ? x : acc[32 * g + e] + x;
+                        }
+                    }
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&bars.acc_free[use & 1]));
+                }
+                if (!ok) break;
+            } else {
+                ok = mbar_wait(smem_u32(&bars.acc_full[use & 1]), (uint32_t)(use >> 1) & 1u, abort_flag);
+                if (!ok) break;
+                tc_fence_after();
+            }
+            const uint32_t src = c.tmem + (use & 1) * 256 + lanes + half * hw;
+            // one block of 32 columns to the output: scale, the positives' remainder, staging, store
+            auto finish = [&](uint32_t (&v)[32], int cb) {
+                const int col = col0 + 32 * cb;
+                if (!F32 && p_row) {
+                    const uint4* pr = reinterpret_cast<const uint4*>(p_row + col);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        if (col + 8 * j >= sd.cols) break;
+                        const uint4 x = __ldg(pr + j);
+                        const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            v[8 * j + 2 * e] = __float_as_uint(fmaf(
+                                r_i, __uint_as_float(w[e] << 16), __uint_as_float(v[8 * j + 2 * e])));
+                            v[8 * j + 2 * e + 1] = __float_as_uint(fmaf(
+                                r_i, __uint_as_float(w[e] & 0xffff0000u), __uint_as_float(v[8 * j + 2 * e + 1])));
+                        }
+                    }
+                }
+                if (lane == 0) asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(SB - 1) : "memory");
+                __syncwarp();
+                const uint32_t buf = stage_buf + (uint32_t)(nstore & (SB - 1)) * 4096u;
+                stage_block(buf, v, p.scale, lane);
+                __syncwarp();
+                if (lane == 0) {                         // (an empty group when nothing is stored)
+                    const CUtensorMap* map = sg.side == 0 ? &mapDQ : &mapDP;
+                    if (row0 >= sd.rows || col >= sd.cols)
+                        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                    else if (sd.add) tma_add_3d(map, buf, col, row0, 0);
+                    else             tma_store_3d(map, buf, col, row0, 0);
+                }
+                ++nstore;
+            };
+            if (whole) {
+#pragma unroll
+                for (int cb = 0; cb < HW / 32; ++cb) {
+                    if (32 * cb >= hw) break;
+                    uint32_t v[32];
+                    if (F32) {
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(acc[F32 ? 32 * cb + e : 0]);
+                    } else {
+                        tmem_ld32(src + 32 * cb, v);
+                        tmem_ld_wait();
+                        if (32 * (cb + 1) >= hw) {
+                            tc_fence_before();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(smem_u32(&bars.acc_free[use & 1]));
+                        }
+                    }
+                    finish(v, cb);
+                }
+            } else {
+                // this group's share of the tile: slot 0 when it starts inside the tile, else 1
+                const int group = walk.group, tn = sd.tiles_n;
+                auto part_of = [&](int g, int slot) {
+                    return reinterpret_cast<float4*>(
+                        p.part + (((size_t)(g * tn + sg.tile_n) * 2 + slot) * 16 + cw) * PART_FLOATS);
+                };
+                // first and last group with a share of this tile
+                const int t1 = sg.t0 + sd.kblocks;
+                int gf = group, gl = group;
+                while (unit_start(p, gf) > sg.t0) --gf;
+                while (unit_start(p, gl + 1) < t1) ++gl;
+                const int tile_id = (sg.side ? p.side[0].tiles : 0) + sg.tile_m * tn + sg.tile_n;
+                int* counter = p.count + tile_id * 16 + cw;
+                auto own_block = [&](int cb, uint32_t (&v)[32]) {
+                    if (F32) {
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(acc[F32 ? 32 * cb + e : 0]);
+                    } else {
+                        tmem_ld32(src + 32 * cb, v);
+                        tmem_ld_wait();
+                    }
+                };
+                auto release_acc = [&]() {
+                    if (F32) return;
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&bars.acc_free[use & 1]));
+                };
+                // Where all other shares are in memory already (as a rule: a group meets the front part
+                // of its first tile long before the neighbour meets the back part of its last), this
+                // share goes into the sum straight from tensor memory.
+                int published = 0;
+                if (lane == 0)
+                    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(published) : "l"(counter) : "memory");
+                published = __shfl_sync(0xffffffffu, published, 0);
+                const bool direct = published == gl - gf;
+                if (!direct) {
+                    float4* mine = part_of(group, sg.kb == 0 ? 1 : 0);
+#pragma unroll
+                    for (int cb = 0; cb < HW / 32; ++cb) {
+                        if (32 * cb >= hw) break;
+                        uint32_t v[32];
+                        own_block(cb, v);
+#pragma unroll
+                        for (int j = 0; j < 8; ++j)
+                            __stcg(mine + (cb * 8 + j) * 32 + lane,
+                                   make_float4(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]),
+                                               __uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3])));
+                    }
+                    release_acc();
+                    __threadfence();
+                    __syncwarp();
+                    if (lane == 0) published = atomicAdd(counter, 1);
+                    published = __shfl_sync(0xffffffffu, published, 0);
+                }
+                if (published == gl - gf) {
+                    __threadfence();
+#pragma unroll
+                    for (int cb = 0; cb < HW / 32; ++cb) {
+                        if (32 * cb >= hw) break;
+                        uint32_t v[32];
+                        if (direct) own_block(cb, v);
+                        float s[32];
+                        for (int g = gf; g <= gl; ++g) {
+                            if (direct && g == group) {
+#pragma unroll
+                                for (int e = 0; e < 32; ++e)
+                                    s[e] = g == gf ? __uint_as_float(v[e]) : s[e] + __uint_as_float(v[e]);
+                                continue;
+                            }
+                            const float4* o = part_of(g, g == gf ? 1 : 0);
+                            float4 x[8];
+#pragma unroll
+                            for (int j = 0; j < 8; ++j) x[j] = __ldcg(o + (cb * 8 + j) * 32 + lane);
+#pragma unroll
+                            for (int j = 0; j < 8; ++j) {
+                                if (g == gf) {
+                                    s[4 * j] = x[j].x; s[4 * j + 1] = x[j].y;
+                                    s[4 * j + 2] = x[j].z; s[4 * j + 3] = x[j].w;
+                                } else {
+                                    s[4 * j] += x[j].x; s[4 * j + 1] += x[j].y;
+                                    s[4 * j + 2] += x[j].z; s[4 * j + 3] += x[j].w;
+                                }
+                            }
+                        }
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(s[e]);
+                        finish(v, cb);
+                    }
+                    if (direct) release_acc();
+                }
+            }
+            if (!F32) ++use;
+        }
+        if (lane == 0) bulk_wait_all();
+        __syncwarp();
+    }
+    pair_teardown(c, abort_flag, p.dev_status);
+}
+
+// ---------------------------------------------------------------------------------------------------
+// Host side
+// ---------------------------------------------------------------------------------------------------
+// A row-major matrix of 16-bit or fp32 values as [planes][rows][cols]; boxes of 128 bytes x box_rows,
+// 128-byte swizzle, out-of-range elements read as zero and are not written.
+bool map3(CUtensorMap* map, bool f32, const void* base, int64_t rows, int64_t cols, int64_t pitch,
+          int64_t planes, int64_t plane_pitch, int box_rows) {
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return false;
+    const cuuint64_t es = f32 ? 4 : 2;
+    cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)planes};
+    cuuint64_t strides[2] = {(cuuint64_t)pitch * es, (cuuint64_t)plane_pitch * es};
+    cuuint32_t box[3] = {(cuuint32_t)(128 / es), (cuuint32_t)box_rows, 1};
+    cuuint32_t estr[3] = {1, 1, 1};
+    return fn(map, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3,
+              const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
+int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
+int pairs_of_device() { return sm_count() / 2; }
+
+constexpr size_t SMEM_L256 = 1024 + 5 * (CHUNK_BYTES + 16384) + NSOFT * 8192;
+constexpr size_t SMEM_L128 = 1024 + 6 * (CHUNK_BYTES + 8192) + NSOFT * 4096;
+constexpr size_t SMEM_LF32 = 1024 + F_NST * F_STAGE + NSOFT * 8192;
+constexpr size_t SMEM_G = 1024 + 5 * (CHUNK_BYTES + 16384) + NSOFT * 8192;
+constexpr size_t SMEM_G128 = 1024 + 6 * (CHUNK_BYTES + 8192) + NSOFT * 8192;
+constexpr size_t SMEM_GF32 = 1024 + 3 * (2 * CHUNK_BYTES + 3 * 8192) + NSOFT * 4096;
+static_assert(SMEM_L256 <= SMEM_LIMIT - 1024 && SMEM_LF32 <= SMEM_LIMIT - 1024 &&
+              SMEM_GF32 <= SMEM_LIMIT - 1024, "shared memory budget");
+
+// Kernel launch with a cluster of `cluster` CTAs (1: none).  Every kernel of this file may start while
+// the kernel before it in the stream runs; it waits for that kernel before it touches memory.
+template <typename... KArgs, typename... Args>
+cudaError_t launch(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, int cluster,
+                   cudaStream_t st, Args&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    int n = 0;
+    if (cluster > 1) {
+        attr[n].id = cudaLaunchAttributeClusterDimension;
+        attr[n].val.clusterDim.x = (unsigned)cluster;
+        attr[n].val.clusterDim.y = 1;
+        attr[n++].val.clusterDim.z = 1;
+    }
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = n;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+
+// The shared-memory limit belongs to the (kernel, device) pair; set once for all kernels here.
+cudaError_t configure_kernels() {
+    static bool done[64] = {false};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    if (done[dev]) return cudaSuccess;
+    const struct { const void* f; size_t bytes; } all[] = {
+        {(const void*)strip_logit_kernel<LOGIT_FWD, 256>, SMEM_L256},
+        {(const void*)strip_logit_kernel<LOGIT_FWD, 128>, SMEM_L128},
+        {(const void*)strip_logit_kernel<LOGIT_STASH, 256>, SMEM_L256},
+        {(const void*)strip_logit_kernel<LOGIT_STASH, 128>, SMEM_L128},
+        {(const void*)strip_logit_kernel<LOGIT_W, 256>, SMEM_L256},
+        {(const void*)strip_logit_kernel<LOGIT_W, 128>, SMEM_L128},
+        {(const void*)strip_logit_kernel<LOGIT_W2, 256>, SMEM_L256},
+        {(const void*)strip_logit_kernel<LOGIT_W2, 128>, SMEM_L128},
+        {(const void*)strip_logit_f32_kernel, SMEM_LF32},
+        {(const void*)strip_grad_kernel<false, 256>, SMEM_G},
+        {(const void*)strip_grad_kernel<false, 128>, SMEM_G128},
+        {(const void*)strip_grad_kernel<true, 128>, SMEM_GF32},
+    };
+    for (const auto& k : all) {
+        const cudaError_t e = cudaFuncSetAttribute(k.f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)k.bytes);
+        if (e != cudaSuccess) return e;
+    }
+    done[dev] = true;
+    return cudaSuccess;
+}
+
+// How the gradient tiles of a strip are dealt out (see GradParams): the cheapest by a count of cycles.
+struct GradDeal { int width, whole, pairs; };
+GradDeal deal_grads(int64_t rows, int64_t N, int d, bool f32, bool dq, bool dp) {
+    const int pairs = pairs_of_device();
+    GradDeal best{};
+    double best_cost = 0;
+    for (int width = f32 ? 128 : 256; width >= 128; width -= 128) {
+        const int tn = (int)ceil_div(d, width);
+        const double unit = f32 ? 1320 : width == 256 ? 560 : 380;      // cycles per contraction block
+        const int64_t kq = ceil_div(N, KB), kp = ceil_div(rows, KB);
+        const int64_t tq = dq ? ceil_div(rows, 256) * tn : 0, tp = dp ? ceil_div(N, 256) * tn : 0;
+        auto offer = [&](double cost, int whole, int used) {
+            if (best.pairs == 0 || cost < best_cost) { best = {width, whole, used}; best_cost = cost; }
+        };
+        // whole tiles, every split of the pairs between the two products
+        if (tq + tp <= pairs) {
+            offer((double)(tq && kq > kp ? kq : tp ? (tq && kq > kp ? kq : kp) : kq) * unit, tq ? (int)tq : 0, (int)(tq + tp));
+        } else {
+            for (int w = tq ? 1 : 0; w <= (tp ? pairs - 1 : pairs); ++w) {
+                if (!tq && w) break;
+                const double a = tq ? (double)(ceil_div(tq, w) * kq) : 0, b = tp ? (double)(ceil_div(tp, pairs - w) * kp) : 0;
+                offer((a > b ? a : b) * unit, w, pairs);
+            }
+        }
+        // equal runs of contraction blocks, at least four to a pair
+        const int64_t units = (tq * kq + tp * kp) / tn;
+        int64_t groups = pairs / tn;
+        if (groups > units / 4) groups = units / 4;
+        if (groups < 1) groups = 1;
+        if (tn <= pairs) offer((double)units / groups * unit + (width == 256 ? 20000 : 9000), -1, (int)(groups * tn));
+    }
+    return best;
+}
+
+struct StripLayout {
+    int64_t rows;                 // of a strip (the last may be shorter)
+    int strips;
+    int64_t ldw;
+    int slot_pitch;
+    size_t zero, slots, pos, res, red, w, part, s, tq, tp, total;
+};
+
+StripLayout strip_layout(int64_t B, int64_t N, int d, int dtype, bool fwd_only = false) {
+    StripLayout l{};
+    const bool f32 = dtype == GC_F32;
+    // Few strips: each costs a read and a write of dP and the fill and drain of three kernels.  Whether
+    // a strip's weights stay in the L2 matters less (8192 x 16384 x 768: 586 us in one strip of 268 MB,
+    // 666 in four of 67 MB; 16384 x 32768: 2.41-2.51 ms against 3.33).  bf16: 512 MB of weights, or 1 GB
+    // where that means fewer than 4096 queries; fp32 holds 8 bytes a pair and does four times the
+    // arithmetic: 64 M pairs.
+    const int64_t pairs = f32 ? 64 : ceil_div(N, 1024) > 64 ? 512 : 256;
+    int64_t r = (pairs << 20) / N / 256 * 256;
+    if (pairs == 512 && r > 4096) r = 4096;
+    if (r < 256) r = 256;
+    const int64_t n = ceil_div(B, r);
+    r = ceil_div(ceil_div(B, n), 256) * 256;
+    l.strips = (int)ceil_div(B, r);
+    l.rows = B < r ? B : r;
+    l.ldw = ceil_div(N, 64) * 64;
+    l.slot_pitch = (int)(ceil_div(N, 256) * 4);
+    const int64_t tiles = ceil_div(l.rows, 256) * ceil_div(d, 128) + ceil_div(N, 256) * ceil_div(d, 128);
+    size_t off = 0;
+    const size_t counters = fwd_only ? 0 : (size_t)tiles * 16;
+    l.zero = off;  off += up256(sizeof(int) * (64 + counters));
+    l.pos = off;   off += up256(sizeof(float) * (size_t)l.rows);
+    l.red = off;   off += up256(sizeof(float) * (size_t)(B + 8 * sm_count()));
+    if (!f32) {
+        const int64_t pitch = fwd_only ? 2 * ceil_div(N, 128) : l.slot_pitch;
+        l.slots = off;  off += up256(sizeof(float2) * (size_t)l.rows * (size_t)pitch);
+    } else {
+        const size_t dp = (size_t)((d + 7) / 8 * 8);
+        l.s = off;   off += up256(4 * (size_t)l.rows * (size_t)l.ldw);
+        l.tq = off;  off += up256(6 * (size_t)B * dp);
+        l.tp = off;  off += up256(6 * (size_t)N * dp);
+    }
+    if (!fwd_only) {
+        l.res = off;   off += up256(sizeof(float) * (size_t)l.rows);
+        l.w = off;     off += up256((f32 ? 4 : 2) * (size_t)l.rows * (size_t)l.ldw);
+        l.part = off;  off += (size_t)pairs_of_device() * 2 * 16 * 32 * (f32 ? 64 : 128) * 4;
+    }
+    l.total = off;
+    return l;
+}
+
+struct StripRun {
+    const Problem& p;
+    StripLayout l;
+    char* ws;
+    cudaStream_t st;
+    int* dev_status;
+    bool f32, shared;
+    const float* col_neg = nullptr;
+    float grad_scale = 1.f;
+
+    StripRun(const Problem& pr, void* w, int* status, cudaStream_t s, bool fwd_only = false)
+        : p(pr), l(strip_layout(pr.B, pr.N, pr.d, pr.dtype, fwd_only)), ws(static_cast<char*>(w)), st(s),
+          dev_status(status), f32(pr.dtype == GC_F32),
+          shared(pr.Q == pr.P && pr.ldq == pr.ldp && pr.B == pr.N) {}
+
+    template <typename T> T* at(size_t off) { return reinterpret_cast<T*>(ws + off); }
+    int64_t rows_of(int s) const { return s == l.strips - 1 ? p.B - (int64_t)s * l.rows : l.rows; }
+    float c1() const { return LOG2E / p.tau; }
+    int shift(int s) const { return (int)(p.mask_shift + (int64_t)s * l.rows); }
+    void* terms_p() { return ws + (shared ? l.tq : l.tp); }
+
+    // planes of 16-bit rows: the inputs themselves, or the terms of fp32 inputs
+    bool rows_map(CUtensorMap* m, bool q, int64_t first, int64_t count, int box) {
+        if (!f32) {
+            const char* base = static_cast<const char*>(q ? p.Q : p.P);
+            const int64_t ld = q ? p.ldq : p.ldp;
+            return map3(m, false, base + first * ld * 2, count, p.d, ld, 1, count * ld, box);
+        }
+        const int64_t all = q ? p.B : p.N;
+        const char* base = static_cast<const char*>(q ? (void*)(ws + l.tq) : terms_p());
+        return map3(m, false, base + first * p.d * 2, count, p.d, p.d, 3, all * p.d, box);
+    }
+
+    cudaError_t split() {
+        const int64_t items = (p.B + (shared ? 0 : p.N)) * (p.d / 4);
+        int64_t blocks = ceil_div(items, 256);
+        if (blocks > 8 * sm_count()) blocks = 8 * sm_count();
+        return launch(split_terms_kernel, (unsigned)blocks, 256, 0, 1, st,
+                      static_cast<const float*>(p.Q), p.ldq, p.B, at<uint2>(l.tq),
+                      static_cast<const float*>(p.P), p.ldp, shared ? (int64_t)0 : p.N, at<uint2>(l.tp),
+                      p.d / 4);
+    }
+
+    cudaError_t logits(int s, int mode, const float* row_lse, bool zero_ticket) {
+        const int64_t row0 = (int64_t)s * l.rows, rows = rows_of(s);
+        const int pairs = pairs_of_device();
+        const int tiles_m = (int)ceil_div(rows, 256);
+        // narrower tiles while 256-wide ones would leave half of the pairs without one
+        const bool narrow = f32 || 2 * tiles_m * ceil_div(p.N, 256) <= pairs;
+        const int bn = narrow ? 128 : 256;
+        LogitParams lp{};
+        lp.rows = (int)rows; lp.N = (int)p.N;
+        lp.kblocks = (int)ceil_div(p.d, KB);
+        lp.tiles_m = tiles_m;
+        lp.tiles_n = (int)ceil_div(p.N, bn);
+        lp.c1 = c1(); lp.inv_tau = 1.f / p.tau;
+        lp.mask_on = p.mask_mode == GC_MASK_SELF; lp.mask_shift = shift(s);
+        lp.pos_idx = p.pos_idx + row0;
+        lp.pos_base = (int)p.pos_base; lp.pos_n = (int)(p.n_total > 0 ? p.n_total : p.N);
+        lp.col_neg = col_neg;
+        lp.row_lse = row_lse ? row_lse + row0 : nullptr;
+        lp.slots = at<float2>(l.slots);
+        lp.slot_pitch = mode == LOGIT_FWD ? 2 * lp.tiles_n : l.slot_pitch;
+        lp.pos_ws = at<float>(l.pos);
+        lp.res = at<float>(l.res);
+        const int skip = zero_ticket ? 0 : 64;
+        lp.zero = at<int>(l.zero) + skip;
+        lp.zero_count = (int)((l.pos - l.zero) / sizeof(int)) - skip;
+        lp.dev_status = dev_status;
+        CUtensorMap mq, mp, mw;
+        if (!rows_map(&mq, true, row0, rows, 128) || !rows_map(&mp, false, 0, p.N, bn / 2)) return cudaErrorInvalidValue;
+        if (!(f32 ? map3(&mw, true, ws + l.s, rows, p.N, l.ldw, 1, rows * l.ldw, 32)
+                  : map3(&mw, false, ws + l.w, rows, p.N, l.ldw, 1, rows * l.ldw, 32)))
+            return cudaErrorInvalidValue;
+        const int total = lp.tiles_m * lp.tiles_n;
+        const unsigned grid = 2u * (unsigned)(total < pairs ? total : pairs);
+        if (f32) return launch(strip_logit_f32_kernel, grid, ST_THREADS, SMEM_LF32, 2, st, mq, mp, mw, lp);
+        auto go = [&](auto k256, auto k128) {
+            return bn == 256 ? launch(k256, grid, ST_THREADS, SMEM_L256, 2, st, mq, mp, mw, lp)
+                             : launch(k128, grid, ST_THREADS, SMEM_L128, 2, st, mq, mp, mw, lp);
+        };
+        if (mode == LOGIT_FWD) return go(strip_logit_kernel<LOGIT_FWD, 256>, strip_logit_kernel<LOGIT_FWD, 128>);
+        if (mode == LOGIT_STASH) return go(strip_logit_kernel<LOGIT_STASH, 256>, strip_logit_kernel<LOGIT_STASH, 128>);
+        if (mode == LOGIT_W2) return go(strip_logit_kernel<LOGIT_W2, 256>, strip_logit_kernel<LOGIT_W2, 128>);
+        return go(strip_logit_kernel<LOGIT_W, 256>, strip_logit_kernel<LOGIT_W, 128>);
+    }
+
+    // rows per block of the row kernel: a row of few passages takes a warp's worth of threads
+    int row_blocks(int s) const {
+        if (!f32) return (int)ceil_div(rows_of(s), ROW_BATCH);
+        const int64_t n = rows_of(s), most = 8 * (int64_t)sm_count();
+        return (int)(n < most ? n : most);
+    }
+
+    cudaError_t rows_kernel(int s, bool write, bool lse_given, float* row_lse, float* pos_logit,
+                            float* loss) {
+        const int64_t row0 = (int64_t)s * l.rows, rows = rows_of(s);
+        RowParams rp{};
+        rp.rows = (int)rows; rp.N = (int)p.N; rp.row0 = (int)row0;
+        rp.c1 = c1(); rp.inv_tau = 1.f / p.tau;
+        rp.mask_on = p.mask_mode == GC_MASK_SELF; rp.mask_shift = shift(s);
+        rp.pos_idx = p.pos_idx + row0;
+        rp.pos_base = (int)p.pos_base; rp.pos_n = (int)(p.n_total > 0 ? p.n_total : p.N);
+        rp.slots = at<float2>(l.slots);
+        if (write) {
+            rp.slot_pitch = l.slot_pitch;
+            rp.nslots = (int)ceil_div(p.N, 64);
+        } else {
+            const int tiles_m = (int)ceil_div(rows, 256);
+            const int bn = 2 * tiles_m * ceil_div(p.N, 256) <= pairs_of_device() ? 128 : 256;
+            rp.nslots = rp.slot_pitch = (int)(2 * ceil_div(p.N, bn));
+        }
+        rp.pos_ws = at<float>(l.pos);
+        rp.res = at<float>(l.res);
+        rp.row_lse = row_lse + row0;
+        rp.pos_logit = pos_logit ? pos_logit + row0 : nullptr;
+        rp.loss = loss;
+        rp.red = at<float>(l.red);
+        rp.ticket = at<int>(l.zero);
+        rp.block0 = 0;
+        for (int k = 0; k < s; ++k) rp.block0 += row_blocks(k);
+        rp.blocks_total = 0;
+        for (int k = 0; k < l.strips; ++k) rp.blocks_total += row_blocks(k);
+        rp.inv_mean = 1.f / (float)(p.b_total > 0 ? p.b_total : p.B);
+        rp.ldw = l.ldw;
+        rp.dev_status = dev_status;
+        rp.S = f32 ? at<float>(l.s) : nullptr;
+        rp.lds = l.ldw;
+        rp.lse_given = lse_given; rp.want_w = write;
+        const unsigned grid = (unsigned)row_blocks(s);
+        if (f32) return launch(strip_row_f32_kernel, grid, 256, 0, 1, st, at<uint2>(l.w), rp);
+        auto go = [&](auto k) { return launch(k, grid, 256, 0, 1, st, at<uint4>(l.w), rp); };
+        return write ? go(strip_row_kernel<true>) : go(strip_row_kernel<false>);
+    }
+
+    cudaError_t grads(int s, float* dQ, int64_t lddq, float* dP, int64_t lddp, float* loss) {
+        const int64_t row0 = (int64_t)s * l.rows, rows = rows_of(s);
+        const int planes = f32 ? 2 : 1;
+        const GradDeal deal = deal_grads(rows, p.N, p.d, f32, dQ != nullptr, dP != nullptr);
+        const int width = deal.width, tn = (int)ceil_div(p.d, width);
+        GradParams gp{};
+        gp.side[0] = {dQ ? (int)ceil_div(rows, 256) * tn : 0, tn, (int)ceil_div(p.N, KB), (int)rows, p.d, 0};
+        gp.side[1] = {dP ? (int)ceil_div(p.N, 256) * tn : 0, tn, (int)ceil_div(rows, KB), (int)p.N, p.d, s > 0};
+        gp.whole = deal.whole;
+        gp.pairs = deal.pairs;
+        gp.groups = deal.pairs / tn;
+        gp.units = (gp.side[0].tiles * gp.side[0].kblocks + gp.side[1].tiles * gp.side[1].kblocks) / tn;
+        gp.scale = grad_scale / ((float)(p.b_total > 0 ? p.b_total : p.B) * p.tau);
+        gp.res = f32 ? nullptr : at<float>(l.res);
+        gp.pos_idx = p.pos_idx + row0;
+        gp.P = f32 ? nullptr : static_cast<const __nv_bfloat16*>(p.P);
+        gp.ldp = p.ldp;
+        if (loss && s == l.strips - 1) {
+            gp.terms = at<float>(l.red);
+            gp.n_terms = (int)p.B;
+            gp.loss = loss;
+            gp.inv_mean = 1.f / (float)(p.b_total > 0 ? p.b_total : p.B);
+        }
+        gp.part = at<float>(l.part);
+        gp.count = at<int>(l.zero) + 64;
+        gp.dev_status = dev_status;
+        CUtensorMap wk, wm, mp, mq, mdq, mdp;
+        if (!map3(&wk, false, ws + l.w, rows, p.N, l.ldw, planes, rows * l.ldw, 128) ||
+            !map3(&wm, false, ws + l.w, rows, p.N, l.ldw, planes, rows * l.ldw, 64) ||
+            !rows_map(&mp, false, 0, p.N, 64) || !rows_map(&mq, true, row0, rows, 64))
+            return cudaErrorInvalidValue;
+        mdq = mq; mdp = mq;           // a missing output gets a map that is never used
+        if (dQ && !make_out_map(&mdq, dQ + row0 * lddq, rows, p.d, lddq, 1)) return cudaErrorInvalidValue;
+        if (dP && !make_out_map(&mdp, dP, p.N, p.d, lddp, 1)) return cudaErrorInvalidValue;
+        const unsigned grid = 2u * (unsigned)gp.pairs;
+        auto go = [&](auto k, size_t smem) {
+            return launch(k, grid, ST_THREADS, smem, 2, st, wk, wm, mp, mq, mdq, mdp, gp);
+        };
+        return f32 ? go(strip_grad_kernel<true, 128>, SMEM_GF32)
+               : width == 128 ? go(strip_grad_kernel<false, 128>, SMEM_G128)
+                              : go(strip_grad_kernel<false, 256>, SMEM_G);
+    }
+};
+
+}  // namespace
+
+// Which problems take the strip plan.  fp32 and bf16 widths that are no multiple of 64: those of
+// small_tiled_applicable (up to 2 GiB of tile-pair planes, 64 tile pairs).  bf16 rows of more than 384
+// values in whole 64s: always, up to N = 2^18 (a strip's weights are bounded, so more passages mean
+// fewer queries per strip and more passes over dP).  Narrower rows: while the exponentials, which the
+// strip plan writes, converts and reads twice, cost less than forming every logit twice (the sweeps of
+// gc_narrow.cu and gc_tc.cu keep them on the chip).  Measured, us per gc_build_cache, sweeps / strips:
+//   d = 128:  3000 x 6000  67 / 51    4096 x 8192  73 / 72     6000 x 6000   77 / 103
+//   d = 256:  2048 x 4096  70 / 38    4096 x 8192  95 / 82     6000 x 12000 155 / 194
+//   d = 384:  4096 x 8192 154 / 101   8192 x 16384 447 / 418  16384 x 32768 1635 / 1731
+//   d = 768:  1024 x 2048  72 / 28    8192 x 16384 684 / 586  32768 x 65536 11.9 / 10.0 ms
+// GRADCACHE_PLAN=sweeps: as in gc_small.cu.
+bool strip_applicable(int64_t B, int64_t N, int d, int dtype) {
+    const char* e = getenv("GRADCACHE_PLAN");
+    if (e && strcmp(e, "sweeps") == 0) return false;
+    if (d % 8 != 0 || d > MAX_D || small_applicable(B, N, d, dtype)) return false;
+    if (N > (1 << 24) || B > (1 << 24)) return false;
+    if (dtype == GC_F32 || d % 64 != 0) return small_tiled_applicable(B, N, d, dtype);
+    if (d > 384) return N <= 1 << 18;
+    const int64_t most = d <= 128 ? 24 : d <= 256 ? 36 : 144;
+    return B * N <= most << 20;
+}
+
+size_t strip_workspace_bytes(int64_t B, int64_t N, int d, int dtype) {
+    return strip_layout(B, N, d, dtype).total;
+}
+size_t strip_forward_bytes(int64_t B, int64_t N, int d, int dtype) {
+    return strip_layout(B, N, d, dtype, true).total;
+}
+
+int strip_launches(int op, int64_t B, int64_t N, int d, int dtype) {
+    const int strips = strip_layout(B, N, d, dtype).strips, pre = dtype == GC_F32 ? 1 : 0;
+    if (op == GC_OP_FWD) return pre + 2 * strips;
+    if (op == GC_OP_BWD) return pre + (dtype == GC_F32 ? 3 : 2) * strips;
+    return pre + 3 * strips;
+}
+
+cudaError_t strip_forward(const Problem& p, void* ws, float* loss, float* row_lse, float* pos_logit,
+                          int* dev_status, cudaStream_t st) {
+    cudaError_t e = configure_kernels();
+    StripRun r(p, ws, dev_status, st, true);
+    if (e == cudaSuccess && r.f32) e = r.split();
+    for (int s = 0; s < r.l.strips && e == cudaSuccess; ++s) {
+        e = r.logits(s, LOGIT_FWD, nullptr, s == 0);
+        if (e == cudaSuccess) e = r.rows_kernel(s, false, false, row_lse, pos_logit, loss);
+    }
+    return e;
+}
+
+cudaError_t strip_build(const Problem& p, void* ws, float* loss, float* row_lse, float* pos_logit,
+                        float* dQ, int64_t lddq, float* dP, int64_t lddp, int* dev_status,
+                        cudaStream_t st) {
+    cudaError_t e = configure_kernels();
+    StripRun r(p, ws, dev_status, st);
+    if (e == cudaSuccess && r.f32) e = r.split();
+    for (int s = 0; s < r.l.strips && e == cudaSuccess; ++s) {
+        e = r.logits(s, LOGIT_STASH, nullptr, s == 0);
+        if (e == cudaSuccess) e = r.rows_kernel(s, true, false, row_lse, pos_logit, loss);
+        if (e == cudaSuccess) e = r.grads(s, dQ, lddq, dP, lddp, loss);
+    }
+    return e;
+}
+
+cudaError_t strip_backward(const Problem& p, void* ws, const float* row_lse, float* dQ, int64_t lddq,
+                           float* dP, int64_t lddp, int* dev_status, cudaStream_t st,
+                           const float* col_neg, float grad_scale) {
+    cudaError_t e = configure_kernels();
+    StripRun r(p, ws, dev_status, st);
+    r.col_neg = col_neg;
+    r.grad_scale = grad_scale;
+    if (e == cudaSuccess && r.f32) e = r.split();
+    for (int s = 0; s < r.l.strips && e == cudaSuccess; ++s) {
+        e = r.logits(s, col_neg ? LOGIT_W2 : LOGIT_W, row_lse, s == 0);
+        if (e == cudaSuccess && r.f32)
+            e = r.rows_kernel(s, true, true, const_cast<float*>(row_lse), nullptr, nullptr);
+        if (e == cudaSuccess) e = r.grads(s, dQ, lddq, dP, lddp, nullptr);
+    }
+    return e;
+}
+
+}  // namespace gc

@@ -1,0 +1,75 @@
+"""GPU parity of the strip plan (three products over strips of query rows) against the CPU oracle, at
+the sizes where it can go wrong: single columns and rows, ragged last tiles and groups of 64 columns,
+column tiles of every width, whole-tile and cut-tile dealing of the gradients, several strips with the
+masked diagonal running through them, one gradient without the other, rows whose logits span hundreds
+of powers of two.  Tolerances are those of the other parity tests."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2101_06983_b200 import inputs
+
+from gpu_util import TOL, check_against_oracle, grad_err, run_build, to_device
+from test_gpu_parity import _check_properties, _check_sampled, _oracle_full
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def binding():
+    if not torch.cuda.is_available():
+        pytest.fail("GPU tests need a CUDA device")
+    from paper_2101_06983_b200 import binding as b
+    return b
+
+
+SHAPES = [
+    # B, N, d, dtype, mask, tau
+    (129, 1, 64, "bf16", 0, 1.0), (1, 257, 8, "bf16", 0, 1.0), (1, 129, 8, "f32", 0, 1.0),
+    (255, 321, 72, "bf16", 1, 0.3), (257, 511, 136, "f32", 1, 0.3), (400, 1601, 448, "bf16", 0, 0.5),
+    (1100, 63, 1088, "bf16", 0, 0.5), (2305, 2561, 192, "bf16", 1, 0.2), (3000, 5000, 576, "bf16", 0, 0.5),
+    (5200, 700, 768, "bf16", 0, 0.5), (1900, 2100, 384, "f32", 0, 0.5), (600, 9001, 512, "f32", 0, 0.5),
+    # logits spanning hundreds of powers of two.  fp32: a weight is 2^(s - lse) of two fp32 numbers, so its
+    # relative error is at least ln 2 times half an ulp of lse log2(e): at tau = 0.01 lse reaches 2800
+    # (4000 in log2 units, 1.7e-4, beyond the 1e-4 of these tests), at 0.1 it stays below 300 (1.1e-5).
+    (300, 520, 768, "bf16", 0, 0.004), (300, 520, 64, "f32", 0, 0.1),
+]
+
+
+@pytest.mark.parametrize("B,N,d,dtype,mask,tau", SHAPES)
+def test_build_and_split_calls(binding, oracle, B, N, d, dtype, mask, tau):
+    prob = inputs.random_problem(B, N, d, dtype, seed=B + N + d, tau=tau, mask_mode=mask,
+                                 scale=1.0 if tau <= 0.1 else d ** -0.5)
+    out = run_build(prob)
+    ref = _oracle_full(oracle, prob)
+    check_against_oracle(prob, out, ref)
+    Q, P, pos = to_device(prob)
+    b = binding.Outputs(B, N, d, binding._dtype_code(Q))
+    args = (Q, P, pos, prob.tau, prob.mask_mode)
+    binding.gc_loss_fwd(*args, b.loss, b.row_lse, b.pos_logit, b.ws, b.dev_status)
+    binding.gc_loss_bwd(*args, b.row_lse, b.dQ, None, b.ws, b.dev_status)
+    binding.gc_loss_bwd(*args, b.row_lse, None, b.dP, b.ws, b.dev_status)
+    torch.cuda.synchronize()
+    check_against_oracle(prob, b, ref)
+
+
+def test_several_strips_f32_self_mask(binding, oracle):
+    """8200 x 8200 pairs are two strips; the diagonal runs through both."""
+    prob = inputs.random_problem(8200, 8200, 16, "f32", seed=5, tau=0.5, mask_mode=inputs.MASK_SELF,
+                                 scale=0.25)
+    assert binding.gc_kernel_launches(binding.GC_OP_BUILD, 8200, 8200, 16, binding.GC_F32) == 1 + 2 * 3
+    out = run_build(prob)
+    check_against_oracle(prob, out, _oracle_full(oracle, prob))
+
+
+def test_several_strips_bf16_self_mask(binding, oracle):
+    """17 000 x 17 000 pairs are two strips: sampled rows of both, and the identities."""
+    n, d = 17000, 448
+    prob = inputs.random_problem(n, n, d, "bf16", seed=6, tau=0.5, mask_mode=inputs.MASK_SELF,
+                                 scale=d ** -0.5)
+    assert binding.gc_kernel_launches(binding.GC_OP_BUILD, n, n, d, binding.GC_BF16) == 2 * 3
+    out = run_build(prob)
+    assert int(out.dev_status.item()) == 0
+    _check_sampled(oracle, prob, out, 48, 24, full_lse=out.row_lse.cpu().numpy().astype(np.float64))
+    Q, P, _ = to_device(prob)
+    _check_properties(prob, out, Q, P)
