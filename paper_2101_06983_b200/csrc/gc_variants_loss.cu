@@ -212,6 +212,31 @@ gather_rows_kernel(const uint4* __restrict__ P, int64_t ldp16, const int32_t* __
     }
 }
 
+// Two-direction loss on the strip plan: how often passage j is a positive (mult[j]) and the first query
+// it is the positive of (first[j] = B - i; both cleared beforehand; 0 where there is none).
+__global__ void __launch_bounds__(256)
+count_positives_kernel(const int32_t* __restrict__ pos, int64_t B, int64_t N, int* __restrict__ mult,
+                       int* __restrict__ first) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= B) return;
+    const int32_t r = pos[i];
+    if (r < 0 || r >= N) return;
+    atomicAdd(mult + r, 1);
+    atomicMax(first + r, (int)(B - i));
+}
+// col_neg[j] = log2(mult_j) - log2e lse_col_j with lse_col_j = lse2 of a query j is the positive of;
+// -inf where j is nobody's positive.  Also loss = (loss + loss2) / 2.
+__global__ void __launch_bounds__(256)
+column_factor_kernel(const int* __restrict__ mult, const int* __restrict__ first,
+                     const float* __restrict__ lse2, int64_t B, int64_t N, float* __restrict__ col_neg,
+                     float* __restrict__ loss, const float* __restrict__ loss2) {
+    const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (j == 0) *loss = 0.5f * (*loss + *loss2);
+    if (j >= (N + 3) / 4 * 4) return;
+    const int m = j < N ? mult[j] : 0;
+    col_neg[j] = m > 0 ? log2f((float)m) - lse2[B - first[j]] * 1.4426950408889634f : -INFINITY;
+}
+
 // dQ = (dQ + dQ2) / 2, dP = dP / 2, loss = (loss + loss2) / 2.
 __global__ void __launch_bounds__(256)
 two_dir_combine_kernel(float* __restrict__ dQ, int64_t lddq, const float* __restrict__ dQ2,
@@ -265,7 +290,13 @@ MultiLayout multi_layout(int64_t B, int64_t N, int d, int dtype, int64_t n_pos) 
     return l;
 }
 
-struct TwoDirLayout { size_t A, ident, dA, dQ2, lse2, loss2, inner, total; };
+// bf16: both directions in one set of weights (strip plan), W_ij = p_ij + m_j p'_ij - 2 [j = r_i] with p'
+// the softmax over the queries and m_j the number of queries j is the positive of.
+bool two_dir_strips(int64_t B, int64_t N, int d, int dtype) {
+    return dtype == GC_BF16 && strip_applicable(B, N, d, dtype);
+}
+
+struct TwoDirLayout { size_t A, ident, dA, dQ2, lse2, loss2, count, col_neg, inner, total; };
 TwoDirLayout two_dir_layout(int64_t B, int64_t N, int d, int dtype) {
     TwoDirLayout l{};
     const size_t es = dtype == GC_BF16 ? 2 : 4;
@@ -276,8 +307,13 @@ TwoDirLayout two_dir_layout(int64_t B, int64_t N, int d, int dtype) {
     l.dQ2 = off;    off += align256v(sizeof(float) * (size_t)B * (size_t)d);
     l.lse2 = off;   off += align256v(sizeof(float) * (size_t)B);
     l.loss2 = off;  off += 256;
-    const size_t w1 = gc_workspace_bytes(GC_OP_BUILD, B, N, d, dtype);
-    const size_t w2 = gc_workspace_bytes(GC_OP_BUILD, B, B, d, dtype);
+    size_t w1 = gc_workspace_bytes(GC_OP_BUILD, B, N, d, dtype);
+    size_t w2 = gc_workspace_bytes(GC_OP_BUILD, B, B, d, dtype);
+    if (two_dir_strips(B, N, d, dtype)) {
+        l.count = off;    off += align256v(2 * sizeof(int) * (size_t)N);
+        l.col_neg = off;  off += align256v(sizeof(float) * (size_t)(N + 4));
+        w2 = strip_workspace_bytes(B, B, d, dtype);
+    }
     l.inner = off;  off += w1 > w2 ? w1 : w2;
     l.total = off;
     return l;
@@ -365,6 +401,40 @@ int gc_build_cache_two_direction(const void* Q, int64_t ldq, const void* P, int6
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     char* w = static_cast<char*>(ws);
     const int es = dtype == GC_BF16 ? 2 : 4;
+    if (two_dir_strips(B, N, d, dtype)) {
+        if (lddq < d || lddp < d) return GC_ERR_SHAPE;
+        if (((uintptr_t)dQ & 15) || ((uintptr_t)dP & 15) || lddq % 4 || lddp % 4) return GC_ERR_ALIGN;
+        // row direction's logsumexp and loss (validates the other arguments), the column direction's
+        // on the anchors A_i = P[r_i] with the queries as candidates, then one set of weights
+        int rc = gc_loss_fwd(Q, ldq, P, ldp, pos_idx, B, N, d, tau, GC_MASK_NONE, dtype, loss, row_lse,
+                             nullptr, w + l.inner, ws_bytes - l.inner, dev_status, cuda_stream);
+        if (rc) return rc;
+        void* A = w + l.A;
+        int32_t* ident = reinterpret_cast<int32_t*>(w + l.ident);
+        float* lse2 = reinterpret_cast<float*>(w + l.lse2);
+        float* loss2 = reinterpret_cast<float*>(w + l.loss2);
+        int* mult = reinterpret_cast<int*>(w + l.count);
+        float* col_neg = reinterpret_cast<float*>(w + l.col_neg);
+        if (cudaMemsetAsync(mult, 0, 2 * sizeof(int) * (size_t)N, st) != cudaSuccess) return GC_ERR_CUDA;
+        count_positives_kernel<<<(unsigned)((B + 255) / 256), 256, 0, st>>>(pos_idx, B, N, mult, mult + N);
+        const int d8 = d * es / 16;
+        gather_rows_kernel<<<grid_for(B * d8, 256), 256, 0, st>>>(
+            static_cast<const uint4*>(P), ldp * es / 16, pos_idx, B, N, d8, static_cast<uint4*>(A), ident);
+        if (cudaGetLastError() != cudaSuccess) return GC_ERR_CUDA;
+        Problem pc{};
+        pc.Q = A; pc.P = Q; pc.pos_idx = ident; pc.ldq = d; pc.ldp = ldq; pc.B = B; pc.N = B; pc.d = d;
+        pc.tau = tau; pc.mask_mode = GC_MASK_NONE; pc.dtype = dtype;
+        if (strip_forward(pc, w + l.inner, loss2, lse2, nullptr, dev_status, st) != cudaSuccess)
+            return GC_ERR_CUDA;
+        column_factor_kernel<<<(unsigned)((N + 3 + 255) / 256), 256, 0, st>>>(mult, mult + N, lse2, B, N,
+                                                                             col_neg, loss, loss2);
+        if (cudaGetLastError() != cudaSuccess) return GC_ERR_CUDA;
+        Problem pr{};
+        pr.Q = Q; pr.P = P; pr.pos_idx = pos_idx; pr.ldq = ldq; pr.ldp = ldp; pr.B = B; pr.N = N; pr.d = d;
+        pr.tau = tau; pr.mask_mode = GC_MASK_NONE; pr.dtype = dtype;
+        return strip_backward(pr, w + l.inner, row_lse, dQ, lddq, dP, lddp, dev_status, st, col_neg,
+                              0.5f) == cudaSuccess ? GC_OK : GC_ERR_CUDA;
+    }
     // row direction: Eq. 1 as it stands (validates the arguments)
     int rc = gc_build_cache(Q, ldq, P, ldp, pos_idx, B, N, d, tau, GC_MASK_NONE, dtype, loss,
                             row_lse, nullptr, dQ, lddq, dP, lddp, w + l.inner, ws_bytes - l.inner,
