@@ -216,7 +216,9 @@ strip_logit_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
     volatile int* abort_flag = &abort_s;
     const PairCtx c = pair_setup(smem_raw, bars, &tmem_s, &abort_s);
     constexpr uint32_t A_BYTES = CHUNK_BYTES, B_BYTES = BN / 2 * 128, STAGE = A_BYTES + B_BYTES;
-    constexpr int NST = BN == 256 ? 5 : 6;
+    // (weights are formed in the epilogue with row_lse given: it is the longer part there, and a second
+    // staging buffer gives more than a sixth stage: 4096 x 8192 x 1024, 246 against 249 us per pass)
+    constexpr int SB = MODE >= LOGIT_W && BN == 256 ? 2 : 1, NST = SB == 2 ? 5 : 6;
     const int total = p.tiles_m * p.tiles_n;
     const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
     dep_release();
@@ -287,7 +289,7 @@ strip_logit_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
             for (int e = blockIdx.x * 256 + (ew * 32 + lane); e < p.zero_count; e += 8 * 256)
                 p.zero[e] = 0;
         }
-        const uint32_t stage_buf = c.smem + NST * STAGE + (uint32_t)ew * (uint32_t)(HC * 64);
+        const uint32_t stage_buf = c.smem + NST * STAGE + (uint32_t)ew * (SB * 4096u);
         const uint64_t c1_2 = pack2(p.c1, p.c1);
         int use = 0;
         for (int t = pair; t < total; t += pairs, ++use) {
@@ -354,7 +356,9 @@ strip_logit_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
                                 if (MODE == LOGIT_W) pos_raw = s[e];
                                 else p.pos_ws[i] = s[e];
                             }
-                            if (e == dm || jg + e >= p.N) s[e] = -INFINITY;
+                            // the stored exponentials and their group's maximum leave the positive out:
+                            // where it dominates its row, its neighbours keep their precision
+                            if (e == dm || jg + e >= p.N || (MODE != LOGIT_FWD && e == dp)) s[e] = -INFINITY;
                         }
                     }
                     float mx[4] = {s[0], s[1], s[2], s[3]};
@@ -422,12 +426,9 @@ strip_logit_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
                 }
                 if (MODE != LOGIT_FWD) {
                     // 32 rows x 64 columns of 16 bits, 128-byte swizzle, one bulk tensor store
-                    if (lane == 0) {
-                        if (HC == 128) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
-                        else           bulk_wait_read0();
-                    }
+                    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(SB - 1) : "memory");
                     __syncwarp();
-                    const uint32_t buf = stage_buf + (uint32_t)g * 4096u + lane * 128;
+                    const uint32_t box = stage_buf + (uint32_t)(g & (SB - 1)) * 4096u, buf = box + lane * 128;
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
                         uint32_t w[4];
@@ -441,7 +442,7 @@ strip_logit_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
                     __syncwarp();
                     if (lane == 0) {                     // (an empty group when nothing is stored)
                         if (row0 < p.rows && jg < p.N)
-                            tma_store_3d(&mapW, stage_buf + (uint32_t)g * 4096u, jg, row0, 0);
+                            tma_store_3d(&mapW, box, jg, row0, 0);
                         else
                             asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                     }
@@ -659,6 +660,7 @@ struct RowParams {
     int block0, blocks_total;     // this launch's first block and the blocks of all strips
     float inv_mean;
     int64_t ldw;                  // elements
+    int seg_rounds;               // strip_row_kernel<true>: rounds of 2048 columns per segment
     int* dev_status;
     // fp32 inputs
     const float* S;
@@ -680,13 +682,14 @@ __device__ __forceinline__ void loss_share(const RowParams& p, float mine) {
     if (!last_s) return;
     __threadfence();
     float v = 0.f;
-    for (int b = threadIdx.x; b < p.blocks_total; b += 256) v += __ldcg(p.red + b);
+#pragma unroll 4
+    for (int b = threadIdx.x; b < p.blocks_total; b += blockDim.x) v += __ldcg(p.red + b);
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     if ((threadIdx.x & 31) == 0) warp_s[threadIdx.x >> 5] = v;
     __syncthreads();
     if (threadIdx.x == 0) {
         float s = 0.f;
-        for (int w = 0; w < 8; ++w) s += warp_s[w];
+        for (int w = 0; w < (int)blockDim.x / 32; ++w) s += warp_s[w];
         *p.loss = s * p.inv_mean;
     }
 }
@@ -699,64 +702,55 @@ __device__ __forceinline__ int row_pos(const RowParams& p, int i, int* flags) {
     return *flags || pos < 0 || pos >= p.N ? -1 : pos;
 }
 
-// bf16 inputs, ROW_BATCH rows per block.  A warp per row merges the row's slots; then all threads turn
-// the rows' fp16 exponentials into bf16 weights in place (WRITE), the first of them requested before
-// the merge so that its chain of dependent loads and reductions is paid once per block.  Bound by the
-// L2: 4 bytes moved per pair.
-constexpr int ROW_BATCH = 4;
+// bf16 inputs: a warp per row (WRITE: per row and segment of its columns; each merges the row's slots
+// for itself).  It forms row_lse, the positive's weight and the loss term, then turns the row's fp16
+// exponentials into bf16 weights in place: eight 16-byte pieces in flight per lane, the first of them
+// requested before the merge, each one's successor as soon as it has been used; one special-function
+// operation per group of 64 columns, its result passed around by shuffles.  Bound by the latency and
+// bandwidth of the L2 (4 bytes moved per pair).
+constexpr int row_warps(bool write) { return write ? 4 : 8; }      // rows per block
+constexpr int ROW_PIECES = 8;                       // of 8 columns, per lane and round
+constexpr int ROW_ROUND = 32 * ROW_PIECES;          // pieces per warp and round: 32 groups of 64 columns
 template <bool WRITE>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(WRITE ? 128 : 256, WRITE ? 8 : 1)
 strip_row_kernel(uint4* __restrict__ W, const RowParams p) {
-    struct RowHead { float lse2, pw; int wpos; };
-    __shared__ RowHead heads[ROW_BATCH];
-    __shared__ float terms[ROW_BATCH];
+    constexpr int ROW_WARPS = WRITE ? 4 : 8;
+    __shared__ float terms[ROW_WARPS];
     dep_release();
     dep_wait();
-    const int i0 = blockIdx.x * ROW_BATCH;
-    const int rows = min(ROW_BATCH, p.rows - i0);
-    const int n8 = (p.N + 7) / 8, pitch8 = (int)(p.ldw / 8);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    W += (int64_t)i0 * pitch8;
-    const float2* sl0 = p.slots + (int64_t)i0 * p.slot_pitch;
-    // pieces of 8 columns, row after row; each thread takes every 256th
-    constexpr int PIECES = 4;
-    int r = 0, k = threadIdx.x;
-    auto wrap = [&]() { while (k >= n8) { k -= n8; ++r; } };
-    wrap();
-    uint4 raw[PIECES];
-    float gm[PIECES];
-    int at[PIECES], of[PIECES];
-    auto fetch = [&]() {
+    const int i = blockIdx.x * ROW_WARPS + warp;
+    const bool live = i < p.rows;
+    const int n8 = (p.N + 7) / 8;
+    const int k0 = WRITE ? (int)blockIdx.y * p.seg_rounds * ROW_ROUND : 0;
+    const int k1 = WRITE ? min(n8, k0 + p.seg_rounds * ROW_ROUND) : 0;
+    const float2* sl = p.slots + (int64_t)(live ? i : 0) * p.slot_pitch;
+    uint4* row = W + (int64_t)(live ? i : 0) * (p.ldw / 8);
+    uint4 raw[ROW_PIECES];
+    if (WRITE && live) {
 #pragma unroll
-        for (int x = 0; x < PIECES; ++x) {
-            of[x] = r;
-            at[x] = k;
-            if (r < rows) {
-                raw[x] = __ldcg(W + (int64_t)r * pitch8 + k);
-                gm[x] = __ldcg(&sl0[(int64_t)r * p.slot_pitch + (k >> 3)].x);
-            }
-            k += 256;
-            wrap();
+        for (int x = 0; x < ROW_PIECES; ++x) {
+            const int k = k0 + lane + 32 * x;
+            if (k < k1) raw[x] = __ldcg(row + k);
         }
-    };
-    if (WRITE) fetch();
-    if (warp < rows) {
-        const int i = i0 + warp;
-        const float2* sl = sl0 + (int64_t)warp * p.slot_pitch;
+    }
+    if (live) {
         int flags;
         const int pos = row_pos(p, i, &flags);
-        const float pos_raw = __ldcg(p.pos_ws + i);
+        const float pos_raw = pos < 0 ? -INFINITY : __ldcg(p.pos_ws + i);
         constexpr int KEEP = 4;                     // slots held in registers (N <= 8192: all)
         float2 kept[KEEP];
 #pragma unroll
         for (int x = 0; x < KEEP; ++x)
             kept[x] = lane + 32 * x < p.nslots ? __ldcg(sl + lane + 32 * x) : make_float2(-INFINITY, 0.f);
-        float m = -INFINITY, l = 0.f;
+        // with weights, the positive is not in the slots: it is a term of its own
+        float m = WRITE ? pos_raw : -INFINITY;
 #pragma unroll
         for (int x = 0; x < KEEP; ++x) m = fmaxf(m, kept[x].x);
         for (int s = lane + 32 * KEEP; s < p.nslots; s += 32) m = fmaxf(m, __ldcg(&sl[s].x));
         for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
         const float ref = m == -INFINITY ? 0.f : m;
+        float l = WRITE && lane == 0 ? ex2((pos_raw - ref) * p.c1) : 0.f;
 #pragma unroll
         for (int x = 0; x < KEEP; ++x) l = fmaf(kept[x].y, ex2((kept[x].x - ref) * p.c1), l);
         for (int s = lane + 32 * KEEP; s < p.nslots; s += 32) {
@@ -764,57 +758,60 @@ strip_row_kernel(uint4* __restrict__ W, const RowParams p) {
             l = fmaf(v.y, ex2((v.x - ref) * p.c1), l);
         }
         for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+        const float lse = m * p.inv_tau + log2f(l) * LN2;
+        const float pl = pos < 0 ? 0.f : pos_raw * p.inv_tau;
+        const float pw = positive_weight(pos_raw, p.inv_tau, lse);
         if (lane == 0) {
-            const float lse = m * p.inv_tau + log2f(l) * LN2;
-            const float pl = pos < 0 ? 0.f : pos_raw * p.inv_tau;
-            RowHead h;
-            h.lse2 = lse * LOG2E;
-            h.pw = positive_weight(pos_raw, p.inv_tau, lse);
-            h.wpos = pos;
-            heads[warp] = h;
             terms[warp] = lse - pl;
-            p.row_lse[i] = lse;
-            if (p.pos_logit) p.pos_logit[i] = pl;
-            if (flags && p.dev_status) atomicOr(p.dev_status, flags);
-            if (WRITE) {
-                p.red[p.row0 + i] = lse - pl;
-                p.res[i] = pos < 0 ? 0.f : h.pw - __bfloat162float(__float2bfloat16_rn(h.pw));
+            if (!WRITE || blockIdx.y == 0) {
+                p.row_lse[i] = lse;
+                if (p.pos_logit) p.pos_logit[i] = pl;
+                if (flags && p.dev_status) atomicOr(p.dev_status, flags);
+                if (WRITE) {
+                    p.red[p.row0 + i] = lse - pl;
+                    p.res[i] = pos < 0 ? 0.f : pw - __bfloat162float(__float2bfloat16_rn(pw));
+                }
+            }
+        }
+        if (WRITE) {
+            const float neg = -(lse * LOG2E);
+            const int wk = pos < 0 ? -1 : pos >> 3;
+            // round after round: lane g of a round holds the factor of its group of 64 columns
+            for (int kr = k0; kr < k1; kr += ROW_ROUND) {
+                const int g = (kr >> 3) + lane;
+                // (a group with no allowed column holds zeros)
+                const float gm = g < p.nslots ? __ldcg(&sl[g].x) : -INFINITY;
+                const float fg = gm > -INFINITY ? ex2(fmaf(gm, p.c1, neg)) : 0.f;
+#pragma unroll
+                for (int x = 0; x < ROW_PIECES; ++x) {
+                    const float f = __shfl_sync(0xffffffffu, fg, 4 * x + (lane >> 3));
+                    const int k = kr + lane + 32 * x;
+                    if (k >= k1) continue;
+                    const __half2* e2 = reinterpret_cast<const __half2*>(&raw[x]);
+                    float w[8];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const float2 v = __half22float2(e2[e]);
+                        w[2 * e] = v.x * f;
+                        w[2 * e + 1] = v.y * f;
+                    }
+                    if (wk == k) {
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) if (e == (pos & 7)) w[e] = pw;
+                    }
+                    row[k] = make_uint4(pack_b2(w[0], w[1]), pack_b2(w[2], w[3]),
+                                        pack_b2(w[4], w[5]), pack_b2(w[6], w[7]));
+                    if (k + ROW_ROUND < k1) raw[x] = __ldcg(row + k + ROW_ROUND);
+                }
             }
         }
     }
-    __syncthreads();
     if (!WRITE) {
+        __syncthreads();
         float share = 0.f;
         if (threadIdx.x == 0)
-            for (int w = 0; w < rows; ++w) share += terms[w];
+            for (int w = 0; w < ROW_WARPS && blockIdx.x * ROW_WARPS + w < p.rows; ++w) share += terms[w];
         loss_share(p, share);
-        return;
-    }
-    if constexpr (WRITE) {
-        while (of[0] < rows) {
-#pragma unroll
-            for (int x = 0; x < PIECES; ++x) {
-                if (of[x] >= rows) break;
-                const RowHead h = heads[of[x]];
-                // (a group with no allowed column holds zeros)
-                const float f = gm[x] > -INFINITY ? ex2(fmaf(gm[x], p.c1, -h.lse2)) : 0.f;
-                const __half2* e2 = reinterpret_cast<const __half2*>(&raw[x]);
-                float w[8];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const float2 v = __half22float2(e2[e]);
-                    w[2 * e] = v.x * f;
-                    w[2 * e + 1] = v.y * f;
-                }
-                if ((h.wpos >> 3) == at[x]) {
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) if (e == (h.wpos & 7)) w[e] = h.pw;
-                }
-                W[(int64_t)of[x] * pitch8 + at[x]] =
-                    make_uint4(pack_b2(w[0], w[1]), pack_b2(w[2], w[3]), pack_b2(w[4], w[5]), pack_b2(w[6], w[7]));
-            }
-            fetch();
-        }
     }
 }
 
@@ -961,10 +958,13 @@ struct Segment {
 __device__ __forceinline__ int unit_start(const GradParams& p, int g) {
     return (int)((int64_t)p.units * g / p.groups);
 }
-// Iterates over a pair's segments.
+// Iterates over a pair's segments.  In a cut run the two cut tiles come first (their partial sums meet
+// under the products of the tiles that follow), the whole ones after them.
 struct SegmentWalk {
     int u, end, group, tile_n;    // whole >= 0: u counts tiles
+    int phase;
     __device__ __forceinline__ SegmentWalk(const GradParams& p, int pair) {
+        phase = 0;
         if (p.whole >= 0) {
             const bool q = pair < p.whole;
             u = q ? pair : pair - p.whole;
@@ -978,6 +978,18 @@ struct SegmentWalk {
             end = unit_start(p, group + 1);
         }
     }
+    // the tile that unit v lies in, and the part of it in [u, end)
+    __device__ __forceinline__ void locate(const GradParams& p, int v, Segment& s) const {
+        const int first_p = p.side[0].tiles / p.side[0].tiles_n * p.side[0].kblocks;
+        s.side = v >= first_p;
+        const int k = s.side ? p.side[1].kblocks : p.side[0].kblocks;
+        const int local = v - (s.side ? first_p : 0);
+        s.tile_m = local / k;
+        s.tile_n = tile_n;
+        s.t0 = v - (local - s.tile_m * k);
+        s.kb = max(u - s.t0, 0);
+        s.n = min(k, end - s.t0) - s.kb;
+    }
     __device__ __forceinline__ bool next(const GradParams& p, Segment& s) {
         if (u >= end) return false;
         if (p.whole >= 0) {
@@ -988,18 +1000,20 @@ struct SegmentWalk {
             s.n = s.side ? p.side[1].kblocks : p.side[0].kblocks;
             s.t0 = 0;
             u += group;
-        } else {
-            const int first_p = p.side[0].tiles / p.side[0].tiles_n * p.side[0].kblocks;
-            s.side = u >= first_p;
-            const int k = s.side ? p.side[1].kblocks : p.side[0].kblocks;
-            const int local = u - (s.side ? first_p : 0);
-            s.tile_m = local / k;
-            s.tile_n = tile_n;
-            s.kb = local - s.tile_m * k;
-            s.n = min(k - s.kb, end - u);
-            s.t0 = u - s.kb;
-            u += s.n;
+            return true;
         }
+        if (phase == 0) {
+            phase = 1;
+            locate(p, u, s);
+            if (s.kb > 0) { u += s.n; return true; }
+        }
+        if (phase == 1) {
+            phase = 2;
+            locate(p, end - 1, s);
+            if (s.n < (s.side ? p.side[1].kblocks : p.side[0].kblocks)) { end -= s.n; return true; }
+        }
+        locate(p, u, s);
+        u += s.n;
         return true;
     }
 };
@@ -1026,7 +1040,7 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
     constexpr int TA = F32 ? 2 : 1, TB = F32 ? 3 : 1;     // operand terms
     constexpr uint32_t B_TERM = WIDTH / 2 * 128;          // 64 contraction rows x WIDTH / 2 columns
     constexpr uint32_t A_BYTES = TA * CHUNK_BYTES, STAGE = A_BYTES + TB * B_TERM;
-    constexpr int NST = F32 ? 3 : WIDTH == 128 ? 6 : 5;
+    constexpr int NST = F32 ? 3 : 6;
     constexpr int CHUNK_KB = 2;                           // F32: blocks per accumulator read-out
     constexpr int HW = WIDTH / 2;                         // columns of an epilogue warp
     const int pair = blockIdx.x >> 1;
@@ -1141,7 +1155,7 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
     } else {
         const int ew = c.warp - (NPROD + 1);
         const int q = c.warp & 3, half = ew >> 2, lane = c.lane;
-                constexpr int SB = F32 ? 1 : 2;                   // staging buffers of 4 KB
+        constexpr int SB = F32 || WIDTH == 256 ? 1 : 2;   // staging buffers of 4 KB
         const uint32_t stage_buf = c.smem + NST * STAGE + (uint32_t)ew * (SB * 4096u);
         const int cw = (int)c.rank * 8 + ew;              // this warp among the 16 of a tile
         constexpr size_t PART_FLOATS = 32 * HW;
@@ -1385,10 +1399,10 @@ size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
 int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 int pairs_of_device() { return sm_count() / 2; }
 
-constexpr size_t SMEM_L256 = 1024 + 5 * (CHUNK_BYTES + 16384) + NSOFT * 8192;
+constexpr size_t SMEM_L256 = 1024 + 6 * (CHUNK_BYTES + 16384) + NSOFT * 4096;    // or 5 stages, NSOFT * 8192
 constexpr size_t SMEM_L128 = 1024 + 6 * (CHUNK_BYTES + 8192) + NSOFT * 4096;
 constexpr size_t SMEM_LF32 = 1024 + F_NST * F_STAGE + NSOFT * 8192;
-constexpr size_t SMEM_G = 1024 + 5 * (CHUNK_BYTES + 16384) + NSOFT * 8192;
+constexpr size_t SMEM_G = 1024 + 6 * (CHUNK_BYTES + 16384) + NSOFT * 4096;
 constexpr size_t SMEM_G128 = 1024 + 6 * (CHUNK_BYTES + 8192) + NSOFT * 8192;
 constexpr size_t SMEM_GF32 = 1024 + 3 * (2 * CHUNK_BYTES + 3 * 8192) + NSOFT * 4096;
 static_assert(SMEM_L256 <= SMEM_LIMIT - 1024 && SMEM_LF32 <= SMEM_LIMIT - 1024 &&
@@ -1397,10 +1411,10 @@ static_assert(SMEM_L256 <= SMEM_LIMIT - 1024 && SMEM_LF32 <= SMEM_LIMIT - 1024 &
 // Kernel launch with a cluster of `cluster` CTAs (1: none).  Every kernel of this file may start while
 // the kernel before it in the stream runs; it waits for that kernel before it touches memory.
 template <typename... KArgs, typename... Args>
-cudaError_t launch(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, int cluster,
+cudaError_t launch(void (*kernel)(KArgs...), dim3 grid, unsigned block, size_t smem, int cluster,
                    cudaStream_t st, Args&&... args) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3(block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
@@ -1620,8 +1634,8 @@ struct StripRun {
     }
 
     // rows per block of the row kernel: a row of few passages takes a warp's worth of threads
-    int row_blocks(int s) const {
-        if (!f32) return (int)ceil_div(rows_of(s), ROW_BATCH);
+    int row_blocks(int s, bool write) const {
+        if (!f32) return (int)ceil_div(rows_of(s), row_warps(write));
         const int64_t n = rows_of(s), most = 8 * (int64_t)sm_count();
         return (int)(n < most ? n : most);
     }
@@ -1652,19 +1666,24 @@ struct StripRun {
         rp.red = at<float>(l.red);
         rp.ticket = at<int>(l.zero);
         rp.block0 = 0;
-        for (int k = 0; k < s; ++k) rp.block0 += row_blocks(k);
+        for (int k = 0; k < s; ++k) rp.block0 += row_blocks(k, write);
         rp.blocks_total = 0;
-        for (int k = 0; k < l.strips; ++k) rp.blocks_total += row_blocks(k);
+        for (int k = 0; k < l.strips; ++k) rp.blocks_total += row_blocks(k, write);
         rp.inv_mean = 1.f / (float)(p.b_total > 0 ? p.b_total : p.B);
         rp.ldw = l.ldw;
         rp.dev_status = dev_status;
         rp.S = f32 ? at<float>(l.s) : nullptr;
         rp.lds = l.ldw;
         rp.lse_given = lse_given; rp.want_w = write;
-        const unsigned grid = (unsigned)row_blocks(s);
+        const unsigned grid = (unsigned)row_blocks(s, write);
         if (f32) return launch(strip_row_f32_kernel, grid, 256, 0, 1, st, at<uint2>(l.w), rp);
-        auto go = [&](auto k) { return launch(k, grid, 256, 0, 1, st, at<uint4>(l.w), rp); };
-        return write ? go(strip_row_kernel<true>) : go(strip_row_kernel<false>);
+        // segments of whole rounds while there are fewer rows than warps the device holds
+        const int64_t rounds = ceil_div(p.N, 8 * ROW_ROUND), room = 28 * (int64_t)sm_count() / rows;
+        const int64_t segs = room < 1 ? 1 : room < rounds ? room : rounds;
+        rp.seg_rounds = (int)ceil_div(rounds, segs);
+        auto go = [&](auto k, dim3 g) { return launch(k, g, 32 * row_warps(write), 0, 1, st, at<uint4>(l.w), rp); };
+        return write ? go(strip_row_kernel<true>, dim3(grid, (unsigned)ceil_div(rounds, rp.seg_rounds)))
+                     : go(strip_row_kernel<false>, dim3(grid));
     }
 
     cudaError_t grads(int s, float* dQ, int64_t lddq, float* dP, int64_t lddp, float* loss) {
