@@ -166,11 +166,12 @@ int gc_build_cache_stored(const void* Q, int64_t ldq, const void* P, int64_t ldp
  * Each u is used as the sum of two bf16 terms (its rounding and the rounding of the remainder,
  * together exact to 2^-17 |u|), products are exact and accumulation is fp32 on the tensor cores.
  * Limits: d a multiple of 8, d_in a multiple of 64 and at most 4096 (else GC_ERR_LIMIT); rows of
- * U, X and dW start on 16-byte boundaries.  One kernel launch; the partial sums over parts of the
- * sub-batch are exchanged through shared memory, so the workspace is nominal:
- * gc_cache_apply_workspace_bytes returns 256 (0 for sizes outside the limits) and ws must be a
- * 256-byte aligned, caller-owned buffer of at least that size.  Asynchronous on cuda_stream;
- * deterministic; GC_DEV_WAIT_LIMIT in *dev_status (may be NULL) as for the other calls.
+ * U, X and dW start on 16-byte boundaries.  Up to two kernel launches: where the widths leave CTA
+ * pairs over, the sub-batch's rows are split into parts whose sums are planes of the workspace, added
+ * in order.  gc_cache_apply_workspace_bytes returns the bytes that takes for any number of rows (0 for
+ * sizes outside the limits); ws must be a 256-byte aligned, caller-owned buffer of at least that size.
+ * Asynchronous on cuda_stream; deterministic; GC_DEV_WAIT_LIMIT in *dev_status (may be NULL) as for
+ * the other calls.
  */
 size_t gc_cache_apply_workspace_bytes(int64_t rows, int d, int d_in);
 int gc_cache_apply(const float* U, int64_t ldu, const void* X, int64_t ldx, int64_t rows, int d,

@@ -4,22 +4,26 @@
 //
 //     dW[a][b] (+)= sum_i U[i][a] X[i][b]          U: rows x d fp32 (cache slice), X: rows x d_in bf16
 //
-// in ONE launch, reading U and X once as they are.  The cache is fp32 and the tensor cores take
-// bf16, so every u is used as two bf16 terms, hi = rn(u) and lo = rn(u - hi), whose sum misses u
-// by at most 2^-17 |u|; both terms accumulate into the same fp32 accumulator.
+// The cache is fp32 and the tensor cores take bf16, so every u is used as two bf16 terms,
+// hi = rn(u) and lo = rn(u - hi), whose sum misses u by at most 2^-17 |u|; both terms accumulate
+// into the same fp32 accumulator.
 //
-// A CTA owns a tile of 128 output rows (columns of U) x up to 384 output columns (columns of X)
-// and one part of the contraction range (the rows of the sub-batch).  Per step of 32 rows:
-//   producer warp   one bulk tensor load of the fp32 U block (32 x 128) and of the X block
-//                   (32 x 384, an MN-major B operand as it lies in memory);
-//   4 converter warps  read the fp32 block from shared memory, form hi and lo and write them as
-//                   two MN-major A operands in the 128-byte swizzle the tensor core expects;
-//   MMA warp        up to 8 instructions (two steps of 16 rows, hi and lo, columns 0..255 and
-//                   256..383 of the tile).
-// The parts of a tile's contraction range are the CTAs of one thread-block cluster (1, 2, 4 or 8):
-// every CTA owns a slice of the tile's rows, the CTAs send the rows of their accumulators to the
-// owners' shared memory, and an owner adds the parts in rank order and writes (or adds to) dW.  Nothing goes through a workspace, there are no atomics on
-// data, the result is deterministic, and every mbarrier wait is bounded.
+// A CTA pair owns a tile of 256 output rows (columns of U) x 256 output columns (columns of X) and
+// one part of the contraction range (the rows of the sub-batch), in blocks of 64 rows:
+//   16 converter warps read U straight from global memory (two blocks ahead, in registers), form hi and
+//                   lo and write them as two MN-major A operands in the 128-byte swizzle; they run the
+//                   epilogue too
+//   producer warp   bulk tensor loads of X, an MN-major B operand as it lies in memory
+//   MMA warp        the leader's: 8 instructions of M = 256, N = 256 per block
+// With one part the tile goes to dW; otherwise each part is a plane of the workspace and a second
+// kernel adds the planes in order.  No atomics, deterministic, every mbarrier wait is bounded.
+//
+// What bounds it at 4096 x 768 x 768 (9 tiles x 8 parts, 18.8 us): reading U and X once (3 us from
+// memory, 3.6 until the first product), a block each 0.72 us against 0.55 of products, 3.8 us from the
+// last product to the stored planes, 5 us for the second launch.  Sixteen converter warps, a float4
+// of a row per lane: with eight, and two float4 per lane, a block took 0.85-1.1 us.  Before, one launch
+// of clusters of single CTAs that exchanged their parts through shared memory: 22.8 us (32768 x 384 x
+// 384: 84 / 35, 8192 x 128 x 384: 31 / 15, 4096 x 2048 x 2048: 93 / 50).
 #include <cuda_bf16.h>
 
 #include "tc_common.cuh"
@@ -28,277 +32,273 @@ namespace gc {
 
 namespace {
 
-constexpr int AK = 32;                         // contraction rows per pipeline step
-constexpr int ATM = 128;                       // output rows per CTA = MMA M
-constexpr int ATN = 384;                       // output columns per CTA (at most): MMAs of N <= 256
-constexpr int A_NS = 4;                        // load stages
-constexpr int A_NA = 2;                        // converted-operand stages
-constexpr uint32_t BLOCK_BYTES = AK * 128;     // 32 rows of 128 bytes: one box, one operand atom
-constexpr uint32_t U_STAGE = 4 * BLOCK_BYTES;  // 128 fp32 columns = 4 boxes of 32
-constexpr uint32_t X_STAGE = 6 * BLOCK_BYTES;  // 384 bf16 columns = 6 boxes of 64
-constexpr uint32_t LD_STAGE = U_STAGE + X_STAGE;
-constexpr uint32_t A_HALF = 2 * BLOCK_BYTES;   // hi (or lo) of 128 output rows x 32
-constexpr uint32_t A_STAGE = 2 * A_HALF;
-constexpr int CONV_WARPS = 4;
-constexpr int APPLY_PROD_WARP = CONV_WARPS;
-constexpr int APPLY_MMA_WARP = CONV_WARPS + 1;
-constexpr int APPLY_THREADS = 32 * (CONV_WARPS + 2);
-constexpr int APPLY_TMEM_COLS = 512;
-constexpr size_t APPLY_DYN_SMEM = 1024 + (size_t)A_NS * LD_STAGE + (size_t)A_NA * A_STAGE;
-constexpr int MAX_SPLITS = 8;                  // portable cluster size
+constexpr int AP_KB = 64;                      // contraction rows per stage
+constexpr int AP_CONV = 16;                    // converter / epilogue warps
+constexpr int AP_PROD_WARP = AP_CONV;
+constexpr int AP_MMA_WARP = AP_CONV + 1;
+constexpr int AP_THREADS = 32 * (AP_CONV + 2);
+constexpr int AP_STAGES = 3;
+constexpr int AP_AHEAD = 3;                    // blocks of U held in registers
+constexpr uint32_t AP_ATOM = 64 * 128;         // 64 contraction rows x 64 columns of bf16
+constexpr uint32_t AP_STAGE = 6 * AP_ATOM;     // hi (2 atoms), lo (2 atoms), X (2 atoms)
+constexpr size_t AP_SMEM = 1024 + (size_t)AP_STAGES * AP_STAGE + AP_CONV * 4096;
+constexpr int AP_MAX_PARTS = 32;
 
-static_assert((size_t)ATM * ATN * 4 <= (size_t)A_NS * LD_STAGE + (size_t)A_NA * A_STAGE,
-              "the accumulator copy fits the pipeline's shared memory");
-
-static_assert(APPLY_DYN_SMEM <= SMEM_LIMIT - SMEM_STATIC_RESERVE, "shared memory budget");
+static_assert(AP_SMEM <= SMEM_LIMIT - 1024, "shared memory budget");
 
 struct ApplyParams {
-    int64_t rows;
+    const float* U;
+    int64_t ldu, rows;
     int d, d_in;
-    int tiles_n;              // tiles along d_in
-    int splits;               // parts of the contraction range = cluster size
-    float* dW;
-    int64_t lddw;
-    int accumulate;
+    int tiles_n, tiles;           // column tiles, all tiles
+    int parts, kblocks;
+    int add;                      // one part: add to dW
     int* dev_status;
 };
 
-struct ApplyBars {
-    uint64_t full[A_NS];
-    uint64_t empty[A_NS];
-    uint64_t a_full[A_NA];
-    uint64_t a_empty[A_NA];
+struct __align__(16) ApplyBars {
+    uint64_t signal[2 * AP_CONV];         // what the second CTA's converters send along with their signal
+    uint64_t full[AP_STAGES];             // leader: X of both CTAs
+    uint64_t conv[AP_STAGES];             // leader: hi and lo of both CTAs
+    uint64_t empty[AP_STAGES];
     uint64_t acc_full;
+    uint64_t acc_free, acc_free_peer;
 };
 
-__device__ __forceinline__ float4 lds128(uint32_t addr) {
-    float4 v;
-    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
-                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
-    return v;
-}
-__device__ __forceinline__ void st_cluster128(uint32_t cluster_addr, uint32_t a, uint32_t b,
-                                              uint32_t c, uint32_t d) {
-    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};"
-                 ::"r"(cluster_addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
-}
-__device__ __forceinline__ void sts128(uint32_t addr, uint32_t a, uint32_t b, uint32_t c,
-                                       uint32_t d) {
-    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};"
-                 ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
-}
-// (x, y) -> packed bf16 pair hi and the packed pair of the rounded remainders
-__device__ __forceinline__ void split2(float x, float y, uint32_t* hi, uint32_t* lo) {
-    const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
-    const uint32_t hb = *reinterpret_cast<const uint32_t*>(&h);
-    const float hx = __uint_as_float(hb << 16), hy = __uint_as_float(hb & 0xffff0000u);
-    const __nv_bfloat162 l = __floats2bfloat162_rn(x - hx, y - hy);
-    *hi = hb;
-    *lo = *reinterpret_cast<const uint32_t*>(&l);
-}
-
-__global__ void __launch_bounds__(APPLY_THREADS, 1)
-apply_kernel(const __grid_constant__ CUtensorMap mapU, const __grid_constant__ CUtensorMap mapX,
+__global__ void __launch_bounds__(AP_THREADS, 1)
+apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapO,
              const ApplyParams p) {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) ApplyBars bars;
-    __shared__ uint32_t tmem_base_s;
+    __shared__ ApplyBars bars;
+    __shared__ uint32_t tmem_s;
     __shared__ int abort_s;
     volatile int* abort_flag = &abort_s;
-
-    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);   // warp-uniform
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
     const int lane = threadIdx.x & 31;
-
-    // work item: (row tile, column tile, part of the contraction range); the parts of a tile are
-    // the CTAs of one cluster
-    const int split = (int)cluster_ctarank();
-    const int tile = (int)(blockIdx.x / (unsigned)p.splits);
-    const int m0 = (tile / p.tiles_n) * ATM;
-    const int n0 = (tile % p.tiles_n) * ATN;
-    const int n_cols = min(ATN, p.d_in - n0);          // a multiple of 64
-    int64_t lo, hi;
-    part_range((p.rows + AK - 1) / AK, p.splits, split, &lo, &hi);
-    const int T = (int)(hi - lo);
-
-    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    const uint32_t ld_smem = base;
-    const uint32_t a_smem = base + A_NS * LD_STAGE;
-
+    const uint32_t rank = cluster_ctarank();
+    const uint32_t smem = (smem_u32(smem_raw) + 1023u) & ~1023u;
     if (threadIdx.x == 0) {
         abort_s = 0;
-        for (int s = 0; s < A_NS; ++s) {
+        for (int s = 0; s < AP_STAGES; ++s) {
             mbar_init(smem_u32(&bars.full[s]), 1);
+            mbar_init(smem_u32(&bars.conv[s]), AP_CONV);
             mbar_init(smem_u32(&bars.empty[s]), 1);
         }
-        for (int s = 0; s < A_NA; ++s) {
-            mbar_init(smem_u32(&bars.a_full[s]), CONV_WARPS);
-            mbar_init(smem_u32(&bars.a_empty[s]), 1);
-        }
         mbar_init(smem_u32(&bars.acc_full), 1);
+        mbar_init(smem_u32(&bars.acc_free), AP_CONV);
+        mbar_init(smem_u32(&bars.acc_free_peer), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == APPLY_MMA_WARP) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     ::"r"(smem_u32(&tmem_base_s)), "r"((uint32_t)APPLY_TMEM_COLS) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if (warp == AP_MMA_WARP) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;"
+                     ::"r"(smem_u32(&tmem_s)), "r"(256u) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
     tc_fence_before();
     __syncthreads();
+    cluster_sync_all();
     tc_fence_after();
-    const uint32_t tmem = tmem_base_s;
-    bool acc_ok = false;
+    const uint32_t tmem = tmem_s;
+    dep_release();
+    dep_wait();
 
-    if (warp == APPLY_PROD_WARP) {
-        // ------------------------------ loads -----------------------------------------------------
-        // Columns past d (of U) or rows past the sub-batch read as zeros and add nothing.
-        const int atoms = n_cols / 64;
+    const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
+    const int units = p.tiles * p.parts;           // unit: (part, tile), tiles fastest
+    struct Unit { int m0, n0, bw, part, kb, kb_end; };
+    auto unit_at = [&](int u) {
+        Unit t;
+        t.part = u / p.tiles;
+        const int tile = u - t.part * p.tiles;
+        t.m0 = tile / p.tiles_n * 256 + (int)rank * 128;
+        t.n0 = tile % p.tiles_n * 256;
+        t.bw = p.d_in - t.n0 <= 128 ? 64 : 128;    // columns of X this CTA loads
+        t.kb = (int)((int64_t)p.kblocks * t.part / p.parts);
+        t.kb_end = (int)((int64_t)p.kblocks * (t.part + 1) / p.parts);
+        return t;
+    };
+
+    if (warp == AP_PROD_WARP) {
         int stage = 0;
         uint32_t phase = 0;
-        for (int t = 0; t < T; ++t) {
-            if (!mbar_wait(smem_u32(&bars.empty[stage]), phase ^ 1u, abort_flag)) break;
-            const uint32_t full = smem_u32(&bars.full[stage]);
-            const uint32_t dst = ld_smem + stage * LD_STAGE;
-            const int k0 = (int)(lo + t) * AK;
-            if (elect_one()) {
-                mbar_expect_tx(full, U_STAGE + (uint32_t)atoms * BLOCK_BYTES);
-#pragma unroll
-                for (int b = 0; b < 4; ++b)
-                    tma_load_2d(dst + b * BLOCK_BYTES, &mapU, m0 + 32 * b, k0, full);
-                for (int b = 0; b < atoms; ++b)
-                    tma_load_2d(dst + U_STAGE + b * BLOCK_BYTES, &mapX, n0 + 64 * b, k0, full);
-            }
-            if (++stage == A_NS) { stage = 0; phase ^= 1u; }
-        }
-    } else if (warp == APPLY_MMA_WARP) {
-        // ------------------------------ MMA issuer ------------------------------------------------
-        const int n1 = min(256, n_cols), n2 = n_cols - n1;        // n2 = 0, 64 or 128
-        const uint32_t idesc1 = instr_desc(n1, true, ATM, true);
-        const uint32_t idesc2 = instr_desc(n2 > 0 ? n2 : 64, true, ATM, true);
-        constexpr uint32_t B2 = (4 * BLOCK_BYTES) >> 4;           // columns 256.. of the X block
-        int s = 0, a = 0;
-        uint32_t ps = 0, pa = 0;
         bool ok = true;
-        for (int t = 0; t < T; ++t) {
-            ok = mbar_wait(smem_u32(&bars.full[s]), ps, abort_flag) &&
-                 mbar_wait(smem_u32(&bars.a_full[a]), pa, abort_flag);
-            if (!ok) break;
-            tc_fence_after();
-            const uint32_t hi_lo = desc_lo(a_smem + a * A_STAGE, BLOCK_BYTES);
-            const uint32_t lo_lo = desc_lo(a_smem + a * A_STAGE + A_HALF, BLOCK_BYTES);
-            const uint32_t b_lo = desc_lo(ld_smem + s * LD_STAGE + U_STAGE, BLOCK_BYTES);
-            if (elect_one()) {
+        for (int u = pair; u < units && ok; u += pairs) {
+            const Unit t = unit_at(u);
+            for (int kb = t.kb; kb < t.kb_end; ++kb) {
+                ok = mbar_wait(smem_u32(&bars.empty[stage]), phase ^ 1u, abort_flag);
+                if (!ok) break;
+                const uint32_t full = smem_u32(&bars.full[stage]), full_leader = mapa_u32(full, 0);
+                const uint32_t dst = smem + stage * AP_STAGE + 4 * AP_ATOM;
+                const int n = t.n0 + (int)rank * t.bw;
+                if (elect_one()) {
+                    if (rank == 0) mbar_expect_tx(full, 2u * 128u * (uint32_t)t.bw);
+                    tma_load_2d_pair(dst, &mapX, n, kb * AP_KB, full_leader);
+                    if (t.bw == 128) tma_load_2d_pair(dst + AP_ATOM, &mapX, n + 64, kb * AP_KB, full_leader);
+                }
+                if (++stage == AP_STAGES) { stage = 0; phase ^= 1u; }
+            }
+        }
+    } else if (warp == AP_MMA_WARP) {
+        int n_unit = 0;
+        bool ok = true;
+        if (rank == 0) {
+            int stage = 0;
+            uint32_t phase = 0;
+            for (int u = pair; u < units && ok; u += pairs, ++n_unit) {
+                const Unit t = unit_at(u);
+                const uint32_t idesc = instr_desc(2 * t.bw, true, 256, true);
+                const uint32_t par = ((uint32_t)n_unit & 1u) ^ 1u;
+                ok = mbar_wait(smem_u32(&bars.acc_free), par, abort_flag) &&
+                     mbar_wait(smem_u32(&bars.acc_free_peer), par, abort_flag);
+                if (!ok) break;
+                tc_fence_after();
+                for (int kb = t.kb; kb < t.kb_end; ++kb) {
+                    ok = mbar_wait(smem_u32(&bars.full[stage]), phase, abort_flag) &&
+                         mbar_wait(smem_u32(&bars.conv[stage]), phase, abort_flag);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t a = desc_lo(smem + stage * AP_STAGE, AP_ATOM);
+                    const uint32_t b = desc_lo(smem + stage * AP_STAGE + 4 * AP_ATOM, AP_ATOM);
+                    if (elect_one()) {
 #pragma unroll
-                for (int k = 0; k < AK / 16; ++k) {      // 16 rows of an MN-major operand: 2 KB
-                    const uint32_t ah = hi_lo + k * 128, al = lo_lo + k * 128, b = b_lo + k * 128;
-                    if (t == 0 && k == 0) mma_ss<false, false>(tmem, ah, b, idesc1);
-                    else                  mma_ss<true, false>(tmem, ah, b, idesc1);
-                    mma_ss<true, false>(tmem, al, b, idesc1);
-                    if (n2 > 0) {
-                        if (t == 0 && k == 0) mma_ss<false, false>(tmem + 256, ah, b + B2, idesc2);
-                        else                  mma_ss<true, false>(tmem + 256, ah, b + B2, idesc2);
-                        mma_ss<true, false>(tmem + 256, al, b + B2, idesc2);
+                        for (int k = 0; k < AP_KB / 16; ++k) {
+                            if (k == 0 && kb == t.kb) mma_ss<false, true>(tmem, a, b, idesc);
+                            else mma_ss<true, true>(tmem, a + 128 * k, b + 128 * k, idesc);
+                            mma_ss<true, true>(tmem, a + (2 * AP_ATOM >> 4) + 128 * k, b + 128 * k, idesc);
+                        }
+                        tc_commit_pair(smem_u32(&bars.empty[stage]));
+                        if (kb == t.kb_end - 1) tc_commit_pair(smem_u32(&bars.acc_full));
+                    }
+                    if (++stage == AP_STAGES) { stage = 0; phase ^= 1u; }
+                }
+            }
+        } else {
+            for (int u = pair; u < units && ok; u += pairs, ++n_unit) {
+                ok = mbar_wait(smem_u32(&bars.acc_free), (uint32_t)n_unit & 1u, abort_flag);
+                if (ok && elect_one()) mbar_arrive_cluster(mapa_u32(smem_u32(&bars.acc_free_peer), 0));
+            }
+        }
+    } else {
+        // Piece of a block: one contraction row x 4 columns of U, one 16-byte load in, one 8-byte store
+        // per term out.  A warp takes whole rows of 128 columns: loads are contiguous, and the stores of
+        // a half warp fall on distinct banks.
+        constexpr int ROWS = AP_KB / AP_CONV;      // of a warp: warp, warp + 16, ...
+        const int col = lane * 4, row0 = warp;
+        const int q = warp & 3, group = warp >> 2; // epilogue: lane quarter, quarter of the columns
+        // the same place in every row and stage: 16 rows further is the same phase of the swizzle
+        const uint32_t place = (uint32_t)(col >> 6) * AP_ATOM + (uint32_t)row0 * 128u +
+                               (uint32_t)((((col & 63) >> 3) ^ (row0 & 7)) << 4) + (uint32_t)(col & 4) * 2u;
+        const int64_t step = (int64_t)AP_CONV * p.ldu;
+        const uint32_t slot = smem + AP_STAGES * AP_STAGE + (uint32_t)warp * 4096u;
+        int stage = 0, n_unit = 0;
+        uint32_t phase = 0;
+        bool ok = true;
+        for (int u = pair; u < units && ok; u += pairs, ++n_unit) {
+            const Unit t = unit_at(u);
+            const bool live = t.m0 + col < p.d;    // d is a multiple of 8
+            const float* src = p.U + (live ? t.m0 + col : 0) + ((int64_t)t.kb * AP_KB + row0) * p.ldu;
+            float4 x[AP_AHEAD][ROWS];
+            // block kb; called once for every block in order
+            auto fetch = [&](float4 (&v)[ROWS], int kb) {
+                const int64_t left = p.rows - (int64_t)kb * AP_KB;         // rows from the block's first on
+                if (kb < t.kb_end && live && left >= AP_KB) {
+#pragma unroll
+                    for (int i = 0; i < ROWS; ++i) v[i] = __ldg(reinterpret_cast<const float4*>(src + i * step));
+                } else {
+#pragma unroll
+                    for (int i = 0; i < ROWS; ++i) {
+                        const bool in = kb < t.kb_end && live && row0 + AP_CONV * i < left;
+                        v[i] = in ? __ldg(reinterpret_cast<const float4*>(src + i * step))
+                                  : make_float4(0.f, 0.f, 0.f, 0.f);
                     }
                 }
-                tc_commit(smem_u32(&bars.empty[s]));
-                tc_commit(smem_u32(&bars.a_empty[a]));
-            }
-            if (++s == A_NS) { s = 0; ps ^= 1u; }
-            if (++a == A_NA) { a = 0; pa ^= 1u; }
-        }
-        if (ok && elect_one()) tc_commit(smem_u32(&bars.acc_full));
-    } else {
-        // ------------------------------ converter warps -------------------------------------------
-        // Item = 8 consecutive output rows m (one 16-byte piece of bf16) of contraction row k.
-        // Eight neighbouring threads share k and cover one 128-byte operand row, so their stores
-        // fall on distinct banks; their fp32 sources are two boxes, and the halves of a thread's
-        // 32 bytes are fetched in opposite order in the two boxes so that the loads do too.
-        const int tid = threadIdx.x;
-        int s = 0, a = 0;
-        uint32_t ps = 0, pa = 0;
-        for (int t = 0; t < T; ++t) {
-            if (!mbar_wait(smem_u32(&bars.full[s]), ps, abort_flag)) break;
-            if (!mbar_wait(smem_u32(&bars.a_empty[a]), pa ^ 1u, abort_flag)) break;
-            const uint32_t u_base = ld_smem + s * LD_STAGE;
-            const uint32_t hi_base = a_smem + a * A_STAGE, lo_base = hi_base + A_HALF;
+                src += (int64_t)AP_KB * p.ldu;
+            };
+            auto convert = [&](const float4 (&v)[ROWS]) {
+                const uint32_t dst0 = smem + stage * AP_STAGE + place;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int id = tid + 128 * i;
-                const int j = id & 7, atom = (id >> 3) & 1, k = id >> 4;
-                const int sw = k & 7;
-                const int odd = j >> 2;
-                const int c = 2 * (j & 3);
-                const uint32_t row = u_base + (uint32_t)(2 * atom + odd) * BLOCK_BYTES + k * 128;
-                const float4 A = lds128(row + (uint32_t)(((c ^ odd) ^ sw) << 4));
-                const float4 B = lds128(row + (uint32_t)(((c ^ odd ^ 1) ^ sw) << 4));
-                const float4 f0 = odd ? B : A, f1 = odd ? A : B;
-                uint32_t h[4], l[4];
-                split2(f0.x, f0.y, &h[0], &l[0]);
-                split2(f0.z, f0.w, &h[1], &l[1]);
-                split2(f1.x, f1.y, &h[2], &l[2]);
-                split2(f1.z, f1.w, &h[3], &l[3]);
-                const uint32_t off = (uint32_t)atom * BLOCK_BYTES + k * 128 + ((j ^ sw) << 4);
-                sts128(hi_base + off, h[0], h[1], h[2], h[3]);
-                sts128(lo_base + off, l[0], l[1], l[2], l[3]);
+                for (int i = 0; i < ROWS; ++i) {
+                    const float f[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+                    uint32_t hi[2], lo[2];
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const __nv_bfloat162 h = __floats2bfloat162_rn(f[2 * e], f[2 * e + 1]);
+                        hi[e] = *reinterpret_cast<const uint32_t*>(&h);
+                        const __nv_bfloat162 g =
+                            __floats2bfloat162_rn(f[2 * e] - __uint_as_float(hi[e] << 16),
+                                                  f[2 * e + 1] - __uint_as_float(hi[e] & 0xffff0000u));
+                        lo[e] = *reinterpret_cast<const uint32_t*>(&g);
+                    }
+                    const uint32_t dst = dst0 + (uint32_t)i * (AP_CONV * 128u);
+                    asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(dst), "r"(hi[0]), "r"(hi[1]) : "memory");
+                    asm volatile("st.shared.v2.b32 [%0], {%1, %2};"
+                                 ::"r"(dst + 2 * AP_ATOM), "r"(lo[0]), "r"(lo[1]) : "memory");
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                // a remote arrival would stall the warp; 16 bytes that the leader's barrier counts do not
+                if (lane == 0) {
+                    const uint32_t bar = smem_u32(&bars.conv[stage]);
+                    const uint32_t box = smem_u32(&bars.signal[2 * warp]);
+                    if (rank != 0)
+                        asm volatile(
+                            "cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes "
+                            "[%0], [%1], 16, [%2];"
+                            ::"r"(mapa_u32(box, 0)), "r"(box), "r"(mapa_u32(bar, 0)) : "memory");
+                    else if (warp == 0) mbar_expect_tx(bar, 16 * AP_CONV);
+                    else                mbar_arrive(bar);
+                }
+            };
+#pragma unroll
+            for (int a = 0; a < AP_AHEAD; ++a) fetch(x[a], t.kb + a);
+            for (int kb = t.kb; kb < t.kb_end && ok; kb += AP_AHEAD) {
+#pragma unroll
+                for (int a = 0; a < AP_AHEAD; ++a) {
+                    if (kb + a >= t.kb_end) break;
+                    ok = mbar_wait(smem_u32(&bars.empty[stage]), phase ^ 1u, abort_flag);
+                    if (!ok) break;
+                    convert(x[a]);
+                    fetch(x[a], kb + a + AP_AHEAD);
+                    if (++stage == AP_STAGES) { stage = 0; phase ^= 1u; }
+                }
             }
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // visible to the MMAs
+            if (!ok) break;
+            ok = mbar_wait(smem_u32(&bars.acc_full), (uint32_t)n_unit & 1u, abort_flag);
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t src_t = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(group * (t.bw / 2));
+            const int r_out = t.m0 + 32 * q;
+            for (int cb = 0; 32 * cb < t.bw / 2; ++cb) {
+                uint32_t v[32];
+                tmem_ld32(src_t + 32 * cb, v);
+                if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+                __syncwarp();
+                tmem_ld_wait();
+                stage_block(slot, v, 1.f, lane);
+                __syncwarp();
+                const int c_out = t.n0 + group * (t.bw / 2) + 32 * cb;
+                if (lane == 0 && r_out < p.d && c_out < p.d_in) {
+                    if (p.add) {
+                        asm volatile(
+                            "cp.reduce.async.bulk.tensor.3d.global.shared::cta.add.bulk_group "
+                            "[%0, {%2, %3, %4}], [%1];"
+                            ::"l"(reinterpret_cast<uint64_t>(&mapO)), "r"(slot), "r"(c_out), "r"(r_out), "r"(0)
+                            : "memory");
+                        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                    } else {
+                        tma_store_3d(&mapO, slot, c_out, r_out, p.parts > 1 ? t.part : 0);
+                    }
+                }
+            }
+            tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&bars.a_full[a]));
-            if (++s == A_NS) { s = 0; ps ^= 1u; }
-            if (++a == A_NA) { a = 0; pa ^= 1u; }
+            if (lane == 0) mbar_arrive(smem_u32(&bars.acc_free));
         }
-        acc_ok = mbar_wait(smem_u32(&bars.acc_full), 0, abort_flag);   // all MMAs have completed
-    }
-
-    // ------------------------------ sum over the parts -------------------------------------------
-    // Rank g of the cluster owns rows [g, g + 1) * 128 / splits of the tile.  Once every CTA's
-    // pipeline buffers are free (first cluster barrier) each CTA sends the rows of its accumulator
-    // to their owners' shared memory, slot [sender][float4 piece q][row]; after the second barrier
-    // an owner adds the senders' slots in rank order and writes (or adds to) dW.
-    const int rows_per = ATM / p.splits;
-    tc_fence_before();
-    cluster_sync_all();            // every CTA gets here, aborted or not
-    if (warp < CONV_WARPS && acc_ok) {
-        tc_fence_after();
-        const int r = threadIdx.x;                              // warp w reads lanes 32 w ..
-        const int owner = r / rows_per, r_local = r - owner * rows_per;
-        const uint32_t dst = mapa_u32(base, (uint32_t)owner) +
-                             (uint32_t)((split * (ATN / 4)) * rows_per + r_local) * 16;
-        const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16);
-        for (int cb = 0; cb < n_cols / 32; ++cb) {
-            uint32_t v[32];
-            tmem_ld32(taddr + cb * 32, v);
-            tmem_ld_wait();
-#pragma unroll
-            for (int q = 0; q < 8; ++q)
-                st_cluster128(dst + (uint32_t)((cb * 8 + q) * rows_per) * 16, v[4 * q], v[4 * q + 1],
-                              v[4 * q + 2], v[4 * q + 3]);
-        }
-    }
-    tc_fence_before();
-    cluster_sync_all();            // the slots of this CTA are complete
-    if (!*abort_flag) {
-        const int items = (n_cols / 4) * rows_per;
-        for (int idx = threadIdx.x; idx < items; idx += APPLY_THREADS) {
-            const int q = idx / rows_per;
-            const int r_local = idx - q * rows_per;
-            const int r = split * rows_per + r_local;
-            if (m0 + r >= p.d) continue;
-            const uint32_t src = base + (uint32_t)(q * rows_per + r_local) * 16;
-            float4* dst = reinterpret_cast<float4*>(p.dW + (int64_t)(m0 + r) * p.lddw + n0 + 4 * q);
-            float4 v[MAX_SPLITS];
-#pragma unroll
-            for (int g = 0; g < MAX_SPLITS; ++g)
-                if (g < p.splits) v[g] = lds128(src + (uint32_t)(g * (ATN / 4) * rows_per) * 16);
-            float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (p.accumulate) sum = *dst;
-#pragma unroll
-            for (int g = 0; g < MAX_SPLITS; ++g)
-                if (g < p.splits) { sum.x += v[g].x; sum.y += v[g].y; sum.z += v[g].z; sum.w += v[g].w; }
-            *dst = sum;
-        }
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+        __syncwarp();
     }
 
     // ------------------------------ teardown ------------------------------------------------------
+    tc_fence_before();
     __syncthreads();
     if (*abort_flag) {
         // let bulk copies still in flight land before the shared memory is released
@@ -307,37 +307,64 @@ apply_kernel(const __grid_constant__ CUtensorMap mapU, const __grid_constant__ C
         if (threadIdx.x == 0 && p.dev_status) atomicOr(p.dev_status, GC_DEV_WAIT_LIMIT);
         __syncthreads();
     }
-    if (warp == APPLY_MMA_WARP) {
+    cluster_sync_all();   // the peer's MMAs, loads and signals no longer touch this CTA
+    if (warp == AP_MMA_WARP) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;"
-                     ::"r"(tmem), "r"((uint32_t)APPLY_TMEM_COLS) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;"
+                     ::"r"(tmem), "r"(256u) : "memory");
+    }
+}
+
+// dW (+)= sum of the planes, in order.
+__global__ void __launch_bounds__(256)
+apply_reduce_kernel(const float4* __restrict__ planes, int parts, int64_t plane, int n4,
+                    float* __restrict__ dW, int64_t lddw, int add) {
+    dep_release();
+    dep_wait();
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < plane;
+         e += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t r = e / n4;
+        float4* dst = reinterpret_cast<float4*>(dW + r * lddw) + (e - r * n4);
+        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (add) s = *dst;
+#pragma unroll 8
+        for (int g = 0; g < parts; ++g) {
+            const float4 v = __ldcg(planes + g * plane + e);
+            s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+        }
+        *dst = s;
     }
 }
 
 struct ApplyPlan {
-    int tiles_m, tiles_n, splits;
+    int tiles_m, tiles_n, parts, kblocks;
 };
 
-// Parts of the contraction range = cluster size: the largest of 8, 4, 2, 1 whose clusters can
-// all be resident at once (a cluster of c CTAs needs c free SMs in one GPC: about SMs / 9
-// clusters of 8, SMs / 4.5 of 4, SMs / 2 of 2) with at least four steps per part.
+// As many parts as pairs are left per tile (one wave), up to AP_MAX_PARTS and one block each: the
+// products of a second wave would cost more than the planes of a part save.
+int most_parts(int64_t tiles) {
+    const int64_t per = sm_count() / 2 / tiles;
+    return per < 1 ? 1 : per > AP_MAX_PARTS ? AP_MAX_PARTS : (int)per;
+}
 ApplyPlan make_apply_plan(int64_t rows, int d, int d_in) {
     ApplyPlan pl{};
-    pl.tiles_m = (d + ATM - 1) / ATM;
-    pl.tiles_n = (d_in + ATN - 1) / ATN;
-    const int64_t tiles = (int64_t)pl.tiles_m * pl.tiles_n;
-    const int64_t steps = (rows + AK - 1) / AK;
-    const int sms = sm_count();
-    int c = 1;
-    if (tiles <= sms / 2 && steps >= 8) c = 2;
-    if (tiles * 2 <= sms * 4 / 9 && steps >= 16) c = 4;
-    if (tiles * 9 <= sms && steps >= 32) c = 8;
-    pl.splits = c;
+    pl.tiles_m = (d + 255) / 256;
+    pl.tiles_n = (d_in + 255) / 256;
+    pl.kblocks = (int)((rows + AP_KB - 1) / AP_KB);
+    pl.parts = most_parts((int64_t)pl.tiles_m * pl.tiles_n);
+    if (pl.parts > pl.kblocks) pl.parts = pl.kblocks;
     return pl;
 }
 
 bool apply_shape_ok(int64_t rows, int d, int d_in) {
     return rows > 0 && rows <= ((int64_t)1 << 30) && d > 0 && d_in > 0 && d <= (1 << 20);
+}
+
+// The planes of the most parts these widths can take, whatever the rows.
+size_t apply_ws(int d, int d_in) {
+    const int parts = most_parts((int64_t)((d + 255) / 256) * ((d_in + 255) / 256));
+    if (parts == 1) return 256;
+    return ((size_t)parts * (size_t)d * (size_t)d_in * 4 + 255) & ~(size_t)255;
 }
 
 }  // namespace
@@ -350,7 +377,7 @@ extern "C" {
 
 size_t gc_cache_apply_workspace_bytes(int64_t rows, int d, int d_in) {
     if (!apply_shape_ok(rows, d, d_in) || d % 8 != 0 || d_in % 64 != 0 || d_in > 4096) return 0;
-    return 256;       // nothing is staged in global memory; the call accepts any such buffer
+    return apply_ws(d, d_in);
 }
 
 int gc_cache_apply(const float* U, int64_t ldu, const void* X, int64_t ldx, int64_t rows, int d,
@@ -363,8 +390,7 @@ int gc_cache_apply(const float* U, int64_t ldu, const void* X, int64_t ldx, int6
     if (((uintptr_t)U & 15) || ((uintptr_t)X & 15) || ((uintptr_t)dW & 15) || (ldu * 4) % 16 ||
         (ldx * 2) % 16 || (lddw * 4) % 16)
         return GC_ERR_ALIGN;
-    const ApplyPlan pl = make_apply_plan(rows, d, d_in);
-    if (!ws || ((uintptr_t)ws & 255) || ws_bytes < 256) return GC_ERR_WORKSPACE;
+    if (!ws || ((uintptr_t)ws & 255) || ws_bytes < apply_ws(d, d_in)) return GC_ERR_WORKSPACE;
     int dev = 0, major = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess) {
@@ -374,38 +400,55 @@ int gc_cache_apply(const float* U, int64_t ldu, const void* X, int64_t ldx, int6
     if (major != 10) return GC_ERR_ARCH;
     if (dev < 0 || dev >= 64) return GC_ERR_CUDA;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-
-    CUtensorMap mu, mx;
-    if (!make_map_f32(&mu, U, rows, d, ldu, AK) || !make_map(&mx, X, rows, d_in, ldx, AK))
+    const ApplyPlan pl = make_apply_plan(rows, d, d_in);
+    float* planes = static_cast<float*>(ws);
+    CUtensorMap mx, mo;
+    if (!make_map(&mx, X, rows, d_in, ldx, AP_KB) ||
+        !(pl.parts > 1 ? make_out_map(&mo, planes, d, d_in, d_in, pl.parts)
+                       : make_out_map(&mo, dW, d, d_in, lddw, 1)))
         return GC_ERR_CUDA;
     ApplyParams p{};
-    p.rows = rows; p.d = d; p.d_in = d_in;
-    p.tiles_n = pl.tiles_n; p.splits = pl.splits;
-    p.dW = dW; p.lddw = lddw; p.accumulate = accumulate ? 1 : 0;
+    p.U = U; p.ldu = ldu; p.rows = rows; p.d = d; p.d_in = d_in;
+    p.tiles_n = pl.tiles_n; p.tiles = pl.tiles_m * pl.tiles_n;
+    p.parts = pl.parts; p.kblocks = pl.kblocks;
+    p.add = pl.parts == 1 && accumulate;
     p.dev_status = dev_status;
 
     static bool configured_on[64] = {false};      // the attribute belongs to (kernel, device)
     if (!configured_on[dev]) {
         if (cudaFuncSetAttribute(apply_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)APPLY_DYN_SMEM) != cudaSuccess) {
+                                 (int)AP_SMEM) != cudaSuccess) {
             cudaGetLastError();
             return GC_ERR_CUDA;
         }
         configured_on[dev] = true;
     }
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((int64_t)pl.tiles_m * pl.tiles_n * pl.splits));
-    cfg.blockDim = dim3(APPLY_THREADS);
-    cfg.dynamicSmemBytes = APPLY_DYN_SMEM;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 2;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)pl.splits;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, apply_kernel, mu, mx, p);
+    const int64_t units = (int64_t)p.tiles * p.parts, pairs = sm_count() / 2;
+    cfg.gridDim = dim3(2u * (unsigned)(units < pairs ? units : pairs));
+    cfg.blockDim = dim3(AP_THREADS);
+    cfg.dynamicSmemBytes = AP_SMEM;
+    cfg.numAttrs = 2;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, apply_kernel, mx, mo, p);
+    if (e == cudaSuccess && pl.parts > 1) {
+        const int64_t plane = (int64_t)d * (d_in / 4);
+        const int64_t blocks = (plane + 255) / 256, most = 8 * (int64_t)sm_count();
+        cfg.gridDim = dim3((unsigned)(blocks < most ? blocks : most));
+        cfg.blockDim = dim3(256);
+        cfg.dynamicSmemBytes = 0;
+        cfg.numAttrs = 1;
+        e = cudaLaunchKernelEx(&cfg, apply_reduce_kernel, reinterpret_cast<const float4*>(planes), pl.parts,
+                               plane, d_in / 4, dW, lddw, accumulate ? 1 : 0);
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
         return GC_ERR_CUDA;
