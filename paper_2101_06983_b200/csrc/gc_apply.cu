@@ -423,31 +423,15 @@ int gc_cache_apply(const float* U, int64_t ldu, const void* X, int64_t ldx, int6
         }
         configured_on[dev] = true;
     }
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = 2;
-    attr[1].val.clusterDim.y = 1;
-    attr[1].val.clusterDim.z = 1;
-    cfg.stream = st;
-    cfg.attrs = attr;
     const int64_t units = (int64_t)p.tiles * p.parts, pairs = sm_count() / 2;
-    cfg.gridDim = dim3(2u * (unsigned)(units < pairs ? units : pairs));
-    cfg.blockDim = dim3(AP_THREADS);
-    cfg.dynamicSmemBytes = AP_SMEM;
-    cfg.numAttrs = 2;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, apply_kernel, mx, mo, p);
+    cudaError_t e = launch_chained(apply_kernel, dim3(2u * (unsigned)(units < pairs ? units : pairs)),
+                                   AP_THREADS, AP_SMEM, 2, st, mx, mo, p);
     if (e == cudaSuccess && pl.parts > 1) {
         const int64_t plane = (int64_t)d * (d_in / 4);
         const int64_t blocks = (plane + 255) / 256, most = 8 * (int64_t)sm_count();
-        cfg.gridDim = dim3((unsigned)(blocks < most ? blocks : most));
-        cfg.blockDim = dim3(256);
-        cfg.dynamicSmemBytes = 0;
-        cfg.numAttrs = 1;
-        e = cudaLaunchKernelEx(&cfg, apply_reduce_kernel, reinterpret_cast<const float4*>(planes), pl.parts,
-                               plane, d_in / 4, dW, lddw, accumulate ? 1 : 0);
+        e = launch_chained(apply_reduce_kernel, dim3((unsigned)(blocks < most ? blocks : most)), 256, 0, 1,
+                           st, reinterpret_cast<const float4*>(planes), pl.parts, plane, d_in / 4, dW, lddw,
+                           accumulate ? 1 : 0);
     }
     if (e != cudaSuccess) {
         cudaGetLastError();

@@ -5,6 +5,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <utility>
+
 #include "gradcache.h"
 
 namespace gc {
@@ -26,6 +28,27 @@ __device__ __forceinline__ void dep_release() {
 }
 __device__ __forceinline__ bool gate_closed(const Gate& g) {
     return g.flag && ((*g.flag != 0) != (g.want != 0));
+}
+// Kernel launch with a cluster of `cluster` CTAs (1: none) that may start while the kernel before it in
+// the stream runs: only for kernels that call dep_wait() before they touch memory.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, unsigned block, size_t smem,
+                                  int cluster, cudaStream_t st, Args&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 // Logsumexp of row i from its per-part (scale, sum) slots, slot g at [g * pitch + i]: the one
 // definition every kernel that merges slots uses, with explicit roundings so that all of them
@@ -219,11 +242,20 @@ bool strip_applicable(int64_t B, int64_t N, int d, int dtype);
 size_t strip_workspace_bytes(int64_t B, int64_t N, int d, int dtype);
 size_t strip_forward_bytes(int64_t B, int64_t N, int d, int dtype);     // strip_forward's share of it
 int strip_launches(int op, int64_t B, int64_t N, int d, int dtype);
+// What the passes of the two-direction loss hand on (gc_variants_loss.cu).
+struct TwoDirection {
+    bool columns;           // this pass: rows are passages (no positives), candidates the queries
+    int* mult;              // [N] queries per passage: cleared and counted by the row direction's forward
+    float* col_neg;         // [N] column factors, written by the column direction's forward
+    const float* col_lse;   // [N] its logsumexp, and [B] the positives' logits, for the loss
+    const float* pos_logit;
+};
 cudaError_t strip_forward(const Problem& p, void* ws, float* loss, float* row_lse, float* pos_logit,
-                          int* dev_status, cudaStream_t st);
+                          int* dev_status, cudaStream_t st, const TwoDirection* two = nullptr);
 cudaError_t strip_backward(const Problem& p, void* ws, const float* row_lse, float* dQ, int64_t lddq,
                            float* dP, int64_t lddp, int* dev_status, cudaStream_t st,
-                           const float* col_neg = nullptr, float grad_scale = 1.f);
+                           const float* col_neg = nullptr, float grad_scale = 1.f,
+                           const TwoDirection* two = nullptr, float* loss = nullptr);
 // dP may be NULL
 cudaError_t strip_build(const Problem& p, void* ws, float* loss, float* row_lse, float* pos_logit,
                         float* dQ, int64_t lddq, float* dP, int64_t lddp, int* dev_status,

@@ -26,8 +26,6 @@
 #include <stdlib.h>
 #include <string.h>
 
-#include <utility>
-
 #include "tc_common.cuh"
 
 namespace gc {
@@ -184,12 +182,18 @@ struct LogitParams {
     const float* row_lse;        // LOGIT_W, LOGIT_W2
     const float* col_neg;        // LOGIT_W2: per passage, log2 of its multiplicity as a positive minus
                                  // its own logsumexp over the queries (log2 units; -inf: none)
+    const float* col_lse;        // LOGIT_W2, may be NULL: that logsumexp; the terms of the loss of both
+    const float* pos_logit;      // directions are then formed here
+    float zero_anchor_lse;       // log B
+    float* terms;
     float2* slots;               // [rows][slot_pitch] (raw maximum, sum)
     int slot_pitch;
     float* pos_ws;               // positive's raw logit
     float* res;                  // LOGIT_W: what the positive's weight lost to bf16
     int* zero;                   // counters of the kernels that follow, cleared here
     int zero_count;
+    int* zero2;                  // LOGIT_FWD, may be NULL: likewise
+    int zero2_count;
     int* dev_status;
 };
 
@@ -289,6 +293,10 @@ strip_logit_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
             for (int e = blockIdx.x * 256 + (ew * 32 + lane); e < p.zero_count; e += 8 * 256)
                 p.zero[e] = 0;
         }
+        if (MODE == LOGIT_FWD && p.zero2) {
+            for (int e = (int)blockIdx.x * 256 + (ew * 32 + lane); e < p.zero2_count; e += (int)gridDim.x * 256)
+                p.zero2[e] = 0;
+        }
         const uint32_t stage_buf = c.smem + NST * STAGE + (uint32_t)ew * (SB * 4096u);
         const uint64_t c1_2 = pack2(p.c1, p.c1);
         int use = 0;
@@ -302,7 +310,7 @@ strip_logit_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
             int pos = -1, masked = -1;
             float neg_lse = -INFINITY, lse_i = 0.f;
             if (i < p.rows) {
-                pos = p.pos_idx[i];
+                pos = p.pos_idx ? p.pos_idx[i] : -1;
                 int flag = pos < 0 || pos >= p.pos_n ? GC_DEV_POS_RANGE : 0;
                 pos -= p.pos_base;
                 if (p.mask_on) {
@@ -316,6 +324,11 @@ strip_logit_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
                     if (n == 0 && half == 0) {
                         if (pos < 0) p.res[i] = 0.f;     // no usable positive: nothing is lost to rounding
                         if (flag && p.dev_status) atomicOr(p.dev_status, flag);
+                        // (the column direction of an unusable positive: a zero anchor row)
+                        if (MODE == LOGIT_W2 && p.terms) {
+                            const float pl = p.pos_logit[i];
+                            p.terms[i] = 0.5f * ((lse_i - pl) + (flag ? p.zero_anchor_lse : p.col_lse[pos] - pl));
+                        }
                     }
                 }
             }
@@ -666,6 +679,10 @@ struct RowParams {
     const float* S;
     int64_t lds;
     int lse_given, want_w;
+    // two-direction loss
+    int* count;                   // queries per passage, counted here
+    const int* mult;              // rows are passages: their counts, and
+    float* col_neg;               // where LOGIT_W2's column factors go
 };
 
 // Shares of the loss are added in a fixed order: a block's rows in row order, then the blocks in a fixed
@@ -696,7 +713,7 @@ __device__ __forceinline__ void loss_share(const RowParams& p, float mine) {
 
 // The positive of strip row i as a column of the strip (-1: none there), and what is wrong with it.
 __device__ __forceinline__ int row_pos(const RowParams& p, int i, int* flags) {
-    const int raw = p.pos_idx[i], pos = raw - p.pos_base;
+    const int raw = p.pos_idx ? p.pos_idx[i] : -1, pos = raw - p.pos_base;
     *flags = raw < 0 || raw >= p.pos_n ? GC_DEV_POS_RANGE
              : p.mask_on && pos == i + p.mask_shift ? GC_DEV_POS_MASKED : 0;
     return *flags || pos < 0 || pos >= p.N ? -1 : pos;
@@ -767,6 +784,11 @@ strip_row_kernel(uint4* __restrict__ W, const RowParams p) {
                 p.row_lse[i] = lse;
                 if (p.pos_logit) p.pos_logit[i] = pl;
                 if (flags && p.dev_status) atomicOr(p.dev_status, flags);
+                if (!WRITE && p.count && pos >= 0) atomicAdd(p.count + pos, 1);
+                if (!WRITE && p.col_neg) {
+                    const int n = p.mult[i];
+                    p.col_neg[i] = n > 0 ? log2f((float)n) - lse * LOG2E : -INFINITY;
+                }
                 if (WRITE) {
                     p.red[p.row0 + i] = lse - pl;
                     p.res[i] = pos < 0 ? 0.f : pw - __bfloat162float(__float2bfloat16_rn(pw));
@@ -1408,31 +1430,6 @@ constexpr size_t SMEM_GF32 = 1024 + 3 * (2 * CHUNK_BYTES + 3 * 8192) + NSOFT * 4
 static_assert(SMEM_L256 <= SMEM_LIMIT - 1024 && SMEM_LF32 <= SMEM_LIMIT - 1024 &&
               SMEM_GF32 <= SMEM_LIMIT - 1024, "shared memory budget");
 
-// Kernel launch with a cluster of `cluster` CTAs (1: none).  Every kernel of this file may start while
-// the kernel before it in the stream runs; it waits for that kernel before it touches memory.
-template <typename... KArgs, typename... Args>
-cudaError_t launch(void (*kernel)(KArgs...), dim3 grid, unsigned block, size_t smem, int cluster,
-                   cudaStream_t st, Args&&... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[2];
-    int n = 0;
-    if (cluster > 1) {
-        attr[n].id = cudaLaunchAttributeClusterDimension;
-        attr[n].val.clusterDim.x = (unsigned)cluster;
-        attr[n].val.clusterDim.y = 1;
-        attr[n++].val.clusterDim.z = 1;
-    }
-    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[n++].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = n;
-    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
-}
-
 // The shared-memory limit belongs to the (kernel, device) pair; set once for all kernels here.
 cudaError_t configure_kernels() {
     static bool done[64] = {false};
@@ -1554,6 +1551,7 @@ struct StripRun {
     int* dev_status;
     bool f32, shared;
     const float* col_neg = nullptr;
+    const TwoDirection* two = nullptr;
     float grad_scale = 1.f;
 
     StripRun(const Problem& pr, void* w, int* status, cudaStream_t s, bool fwd_only = false)
@@ -1583,7 +1581,7 @@ struct StripRun {
         const int64_t items = (p.B + (shared ? 0 : p.N)) * (p.d / 4);
         int64_t blocks = ceil_div(items, 256);
         if (blocks > 8 * sm_count()) blocks = 8 * sm_count();
-        return launch(split_terms_kernel, (unsigned)blocks, 256, 0, 1, st,
+        return launch_chained(split_terms_kernel, (unsigned)blocks, 256, 0, 1, st,
                       static_cast<const float*>(p.Q), p.ldq, p.B, at<uint2>(l.tq),
                       static_cast<const float*>(p.P), p.ldp, shared ? (int64_t)0 : p.N, at<uint2>(l.tp),
                       p.d / 4);
@@ -1603,9 +1601,16 @@ struct StripRun {
         lp.tiles_n = (int)ceil_div(p.N, bn);
         lp.c1 = c1(); lp.inv_tau = 1.f / p.tau;
         lp.mask_on = p.mask_mode == GC_MASK_SELF; lp.mask_shift = shift(s);
-        lp.pos_idx = p.pos_idx + row0;
+        lp.pos_idx = p.pos_idx ? p.pos_idx + row0 : nullptr;
         lp.pos_base = (int)p.pos_base; lp.pos_n = (int)(p.n_total > 0 ? p.n_total : p.N);
         lp.col_neg = col_neg;
+        if (two) {
+            lp.col_lse = two->col_lse; lp.pos_logit = two->pos_logit;
+            lp.terms = mode == LOGIT_W2 ? at<float>(l.red) + row0 : nullptr;
+            if (mode == LOGIT_FWD && zero_ticket && !two->columns) { lp.zero2 = two->mult; lp.zero2_count = (int)p.N; }
+            if (mode == LOGIT_W2) lp.pos_logit += row0;
+            lp.zero_anchor_lse = logf((float)p.B);
+        }
         lp.row_lse = row_lse ? row_lse + row0 : nullptr;
         lp.slots = at<float2>(l.slots);
         lp.slot_pitch = mode == LOGIT_FWD ? 2 * lp.tiles_n : l.slot_pitch;
@@ -1622,10 +1627,10 @@ struct StripRun {
             return cudaErrorInvalidValue;
         const int total = lp.tiles_m * lp.tiles_n;
         const unsigned grid = 2u * (unsigned)(total < pairs ? total : pairs);
-        if (f32) return launch(strip_logit_f32_kernel, grid, ST_THREADS, SMEM_LF32, 2, st, mq, mp, mw, lp);
+        if (f32) return launch_chained(strip_logit_f32_kernel, grid, ST_THREADS, SMEM_LF32, 2, st, mq, mp, mw, lp);
         auto go = [&](auto k256, auto k128) {
-            return bn == 256 ? launch(k256, grid, ST_THREADS, SMEM_L256, 2, st, mq, mp, mw, lp)
-                             : launch(k128, grid, ST_THREADS, SMEM_L128, 2, st, mq, mp, mw, lp);
+            return bn == 256 ? launch_chained(k256, grid, ST_THREADS, SMEM_L256, 2, st, mq, mp, mw, lp)
+                             : launch_chained(k128, grid, ST_THREADS, SMEM_L128, 2, st, mq, mp, mw, lp);
         };
         if (mode == LOGIT_FWD) return go(strip_logit_kernel<LOGIT_FWD, 256>, strip_logit_kernel<LOGIT_FWD, 128>);
         if (mode == LOGIT_STASH) return go(strip_logit_kernel<LOGIT_STASH, 256>, strip_logit_kernel<LOGIT_STASH, 128>);
@@ -1647,7 +1652,7 @@ struct StripRun {
         rp.rows = (int)rows; rp.N = (int)p.N; rp.row0 = (int)row0;
         rp.c1 = c1(); rp.inv_tau = 1.f / p.tau;
         rp.mask_on = p.mask_mode == GC_MASK_SELF; rp.mask_shift = shift(s);
-        rp.pos_idx = p.pos_idx + row0;
+        rp.pos_idx = p.pos_idx ? p.pos_idx + row0 : nullptr;
         rp.pos_base = (int)p.pos_base; rp.pos_n = (int)(p.n_total > 0 ? p.n_total : p.N);
         rp.slots = at<float2>(l.slots);
         if (write) {
@@ -1675,13 +1680,17 @@ struct StripRun {
         rp.S = f32 ? at<float>(l.s) : nullptr;
         rp.lds = l.ldw;
         rp.lse_given = lse_given; rp.want_w = write;
+        if (two && !write) {
+            if (two->columns) { rp.mult = two->mult + row0; rp.col_neg = two->col_neg + row0; }
+            else              rp.count = two->mult;
+        }
         const unsigned grid = (unsigned)row_blocks(s, write);
-        if (f32) return launch(strip_row_f32_kernel, grid, 256, 0, 1, st, at<uint2>(l.w), rp);
+        if (f32) return launch_chained(strip_row_f32_kernel, grid, 256, 0, 1, st, at<uint2>(l.w), rp);
         // segments of whole rounds while there are fewer rows than warps the device holds
         const int64_t rounds = ceil_div(p.N, 8 * ROW_ROUND), room = 28 * (int64_t)sm_count() / rows;
         const int64_t segs = room < 1 ? 1 : room < rounds ? room : rounds;
         rp.seg_rounds = (int)ceil_div(rounds, segs);
-        auto go = [&](auto k, dim3 g) { return launch(k, g, 32 * row_warps(write), 0, 1, st, at<uint4>(l.w), rp); };
+        auto go = [&](auto k, dim3 g) { return launch_chained(k, g, 32 * row_warps(write), 0, 1, st, at<uint4>(l.w), rp); };
         return write ? go(strip_row_kernel<true>, dim3(grid, (unsigned)ceil_div(rounds, rp.seg_rounds)))
                      : go(strip_row_kernel<false>, dim3(grid));
     }
@@ -1722,7 +1731,7 @@ struct StripRun {
         if (dP && !make_out_map(&mdp, dP, p.N, p.d, lddp, 1)) return cudaErrorInvalidValue;
         const unsigned grid = 2u * (unsigned)gp.pairs;
         auto go = [&](auto k, size_t smem) {
-            return launch(k, grid, ST_THREADS, smem, 2, st, wk, wm, mp, mq, mdq, mdp, gp);
+            return launch_chained(k, grid, ST_THREADS, smem, 2, st, wk, wm, mp, mq, mdq, mdp, gp);
         };
         return f32 ? go(strip_grad_kernel<true, 128>, SMEM_GF32)
                : width == 128 ? go(strip_grad_kernel<false, 128>, SMEM_G128)
@@ -1769,9 +1778,10 @@ int strip_launches(int op, int64_t B, int64_t N, int d, int dtype) {
 }
 
 cudaError_t strip_forward(const Problem& p, void* ws, float* loss, float* row_lse, float* pos_logit,
-                          int* dev_status, cudaStream_t st) {
+                          int* dev_status, cudaStream_t st, const TwoDirection* two) {
     cudaError_t e = configure_kernels();
     StripRun r(p, ws, dev_status, st, true);
+    r.two = two;
     if (e == cudaSuccess && r.f32) e = r.split();
     for (int s = 0; s < r.l.strips && e == cudaSuccess; ++s) {
         e = r.logits(s, LOGIT_FWD, nullptr, s == 0);
@@ -1796,17 +1806,18 @@ cudaError_t strip_build(const Problem& p, void* ws, float* loss, float* row_lse,
 
 cudaError_t strip_backward(const Problem& p, void* ws, const float* row_lse, float* dQ, int64_t lddq,
                            float* dP, int64_t lddp, int* dev_status, cudaStream_t st,
-                           const float* col_neg, float grad_scale) {
+                           const float* col_neg, float grad_scale, const TwoDirection* two, float* loss) {
     cudaError_t e = configure_kernels();
     StripRun r(p, ws, dev_status, st);
     r.col_neg = col_neg;
     r.grad_scale = grad_scale;
+    r.two = two;
     if (e == cudaSuccess && r.f32) e = r.split();
     for (int s = 0; s < r.l.strips && e == cudaSuccess; ++s) {
         e = r.logits(s, col_neg ? LOGIT_W2 : LOGIT_W, row_lse, s == 0);
         if (e == cudaSuccess && r.f32)
             e = r.rows_kernel(s, true, true, const_cast<float*>(row_lse), nullptr, nullptr);
-        if (e == cudaSuccess) e = r.grads(s, dQ, lddq, dP, lddp, nullptr);
+        if (e == cudaSuccess) e = r.grads(s, dQ, lddq, dP, lddp, loss);
     }
     return e;
 }

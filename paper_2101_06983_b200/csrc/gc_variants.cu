@@ -9,7 +9,9 @@
 //                        <q_i, dQ_i> = sum_j G_ij <q_i, p_j> / tau (Eq. 5).  gc_dtau reduces the
 //                        cache rows against the rows they belong to, in a fixed order.
 //
-// All three are bound by HBM traffic: one warp per row, 16-byte loads, fp32 arithmetic.
+// All three are bound by HBM traffic, or by launch and load latency for small batches: one warp per row,
+// which holds its pieces in registers (a second read of the row only beyond 1024
+// columns), fp32 arithmetic, launched early (programmatic dependent launch).
 #include <cuda_bf16.h>
 #include <math.h>
 
@@ -46,79 +48,109 @@ __device__ __forceinline__ void store4(void* row, int k, float4 v) {
     }
 }
 
-template <bool BF16>
+// A lane's pieces of a row: 4 columns at 4 lane + 128 x, x < ROW_KEEP, held in registers; the rest is
+// loaded each time it is asked for.  ROW_KEEP is 4 up to 512 columns (more warps per SM), else 8.
+template <int ROW_KEEP, typename Load>
+struct RowPieces {
+    float4 v[ROW_KEEP];
+    Load load;
+    int d, k0;
+    __device__ __forceinline__ RowPieces(Load l, int d_, int lane) : load(l), d(d_), k0(4 * lane) {
+#pragma unroll
+        for (int x = 0; x < ROW_KEEP; ++x)
+            if (k0 + 128 * x < d) v[x] = load(k0 + 128 * x);
+    }
+};
+template <int KEEP, typename Load>
+__device__ __forceinline__ RowPieces<KEEP, Load> row_pieces(Load l, int d, int lane) {
+    return RowPieces<KEEP, Load>(l, d, lane);
+}
+// f(k, piece of a, piece of b) for this lane's pieces in ascending order
+template <int ROW_KEEP, typename A, typename B, typename F>
+__device__ __forceinline__ void each_piece(const RowPieces<ROW_KEEP, A>& a, const RowPieces<ROW_KEEP, B>& b,
+                                           F f) {
+#pragma unroll
+    for (int x = 0; x < ROW_KEEP; ++x)
+        if (a.k0 + 128 * x < a.d) f(a.k0 + 128 * x, a.v[x], b.v[x]);
+    for (int k = a.k0 + 128 * ROW_KEEP; k < a.d; k += 128) f(k, a.load(k), b.load(k));
+}
+
+template <bool BF16, int KEEP>
 __global__ void __launch_bounds__(256)
 row_normalize_kernel(const void* __restrict__ X, int64_t ldx, int64_t rows, int d,
                      void* __restrict__ Xn, int64_t ldxn, float* __restrict__ inv_norm) {
     const int lane = threadIdx.x & 31;
     const size_t es = BF16 ? 2 : 4;
+    dep_release();
+    dep_wait();
     for (int64_t i = blockIdx.x * 8 + (threadIdx.x >> 5); i < rows; i += (int64_t)gridDim.x * 8) {
         const char* src = static_cast<const char*>(X) + (size_t)i * (size_t)ldx * es;
+        const auto x = row_pieces<KEEP>([&](int k) { return load4<BF16>(src, k); }, d, lane);
         float ss = 0.f;
-        for (int k = 4 * lane; k < d; k += 128) {
-            const float4 v = load4<BF16>(src, k);
+        each_piece(x, x, [&](int, const float4& v, const float4&) {
             ss = fmaf(v.x, v.x, ss); ss = fmaf(v.y, v.y, ss);
             ss = fmaf(v.z, v.z, ss); ss = fmaf(v.w, v.w, ss);
-        }
+        });
         ss = warp_sum(ss);
         const float inv = ss > 0.f ? 1.0f / sqrtf(ss) : 0.f;       // a zero row stays zero
         if (lane == 0) inv_norm[i] = inv;
         char* dst = static_cast<char*>(Xn) + (size_t)i * (size_t)ldxn * es;
-        for (int k = 4 * lane; k < d; k += 128) {
-            const float4 v = load4<BF16>(src, k);
+        each_piece(x, x, [&](int k, const float4& v, const float4&) {
             store4<BF16>(dst, k, make_float4(v.x * inv, v.y * inv, v.z * inv, v.w * inv));
-        }
+        });
     }
 }
 
 // dX_i = inv_i (g_i - n_i <n_i, g_i>) with n_i = inv_i x_i formed in fp32 from the original row
-template <bool BF16>
+template <bool BF16, int KEEP>
 __global__ void __launch_bounds__(256)
 cosine_bwd_kernel(const void* __restrict__ X, int64_t ldx, const float* __restrict__ inv_norm,
                   const float* G, int64_t ldg, int64_t rows, int d, float* dX, int64_t lddx) {
     const int lane = threadIdx.x & 31;
     const size_t es = BF16 ? 2 : 4;
+    dep_release();
+    dep_wait();
     for (int64_t i = blockIdx.x * 8 + (threadIdx.x >> 5); i < rows; i += (int64_t)gridDim.x * 8) {
         const char* src = static_cast<const char*>(X) + (size_t)i * (size_t)ldx * es;
         const float* g = G + i * ldg;
         const float inv = inv_norm[i];
+        const auto xs = row_pieces<KEEP>([&](int k) { return load4<BF16>(src, k); }, d, lane);
+        const auto gs = row_pieces<KEEP>([&](int k) { return *reinterpret_cast<const float4*>(g + k); }, d, lane);
         float dot = 0.f;
-        for (int k = 4 * lane; k < d; k += 128) {
-            const float4 x = load4<BF16>(src, k);
-            const float4 gv = *reinterpret_cast<const float4*>(g + k);
+        each_piece(xs, gs, [&](int, const float4& x, const float4& gv) {
             dot = fmaf(x.x * inv, gv.x, dot); dot = fmaf(x.y * inv, gv.y, dot);
             dot = fmaf(x.z * inv, gv.z, dot); dot = fmaf(x.w * inv, gv.w, dot);
-        }
+        });
         dot = warp_sum(dot);
         float* out = dX + i * lddx;
-        for (int k = 4 * lane; k < d; k += 128) {
-            const float4 x = load4<BF16>(src, k);
-            const float4 gv = *reinterpret_cast<const float4*>(g + k);
+        each_piece(xs, gs, [&](int k, const float4& x, const float4& gv) {
             float4 o;
             o.x = inv * (gv.x - x.x * inv * dot); o.y = inv * (gv.y - x.y * inv * dot);
             o.z = inv * (gv.z - x.z * inv * dot); o.w = inv * (gv.w - x.w * inv * dot);
             *reinterpret_cast<float4*>(out + k) = o;
-        }
+        });
     }
 }
 
 // row_dot[i] = <q_i, dQ_i>
-template <bool BF16>
+template <bool BF16, int KEEP>
 __global__ void __launch_bounds__(256)
 row_dot_kernel(const void* __restrict__ Q, int64_t ldq, const float* __restrict__ dQ, int64_t lddq,
                int64_t rows, int d, float* __restrict__ row_dot) {
     const int lane = threadIdx.x & 31;
     const size_t es = BF16 ? 2 : 4;
+    dep_release();
+    dep_wait();
     for (int64_t i = blockIdx.x * 8 + (threadIdx.x >> 5); i < rows; i += (int64_t)gridDim.x * 8) {
         const char* src = static_cast<const char*>(Q) + (size_t)i * (size_t)ldq * es;
         const float* g = dQ + i * lddq;
+        const auto xs = row_pieces<KEEP>([&](int k) { return load4<BF16>(src, k); }, d, lane);
+        const auto gs = row_pieces<KEEP>([&](int k) { return *reinterpret_cast<const float4*>(g + k); }, d, lane);
         float dot = 0.f;
-        for (int k = 4 * lane; k < d; k += 128) {
-            const float4 x = load4<BF16>(src, k);
-            const float4 gv = *reinterpret_cast<const float4*>(g + k);
+        each_piece(xs, gs, [&](int, const float4& x, const float4& gv) {
             dot = fmaf(x.x, gv.x, dot); dot = fmaf(x.y, gv.y, dot);
             dot = fmaf(x.z, gv.z, dot); dot = fmaf(x.w, gv.w, dot);
-        }
+        });
         dot = warp_sum(dot);
         if (lane == 0) row_dot[i] = dot;
     }
@@ -127,8 +159,11 @@ row_dot_kernel(const void* __restrict__ Q, int64_t ldq, const float* __restrict_
 __global__ void __launch_bounds__(1024)
 ordered_sum_kernel(const float* __restrict__ v, int64_t n, float scale, float* __restrict__ out) {
     __shared__ float part[32];
+    dep_release();
+    dep_wait();
     float s = 0.f;
-    for (int64_t i = threadIdx.x; i < n; i += 1024) s += v[i];
+#pragma unroll 8
+    for (int64_t i = threadIdx.x; i < n; i += 1024) s += __ldcg(v + i);
     s = warp_sum(s);
     if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
     __syncthreads();
@@ -176,11 +211,14 @@ int gc_row_normalize(const void* X, int64_t ldx, int64_t rows, int d, int dtype,
     if ((rc = check_rows(Xn, ldxn, rows, d, dtype))) return rc;
     if (!inv_norm) return GC_ERR_NULL;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    if (dtype == GC_BF16)
-        row_normalize_kernel<true><<<grid_for(rows), 256, 0, st>>>(X, ldx, rows, d, Xn, ldxn, inv_norm);
-    else
-        row_normalize_kernel<false><<<grid_for(rows), 256, 0, st>>>(X, ldx, rows, d, Xn, ldxn, inv_norm);
-    return cudaGetLastError() == cudaSuccess ? GC_OK : GC_ERR_CUDA;
+    cudaError_t e;
+    auto go = [&](auto kernel) {
+        return launch_chained(kernel, dim3(grid_for(rows)), 256, 0, 1, st, X, ldx, rows, d, Xn, ldxn,
+                              inv_norm);
+    };
+    if (dtype == GC_BF16) e = d <= 512 ? go(row_normalize_kernel<true, 4>) : go(row_normalize_kernel<true, 8>);
+    else                  e = d <= 512 ? go(row_normalize_kernel<false, 4>) : go(row_normalize_kernel<false, 8>);
+    return e == cudaSuccess ? GC_OK : GC_ERR_CUDA;
 }
 
 int gc_cosine_bwd(const void* X, int64_t ldx, int64_t rows, int d, int dtype, const float* inv_norm,
@@ -191,13 +229,14 @@ int gc_cosine_bwd(const void* X, int64_t ldx, int64_t rows, int d, int dtype, co
     if ((rc = check_f32(dXn, lddxn, d))) return rc;
     if ((rc = check_f32(dX, lddx, d))) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    if (dtype == GC_BF16)
-        cosine_bwd_kernel<true><<<grid_for(rows), 256, 0, st>>>(X, ldx, inv_norm, dXn, lddxn, rows, d,
-                                                               dX, lddx);
-    else
-        cosine_bwd_kernel<false><<<grid_for(rows), 256, 0, st>>>(X, ldx, inv_norm, dXn, lddxn, rows,
-                                                                d, dX, lddx);
-    return cudaGetLastError() == cudaSuccess ? GC_OK : GC_ERR_CUDA;
+    cudaError_t e;
+    auto go = [&](auto kernel) {
+        return launch_chained(kernel, dim3(grid_for(rows)), 256, 0, 1, st, X, ldx, inv_norm, dXn, lddxn,
+                              rows, d, dX, lddx);
+    };
+    if (dtype == GC_BF16) e = d <= 512 ? go(cosine_bwd_kernel<true, 4>) : go(cosine_bwd_kernel<true, 8>);
+    else                  e = d <= 512 ? go(cosine_bwd_kernel<false, 4>) : go(cosine_bwd_kernel<false, 8>);
+    return e == cudaSuccess ? GC_OK : GC_ERR_CUDA;
 }
 
 size_t gc_dtau_workspace_bytes(int64_t B) {
@@ -213,14 +252,16 @@ int gc_dtau(const void* Q, int64_t ldq, const float* dQ, int64_t lddq, int64_t B
     if (!(tau > 0.f) || !isfinite(tau)) return GC_ERR_SHAPE;
     if (!ws || ((uintptr_t)ws & 255) != 0 || ws_bytes < gc_dtau_workspace_bytes(B)) return GC_ERR_WORKSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+    cudaError_t e;
     float* row_dot = static_cast<float*>(ws);
-    if (dtype == GC_BF16)
-        row_dot_kernel<true><<<grid_for(B), 256, 0, st>>>(Q, ldq, dQ, lddq, B, d, row_dot);
-    else
-        row_dot_kernel<false><<<grid_for(B), 256, 0, st>>>(Q, ldq, dQ, lddq, B, d, row_dot);
-    if (cudaGetLastError() != cudaSuccess) return GC_ERR_CUDA;
-    ordered_sum_kernel<<<1, 1024, 0, st>>>(row_dot, B, -1.f / tau, dtau);
-    return cudaGetLastError() == cudaSuccess ? GC_OK : GC_ERR_CUDA;
+    auto go = [&](auto kernel) {
+        return launch_chained(kernel, dim3(grid_for(B)), 256, 0, 1, st, Q, ldq, dQ, lddq, B, d, row_dot);
+    };
+    if (dtype == GC_BF16) e = d <= 512 ? go(row_dot_kernel<true, 4>) : go(row_dot_kernel<true, 8>);
+    else                  e = d <= 512 ? go(row_dot_kernel<false, 4>) : go(row_dot_kernel<false, 8>);
+    if (e != cudaSuccess) return GC_ERR_CUDA;
+    e = launch_chained(ordered_sum_kernel, dim3(1), 1024, 0, 1, st, row_dot, B, -1.f / tau, dtau);
+    return e == cudaSuccess ? GC_OK : GC_ERR_CUDA;
 }
 
 }  // extern "C"

@@ -73,3 +73,29 @@ def test_several_strips_bf16_self_mask(binding, oracle):
     _check_sampled(oracle, prob, out, 48, 24, full_lse=out.row_lse.cpu().numpy().astype(np.float64))
     Q, P, _ = to_device(prob)
     _check_properties(prob, out, Q, P)
+
+
+@pytest.mark.parametrize("B,N,d,tau", [(300, 310, 136, 0.3), (500, 320, 64, 0.2), (1030, 1200, 448, 0.5)])
+def test_two_directions_with_few_spare_passages(binding, oracle, B, N, d, tau):
+    """Up to 1.25 B passages the column direction runs over all passages: passages that are nobody's
+    positive, and passages that are the positive of several queries."""
+    prob = inputs.random_problem(B, N, d, "bf16", seed=B + N, tau=tau, scale=d ** -0.5)
+    ref = oracle.build_variant(prob.Q, prob.P, prob.pos_idx, prob.tau, 0, two_direction=True)
+    assert np.unique(prob.pos_idx).size < min(B, N)
+    Q, P, pos = to_device(prob)
+    f = dict(dtype=torch.float32, device="cuda")
+    loss, lse = torch.zeros(1, **f), torch.empty(B, **f)
+    dQ, dP = torch.full((B, d), float("nan"), **f), torch.full((N, d), float("nan"), **f)
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    binding.gc_build_cache_two_direction(Q, P, pos, prob.tau, loss, lse, dQ, dP, dev_status=st)
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0
+    tol = TOL["bf16"]
+    assert abs(loss.item() - ref["loss"]) <= tol["loss"] * abs(ref["loss"])
+    assert grad_err(dQ.cpu().numpy(), ref["dQ"]) <= tol["grad"]
+    assert grad_err(dP.cpu().numpy(), ref["dP"]) <= tol["grad"]
+    bad = pos.clone()
+    bad[3] = N
+    binding.gc_build_cache_two_direction(Q, P, bad, prob.tau, loss, lse, dQ, dP, dev_status=st)
+    torch.cuda.synchronize()
+    assert int(st.item()) == binding.GC_DEV_POS_RANGE and bool(torch.isfinite(dP).all())
