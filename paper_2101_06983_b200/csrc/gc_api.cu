@@ -42,11 +42,7 @@ Plan make_plan(int64_t B, int64_t N, int d, int dtype, bool stored) {
         pl.g_dq = simt_sweep_groups(B, N, d);
         pl.g_dp = simt_sweep_groups(N, B, d);
     }
-    // fp32 batches of a few tiles: the one-tile tcgen05 kernel per tile pair (gc_small.cu); its
-    // slots and partial planes share the regions of the plan it replaces
-    pl.tiles = small_tiled_applicable(B, N, d, dtype) ? 1 : 0;
-    pl.tiles_y = pl.tiles ? small_tiles_y(N, dtype) : 0;
-    const int tiles_x = pl.tiles ? small_tiles_x(B) : 0, tiles_y = pl.tiles ? small_tiles_y(N, dtype) : 0;
+    pl.tiles_y = dtype == GC_F32 && small_tiled_applicable(B, N, d, dtype) ? (int)((N + 127) / 128) : 0;
     pl.fused = (pl.tc && tc_fused_applicable(d)) ? 1 : 0;
     // 1: four-CTA sweeps (rows of two column halves); 2: narrow rows (two S buffers)
     pl.anchored = (pl.fused && quad_applicable(B, d)) ? 1
@@ -58,19 +54,16 @@ Plan make_plan(int64_t B, int64_t N, int d, int dtype, bool stored) {
     if (pl.fused && (size_t)(2 * pl.g_dq) > slots) slots = (size_t)(2 * pl.g_dq);
     if (pl.anchored == 1 && (size_t)(4 * pl.g_dq) > slots) slots = (size_t)(4 * pl.g_dq);
     if (pl.anchored == 2 && (size_t)(4 * pl.g_dq) > slots) slots = (size_t)(4 * pl.g_dq);
-    if ((size_t)tiles_y > slots) slots = (size_t)tiles_y;
-    const int planes_q = pl.g_dq > tiles_y ? pl.g_dq : tiles_y;
-    const int planes_p = pl.g_dp > tiles_x ? pl.g_dp : tiles_x;
     size_t off = 0;
     pl.off_m = off;    off += align256(sizeof(float) * slots * (size_t)B);
     pl.off_l = off;    off += align256(sizeof(float) * slots * (size_t)B);
     pl.off_pos = off;  off += align256(sizeof(float) * (size_t)B);
     pl.off_red = off;  off += 2048;      // loss reduction: block ticket + up to 256 block sums
     pl.off_accq = off;
-    if (planes_q > 1 || pl.fused || pl.anchored)
-        off += align256(sizeof(float) * (size_t)planes_q * (size_t)B * dpad);
+    if (pl.g_dq > 1 || pl.fused || pl.anchored)
+        off += align256(sizeof(float) * (size_t)pl.g_dq * (size_t)B * dpad);
     pl.off_accp = off;
-    if (planes_p > 1) off += align256(sizeof(float) * (size_t)planes_p * (size_t)N * dpad);
+    if (pl.g_dp > 1) off += align256(sizeof(float) * (size_t)pl.g_dp * (size_t)N * dpad);
     pl.launches_fwd = 2;  // sweep + combine
     pl.launches_bwd = 2 + (pl.g_dq > 1 ? 1 : 0) + (pl.g_dp > 1 ? 1 : 0);
     pl.launches_build = pl.fused ? 4 + (pl.g_dp > 1 ? 1 : 0) : pl.launches_fwd + pl.launches_bwd;
@@ -543,8 +536,7 @@ int run_small(int op, const Problem& p, const float* row_lse_in, float* loss, fl
                         st) == cudaSuccess ? GC_OK : GC_ERR_CUDA;
 }
 
-// fp32 batches of a few tiles (gc_small.cu): forward = tile kernel + combine, gradients = tile
-// kernel + one reduce per side that has several planes.
+// Forward of fp32 batches whose logits do not fit the static array: one slot per passage tile, combine.
 int run_tiles_fwd(const Problem& p, const Plan& pl, char* ws, float* loss, float* row_lse,
                   float* pos_logit, int* dev_status, cudaStream_t st) {
     float* part_m = reinterpret_cast<float*>(ws + pl.off_m);
@@ -557,31 +549,10 @@ int run_tiles_fwd(const Problem& p, const Plan& pl, char* ws, float* loss, float
         e = launch_small_tiled_fwd(p, part_m, part_l, pos_ws, red, dev_status, st);
     }
     if (e != cudaSuccess) return GC_ERR_CUDA;
-    e = launch_lse_combine(part_m, part_l, pos_ws, p.pos_idx, small_tiles_y(p.N, p.dtype), p.B, p.N,
+    e = launch_lse_combine(part_m, part_l, pos_ws, p.pos_idx, pl.tiles_y, p.B, p.N,
                            p.mask_mode, row_lse, pos_logit, loss, red, dev_status, kOpen, st,
                            p.b_total, p.mask_shift);
     return e == cudaSuccess ? GC_OK : GC_ERR_CUDA;
-}
-
-int run_tiles_bwd(const Problem& p, const Plan& pl, char* ws, const float* row_lse, float* dQ,
-                  int64_t lddq, float* dP, int64_t lddp, int* dev_status, cudaStream_t st) {
-    float* partial_q = reinterpret_cast<float*>(ws + pl.off_accq);
-    float* partial_p = reinterpret_cast<float*>(ws + pl.off_accp);
-    cudaError_t e;
-    {
-        KernelTimer t(1, st);
-        e = launch_small_tiled_bwd(p, row_lse, dQ, lddq, partial_q, dP, lddp, partial_p, dev_status,
-                                   st);
-    }
-    if (e != cudaSuccess) return GC_ERR_CUDA;
-    const int tx = small_tiles_x(p.B), ty = small_tiles_y(p.N, p.dtype);
-    if (dQ && ty > 1 &&
-        launch_partial_reduce(partial_q, ty, p.B, p.d, grad_scale(p), dQ, lddq, kOpen, st) != cudaSuccess)
-        return GC_ERR_CUDA;
-    if (dP && tx > 1 &&
-        launch_partial_reduce(partial_p, tx, p.N, p.d, grad_scale(p), dP, lddp, kOpen, st) != cudaSuccess)
-        return GC_ERR_CUDA;
-    return GC_OK;
 }
 
 }  // namespace
@@ -597,7 +568,7 @@ namespace {
 // other calls reserves the slots of the widest build plan) and returns the bytes they take.
 size_t forward_layout(Plan* pl, int64_t B, int64_t N) {
     size_t slots = (size_t)pl->g_fwd;
-    if (pl->tiles && (size_t)pl->tiles_y > slots) slots = (size_t)pl->tiles_y;
+    if ((size_t)pl->tiles_y > slots) slots = (size_t)pl->tiles_y;
     size_t off = 0;
     pl->off_m = off;    off += align256(sizeof(float) * slots * (size_t)B);
     pl->off_l = off;    off += align256(sizeof(float) * slots * (size_t)B);
@@ -659,12 +630,6 @@ int gc_kernel_launches(int op, int64_t B, int64_t N, int d, int dtype) {
     if (op >= GC_OP_FWD && op <= GC_OP_BUILD && small_applicable(B, N, d, dtype)) return 1;
     if (op >= GC_OP_FWD && op <= GC_OP_BUILD && strip_applicable(B, N, d, dtype))
         return strip_launches(op, B, N, d, dtype);
-    if (op >= GC_OP_FWD && op <= GC_OP_BUILD && small_tiled_applicable(B, N, d, dtype)) {
-        const int reduces = (small_tiles_y(N, dtype) > 1 ? 1 : 0) + (small_tiles_x(B) > 1 ? 1 : 0);
-        if (op == GC_OP_FWD) return 2;                  // tile kernel, combine
-        if (op == GC_OP_BWD) return 2 + reduces;        // pos_idx validation, tile kernel, reduces
-        return 3 + reduces;
-    }
     Plan pl = make_plan(B, N, d, dtype);
     if (op == GC_OP_FWD) return pl.launches_fwd;
     if (op == GC_OP_BWD) return pl.launches_bwd + 1;   // + pos_idx validation
@@ -693,9 +658,6 @@ int gc_loss_fwd(const void* Q, int64_t ldq, const void* P, int64_t ldp, const in
         return strip_forward(p, ws, loss, row_lse, pos_logit, dev_status,
                              static_cast<cudaStream_t>(cuda_stream)) == cudaSuccess ? GC_OK : GC_ERR_CUDA;
     }
-    if (pl.tiles)
-        return run_tiles_fwd(p, pl, static_cast<char*>(ws), loss, row_lse, pos_logit, dev_status,
-                             static_cast<cudaStream_t>(cuda_stream));
     return run_fwd(p, pl, static_cast<char*>(ws), loss, row_lse, pos_logit, dev_status,
                    static_cast<cudaStream_t>(cuda_stream));
 }
@@ -728,7 +690,7 @@ int gc_loss_fwd_static(const void* Q, int64_t ldq, const void* P, int64_t ldp,
     if (strips)
         return strip_forward(p, scratch, loss, row_lse, pos_logit, dev_status,
                              static_cast<cudaStream_t>(cuda_stream)) == cudaSuccess ? GC_OK : GC_ERR_CUDA;
-    if (pl.tiles)
+    if (pl.tiles_y)
         return run_tiles_fwd(p, pl, static_cast<char*>(scratch), loss, row_lse, pos_logit,
                              dev_status, static_cast<cudaStream_t>(cuda_stream));
     return run_fwd(p, pl, static_cast<char*>(scratch), loss, row_lse, pos_logit, dev_status,
@@ -761,8 +723,6 @@ int gc_loss_bwd(const void* Q, int64_t ldq, const void* P, int64_t ldp, const in
     if (dev_status && launch_pos_check(pos_idx, B, N, mask_mode, dev_status, st) != cudaSuccess)
         return GC_ERR_CUDA;
     char* w = static_cast<char*>(ws);
-    if (pl.tiles && (dQ || dP))
-        return run_tiles_bwd(p, pl, w, row_lse, dQ, lddq, dP, lddp, dev_status, st);
     if (dQ && (rc = run_sweep(p, pl, w, SWEEP_DQ, row_lse, dQ, lddq, dev_status, st))) return rc;
     if (dP && (rc = run_sweep(p, pl, w, SWEEP_DP, row_lse, dP, lddp, dev_status, st))) return rc;
     return GC_OK;
@@ -791,10 +751,6 @@ int gc_build_cache(const void* Q, int64_t ldq, const void* P, int64_t ldp, const
         KernelTimer t(1, st);
         return strip_build(p, ws, loss, row_lse, pos_logit, dQ, lddq, dP, lddp, dev_status, st) ==
                        cudaSuccess ? GC_OK : GC_ERR_CUDA;
-    }
-    if (pl.tiles) {
-        if ((rc = run_tiles_fwd(p, pl, w, loss, row_lse, pos_logit, dev_status, st))) return rc;
-        return run_tiles_bwd(p, pl, w, row_lse, dQ, lddq, dP, lddp, dev_status, st);
     }
     return run_build_sweeps(p, pl, w, loss, row_lse, pos_logit, dQ, lddq, dP, lddp, dev_status, st);
 }

@@ -136,8 +136,7 @@ struct FwdArgs {
 // How one call is carried out for given sizes on the current device.
 struct Plan {
     int tc;                 // 1: tcgen05 kernels, 0: SIMT kernels
-    int tiles;              // 1: batch of a few tiles on the one-tile tcgen05 kernel
-    int tiles_y;            // its passage tiles (slots per row of its forward)
+    int tiles_y;            // fp32: passage tiles of the forward that gc_loss_fwd_static falls back to
     int strips;             // 1: three products over strips of query rows (gc_strip.cu)
     int g_fwd, g_dq, g_dp;  // split factors of the streamed range
     size_t off_m, off_l, off_pos, off_red, off_accq, off_accp;
@@ -229,13 +228,12 @@ cudaError_t launch_small(int op, const Problem& pr, const float* row_lse_in, flo
                          int64_t lddp, int* dev_status, cudaStream_t st);
 
 bool small_tiled_applicable(int64_t B, int64_t N, int d, int dtype);
-int small_tiles_x(int64_t B);
-int small_tiles_y(int64_t N, int dtype);
+// gc_small_f32.cu
+cudaError_t launch_small_f32(int op, const Problem& pr, const float* row_lse_in, float* loss, float* row_lse,
+                             float* pos_logit, float* dQ, int64_t lddq, float* dP, int64_t lddp,
+                             int* dev_status, cudaStream_t st);
 cudaError_t launch_small_tiled_fwd(const Problem& pr, float* part_m, float* part_l, float* pos_ws,
                                    float* red, int* dev_status, cudaStream_t st);
-cudaError_t launch_small_tiled_bwd(const Problem& pr, const float* row_lse, float* dQ, int64_t lddq,
-                                   float* partial_q, float* dP, int64_t lddp, float* partial_p,
-                                   int* dev_status, cudaStream_t st);
 
 // gc_strip.cu
 bool strip_applicable(int64_t B, int64_t N, int d, int dtype);

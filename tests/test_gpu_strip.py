@@ -99,3 +99,21 @@ def test_two_directions_with_few_spare_passages(binding, oracle, B, N, d, tau):
     binding.gc_build_cache_two_direction(Q, P, bad, prob.tau, loss, lse, dQ, dP, dev_status=st)
     torch.cuda.synchronize()
     assert int(st.item()) == binding.GC_DEV_POS_RANGE and bool(torch.isfinite(dP).all())
+
+
+@pytest.mark.parametrize("B,N,d,mask", [(128, 128, 8, 0), (33, 127, 72, 0), (97, 97, 136, 1),
+                                        (128, 1, 192, 0), (1, 128, 264, 0), (65, 66, 1000, 1)])
+def test_one_tile_f32_clusters(binding, oracle, B, N, d, mask):
+    """One, two and four CTAs per cluster, slices that do not fill the last cluster; both gradients from
+    the build and each alone from the backward call."""
+    prob = inputs.random_problem(B, N, d, "f32", seed=B + N + d, tau=0.5, mask_mode=mask, scale=d ** -0.5)
+    ref = _oracle_full(oracle, prob)
+    check_against_oracle(prob, run_build(prob), ref)
+    Q, P, pos = to_device(prob)
+    b = binding.Outputs(B, N, d, binding.GC_F32)
+    args = (Q, P, pos, prob.tau, prob.mask_mode)
+    binding.gc_loss_fwd(*args, b.loss, b.row_lse, b.pos_logit, b.ws, b.dev_status)
+    binding.gc_loss_bwd(*args, b.row_lse, b.dQ, None, b.ws, b.dev_status)
+    binding.gc_loss_bwd(*args, b.row_lse, None, b.dP, b.ws, b.dev_status)
+    torch.cuda.synchronize()
+    check_against_oracle(prob, b, ref)
