@@ -307,7 +307,7 @@ apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ C
         if (threadIdx.x == 0 && p.dev_status) atomicOr(p.dev_status, GC_DEV_WAIT_LIMIT);
         __syncthreads();
     }
-    cluster_sync_all();   // the peer's MMAs, loads and signals no longer touch this CTA
+    cluster_meet();       // the peer's MMAs, loads and signals no longer touch this CTA
     if (warp == AP_MMA_WARP) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;"

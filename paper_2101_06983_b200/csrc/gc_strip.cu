@@ -143,7 +143,7 @@ __device__ __forceinline__ void pair_teardown(const PairCtx& c, volatile int* ab
         if (threadIdx.x == 0 && dev_status) atomicOr(dev_status, GC_DEV_WAIT_LIMIT);
         __syncthreads();
     }
-    cluster_sync_all();   // the peer's MMAs, loads and arrivals no longer touch this CTA
+    cluster_meet();       // the peer's MMAs, loads and arrivals no longer touch this CTA
     if (c.warp == MMA_WARP) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;"
