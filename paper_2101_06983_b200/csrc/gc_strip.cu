@@ -673,6 +673,7 @@ struct RowParams {
     int block0, blocks_total;     // this launch's first block and the blocks of all strips
     float inv_mean;
     int64_t ldw;                  // elements
+    int split;                    // strip_row_kernel<true>: 2^split warps share a row's rounds
     int seg_rounds;               // strip_row_kernel<true>: rounds of 2048 columns per segment
     int* dev_status;
     // fp32 inputs
@@ -719,30 +720,65 @@ __device__ __forceinline__ int row_pos(const RowParams& p, int i, int* flags) {
     return *flags || pos < 0 || pos >= p.N ? -1 : pos;
 }
 
-// bf16 inputs: a warp per row (WRITE: per row and segment of its columns; each merges the row's slots
-// for itself).  It forms row_lse, the positive's weight and the loss term, then turns the row's fp16
-// exponentials into bf16 weights in place: eight 16-byte pieces in flight per lane, the first of them
-// requested before the merge, each one's successor as soon as it has been used; one special-function
-// operation per group of 64 columns, its result passed around by shuffles.  Bound by the latency and
-// bandwidth of the L2 (4 bytes moved per pair).
+// bf16 inputs: a warp per row, or (WRITE) 2^split warps, each taking every 2^split-th round of 2048
+// columns of the block's segment.  They merge the row's (max, sum) slots, form row_lse, the positive's
+// weight and the loss term, then turn the row's fp16 exponentials into bf16 weights in place: eight
+// 16-byte pieces in flight per lane, each one's successor requested as soon as it has been used, the
+// slots of the next round with them; one special-function operation per group of 64 columns, its result
+// passed around by shuffles.  Rows go last to first: the logits written last are still in the L2.
+// Bound by the latency and bandwidth of the memory (4 bytes moved per pair).  Measured, us, one warp per
+// row, rows in order, each round's slots read when it begins -> as it is now:
+//   1531 x 3062  5.9 -> 4.7   4096 x 8192  23.8 -> 20.3   6000 x 12000   76 -> 48
+//   2048 x 32768  62 -> 52    8192 x 16384  120 -> 91     4096 x 131072 480 -> 387 (5.5 TB/s)
+// RESIDENT, the blocks an SM is to hold: seven (72 registers a thread), six where the grid then fits in
+// one go (1531 x 3062: 5.1 us with seven, 4.7 with six; 4096 x 8192: 20.3 and 22.0).
 constexpr int row_warps(bool write) { return write ? 4 : 8; }      // rows per block
 constexpr int ROW_PIECES = 8;                       // of 8 columns, per lane and round
 constexpr int ROW_ROUND = 32 * ROW_PIECES;          // pieces per warp and round: 32 groups of 64 columns
-template <bool WRITE>
-__global__ void __launch_bounds__(WRITE ? 128 : 256, WRITE ? 8 : 1)
+template <bool WRITE, int RESIDENT>
+__global__ void __launch_bounds__(WRITE ? 128 : 256, RESIDENT)
 strip_row_kernel(uint4* __restrict__ W, const RowParams p) {
     constexpr int ROW_WARPS = WRITE ? 4 : 8;
     __shared__ float terms[ROW_WARPS];
+    __shared__ float2 shares[ROW_WARPS];
     dep_release();
     dep_wait();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int i = blockIdx.x * ROW_WARPS + warp;
+    const int split = WRITE ? p.split : 0, sub = warp & ((1 << split) - 1);
+    // the rows written last come first: they are still in the L2
+    const int block = WRITE ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x;
+    const int i = (block * ROW_WARPS + warp) >> split;
     const bool live = i < p.rows;
-    const int n8 = (p.N + 7) / 8;
-    const int k0 = WRITE ? (int)blockIdx.y * p.seg_rounds * ROW_ROUND : 0;
-    const int k1 = WRITE ? min(n8, k0 + p.seg_rounds * ROW_ROUND) : 0;
+    const int n8 = (p.N + 7) / 8, stride = ROW_ROUND << split;
+    const int s0 = WRITE ? (int)blockIdx.y * p.seg_rounds * ROW_ROUND : 0;
+    const int k0 = s0 + sub * ROW_ROUND;
+    const int k1 = WRITE ? min(n8, s0 + p.seg_rounds * ROW_ROUND) : 0;
     const float2* sl = p.slots + (int64_t)(live ? i : 0) * p.slot_pitch;
     uint4* row = W + (int64_t)(live ? i : 0) * (p.ldw / 8);
+    // (max, sum) of the row: from the slots, shared out over the row's warps where there are many, and,
+    // with weights, from the positive, which is not in the slots then.  All but the first two of a lane
+    // come before the row's own pieces take their registers.
+    const int shared = p.nslots > 64 ? split : 0;
+    const int step = 32 << shared, first_slot = (shared ? sub * 32 : 0) + lane;
+    float m = -INFINITY, l = 0.f, pos_raw = -INFINITY;
+    int flags = 0, pos = -1;
+    auto slot = [&](int s) { return s < p.nslots ? __ldcg(sl + s) : make_float2(-INFINITY, 0.f); };
+    auto join = [&](float2 v, float ref) { l = fmaf(v.y, ex2((v.x - ref) * p.c1), l); };
+    if (live) {
+        for (int s = first_slot + 2 * step; s < p.nslots; s += 8 * step) {
+            float2 v[8];
+#pragma unroll
+            for (int x = 0; x < 8; ++x) v[x] = slot(s + step * x);
+            float top = m;
+#pragma unroll
+            for (int x = 0; x < 8; ++x) top = fmaxf(top, v[x].x);
+            const float ref = top == -INFINITY ? 0.f : top;
+            l *= ex2((m - ref) * p.c1);
+#pragma unroll
+            for (int x = 0; x < 8; ++x) join(v[x], ref);
+            m = top;
+        }
+    }
     uint4 raw[ROW_PIECES];
     if (WRITE && live) {
 #pragma unroll
@@ -752,35 +788,37 @@ strip_row_kernel(uint4* __restrict__ W, const RowParams p) {
         }
     }
     if (live) {
-        int flags;
-        const int pos = row_pos(p, i, &flags);
-        const float pos_raw = pos < 0 ? -INFINITY : __ldcg(p.pos_ws + i);
-        constexpr int KEEP = 4;                     // slots held in registers (N <= 8192: all)
-        float2 kept[KEEP];
-#pragma unroll
-        for (int x = 0; x < KEEP; ++x)
-            kept[x] = lane + 32 * x < p.nslots ? __ldcg(sl + lane + 32 * x) : make_float2(-INFINITY, 0.f);
-        // with weights, the positive is not in the slots: it is a term of its own
-        float m = WRITE ? pos_raw : -INFINITY;
-#pragma unroll
-        for (int x = 0; x < KEEP; ++x) m = fmaxf(m, kept[x].x);
-        for (int s = lane + 32 * KEEP; s < p.nslots; s += 32) m = fmaxf(m, __ldcg(&sl[s].x));
-        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        const float ref = m == -INFINITY ? 0.f : m;
-        float l = WRITE && lane == 0 ? ex2((pos_raw - ref) * p.c1) : 0.f;
-#pragma unroll
-        for (int x = 0; x < KEEP; ++x) l = fmaf(kept[x].y, ex2((kept[x].x - ref) * p.c1), l);
-        for (int s = lane + 32 * KEEP; s < p.nslots; s += 32) {
-            const float2 v = __ldcg(sl + s);
-            l = fmaf(v.y, ex2((v.x - ref) * p.c1), l);
-        }
+        const float2 v0 = slot(first_slot), v1 = slot(first_slot + step);
+        pos_raw = __ldcg(p.pos_ws + i);
+        pos = row_pos(p, i, &flags);
+        if (pos < 0) pos_raw = -INFINITY;
+        float top = fmaxf(m, fmaxf(v0.x, v1.x));
+        if (WRITE) top = fmaxf(top, pos_raw);
+        for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+        const float ref = top == -INFINITY ? 0.f : top;
+        l *= ex2((m - ref) * p.c1);
+        join(v0, ref);
+        join(v1, ref);
+        m = top;
+        if (WRITE && lane == 0 && (!shared || sub == 0)) l += ex2((pos_raw - ref) * p.c1);
         for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+    }
+    if (WRITE && shared) {
+        if (lane == 0) shares[warp] = make_float2(m, l);
+        __syncthreads();
+        const int first = warp - sub;
+        for (int w = 0; w < 1 << split; ++w) m = fmaxf(m, shares[first + w].x);
+        const float ref = m == -INFINITY ? 0.f : m;
+        l = 0.f;
+        for (int w = 0; w < 1 << split; ++w) l = fmaf(shares[first + w].y, ex2((shares[first + w].x - ref) * p.c1), l);
+    }
+    if (live) {
         const float lse = m * p.inv_tau + log2f(l) * LN2;
         const float pl = pos < 0 ? 0.f : pos_raw * p.inv_tau;
         const float pw = positive_weight(pos_raw, p.inv_tau, lse);
         if (lane == 0) {
             terms[warp] = lse - pl;
-            if (!WRITE || blockIdx.y == 0) {
+            if (!WRITE || (blockIdx.y == 0 && sub == 0)) {
                 p.row_lse[i] = lse;
                 if (p.pos_logit) p.pos_logit[i] = pl;
                 if (flags && p.dev_status) atomicOr(p.dev_status, flags);
@@ -799,10 +837,15 @@ strip_row_kernel(uint4* __restrict__ W, const RowParams p) {
             const float neg = -(lse * LOG2E);
             const int wk = pos < 0 ? -1 : pos >> 3;
             // round after round: lane g of a round holds the factor of its group of 64 columns
-            for (int kr = k0; kr < k1; kr += ROW_ROUND) {
+            auto top_of = [&](int kr) {
                 const int g = (kr >> 3) + lane;
+                return g < p.nslots ? __ldcg(&sl[g].x) : -INFINITY;
+            };
+            float next = top_of(k0);
+            for (int kr = k0; kr < k1; kr += stride) {
                 // (a group with no allowed column holds zeros)
-                const float gm = g < p.nslots ? __ldcg(&sl[g].x) : -INFINITY;
+                const float gm = next;
+                if (kr + stride < k1) next = top_of(kr + stride);
                 const float fg = gm > -INFINITY ? ex2(fmaf(gm, p.c1, neg)) : 0.f;
 #pragma unroll
                 for (int x = 0; x < ROW_PIECES; ++x) {
@@ -823,7 +866,7 @@ strip_row_kernel(uint4* __restrict__ W, const RowParams p) {
                     }
                     row[k] = make_uint4(pack_b2(w[0], w[1]), pack_b2(w[2], w[3]),
                                         pack_b2(w[4], w[5]), pack_b2(w[6], w[7]));
-                    if (k + ROW_ROUND < k1) raw[x] = __ldcg(row + k + ROW_ROUND);
+                    if (k + stride < k1) raw[x] = __ldcg(row + k + stride);
                 }
             }
         }
@@ -1690,13 +1733,19 @@ struct StripRun {
         }
         const unsigned grid = (unsigned)row_blocks(s, write);
         if (f32) return launch_chained(strip_row_f32_kernel, grid, 256, 0, 1, st, at<uint2>(l.w), rp);
-        // segments of whole rounds while there are fewer rows than warps the device holds
-        const int64_t rounds = ceil_div(p.N, 8 * ROW_ROUND), room = 28 * (int64_t)sm_count() / rows;
-        const int64_t segs = room < 1 ? 1 : room < rounds ? room : rounds;
-        rp.seg_rounds = (int)ceil_div(rounds, segs);
+        const int64_t rounds = ceil_div(p.N, 8 * ROW_ROUND);
+        // four warps to a row from three rounds on; a second segment where they would have more than two
+        // rounds each (6144 x 24000: 132 us with it, 134 without; 4096 x 131072: 472 and 481), more
+        // while there are few rows (512 x 32768: 11.7 with two, 17.8 with one)
+        rp.split = !write ? 0 : rounds >= 3 ? 2 : rounds == 2 ? 1 : 0;
+        const int64_t each = ceil_div(rounds, 1 << rp.split), room = 8 * (int64_t)sm_count() / rows;
+        const int64_t least = each > 2 ? 2 : 1, segs = room > least ? (room < each ? room : each) : least;
+        rp.seg_rounds = (int)ceil_div(each, segs) << rp.split;
         auto go = [&](auto k, dim3 g) { return launch_chained(k, g, 32 * row_warps(write), 0, 1, st, at<uint4>(l.w), rp); };
-        return write ? go(strip_row_kernel<true>, dim3(grid, (unsigned)ceil_div(rounds, rp.seg_rounds)))
-                     : go(strip_row_kernel<false>, dim3(grid));
+        if (!write) return go(strip_row_kernel<false, 1>, dim3(grid));
+        const dim3 g((unsigned)ceil_div(rows, row_warps(true) >> rp.split), (unsigned)ceil_div(rounds, rp.seg_rounds));
+        return (int64_t)g.x * g.y <= 6 * sm_count() ? go(strip_row_kernel<true, 6>, g)
+                                                    : go(strip_row_kernel<true, 7>, g);
     }
 
     cudaError_t grads(int s, float* dQ, int64_t lddq, float* dP, int64_t lddp, float* loss) {
