@@ -1510,11 +1510,13 @@ GradDeal deal_grads(int64_t rows, int64_t N, int d, bool f32, bool dq, bool dp) 
     double best_cost = 0;
     for (int width = f32 ? 128 : 256; width >= 128; width -= 128) {
         const int tn = (int)ceil_div(d, width);
-        // cycles per contraction block, and what cutting tiles costs beyond its share of them: fitted to 168
-        // shapes (150 to 6000 queries, 128 to 1024 columns) with every choice forced; the choice this makes
-        // is within 7 % of the best one at each, 0.3 % on average
-        const double unit = f32 ? 1320 : width == 256 ? 560 : 360;
-        const double cut = f32 ? 9000 : width == 256 ? 18000 : 15000;
+        // Cycles per contraction block; what cutting tiles costs by itself; and per part of a tile, whose
+        // sums its last pair adds up one after the other (dQ alone of 512 x 8192 x 64: 64 runs 49 us, 12 runs
+        // 28).  Fitted to 258 shapes (150 to 16384 queries, 64 to 1024 columns, one gradient or both) with
+        // every choice forced: the choice this makes is within 7 % of the best at each, 0.3 % on average.
+        const double unit = f32 ? 1320 : width == 256 ? 560 : 364;
+        const double cut = f32 ? 6300 : width == 256 ? 18000 : 8800;
+        const double part = f32 ? 970 : width == 256 ? 3080 : 1580;
         const int64_t kq = ceil_div(N, KB), kp = ceil_div(rows, KB);
         const int64_t tq = dq ? ceil_div(rows, 256) * tn : 0, tp = dp ? ceil_div(N, 256) * tn : 0;
         auto offer = [&](double cost, int whole, int used) {
@@ -1530,12 +1532,14 @@ GradDeal deal_grads(int64_t rows, int64_t N, int d, bool f32, bool dq, bool dp) 
                 offer((a > b ? a : b) * unit, w, pairs);
             }
         }
-        // equal runs of contraction blocks, at least four to a pair
-        const int64_t units = (tq * kq + tp * kp) / tn;
-        int64_t groups = pairs / tn;
-        if (groups > units / 4) groups = units / 4;
+        // equal runs of contraction blocks, at least four to a pair: as many as cost least
+        if (tn > pairs) continue;
+        const double units = (double)((tq * kq + tp * kp) / tn), longest = (double)(tq && (kq > kp || !tp) ? kq : kp);
+        int groups = (int)(units * sqrt(unit / (part * longest)));
+        if (groups > pairs / tn) groups = pairs / tn;
+        if (groups > units / 4) groups = (int)(units / 4);
         if (groups < 1) groups = 1;
-        if (tn <= pairs) offer((double)units / groups * unit + cut, -1, (int)(groups * tn));
+        offer(units / groups * unit + cut + part * longest * groups / units, -1, groups * tn);
     }
     return best;
 }
