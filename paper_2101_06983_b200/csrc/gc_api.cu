@@ -101,9 +101,11 @@ Plan make_plan(int64_t B, int64_t N, int d, int dtype, bool stored) {
         // positive terms, then the gated fallback sequence
         pl.launches_build = 8 + (pl.g_mp > 1 ? 1 : 0) + pl.launches_build;
     }
-    pl.strips = strip_applicable(B, N, d, dtype) ? 1 : 0;
+    for (int u = STRIP_FWD; u < STRIP_TWO_DIR; ++u)
+        pl.strips |= strip_applicable((StripUse)u, B, N, d, dtype) ? 1 << u : 0;
     if (pl.strips) {
-        const size_t need = strip_workspace_bytes(B, N, d, dtype);
+        const size_t need = pl.strips == 1 << STRIP_FWD ? strip_forward_bytes(B, N, d, dtype)
+                                                        : strip_workspace_bytes(B, N, d, dtype);
         if (need > off) off = need;
     }
     pl.total = off;
@@ -577,10 +579,14 @@ size_t forward_layout(Plan* pl, int64_t B, int64_t N) {
     return off;
 }
 
+StripUse strip_use(int op) {
+    return op == GC_OP_FWD ? STRIP_FWD : op == GC_OP_BWD ? STRIP_BWD : STRIP_BUILD;
+}
+
 // Scratch of the strip plan's forward where it serves this problem from the static array, else 0:
 // problems whose logits (fp32) or slots do not fit keep the plans that need less.
 size_t static_strip_need(int64_t B, int64_t N, int d, int dtype) {
-    if (!strip_applicable(B, N, d, dtype)) return 0;
+    if (!strip_applicable(STRIP_FWD, B, N, d, dtype)) return 0;
     const size_t need = strip_forward_bytes(B, N, d, dtype);
     return need <= (size_t)GC_STATIC_SCRATCH_BYTES ? need : 0;
 }
@@ -620,7 +626,7 @@ const char* gc_plan_name(int op, int64_t B, int64_t N, int d, int dtype) {
     if (op < GC_OP_FWD || op > GC_OP_BUILD_STORED || B <= 0 || N <= 0 || d <= 0) return "invalid";
     if (op == GC_OP_BUILD_STORED && !make_plan(B, N, d, dtype, true).mat) return "invalid";
     if (op != GC_OP_BUILD_STORED && small_applicable(B, N, d, dtype)) return "tcgen05-one-tile";
-    if (op != GC_OP_BUILD_STORED && strip_applicable(B, N, d, dtype))
+    if (op != GC_OP_BUILD_STORED && strip_applicable(strip_use(op), B, N, d, dtype))
         return small_tiled_applicable(B, N, d, dtype) ? "tcgen05-tiles" : "tcgen05";
     return tc_supported(B, N, d, dtype) ? "tcgen05" : "simt";
 }
@@ -628,7 +634,7 @@ const char* gc_plan_name(int op, int64_t B, int64_t N, int d, int dtype) {
 int gc_kernel_launches(int op, int64_t B, int64_t N, int d, int dtype) {
     if (B <= 0 || N <= 0 || d <= 0) return 0;
     if (op >= GC_OP_FWD && op <= GC_OP_BUILD && small_applicable(B, N, d, dtype)) return 1;
-    if (op >= GC_OP_FWD && op <= GC_OP_BUILD && strip_applicable(B, N, d, dtype))
+    if (op >= GC_OP_FWD && op <= GC_OP_BUILD && strip_applicable(strip_use(op), B, N, d, dtype))
         return strip_launches(op, B, N, d, dtype);
     Plan pl = make_plan(B, N, d, dtype);
     if (op == GC_OP_FWD) return pl.launches_fwd;
@@ -653,7 +659,7 @@ int gc_loss_fwd(const void* Q, int64_t ldq, const void* P, int64_t ldp, const in
     if (small_applicable(B, N, d, dtype))
         return run_small(GC_OP_FWD, p, nullptr, loss, row_lse, pos_logit, nullptr, 0, nullptr, 0,
                          dev_status, static_cast<cudaStream_t>(cuda_stream));
-    if (pl.strips) {
+    if (pl.strips >> STRIP_FWD & 1) {
         KernelTimer t(0, static_cast<cudaStream_t>(cuda_stream));
         return strip_forward(p, ws, loss, row_lse, pos_logit, dev_status,
                              static_cast<cudaStream_t>(cuda_stream)) == cudaSuccess ? GC_OK : GC_ERR_CUDA;
@@ -715,7 +721,7 @@ int gc_loss_bwd(const void* Q, int64_t ldq, const void* P, int64_t ldp, const in
     if (small_applicable(B, N, d, dtype) && (dQ || dP))
         return run_small(GC_OP_BWD, p, row_lse, nullptr, nullptr, nullptr, dQ, lddq, dP, lddp,
                          dev_status, st);
-    if (pl.strips && (dQ || dP)) {
+    if ((dQ || dP) && pl.strips >> (dQ && dP ? STRIP_BWD : STRIP_BWD_ONE) & 1) {
         KernelTimer t(1, st);
         return strip_backward(p, ws, row_lse, dQ, lddq, dP, lddp, dev_status, st) == cudaSuccess
                    ? GC_OK : GC_ERR_CUDA;
@@ -747,7 +753,7 @@ int gc_build_cache(const void* Q, int64_t ldq, const void* P, int64_t ldp, const
     if (small_applicable(B, N, d, dtype))
         return run_small(GC_OP_BUILD, p, nullptr, loss, row_lse, pos_logit, dQ, lddq, dP, lddp,
                          dev_status, st);
-    if (pl.strips) {
+    if (pl.strips >> STRIP_BUILD & 1) {
         KernelTimer t(1, st);
         return strip_build(p, ws, loss, row_lse, pos_logit, dQ, lddq, dP, lddp, dev_status, st) ==
                        cudaSuccess ? GC_OK : GC_ERR_CUDA;
@@ -803,7 +809,7 @@ int gc_shard_fwd_dq(const void* Q, int64_t ldq, const void* P, int64_t ldp, cons
     Problem p = make_problem(q_first, ldq, P, ldp, pos_idx + q0, q_count, N, d, tau, mask_mode, dtype);
     p.b_total = B;
     p.mask_shift = q0;             // local query i is query q0 + i of the batch
-    if (pl.strips) {
+    if (pl.strips >> STRIP_BUILD_DQ & 1) {
         cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
         KernelTimer t(1, st);
         return strip_build(p, ws, loss_part, row_lse + q0, pos_logit ? pos_logit + q0 : nullptr, dQ, lddq,
@@ -831,7 +837,7 @@ int gc_shard_dp(const void* Q, int64_t ldq, const void* P, int64_t ldp, const in
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     char* w = static_cast<char*>(ws);
     const char* p_first = static_cast<const char*>(P) + (size_t)p0 * (size_t)ldp * elem_size(dtype);
-    if (pl.strips) {
+    if (pl.strips >> STRIP_BWD_ONE & 1) {
         Problem p = make_problem(Q, ldq, p_first, ldp, pos_idx, B, p_count, d, tau, mask_mode, dtype);
         p.mask_shift = -p0;
         p.pos_base = p0;

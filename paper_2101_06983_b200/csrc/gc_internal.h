@@ -137,7 +137,7 @@ struct FwdArgs {
 struct Plan {
     int tc;                 // 1: tcgen05 kernels, 0: SIMT kernels
     int tiles_y;            // fp32: passage tiles of the forward that gc_loss_fwd_static falls back to
-    int strips;             // 1: three products over strips of query rows (gc_strip.cu)
+    int strips;             // bit u: a StripUse u of this problem takes the strip plan (gc_strip.cu)
     int g_fwd, g_dq, g_dp;  // split factors of the streamed range
     size_t off_m, off_l, off_pos, off_red, off_accq, off_accp;
     size_t total;           // workspace bytes (multiple of 256)
@@ -236,7 +236,10 @@ cudaError_t launch_small_tiled_fwd(const Problem& pr, float* part_m, float* part
                                    float* red, int* dev_status, cudaStream_t st);
 
 // gc_strip.cu
-bool strip_applicable(int64_t B, int64_t N, int d, int dtype);
+// What a call wants of the strip plan: the loss alone; both gradients with the loss, or given row_lse; dQ
+// with the loss; one gradient given row_lse; the two-direction loss.
+enum StripUse { STRIP_FWD, STRIP_BUILD, STRIP_BWD, STRIP_BUILD_DQ, STRIP_BWD_ONE, STRIP_TWO_DIR, STRIP_USES };
+bool strip_applicable(StripUse use, int64_t B, int64_t N, int d, int dtype);
 size_t strip_workspace_bytes(int64_t B, int64_t N, int d, int dtype);
 size_t strip_forward_bytes(int64_t B, int64_t N, int d, int dtype);     // strip_forward's share of it
 int strip_launches(int op, int64_t B, int64_t N, int d, int dtype);

@@ -1798,26 +1798,53 @@ struct StripRun {
 
 }  // namespace
 
-// Which problems take the strip plan.  fp32 and bf16 widths that are no multiple of 64: those of
-// small_tiled_applicable (up to 2 GiB of tile-pair planes, 64 tile pairs).  bf16 rows of more than 384
-// values in whole 64s: always, up to N = 2^18 (a strip's weights are bounded, so more passages mean
-// fewer queries per strip and more passes over dP).  Narrower rows: while the exponentials, which the
-// strip plan writes, converts and reads twice, cost less than forming every logit twice (the sweeps of
-// gc_narrow.cu and gc_tc.cu keep them on the chip).  Measured, us per gc_build_cache, sweeps / strips:
-//   d = 128:  3000 x 6000  67 / 51    4096 x 8192  73 / 72     6000 x 6000   77 / 103
-//   d = 256:  2048 x 4096  70 / 38    4096 x 8192  95 / 82     6000 x 12000 155 / 194
-//   d = 384:  4096 x 8192 154 / 101   8192 x 16384 447 / 418  16384 x 32768 1635 / 1731
-//   d = 768:  1024 x 2048  72 / 28    8192 x 16384 684 / 586  32768 x 65536 11.9 / 10.0 ms
+// Which calls take the strip plan.  fp32 and bf16 widths that are no multiple of 64: the problems of
+// small_tiled_applicable (up to 2 GiB of tile-pair planes, 64 tile pairs).  bf16 rows in whole 64s, in one
+// strip or up to N = 2^18 (a strip's weights are bounded, so more passages mean fewer queries per strip
+// and more passes over dP): the loss alone always; with gradients, narrow rows only up to a number of pairs, beyond which
+// the weights, written and read (and, in a build, converted) in memory, cost more than the sweeps of
+// gc_narrow.cu and gc_tc.cu, which keep them on the chip and form the logits again.  Measured, us, sweeps
+// / strips, on both sides of each limit (in units of 2^20 pairs):
+//   build      d =  64  5000 x 5000 61 / 61      4096 x 8192 66 / 68
+//              d = 128  4096 x 8192 72 / 70      6000 x 6000 76 / 78
+//              d = 256  5000 x 10000 140 / 137   6000 x 12000 158 / 165
+//              d = 384  8192 x 16384 421 / 375   16384 x 32768 1812 / 1661
+//   backward   d =  64  4096 x 4096 39 / 37      3000 x 6000 37 / 40     (d = 128: 5000 x 5000 53 / 49,
+//              4096 x 8192 57 / 61; d = 256: 8192 x 16384 262 / 201)
+//   dQ only    d = 128  1024 x 16384 58 / 50     2048 x 16384 60 / 68
+//   (of eight) d = 256  1500 x 24000 88 / 86     2048 x 16384 82 / 87
+//              d = 384  1500 x 24000 109 / 96    2048 x 32768 154 / 182  (d = 512: 247 / 217)
+//   dP only    d = 128  3000 x 750 23 / 23       4096 x 1024 23 / 27
+//   (of eight) d = 256  6000 x 1500 37 / 34      8192 x 2048 44 / 44, 16384 x 2048 65 / 71
+//   both directions, d = 128: 12000 x 12000 431 / 366, 16384 x 16384 585 / 646
+//   loss alone d =  64  16384 x 32768 283 / 238  30000 x 60000 994 / 801
 // GRADCACHE_PLAN=sweeps: as in gc_small.cu.
-bool strip_applicable(int64_t B, int64_t N, int d, int dtype) {
+bool strip_applicable(StripUse use, int64_t B, int64_t N, int d, int dtype) {
     const char* e = getenv("GRADCACHE_PLAN");
     if (e && strcmp(e, "sweeps") == 0) return false;
     if (d % 8 != 0 || d > MAX_D || small_applicable(B, N, d, dtype)) return false;
     if (N > (1 << 24) || B > (1 << 24)) return false;
     if (dtype == GC_F32 || d % 64 != 0) return small_tiled_applicable(B, N, d, dtype);
-    if (d > 384) return N <= 1 << 18;
-    const int64_t most = d <= 128 ? 24 : d <= 256 ? 36 : 144;
-    return B * N <= most << 20;
+    if (N > 1 << 18 && B * N > (int64_t)256 << 20) return false;
+    if (use == STRIP_FWD || d > 384) return true;
+    constexpr int ANY = 0;
+    static const int most[][4] = {      // d <= 64, 128, 256, 384
+        {24, 32, 56, ANY},              // STRIP_BUILD
+        {16, 24, ANY, ANY},             // STRIP_BWD
+        {20, 20, 28, 44},               // STRIP_BUILD_DQ
+        {2, 2, 14, ANY},                // STRIP_BWD_ONE
+        {160, 160, ANY, ANY},           // STRIP_TWO_DIR
+    };
+    const int limit = most[use - STRIP_BUILD][d <= 64 ? 0 : d <= 128 ? 1 : d <= 256 ? 2 : 3];
+    return limit == ANY || B * N <= (int64_t)limit << 20;
+}
+
+// A build that forms the logits twice, for the logsumexp and then for the weights, and has no row pass:
+// rows for which a product costs less than reading, converting and writing the weights out of the memory
+// (384: 12000 x 24000 871 us with the row pass, 812 without, 16384 x 32768 1661 and 1593; 8192 x 16384
+// 375 and 395.  512: 16384 x 16384 808 and 815).
+static bool logits_twice(int64_t B, int64_t N, int d, int dtype) {
+    return dtype != GC_F32 && d <= 384 && B * N > (int64_t)192 << 20;
 }
 
 size_t strip_workspace_bytes(int64_t B, int64_t N, int d, int dtype) {
@@ -1831,6 +1858,7 @@ int strip_launches(int op, int64_t B, int64_t N, int d, int dtype) {
     const int strips = strip_layout(B, N, d, dtype).strips, pre = dtype == GC_F32 ? 1 : 0;
     if (op == GC_OP_FWD) return pre + 2 * strips;
     if (op == GC_OP_BWD) return pre + (dtype == GC_F32 ? 3 : 2) * strips;
+    if (logits_twice(B, N, d, dtype)) return 4 * strips;
     return pre + 3 * strips;
 }
 
@@ -1850,6 +1878,10 @@ cudaError_t strip_forward(const Problem& p, void* ws, float* loss, float* row_ls
 cudaError_t strip_build(const Problem& p, void* ws, float* loss, float* row_lse, float* pos_logit,
                         float* dQ, int64_t lddq, float* dP, int64_t lddp, int* dev_status,
                         cudaStream_t st) {
+    if (dP && logits_twice(p.B, p.N, p.d, p.dtype)) {
+        const cudaError_t f = strip_forward(p, ws, loss, row_lse, pos_logit, dev_status, st);
+        return f == cudaSuccess ? strip_backward(p, ws, row_lse, dQ, lddq, dP, lddp, dev_status, st) : f;
+    }
     cudaError_t e = configure_kernels();
     StripRun r(p, ws, dev_status, st);
     if (e == cudaSuccess && r.f32) e = r.split();

@@ -293,11 +293,11 @@ MultiLayout multi_layout(int64_t B, int64_t N, int d, int dtype, int64_t n_pos) 
 // bf16: both directions in one set of weights (strip plan), W_ij = p_ij + m_j p'_ij - 2 [j = r_i] with p'
 // the softmax over the queries and m_j the number of queries j is the positive of.
 bool two_dir_strips(int64_t B, int64_t N, int d, int dtype) {
-    return dtype == GC_BF16 && strip_applicable(B, N, d, dtype);
+    return dtype == GC_BF16 && strip_applicable(STRIP_TWO_DIR, B, N, d, dtype);
 }
 
 bool two_dir_swapped(int64_t B, int64_t N, int d, int dtype) {
-    return two_dir_strips(B, N, d, dtype) && strip_applicable(N, B, d, dtype) && N <= B + B / 4;
+    return two_dir_strips(B, N, d, dtype) && strip_applicable(STRIP_TWO_DIR, N, B, d, dtype) && N <= B + B / 4;
 }
 // what gc_build_cache would refuse
 int check_two_dir(const void* Q, int64_t ldq, const void* P, int64_t ldp, float tau, int es) {
@@ -329,9 +329,10 @@ TwoDirLayout two_dir_layout(int64_t B, int64_t N, int d, int dtype) {
     if (two_dir_strips(B, N, d, dtype)) {
         l.count = off;    off += align256v(2 * sizeof(int) * (size_t)N);
         l.col_neg = off;  off += align256v(sizeof(float) * (size_t)(N + 4));
-        w2 = strip_workspace_bytes(B, B, d, dtype);
-        if (two_dir_swapped(B, N, d, dtype) && strip_workspace_bytes(N, B, d, dtype) > w2)
-            w2 = strip_workspace_bytes(N, B, d, dtype);
+        const size_t need[] = {strip_workspace_bytes(B, N, d, dtype), strip_forward_bytes(B, B, d, dtype),
+                               strip_forward_bytes(N, B, d, dtype)};
+        w2 = 0;
+        for (const size_t n : need) w2 = n > w2 ? n : w2;
     }
     l.inner = off;  off += w1 > w2 ? w1 : w2;
     l.total = off;

@@ -53,6 +53,27 @@ def test_build_and_split_calls(binding, oracle, B, N, d, dtype, mask, tau):
     check_against_oracle(prob, b, ref)
 
 
+@pytest.mark.parametrize("B,N", [(333, 4100), (66, 33000), (650, 17000), (1300, 16500), (3, 270000)])
+def test_long_rows_of_the_row_pass(binding, oracle, B, N):
+    """Four warps to a row with the last one idle; segments of one, two and three rounds; a grid beyond
+    six blocks per SM; more slots than a lane holds at once."""
+    prob = inputs.random_problem(B, N, 64, "bf16", seed=B + N, tau=0.2, scale=0.125)
+    check_against_oracle(prob, run_build(prob), _oracle_full(oracle, prob))
+
+
+def test_logits_formed_twice(binding, oracle):
+    """Rows of at most 384 values and many pairs: no row pass, two launches more per strip."""
+    n, d = 16700, 320
+    prob = inputs.random_problem(n, n, d, "bf16", seed=7, tau=0.5, mask_mode=inputs.MASK_SELF,
+                                 scale=d ** -0.5)
+    assert binding.gc_kernel_launches(binding.GC_OP_BUILD, n, n, d, binding.GC_BF16) == 2 * 4
+    out = run_build(prob)
+    assert int(out.dev_status.item()) == 0
+    _check_sampled(oracle, prob, out, 48, 24, full_lse=out.row_lse.cpu().numpy().astype(np.float64))
+    Q, P, _ = to_device(prob)
+    _check_properties(prob, out, Q, P)
+
+
 def test_several_strips_f32_self_mask(binding, oracle):
     """8200 x 8200 pairs are two strips; the diagonal runs through both."""
     prob = inputs.random_problem(8200, 8200, 16, "f32", seed=5, tau=0.5, mask_mode=inputs.MASK_SELF,
