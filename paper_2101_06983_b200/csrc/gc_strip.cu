@@ -1557,12 +1557,11 @@ StripLayout strip_layout(int64_t B, int64_t N, int d, int dtype, bool fwd_only =
     const bool f32 = dtype == GC_F32;
     // Few strips: each costs a read and a write of dP and the fill and drain of three kernels.  Whether
     // a strip's weights stay in the L2 matters less (8192 x 16384 x 768: 586 us in one strip of 268 MB,
-    // 666 in four of 67 MB; 16384 x 32768: 2.41-2.51 ms against 3.33).  bf16: 512 MB of weights, or 1 GB
-    // where that means fewer than 4096 queries; fp32 holds 8 bytes a pair and does four times the
-    // arithmetic: 64 M pairs.
-    const int64_t pairs = f32 ? 64 : ceil_div(N, 1024) > 64 ? 512 : 256;
-    int64_t r = (pairs << 20) / N / 256 * 256;
-    if (pairs == 512 && r > 4096) r = 4096;
+    // 666 in four of 67 MB).  bf16: 768 M pairs, 1.5 GB of weights (ms in strips of 0.5 GB, or 1 GB beyond
+    // 65536 passages, and of 1.5-2 GB: 16384 x 32768 x 768 2.38 / 2.33, 40000 x 80000 x 512 11.1 / 10.7,
+    // 65536 x 131072 x 768 38.3 / 37.0, loss and gradients of 40000 x 120000 x 256 11.5 / 11.0; 4 GB would
+    // give 10.5, 37.8 and 10.5); fp32 holds 8 bytes a pair and does four times the arithmetic: 64 M pairs.
+    int64_t r = ((int64_t)(f32 ? 64 : 768) << 20) / N / 256 * 256;
     if (r < 256) r = 256;
     const int64_t n = ceil_div(B, r);
     r = ceil_div(ceil_div(B, n), 256) * 256;
