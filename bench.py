@@ -36,19 +36,16 @@ def metric_name(B, N, d):
 
 NOMINAL_BF16_TFLOPS = 2250.0      # public dense bf16 figure for B200, context only
 # dram__bytes_read.sum + dram__bytes_write.sum of ONE STEP (every launch of a gc_build_cache
-# call summed) from the ncu captures summarised under profiles/ (quad_kernel_cfg2_*, quad_kernel_
-# cfg4_*, small_kernel_*).  Under ncu every launch starts from flushed caches, so a step of
-# several launches counts its inputs once per launch.  A figure is reported only while the
-# sources its kernels come from still have the hash they had when the counters were taken.
-SWEEP_SOURCES = ['gc_api.cu', 'gc_combine.cu', 'gc_internal.h', 'gc_quad.cu', 'gc_tc.cu', 'tc_common.cuh']
-ONE_TILE_SOURCES = ['gc_api.cu', 'gc_internal.h', 'gc_small.cu', 'tc_common.cuh']
-NARROW_SOURCES = SWEEP_SOURCES + ['gc_narrow.cu']
+# call summed) from ncu captures (profiles/strip_kernels_cfg2_*, small_kernel_*).  Under ncu every
+# launch starts from flushed caches, so a step of several launches counts its inputs once per
+# launch.  A figure is reported only while the sources its kernels come from still have the hash
+# they had when the counters were taken.
+STRIP_SOURCES = ['gc_strip.cu', 'tc_common.cuh']
+ONE_TILE_SOURCES = ['gc_small.cu', 'gc_small_f32.cu', 'tc_common.cuh']
 NCU_STEP_TRAFFIC = {
-    "cfg2_": (82.9e6, SWEEP_SOURCES, "984da4d026488e42db1a380f3e3a5b542047d09f"),
-    "cfg4_": (4.80e9, SWEEP_SOURCES, "984da4d026488e42db1a380f3e3a5b542047d09f"),
-    "cfg3_": (26.4e6, NARROW_SOURCES, "44a0d1324795e9d77b5ed87232933502e92ce031"),
-    "cfg1_": (0.629e6, ONE_TILE_SOURCES, "42794198880e3035735ceb1c20a53113fbce4c0e"),
-    "cfg0_": (0.640e6, ONE_TILE_SOURCES, "42794198880e3035735ceb1c20a53113fbce4c0e"),
+    "cfg2_": (287.3e6, STRIP_SOURCES, "cca1fe5a95949c88c1b4569a516c7d996485d6fa"),
+    "cfg1_": (0.627e6, ONE_TILE_SOURCES, "0cd4e6330cdbe269ff964a2ca75e1035488fc56c"),
+    "cfg0_": (0.634e6, ONE_TILE_SOURCES, "0cd4e6330cdbe269ff964a2ca75e1035488fc56c"),
 }
 FP32_LANES_PER_SM = 128           # fp32 FMA lanes of one SM (2 FLOP per lane and clock)
 
@@ -425,9 +422,9 @@ def run_ours(args, rank, local_rank, world):
 
     if rank == 0:
         pk = load_peaks()
-        # dominant kernel: the tile sweep kernel, launched twice per step for the gradients.  The
-        # dP launch delivers one useful GEMM (2 B N d); the dQ launch delivers one, or two when the
-        # forward is fused into it (no separate forward launch was timed).
+        # The tensor-core launches of a step.  Strip plan: all of the step's launches, one figure (the
+        # dQ slot).  Sweeps: two launches; the dP launch delivers one useful GEMM (2 B N d), the dQ
+        # launch one, or two when the forward is fused into it (no separate forward launch was timed).
         # The stored-weights plan has three tensor kernels of one useful GEMM each.
         fused = kern[0] == 0.0
         if stored:
@@ -439,7 +436,7 @@ def run_ours(args, rank, local_rank, world):
         achieved = sweep_flop / (sweep_ms * 1e-3) / 1e12 if sweep_ms > 0 else 0.0
         value = replicas.whole_job_rate(flop, world, ms_per_step) / 1e12
         if plan.startswith("tcgen05"):
-            roof = {"bound": "tensor", "kernel": f"{plan} sweeps (the tensor-core launches of a step)",
+            roof = {"bound": "tensor", "kernel": f"{plan} (the tensor-core launches of a step)",
                     "achieved": achieved, "peak": pk["tf_burst"], "unit": "TFLOP/s",
                     "frac": achieved / pk["tf_burst"], "peak_source": pk["source"]}
         else:
@@ -625,12 +622,12 @@ def run_apply(args):
     ms = sum(a.elapsed_time(b) for a, b in ev) / args.steps
     pk = load_peaks()
     nbytes = 4.0 * rows * d + 2.0 * rows * d_in + 4.0 * d * d_in
-    # dram bytes of the call's one launch at 4096 rows, from
+    # dram bytes of the call's two launches at 4096 rows, from
     # profiles/apply_kernel_rows4096_d768_din768.txt; reported while gc_apply.cu is unchanged
     import hashlib
     with open(os.path.join(ROOT, "paper_2101_06983_b200", "csrc", "gc_apply.cu"), "rb") as fh:
-        same = hashlib.sha1(fh.read()).hexdigest() == "71def43a9090e7af98d500aed9dc7b0ff9170948"
-    traffic = 18.9e6 if same and rows == 4096 else None
+        same = hashlib.sha1(fh.read()).hexdigest() == "ee38bebd7446ec94ae01602901763dce147fab0f"
+    traffic = 37.8e6 if same and rows == 4096 else None
     import oracle
     t0 = time.perf_counter()
     ref = oracle.cache_apply(U, X)
