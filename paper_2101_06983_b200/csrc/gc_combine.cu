@@ -32,18 +32,19 @@ lse_combine_kernel(const float* __restrict__ part_m, const float* __restrict__ p
                    float* __restrict__ pos_logit, float* __restrict__ loss, float* red,
                    int* __restrict__ dev_status, const Gate gate, int64_t mean_over,
                    int64_t mask_shift) {
+    dep_wait();
     if (gate_closed(gate)) return;
     __shared__ float warp_sum[kCombineThreads / 32];
     __shared__ int warp_flag[kCombineThreads / 32];
     __shared__ int is_last;
     float local = 0.f;
     int flags = 0;
-    for (int64_t i = blockIdx.x * (int64_t)kCombineThreads + threadIdx.x; i < B;
-         i += (int64_t)gridDim.x * kCombineThreads) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < B;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        int f = pos_flags(pos_idx[i], i, N, mask_mode, mask_shift);
+        const float pos = pos_ws[i], pl = f ? 0.f : pos;
         const float lse = combined_lse(part_m, part_l, groups, B, i);
         row_lse[i] = lse;
-        int f = pos_flags(pos_idx[i], i, N, mask_mode, mask_shift);
-        float pl = f ? 0.f : pos_ws[i];
         if (pos_logit) pos_logit[i] = pl;
         flags |= f;
         local += lse - pl;
@@ -56,8 +57,8 @@ lse_combine_kernel(const float* __restrict__ part_m, const float* __restrict__ p
     if (lane == 0) { warp_sum[warp] = local; warp_flag[warp] = flags; }
     __syncthreads();
     if (warp == 0) {
-        float v = lane < kCombineThreads / 32 ? warp_sum[lane] : 0.f;
-        int f = lane < kCombineThreads / 32 ? warp_flag[lane] : 0;
+        float v = lane < (int)blockDim.x / 32 ? warp_sum[lane] : 0.f;
+        int f = lane < (int)blockDim.x / 32 ? warp_flag[lane] : 0;
         for (int o = 16; o > 0; o >>= 1) {
             v += __shfl_xor_sync(0xffffffffu, v, o);
             f |= __shfl_xor_sync(0xffffffffu, f, o);
@@ -344,15 +345,16 @@ cudaError_t launch_lse_combine(const float* part_m, const float* part_l, const f
                                int mask_mode, float* row_lse, float* pos_logit, float* loss,
                                float* red, int* dev_status, Gate gate, cudaStream_t st,
                                int64_t mean_over, int64_t mask_shift) {
-    int64_t blocks = (B + kCombineThreads - 1) / kCombineThreads;
+    // Small blocks while they spread the rows over more SMs: the sweep after it waits for this kernel.
+    // 8192 rows, 8 slots: 7.1 us as 128 blocks with their loads in flight together and set up under the
+    // sweep before it, about 10 as 32 blocks that read one slot after the other.
+    const int threads = B <= 64 * (int64_t)sm_count() ? 64 : kCombineThreads;
+    int64_t blocks = (B + threads - 1) / threads;
     if (blocks > sm_count()) blocks = sm_count();
     if (blocks > 256) blocks = 256;          // the scratch holds this many block sums
-    lse_combine_kernel<<<(int)blocks, kCombineThreads, 0, st>>>(part_m, part_l, pos_ws, pos_idx,
-                                                               groups, B, N, mask_mode, row_lse,
-                                                               pos_logit, loss, red, dev_status,
-                                                               gate, mean_over > 0 ? mean_over : B,
-                                                               mask_shift);
-    return cudaGetLastError();
+    return launch_chained(lse_combine_kernel, dim3((unsigned)blocks), (unsigned)threads, 0, 1, st, part_m, part_l,
+                          pos_ws, pos_idx, groups, B, N, mask_mode, row_lse, pos_logit, loss, red, dev_status,
+                          gate, mean_over > 0 ? mean_over : B, mask_shift);
 }
 
 namespace {

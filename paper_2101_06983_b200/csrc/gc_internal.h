@@ -57,11 +57,13 @@ __device__ __forceinline__ float combined_lse(const float* __restrict__ part_m,
                                               const float* __restrict__ part_l, int slots,
                                               int64_t pitch, int64_t i) {
     float m = -INFINITY;
+#pragma unroll 8
     for (int g = 0; g < slots; ++g) m = fmaxf(m, part_m[(int64_t)g * pitch + i]);
     float l = 0.f;
+#pragma unroll 8
     for (int g = 0; g < slots; ++g) {
-        const float mg = part_m[(int64_t)g * pitch + i];
-        if (mg > -INFINITY) l = __fmaf_rn(part_l[(int64_t)g * pitch + i], expf(mg - m), l);
+        const float mg = part_m[(int64_t)g * pitch + i], lg = part_l[(int64_t)g * pitch + i];
+        if (mg > -INFINITY) l = __fmaf_rn(lg, expf(mg - m), l);
     }
     return __fadd_rn(m, logf(l));
 }
