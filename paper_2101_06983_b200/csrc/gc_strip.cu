@@ -1544,6 +1544,15 @@ GradDeal deal_grads(int64_t rows, int64_t N, int d, bool f32, bool dq, bool dp) 
     return best;
 }
 
+// Columns of a logit tile: 128 while there are at most one and a half 256-wide tiles to a CTA pair (more
+// pairs busy, or a shorter last wave, and epilogues that overlap products).  us per build of d = 768 with
+// 256 / 128: 500 x 1000 22.9 / 20.5, 1531 x 3062 35.1 / 33.7 (72 tiles, 74 pairs), 1300 x 3900 43.6 / 40.6 (96),
+// 1700 x 3400 46.3 / 44.1 (98); from there on nothing or a loss: 1800 x 3600 49.8 / 49.7 (120), 2048 x 4096
+// 51.5 / 51.6 (128), 3000 x 6000 78.9 / 81.7 (288).  d = 256 and 512, and the loss alone: the same sides.
+int logit_width(int64_t rows, int64_t N) {
+    return 2 * ceil_div(rows, 256) * ceil_div(N, 256) <= 3 * (int64_t)pairs_of_device() ? 128 : 256;
+}
+
 struct StripLayout {
     int64_t rows;                 // of a strip (the last may be shorter)
     int strips;
@@ -1641,9 +1650,7 @@ struct StripRun {
         const int64_t row0 = (int64_t)s * l.rows, rows = rows_of(s);
         const int pairs = pairs_of_device();
         const int tiles_m = (int)ceil_div(rows, 256);
-        // narrower tiles while 256-wide ones would leave half of the pairs without one
-        const bool narrow = f32 || 2 * tiles_m * ceil_div(p.N, 256) <= pairs;
-        const int bn = narrow ? 128 : 256;
+        const int bn = f32 ? 128 : logit_width(rows, p.N);
         LogitParams lp{};
         lp.rows = (int)rows; lp.N = (int)p.N;
         lp.kblocks = (int)ceil_div(p.d, KB);
@@ -1709,8 +1716,7 @@ struct StripRun {
             rp.slot_pitch = l.slot_pitch;
             rp.nslots = (int)ceil_div(p.N, 64);
         } else {
-            const int tiles_m = (int)ceil_div(rows, 256);
-            const int bn = 2 * tiles_m * ceil_div(p.N, 256) <= pairs_of_device() ? 128 : 256;
+            const int bn = logit_width(rows, p.N);
             rp.nslots = rp.slot_pitch = (int)(2 * ceil_div(p.N, bn));
         }
         rp.pos_ws = at<float>(l.pos);
