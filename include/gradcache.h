@@ -85,7 +85,8 @@ size_t gc_workspace_bytes(int op, int64_t B, int64_t N, int d, int dtype);
  *                       4096; at most two CTAs' worth of 64-column slices per SM)
  *   "tcgen05"           bf16, d a multiple of 64 up to 4096, TMA + tcgen05 MMA.  The strip plan: three
  *                       products over strips of query rows whose weights are held in the workspace;
- *                       or, for rows of at most 384 values and many pairs, sweeps that keep every
+ *                       or, for gradients of narrow rows (at most 256 values; 384 for one rank's dQ)
+ *                       with many pairs and for more than 2^18 passages, sweeps that keep every
  *                       logit on the chip (one CTA, a CTA pair or a cluster of four per tile)
  *   "simt"              fp32 FMA tiles: every other case (other widths, fp32 batches beyond that)
  * "invalid" for an unknown op, non-positive sizes, or a problem GC_OP_BUILD_STORED refuses.
