@@ -206,6 +206,13 @@ __device__ __forceinline__ void logit_tile(int t, int tiles_m, int tiles_n, int*
     *m = 8 * g + (r - *n * h);
 }
 
+// Counters for the kernels that follow, cleared by the epilogue warps of every block of the grid, however
+// few there are (thread: 0 .. 32 NSOFT - 1; NULL: nothing to clear).
+__device__ __forceinline__ void clear_words(int* words, int count, int thread) {
+    if (!words) return;
+    for (int e = (int)blockIdx.x * (32 * NSOFT) + thread; e < count; e += (int)gridDim.x * (32 * NSOFT)) words[e] = 0;
+}
+
 // BN: passages per tile (a CTA loads BN / 2 of them).  What bounds it: tcgen05 at 256 x 256 tiles (a
 // stage of 64 is 512 cycles of products for 32 KB per CTA); the epilogue's two special-function
 // operations per 32 lanes and clock stay below that from d = 256 on.
@@ -289,14 +296,8 @@ strip_logit_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
         const int ew = c.warp - (NPROD + 1);
         const int q = c.warp & 3, half = ew >> 2, lane = c.lane;
         constexpr int HC = BN / 2;                       // columns of this warp
-        if (p.zero && blockIdx.x < 8) {
-            for (int e = blockIdx.x * 256 + (ew * 32 + lane); e < p.zero_count; e += 8 * 256)
-                p.zero[e] = 0;
-        }
-        if (MODE == LOGIT_FWD && p.zero2) {
-            for (int e = (int)blockIdx.x * 256 + (ew * 32 + lane); e < p.zero2_count; e += (int)gridDim.x * 256)
-                p.zero2[e] = 0;
-        }
+        clear_words(p.zero, p.zero_count, ew * 32 + lane);
+        if (MODE == LOGIT_FWD) clear_words(p.zero2, p.zero2_count, ew * 32 + lane);
         const uint32_t stage_buf = c.smem + NST * STAGE + (uint32_t)ew * (SB * 4096u);
         const uint64_t c1_2 = pack2(p.c1, p.c1);
         int use = 0;
@@ -570,10 +571,7 @@ strip_logit_f32_kernel(const __grid_constant__ CUtensorMap mapQ,
     } else {
         const int ew = c.warp - (NPROD + 1);
         const int q = c.warp & 3, half = ew >> 2, lane = c.lane;
-        if (p.zero && blockIdx.x < 8) {
-            for (int e = blockIdx.x * 256 + (ew * 32 + lane); e < p.zero_count; e += 8 * 256)
-                p.zero[e] = 0;
-        }
+        clear_words(p.zero, p.zero_count, ew * 32 + lane);
         const uint32_t slot = c.smem + F_NST * F_STAGE + (uint32_t)ew * 8192u;
         int use = 0;
         for (int t = pair; t < total; t += pairs, ++use) {

@@ -138,3 +138,19 @@ def test_one_tile_f32_clusters(binding, oracle, B, N, d, mask):
     binding.gc_loss_bwd(*args, b.row_lse, None, b.dP, b.ws, b.dev_status)
     torch.cuda.synchronize()
     check_against_oracle(prob, b, ref)
+
+
+@pytest.mark.parametrize("B,N,d", [(768, 64, 3072), (705, 1, 3008), (768, 65, 3072)])
+def test_few_logit_tiles_clear_every_counter(binding, oracle, B, N, d):
+    """Three logit tiles (six CTAs), gradient tiles cut between CTA pairs: the counters of every cut tile
+    start at zero whatever the workspace held, in a first call and in a second one on other inputs."""
+    out = binding.Outputs(B, N, d, binding.GC_F32)
+    out.ws.fill_(0xA5)
+    for seed in (1, 2):
+        prob = inputs.random_problem(B, N, d, "f32", seed=seed, tau=0.5, scale=d ** -0.5)
+        Q, P, pos = to_device(prob)
+        out.dQ.fill_(float("nan"))
+        out.dP.fill_(float("nan"))
+        binding.build_cache(Q, P, pos, prob.tau, prob.mask_mode, out)
+        torch.cuda.synchronize()
+        check_against_oracle(prob, out, _oracle_full(oracle, prob))
