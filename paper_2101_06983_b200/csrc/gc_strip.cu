@@ -7,8 +7,8 @@
 //
 //   logit kernel   S = Q P^T on tcgen05, 256 x 256 tiles; the epilogue leaves, per row and group of
 //                  64 columns, the raw maximum m and sum of e = 2^((s - m) log2e / tau) as a slot and
-//                  the e themselves as fp16 (each in [0, 1], its group's largest exactly 1, so the
-//                  error is 2^-12 of a value, whatever the range of the logits)
+//                  the e themselves, each in [0, 1], in 16 bits (see stash_pack_small: off by at most 2^-11 of a
+//                  value down to 2^-14, by 2^-9 of it down to 2^-126)
 //   row kernel     merges a row's slots into row_lse, its share of the loss, and turns the row, in
 //                  place, into the bf16 weights W_ij = p_ij - [j = r_i] (0 at the masked pair)
 //   grad kernel    dQ = W P and dP += W^T Q in one launch; tiles of both products are dealt out in
@@ -84,6 +84,36 @@ __device__ __forceinline__ uint32_t pack_b2(float lo, float hi) {
     uint32_t r;
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
     return r;
+}
+
+// Exponentials of a group in 16 bits, two to a word.  Relative to the group's largest they cover as many
+// octaves as the logits span (a passage far below a hard negative of its group still has a row of dP), which
+// fp16 alone does not: below 2^-14 it rounds to multiples of 2^-24.  So: from 2^-14 on fp16, ten bits of
+// mantissa, with a sign bit of 0; below, a sign bit of 1 and the upper 15 bits of the fp32 number without
+// its sign, eight bits of mantissa, down to 2^-126.  The logits of most groups span fewer octaves: the second
+// form costs them a minimum over the logits here and a test per 16 bytes in the row kernel.
+// Measured, us, kernels with fp16 alone / as they are: logit kernel of a build 1531 x 3062 x 768 11.7 / 12.0, of
+// gradients 4096 x 8192 x 1024 54.6 / 56.5 and 4096 x 1024 x 768 14.7 / 15.5, row pass 1531 x 3062 6.3 / 6.4.
+constexpr float STASH_FP16 = 6.103515625e-5f;            // 2^-14
+__device__ __forceinline__ uint32_t stash_pack_small(uint32_t h, float a, float b) {
+    if (a < STASH_FP16) h = (h & 0xffff0000u) | 0x8000u | ((__float_as_uint(a) + 0x4000u) >> 15);
+    if (b < STASH_FP16) h = (h & 0xffffu) | 0x80000000u | ((__float_as_uint(b) + 0x4000u) >> 15 << 16);
+    return h;
+}
+// what such a code stands for
+__device__ __forceinline__ float stash_round_small(float a) {
+    return __uint_as_float((__float_as_uint(a) + 0x4000u) & 0xffff8000u);
+}
+// f times the two numbers
+__device__ __forceinline__ float2 stash_times(uint32_t h, float f) {
+    const float2 v = __half22float2(*reinterpret_cast<const __half2*>(&h));
+    return make_float2(v.x * f, v.y * f);
+}
+__device__ __forceinline__ float2 stash_times_small(uint32_t h, float f) {
+    float2 v = stash_times(h, f);
+    if (h & 0x8000u) v.x = __uint_as_float((h & 0x7fffu) << 15) * f;
+    if (h & 0x80000000u) v.y = __uint_as_float((h >> 16 & 0x7fffu) << 15) * f;
+    return v;
 }
 
 // p - 1 of a positive from its raw logit (roundings spelled out: two kernels form it, same bits).
@@ -362,7 +392,15 @@ strip_logit_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
                 const bool special = (unsigned)dp < 64u || (unsigned)dm < 64u;
                 const bool any_special = __any_sync(0xffffffffu, special) || jg + 64 > p.N;
                 float pos_raw = 0.f;
+                uint32_t h[MODE == LOGIT_STASH ? 32 : 1];        // the group's codes
                 if (MODE != LOGIT_W2) {
+                    float least = INFINITY;              // of the raw logits, special columns among them
+                    if (MODE != LOGIT_FWD) {
+                        float mn[4] = {s[0], s[1], s[2], s[3]};
+#pragma unroll
+                        for (int e = 4; e < 64; ++e) mn[e & 3] = fminf(mn[e & 3], s[e]);
+                        least = fminf(fminf(mn[0], mn[1]), fminf(mn[2], mn[3]));
+                    }
                     if (any_special) {
 #pragma unroll
                         for (int e = 0; e < 64; ++e) {
@@ -379,6 +417,8 @@ strip_logit_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
 #pragma unroll
                     for (int e = 4; e < 64; ++e) mx[e & 3] = fmaxf(mx[e & 3], s[e]);
                     const float gm = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+                    // (a little before 2^-14, so that every smaller exponential finds its code)
+                    const bool small = MODE != LOGIT_FWD && __any_sync(0xffffffffu, (least - gm) * p.c1 < -13.9f);
                     const float ref = gm == -INFINITY ? 0.f : gm;
                     const float off = -ref * p.c1;
                     const uint64_t off2 = pack2(off, off);
@@ -396,16 +436,32 @@ strip_logit_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
                     unpack2(add2(sum2, sum2b), sa, sb);
                     const float sum = sa + sb;
                     if (MODE == LOGIT_STASH) {
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) h[e] = pack_h2(s[2 * e], s[2 * e + 1]);
+                        if (small) {
+#pragma unroll
+                            for (int e = 0; e < 32; ++e) h[e] = stash_pack_small(h[e], s[2 * e], s[2 * e + 1]);
+                        }
+                    }
+                    if (MODE == LOGIT_STASH) {
                         if (i < p.rows) p.slots[(int64_t)i * p.slot_pitch + (jg >> 6)] = make_float2(gm, sum);
                     } else if (MODE == LOGIT_W) {
                         // what the row kernel makes of the stored exponentials, bit for bit
                         const float f = gm > -INFINITY ? ex2(fmaf(gm, p.c1, neg_lse)) : 0.f;
+                        if (small) {
 #pragma unroll
-                        for (int e = 0; e < 64; e += 2) {
-                            const uint32_t h = pack_h2(s[e], s[e + 1]);
-                            const float2 v = __half22float2(*reinterpret_cast<const __half2*>(&h));
-                            s[e] = v.x * f;
-                            s[e + 1] = v.y * f;
+                            for (int e = 0; e < 64; e += 2) {
+                                const float2 v = stash_times(pack_h2(s[e], s[e + 1]), f);
+                                s[e] = s[e] < STASH_FP16 ? stash_round_small(s[e]) * f : v.x;
+                                s[e + 1] = s[e + 1] < STASH_FP16 ? stash_round_small(s[e + 1]) * f : v.y;
+                            }
+                        } else {
+#pragma unroll
+                            for (int e = 0; e < 64; e += 2) {
+                                const float2 v = stash_times(pack_h2(s[e], s[e + 1]), f);
+                                s[e] = v.x;
+                                s[e + 1] = v.y;
+                            }
                         }
                         if ((unsigned)dp < 64u) {
                             const float pw = positive_weight(pos_raw, p.inv_tau, lse_i);
@@ -448,7 +504,7 @@ strip_logit_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
                         uint32_t w[4];
 #pragma unroll
                         for (int e = 0; e < 4; ++e)
-                            w[e] = MODE == LOGIT_STASH ? pack_h2(s[8 * j + 2 * e], s[8 * j + 2 * e + 1])
+                            w[e] = MODE == LOGIT_STASH ? h[MODE == LOGIT_STASH ? 4 * j + e : 0]
                                                        : pack_b2(s[8 * j + 2 * e], s[8 * j + 2 * e + 1]);
                         sts_v4(buf + (uint32_t)((j ^ (lane & 7)) << 4), w[0], w[1], w[2], w[3]);
                     }
@@ -720,7 +776,7 @@ __device__ __forceinline__ int row_pos(const RowParams& p, int i, int* flags) {
 
 // bf16 inputs: a warp per row, or (WRITE) 2^split warps, each taking every 2^split-th round of 2048
 // columns of the block's segment.  They merge the row's (max, sum) slots, form row_lse, the positive's
-// weight and the loss term, then turn the row's fp16 exponentials into bf16 weights in place: eight
+// weight and the loss term, then turn the row's 16-bit exponentials into bf16 weights in place: eight
 // 16-byte pieces in flight per lane, each one's successor requested as soon as it has been used, the
 // slots of the next round with them; one special-function operation per group of 64 columns, its result
 // passed around by shuffles.  Rows go last to first: the logits written last are still in the L2.
@@ -850,13 +906,20 @@ strip_row_kernel(uint4* __restrict__ W, const RowParams p) {
                     const float f = __shfl_sync(0xffffffffu, fg, 4 * x + (lane >> 3));
                     const int k = kr + lane + 32 * x;
                     if (k >= k1) continue;
-                    const __half2* e2 = reinterpret_cast<const __half2*>(&raw[x]);
+                    const uint32_t h[4] = {raw[x].x, raw[x].y, raw[x].z, raw[x].w};
                     float w[8];
+                    if ((h[0] | h[1] | h[2] | h[3]) & 0x80008000u) {
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const float2 v = __half22float2(e2[e]);
-                        w[2 * e] = v.x * f;
-                        w[2 * e + 1] = v.y * f;
+                        for (int e = 0; e < 4; ++e) {
+                            const float2 v = stash_times_small(h[e], f);
+                            w[2 * e] = v.x; w[2 * e + 1] = v.y;
+                        }
+                    } else {
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const float2 v = stash_times(h[e], f);
+                            w[2 * e] = v.x; w[2 * e + 1] = v.y;
+                        }
                     }
                     if (wk == k) {
 #pragma unroll

@@ -154,3 +154,42 @@ def test_few_logit_tiles_clear_every_counter(binding, oracle, B, N, d):
         binding.build_cache(Q, P, pos, prob.tau, prob.mask_mode, out)
         torch.cuda.synchronize()
         check_against_oracle(prob, out, _oracle_full(oracle, prob))
+
+
+def _hard_negatives(B, N, d, seed):
+    """Unit rows; passage i is the positive of query i (cosine 0.8), passage B + i its hard negative (0.95)."""
+    rng = np.random.default_rng(seed)
+    unit = lambda x: x / np.linalg.norm(x, axis=1, keepdims=True)
+    Q, P = unit(rng.standard_normal((B, d))), unit(rng.standard_normal((N, d)))
+    for first, cos in ((0, 0.8), (B, 0.95)):
+        side = P[first:first + B] - (P[first:first + B] * Q).sum(1, keepdims=True) * Q
+        P[first:first + B] = cos * Q + (1 - cos * cos) ** 0.5 * unit(side)
+    return Q.astype(np.float32), P.astype(np.float32)
+
+
+@pytest.mark.parametrize("B,N,d,tau", [(512, 2048, 512, 0.05), (512, 2048, 512, 0.02), (300, 1000, 448, 0.012),
+                                       (300, 1111, 512, 0.2), (130, 900, 64, 0.03)])
+def test_rows_of_small_weights_keep_their_precision(binding, B, N, d, tau):
+    """dP row by row, for passages whose every weight lies up to a hundred powers of two below their row's
+    largest.  A weight is rounded at most twice, to 8 bits of mantissa (2^-9 of it) in between and to bf16
+    (2^-8) in the end, and 2^(s - lse) of two fp32 numbers below 2^8 in magnitude is off by 2^-15 at most; a
+    row of dP therefore by at most that share of the sum of its terms' norms."""
+    Qn, Pn = _hard_negatives(B, N, d, seed=B + N)
+    Q, P = (torch.from_numpy(x).to(torch.bfloat16).cuda() for x in (Qn, Pn))
+    pos = torch.arange(B, dtype=torch.int32, device="cuda")
+    o = binding.Outputs(B, N, d, binding.GC_BF16)
+    binding.gc_build_cache(Q, P, pos, tau, 0, o.loss, o.row_lse, o.dQ, o.dP, o.pos_logit, o.ws, o.dev_status)
+    both = torch.empty_like(o.dP)
+    binding.gc_loss_bwd(Q, P, pos, tau, 0, o.row_lse, o.dQ, both, o.ws, o.dev_status)
+    torch.cuda.synchronize()
+    assert int(o.dev_status.item()) == 0
+    Q64, P64 = Q.double().cpu(), P.double().cpu()
+    S = Q64 @ P64.T / tau
+    W = torch.exp(S - torch.logsumexp(S, 1, keepdim=True))
+    W[torch.arange(B), torch.arange(B)] -= 1.0
+    dP = W.T @ Q64 / (B * tau)
+    terms = W.abs().T @ Q64.norm(dim=1) / (B * tau)
+    bound = (2.0 ** -8 + 2.0 ** -9 + 2.0 ** -13) * terms + B * 2.0 ** -118
+    for got in (o.dP, both):
+        err = (got.double().cpu() - dP).norm(dim=1)
+        assert bool((err <= bound).all()), float((err / bound).max())
