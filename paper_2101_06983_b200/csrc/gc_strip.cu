@@ -26,6 +26,8 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <type_traits>
+
 #include "tc_common.cuh"
 
 namespace gc {
@@ -91,9 +93,11 @@ __device__ __forceinline__ uint32_t pack_b2(float lo, float hi) {
 // fp16 alone does not: below 2^-14 it rounds to multiples of 2^-24.  So: from 2^-14 on fp16, ten bits of
 // mantissa, with a sign bit of 0; below, a sign bit of 1 and the upper 15 bits of the fp32 number without
 // its sign, eight bits of mantissa, down to 2^-126.  The logits of most groups span fewer octaves: the second
-// form costs them a minimum over the logits here and a test per 16 bytes in the row kernel.
-// Measured, us, kernels with fp16 alone / as they are: logit kernel of a build 1531 x 3062 x 768 11.7 / 12.0, of
-// gradients 4096 x 8192 x 1024 54.6 / 56.5 and 4096 x 1024 x 768 14.7 / 15.5, row pass 1531 x 3062 6.3 / 6.4.
+// form costs them a minimum over the logits here.  A block of 32 rows x 64 columns that uses it marks its slots
+// with a negative sum, so that the row kernel decides once per round of 2048 columns.
+// Measured, us, kernels with fp16 alone / as they are: logit kernel of a build 1531 x 3062 x 768 11.7 / 12.1, of
+// gradients 4096 x 8192 x 1024 54.6 / 56.5 and 4096 x 1024 x 768 14.7 / 15.5, row pass 6.1 / 6.1 (with a test per
+// 16 bytes in place of the mark 6.4).
 constexpr float STASH_FP16 = 6.103515625e-5f;            // 2^-14
 __device__ __forceinline__ uint32_t stash_pack_small(uint32_t h, float a, float b) {
     if (a < STASH_FP16) h = (h & 0xffff0000u) | 0x8000u | ((__float_as_uint(a) + 0x4000u) >> 15);
@@ -216,7 +220,8 @@ struct LogitParams {
     const float* pos_logit;      // directions are then formed here
     float zero_anchor_lse;       // log B
     float* terms;
-    float2* slots;               // [rows][slot_pitch] (raw maximum, sum)
+    float2* slots;               // [rows][slot_pitch] (raw maximum, sum; LOGIT_STASH: sum negated where the
+                                 // group's codes are of both forms)
     int slot_pitch;
     float* pos_ws;               // positive's raw logit
     float* res;                  // LOGIT_W: what the positive's weight lost to bf16
@@ -444,7 +449,7 @@ strip_logit_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
                         }
                     }
                     if (MODE == LOGIT_STASH) {
-                        if (i < p.rows) p.slots[(int64_t)i * p.slot_pitch + (jg >> 6)] = make_float2(gm, sum);
+                        if (i < p.rows) p.slots[(int64_t)i * p.slot_pitch + (jg >> 6)] = make_float2(gm, small ? -sum : sum);
                     } else if (MODE == LOGIT_W) {
                         // what the row kernel makes of the stored exponentials, bit for bit
                         const float f = gm > -INFINITY ? ex2(fmaf(gm, p.c1, neg_lse)) : 0.f;
@@ -817,7 +822,7 @@ strip_row_kernel(uint4* __restrict__ W, const RowParams p) {
     float m = -INFINITY, l = 0.f, pos_raw = -INFINITY;
     int flags = 0, pos = -1;
     auto slot = [&](int s) { return s < p.nslots ? __ldcg(sl + s) : make_float2(-INFINITY, 0.f); };
-    auto join = [&](float2 v, float ref) { l = fmaf(v.y, ex2((v.x - ref) * p.c1), l); };
+    auto join = [&](float2 v, float ref) { l = fmaf(WRITE ? fabsf(v.y) : v.y, ex2((v.x - ref) * p.c1), l); };
     if (live) {
         for (int s = first_slot + 2 * step; s < p.nslots; s += 8 * step) {
             float2 v[8];
@@ -891,44 +896,41 @@ strip_row_kernel(uint4* __restrict__ W, const RowParams p) {
             const float neg = -(lse * LOG2E);
             const int wk = pos < 0 ? -1 : pos >> 3;
             // round after round: lane g of a round holds the factor of its group of 64 columns
-            auto top_of = [&](int kr) {
+            auto slot_of = [&](int kr) {
                 const int g = (kr >> 3) + lane;
-                return g < p.nslots ? __ldcg(&sl[g].x) : -INFINITY;
+                return g < p.nslots ? __ldcg(sl + g) : make_float2(-INFINITY, 0.f);
             };
-            float next = top_of(k0);
+            float2 next = slot_of(k0);
             for (int kr = k0; kr < k1; kr += stride) {
                 // (a group with no allowed column holds zeros)
-                const float gm = next;
-                if (kr + stride < k1) next = top_of(kr + stride);
-                const float fg = gm > -INFINITY ? ex2(fmaf(gm, p.c1, neg)) : 0.f;
+                const float2 now = next;
+                if (kr + stride < k1) next = slot_of(kr + stride);
+                const float fg = now.x > -INFINITY ? ex2(fmaf(now.x, p.c1, neg)) : 0.f;
+                auto round = [&](auto small) {
 #pragma unroll
-                for (int x = 0; x < ROW_PIECES; ++x) {
-                    const float f = __shfl_sync(0xffffffffu, fg, 4 * x + (lane >> 3));
-                    const int k = kr + lane + 32 * x;
-                    if (k >= k1) continue;
-                    const uint32_t h[4] = {raw[x].x, raw[x].y, raw[x].z, raw[x].w};
-                    float w[8];
-                    if ((h[0] | h[1] | h[2] | h[3]) & 0x80008000u) {
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const float2 v = stash_times_small(h[e], f);
-                            w[2 * e] = v.x; w[2 * e + 1] = v.y;
-                        }
-                    } else {
+                    for (int x = 0; x < ROW_PIECES; ++x) {
+                        const float f = __shfl_sync(0xffffffffu, fg, 4 * x + (lane >> 3));
+                        const int k = kr + lane + 32 * x;
+                        if (k >= k1) continue;
+                        const uint32_t h[4] = {raw[x].x, raw[x].y, raw[x].z, raw[x].w};
+                        float w[8];
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
-                            const float2 v = stash_times(h[e], f);
-                            w[2 * e] = v.x; w[2 * e + 1] = v.y;
+                            const float2 v = decltype(small)::value ? stash_times_small(h[e], f) : stash_times(h[e], f);
+                            w[2 * e] = v.x;
+                            w[2 * e + 1] = v.y;
                         }
-                    }
-                    if (wk == k) {
+                        if (wk == k) {
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) if (e == (pos & 7)) w[e] = pw;
+                            for (int e = 0; e < 8; ++e) if (e == (pos & 7)) w[e] = pw;
+                        }
+                        row[k] = make_uint4(pack_b2(w[0], w[1]), pack_b2(w[2], w[3]),
+                                            pack_b2(w[4], w[5]), pack_b2(w[6], w[7]));
+                        if (k + stride < k1) raw[x] = __ldcg(row + k + stride);
                     }
-                    row[k] = make_uint4(pack_b2(w[0], w[1]), pack_b2(w[2], w[3]),
-                                        pack_b2(w[4], w[5]), pack_b2(w[6], w[7]));
-                    if (k + stride < k1) raw[x] = __ldcg(row + k + stride);
-                }
+                };
+                if (__any_sync(0xffffffffu, now.y < 0.f)) round(std::true_type{});
+                else                                      round(std::false_type{});
             }
         }
     }
