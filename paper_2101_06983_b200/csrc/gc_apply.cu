@@ -137,6 +137,11 @@ apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ C
                 if (++stage == AP_STAGES) { stage = 0; phase ^= 1u; }
             }
         }
+        // the last commits that give stages back, from the leader into both CTAs, have arrived
+        for (int n = 0; n < AP_STAGES && ok; ++n) {
+            ok = mbar_wait(smem_u32(&bars.empty[stage]), phase ^ 1u, abort_flag);
+            if (++stage == AP_STAGES) { stage = 0; phase ^= 1u; }
+        }
     } else if (warp == AP_MMA_WARP) {
         int n_unit = 0;
         bool ok = true;
@@ -172,7 +177,8 @@ apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ C
                 }
             }
         } else {
-            for (int u = pair; u < units && ok; u += pairs, ++n_unit) {
+            // what the leader waits for: every unit's "accumulator read" but the last one's
+            for (int u = pair; u + pairs < units && ok; u += pairs, ++n_unit) {
                 ok = mbar_wait(smem_u32(&bars.acc_free), (uint32_t)n_unit & 1u, abort_flag);
                 if (ok && elect_one()) mbar_arrive_cluster(mapa_u32(smem_u32(&bars.acc_free_peer), 0));
             }
@@ -307,7 +313,7 @@ apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ C
         if (threadIdx.x == 0 && p.dev_status) atomicOr(p.dev_status, GC_DEV_WAIT_LIMIT);
         __syncthreads();
     }
-    cluster_meet();       // the peer's MMAs, loads and signals no longer touch this CTA
+    cluster_meet();       // every load, signal, product, commit and arrival between the CTAs has been waited for
     if (warp == AP_MMA_WARP) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;"

@@ -177,7 +177,9 @@ __device__ __forceinline__ void pair_teardown(const PairCtx& c, volatile int* ab
         if (threadIdx.x == 0 && dev_status) atomicOr(dev_status, GC_DEV_WAIT_LIMIT);
         __syncthreads();
     }
-    cluster_meet();       // the peer's MMAs, loads and arrivals no longer touch this CTA
+    // By here nothing remote is under way: the leader has waited for every load and every forwarded arrival, the
+    // second CTA for every product (its last accumulator) and every commit (ring_drained).
+    cluster_meet();
     if (c.warp == MMA_WARP) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;"
@@ -186,9 +188,11 @@ __device__ __forceinline__ void pair_teardown(const PairCtx& c, volatile int* ab
 }
 
 // The second CTA's idle issuing warp passes "buffer read" on to the leader: one remote arrival per
-// use instead of eight (a remote arrival stalls the arriving warp for more than a thousand cycles).
+// use instead of eight (a remote arrival stalls the arriving warp for more than a thousand cycles).  Only
+// what the leader waits for (wait_acc_free, of use n + 2): an arrival that nobody waits for could reach the
+// leader's shared memory after it has left.
 __device__ __forceinline__ void forward_acc_free(StripBars& bars, int uses, volatile int* abort_flag) {
-    for (int n = 0; n < uses; ++n) {
+    for (int n = 0; n < uses - 2; ++n) {
         const int b = n & 1;
         if (!mbar_wait(smem_u32(&bars.acc_free[b]), (uint32_t)(n >> 1) & 1u, abort_flag)) return;
         if (elect_one()) mbar_arrive_cluster(mapa_u32(smem_u32(&bars.acc_free_peer[b]), 0));
@@ -199,6 +203,16 @@ __device__ __forceinline__ bool wait_acc_free(StripBars& bars, int n, volatile i
     const uint32_t par = ((uint32_t)(n >> 1) & 1u) ^ 1u;
     return mbar_wait(smem_u32(&bars.acc_free[b]), par, abort_flag) &&
            mbar_wait(smem_u32(&bars.acc_free_peer[b]), par, abort_flag);
+}
+
+// The last step of a CTA's first producer, from where its ring stands: all stages have been given back.  The commits that
+// give them back come from the leader into both CTAs; the last of them nobody else waits for.
+__device__ __forceinline__ void ring_drained(StripBars& bars, int stages, int stage, uint32_t phase,
+                                             volatile int* abort_flag) {
+    for (int n = 0; n < stages; ++n) {
+        if (!mbar_wait(smem_u32(&bars.empty[stage]), phase ^ 1u, abort_flag)) return;
+        if (++stage == stages) { stage = 0; phase ^= 1u; }
+    }
 }
 
 // ---------------------------------------------------------------------------------------------------
@@ -293,6 +307,7 @@ strip_logit_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
                 if (++stage == NST) { stage = 0; phase ^= 1u; }
             }
         }
+        if (ok && is_a) ring_drained(bars, NST, stage, phase, abort_flag);
     } else if (c.warp == MMA_WARP) {
         if (c.rank == 0) {
             const uint32_t idesc = instr_desc(BN, false, 256, false);
@@ -582,6 +597,7 @@ strip_logit_f32_kernel(const __grid_constant__ CUtensorMap mapQ,
                 if (++stage == F_NST) { stage = 0; phase ^= 1u; }
             }
         }
+        if (ok && is_a) ring_drained(bars, F_NST, stage, phase, abort_flag);
     } else if (c.warp == MMA_WARP) {
         if (c.rank == 0) {
             const uint32_t idesc = instr_desc(F_BN, false, 256, false);
@@ -623,8 +639,9 @@ strip_logit_f32_kernel(const __grid_constant__ CUtensorMap mapQ,
                 }
             }
         } else {
+            // (the leader waits for every use but the last)
             int n = 0;
-            for (int t = pair; t < total; t += pairs, ++n) {
+            for (int t = pair; t + pairs < total; t += pairs, ++n) {
                 if (!mbar_wait(smem_u32(&bars.acc_free[0]), (uint32_t)n & 1u, abort_flag)) break;
                 if (elect_one()) mbar_arrive_cluster(mapa_u32(smem_u32(&bars.acc_free_peer[0]), 0));
             }
@@ -1224,6 +1241,7 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
                 if (++stage == NST) { stage = 0; phase ^= 1u; }
             }
         }
+        if (ok && is_a) ring_drained(bars, NST, stage, phase, abort_flag);
     } else if (c.warp == MMA_WARP) {
         if (c.rank == 0) {
             int stage = 0, use = 0;

@@ -129,8 +129,9 @@ __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
                  "barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// The same without ordering memory: for a teardown, where all that matters is that nobody leaves early
-// (the releasing form waits for the CTA's global stores).
+// The same without ordering memory: for the teardown of CTAs that have already waited for everything they
+// send one another (the releasing form also waits for the CTA's global stores).  It does not order earlier
+// remote arrivals: one that nobody has waited for may still be on its way when the receiver leaves.
 __device__ __forceinline__ void cluster_meet() {
     asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\t"
                  "barrier.cluster.wait.aligned;" ::: "memory");

@@ -193,3 +193,25 @@ def test_rows_of_small_weights_keep_their_precision(binding, B, N, d, tau):
     for got in (o.dP, both):
         err = (got.double().cpu() - dP).norm(dim=1)
         assert bool((err <= bound).all()), float((err / bound).max())
+
+
+@pytest.mark.parametrize("B,N,d,dtype", [
+    (256, 256, 64, "bf16"), (2048, 2304, 64, "bf16"), (3328, 4096, 64, "bf16"), (4100, 5700, 64, "bf16"),
+    (512, 300, 40, "f32"), (1800, 1900, 72, "f32"), (2600, 2700, 64, "f32"),
+])
+def test_chained_calls_of_pairs_with_one_to_four_tiles(binding, oracle, B, N, d, dtype):
+    """The CTAs of a pair leave together after one, two, three and four uses of their accumulators, and the
+    next kernel takes their place at once: forty calls in a row, no wait that runs out, the same bits."""
+    prob = inputs.random_problem(B, N, d, dtype, seed=B + N, tau=0.5, scale=d ** -0.5)
+    Q, P, pos = to_device(prob)
+    a = binding.Outputs(B, N, d, binding._dtype_code(Q))
+    b = binding.Outputs(B, N, d, binding._dtype_code(Q))
+    args = (Q, P, pos, prob.tau, prob.mask_mode)
+    for o in [a] + [b] * 20:
+        binding.gc_build_cache(*args, o.loss, o.row_lse, o.dQ, o.dP, o.pos_logit, o.ws, o.dev_status)
+        binding.gc_loss_bwd(*args, o.row_lse, o.dQ, None, o.ws, o.dev_status)
+    torch.cuda.synchronize()
+    check_against_oracle(prob, a, _oracle_full(oracle, prob))
+    assert int(b.dev_status.item()) == 0
+    for name in ("loss", "row_lse", "pos_logit", "dQ", "dP"):
+        assert torch.equal(getattr(a, name), getattr(b, name)), name
