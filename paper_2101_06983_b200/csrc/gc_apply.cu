@@ -208,12 +208,12 @@ apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ C
                 const int64_t left = p.rows - (int64_t)kb * AP_KB;         // rows from the block's first on
                 if (kb < t.kb_end && live && left >= AP_KB) {
 #pragma unroll
-                    for (int i = 0; i < ROWS; ++i) v[i] = __ldg(reinterpret_cast<const float4*>(src + i * step));
+                    for (int i = 0; i < ROWS; ++i) v[i] = __ldcg(reinterpret_cast<const float4*>(src + i * step));
                 } else {
 #pragma unroll
                     for (int i = 0; i < ROWS; ++i) {
                         const bool in = kb < t.kb_end && live && row0 + AP_CONV * i < left;
-                        v[i] = in ? __ldg(reinterpret_cast<const float4*>(src + i * step))
+                        v[i] = in ? __ldcg(reinterpret_cast<const float4*>(src + i * step))
                                   : make_float4(0.f, 0.f, 0.f, 0.f);
                     }
                 }
@@ -323,7 +323,7 @@ apply_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ C
 
 // dW (+)= sum of the planes, in order.
 __global__ void __launch_bounds__(256)
-apply_reduce_kernel(const float4* __restrict__ planes, int parts, int64_t plane, int n4,
+apply_reduce_kernel(const float4* planes, int parts, int64_t plane, int n4,
                     float* __restrict__ dW, int64_t lddw, int add) {
     dep_release();
     dep_wait();

@@ -26,8 +26,8 @@ __device__ __forceinline__ int pos_flags(int32_t r, int64_t i, int64_t N, int ma
 // The block that draws the last ticket (red[0], cleared by the sweep before this kernel, and put
 // back to 0 here) adds the block sums in index order: the loss does not depend on block timing.
 __global__ void __launch_bounds__(kCombineThreads)
-lse_combine_kernel(const float* __restrict__ part_m, const float* __restrict__ part_l,
-                   const float* __restrict__ pos_ws, const int32_t* __restrict__ pos_idx,
+lse_combine_kernel(const float* part_m, const float* part_l,
+                   const float* pos_ws, const int32_t* pos_idx,
                    int groups, int64_t B, int64_t N, int mask_mode, float* __restrict__ row_lse,
                    float* __restrict__ pos_logit, float* __restrict__ loss, float* red,
                    int* __restrict__ dev_status, const Gate gate, int64_t mean_over,

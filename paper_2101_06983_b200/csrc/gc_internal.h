@@ -22,6 +22,9 @@ struct Gate {
 // may start while the kernel before it in the stream still runs; dep_wait() returns once that
 // kernel has completed and its writes are visible (at once for an ordinary launch);
 // dep_release() in the earlier kernel lets the later one be scheduled early.
+// What such a kernel reads may have been written while it was already running, by the kernel before it or by
+// one before that: no __ldg and no const __restrict__ pointer in it (loads of memory that is constant for the
+// life of the kernel, which the compiler may also move above the wait).
 __device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void dep_release() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -53,8 +56,8 @@ inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, unsigned 
 // Logsumexp of row i from its per-part (scale, sum) slots, slot g at [g * pitch + i]: the one
 // definition every kernel that merges slots uses, with explicit roundings so that all of them
 // get the same bits.
-__device__ __forceinline__ float combined_lse(const float* __restrict__ part_m,
-                                              const float* __restrict__ part_l, int slots,
+__device__ __forceinline__ float combined_lse(const float* part_m,
+                                              const float* part_l, int slots,
                                               int64_t pitch, int64_t i) {
     float m = -INFINITY;
 #pragma unroll 8

@@ -498,7 +498,7 @@ strip_logit_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
                     const float4* cn = reinterpret_cast<const float4*>(p.col_neg + jg);
 #pragma unroll
                     for (int e = 0; e < 64; e += 4) {
-                        const float4 n4 = jg + e < p.N ? __ldg(cn + (e >> 2)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        const float4 n4 = jg + e < p.N ? __ldcg(cn + (e >> 2)) : make_float4(0.f, 0.f, 0.f, 0.f);
                         const float nn[4] = {n4.x, n4.y, n4.z, n4.w};
 #pragma unroll
                         for (int x = 0; x < 4; ++x)
@@ -702,8 +702,8 @@ __device__ __forceinline__ void split3(float x, uint32_t& t1, uint32_t& t2, uint
     t3 = __float_as_uint(r - __uint_as_float(t2));
 }
 __global__ void __launch_bounds__(256)
-split_terms_kernel(const float* __restrict__ Q, int64_t ldq, int64_t B, uint2* __restrict__ tq,
-                   const float* __restrict__ P, int64_t ldp, int64_t N, uint2* __restrict__ tp,
+split_terms_kernel(const float* Q, int64_t ldq, int64_t B, uint2* __restrict__ tq,
+                   const float* P, int64_t ldp, int64_t N, uint2* __restrict__ tp,
                    int d4) {
     dep_release();
     dep_wait();
@@ -1376,7 +1376,7 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
                         if (col + 8 * j >= sd.cols) break;
-                        const uint4 x = __ldg(pr + j);
+                        const uint4 x = __ldcg(pr + j);
                         const uint32_t w[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {

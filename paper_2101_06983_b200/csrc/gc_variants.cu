@@ -77,7 +77,7 @@ __device__ __forceinline__ void each_piece(const RowPieces<ROW_KEEP, A>& a, cons
 
 template <bool BF16, int KEEP>
 __global__ void __launch_bounds__(256)
-row_normalize_kernel(const void* __restrict__ X, int64_t ldx, int64_t rows, int d,
+row_normalize_kernel(const void* X, int64_t ldx, int64_t rows, int d,
                      void* __restrict__ Xn, int64_t ldxn, float* __restrict__ inv_norm) {
     const int lane = threadIdx.x & 31;
     const size_t es = BF16 ? 2 : 4;
@@ -104,7 +104,7 @@ row_normalize_kernel(const void* __restrict__ X, int64_t ldx, int64_t rows, int 
 // dX_i = inv_i (g_i - n_i <n_i, g_i>) with n_i = inv_i x_i formed in fp32 from the original row
 template <bool BF16, int KEEP>
 __global__ void __launch_bounds__(256)
-cosine_bwd_kernel(const void* __restrict__ X, int64_t ldx, const float* __restrict__ inv_norm,
+cosine_bwd_kernel(const void* X, int64_t ldx, const float* inv_norm,
                   const float* G, int64_t ldg, int64_t rows, int d, float* dX, int64_t lddx) {
     const int lane = threadIdx.x & 31;
     const size_t es = BF16 ? 2 : 4;
@@ -135,7 +135,7 @@ cosine_bwd_kernel(const void* __restrict__ X, int64_t ldx, const float* __restri
 // row_dot[i] = <q_i, dQ_i>
 template <bool BF16, int KEEP>
 __global__ void __launch_bounds__(256)
-row_dot_kernel(const void* __restrict__ Q, int64_t ldq, const float* __restrict__ dQ, int64_t lddq,
+row_dot_kernel(const void* Q, int64_t ldq, const float* dQ, int64_t lddq,
                int64_t rows, int d, float* __restrict__ row_dot) {
     const int lane = threadIdx.x & 31;
     const size_t es = BF16 ? 2 : 4;
@@ -157,7 +157,7 @@ row_dot_kernel(const void* __restrict__ Q, int64_t ldq, const float* __restrict_
 }
 // *out = scale * sum_i v[i]: one block, every thread a fixed strided share, then fixed trees
 __global__ void __launch_bounds__(1024)
-ordered_sum_kernel(const float* __restrict__ v, int64_t n, float scale, float* __restrict__ out) {
+ordered_sum_kernel(const float* v, int64_t n, float scale, float* __restrict__ out) {
     __shared__ float part[32];
     dep_release();
     dep_wait();
