@@ -169,9 +169,10 @@ int gc_build_cache_stored(const void* Q, int64_t ldq, const void* P, int64_t ldp
  * U, X and dW start on 16-byte boundaries.  Up to two kernel launches: where the widths leave CTA
  * pairs over, the sub-batch's rows are split into parts whose sums are planes of the workspace, added
  * in order.  gc_cache_apply_workspace_bytes returns the bytes that takes for any number of rows (0 for
- * sizes outside the limits); ws must be a 256-byte aligned, caller-owned buffer of at least that size.
- * Asynchronous on cuda_stream; deterministic; GC_DEV_WAIT_LIMIT in *dev_status (may be NULL) as for
- * the other calls.
+ * sizes outside the limits); ws must be a 256-byte aligned, caller-owned buffer of at least 256 bytes:
+ * one that holds fewer planes means fewer parts, one that holds fewer than two a single launch.
+ * Asynchronous on cuda_stream; deterministic for a given size of ws; GC_DEV_WAIT_LIMIT in *dev_status
+ * (may be NULL) as for the other calls.
  */
 size_t gc_cache_apply_workspace_bytes(int64_t rows, int d, int d_in);
 int gc_cache_apply(const float* U, int64_t ldu, const void* X, int64_t ldx, int64_t rows, int d,

@@ -352,13 +352,17 @@ int most_parts(int64_t tiles) {
     const int64_t per = sm_count() / 2 / tiles;
     return per < 1 ? 1 : per > AP_MAX_PARTS ? AP_MAX_PARTS : (int)per;
 }
-ApplyPlan make_apply_plan(int64_t rows, int d, int d_in) {
+size_t plane_bytes(int d, int d_in) { return (size_t)d * (size_t)d_in * 4; }
+// ws_bytes: of a workspace that may hold fewer planes than that
+ApplyPlan make_apply_plan(int64_t rows, int d, int d_in, size_t ws_bytes) {
     ApplyPlan pl{};
     pl.tiles_m = (d + 255) / 256;
     pl.tiles_n = (d_in + 255) / 256;
     pl.kblocks = (int)((rows + AP_KB - 1) / AP_KB);
     pl.parts = most_parts((int64_t)pl.tiles_m * pl.tiles_n);
     if (pl.parts > pl.kblocks) pl.parts = pl.kblocks;
+    const size_t room = ws_bytes / plane_bytes(d, d_in);
+    if ((size_t)pl.parts > room) pl.parts = room < 2 ? 1 : (int)room;
     return pl;
 }
 
@@ -370,7 +374,7 @@ bool apply_shape_ok(int64_t rows, int d, int d_in) {
 size_t apply_ws(int d, int d_in) {
     const int parts = most_parts((int64_t)((d + 255) / 256) * ((d_in + 255) / 256));
     if (parts == 1) return 256;
-    return ((size_t)parts * (size_t)d * (size_t)d_in * 4 + 255) & ~(size_t)255;
+    return ((size_t)parts * plane_bytes(d, d_in) + 255) & ~(size_t)255;
 }
 
 }  // namespace
@@ -396,7 +400,7 @@ int gc_cache_apply(const float* U, int64_t ldu, const void* X, int64_t ldx, int6
     if (((uintptr_t)U & 15) || ((uintptr_t)X & 15) || ((uintptr_t)dW & 15) || (ldu * 4) % 16 ||
         (ldx * 2) % 16 || (lddw * 4) % 16)
         return GC_ERR_ALIGN;
-    if (!ws || ((uintptr_t)ws & 255) || ws_bytes < apply_ws(d, d_in)) return GC_ERR_WORKSPACE;
+    if (!ws || ((uintptr_t)ws & 255) || ws_bytes < 256) return GC_ERR_WORKSPACE;
     int dev = 0, major = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess) {
@@ -406,7 +410,7 @@ int gc_cache_apply(const float* U, int64_t ldu, const void* X, int64_t ldx, int6
     if (major != 10) return GC_ERR_ARCH;
     if (dev < 0 || dev >= 64) return GC_ERR_CUDA;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    const ApplyPlan pl = make_apply_plan(rows, d, d_in);
+    const ApplyPlan pl = make_apply_plan(rows, d, d_in, ws_bytes);
     float* planes = static_cast<float*>(ws);
     CUtensorMap mx, mo;
     if (!make_map(&mx, X, rows, d_in, ldx, AP_KB) ||

@@ -33,3 +33,29 @@ def test_parts_and_tiles(oracle, rows, d, d_in):
     assert int(st.item()) == 0 and bool((ws[need:] == 0xA5).all())
     assert grad_err(once.cpu().numpy(), ref) <= 1e-4
     assert grad_err(W.cpu().numpy(), 2 * ref) <= 1e-4
+
+
+@pytest.mark.parametrize("planes", [0, 1, 2, 3])
+def test_workspace_of_fewer_planes(oracle, planes):
+    """256 bytes are enough for any call; what fits beside them is used, and nothing past it is written."""
+    from paper_2101_06983_b200 import binding
+    rows, d, d_in = 1000, 264, 320
+    U = inputs.cache_rows(rows, d, seed=rows)
+    bits, X = inputs.encoder_inputs(rows, d_in, seed=d)
+    ref = oracle.cache_apply(U, X)
+    dU = torch.from_numpy(U).cuda()
+    dX = torch.from_numpy(bits.view(np.int16)).view(torch.bfloat16).cuda()
+    need = max(256, planes * d * d_in * 4)
+    assert need < binding.gc_cache_apply_workspace_bytes(rows, d, d_in)
+    ws = torch.full((need + 4096,), 0xA5, dtype=torch.uint8, device="cuda")
+    W = torch.full((d, d_in), float("nan"), device="cuda")
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    binding.gc_cache_apply(dU, dX, W, False, ws[:need], st)
+    once = W.clone()
+    binding.gc_cache_apply(dU, dX, W, True, ws[:need], st)
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0 and bool((ws[need:] == 0xA5).all())
+    assert grad_err(once.cpu().numpy(), ref) <= 1e-4
+    assert grad_err(W.cpu().numpy(), 2 * ref) <= 1e-4
+    with pytest.raises(binding.GradCacheError):
+        binding.gc_cache_apply(dU, dX, W, True, ws[:255], st)
