@@ -72,8 +72,11 @@ typedef enum { GC_OP_FWD = 0, GC_OP_BWD = 1, GC_OP_BUILD = 2, GC_OP_BUILD_STORED
 enum { GC_DEV_POS_RANGE = 1, GC_DEV_POS_MASKED = 2, GC_DEV_WAIT_LIMIT = 4 };
 
 /* Bytes of workspace the given call needs for these sizes on the current device (a multiple
- * of 256).  O((B + N) d) plus, for the three calls of the paper's path, at most 1.5 GiB of softmax
- * weights of a strip of query rows (more beyond 3 * 2^20 passages: never fewer than 256 queries); GC_OP_BUILD_STORED adds 2 B N bytes for its weight matrix.  Returns 0 for invalid arguments. */
+ * of 256).  O((B + N) d) plus, for the three calls of the paper's path, what a strip of query rows
+ * takes: at most 1.5 GiB of softmax weights (fp32: 512 MiB of logits and weights; rows of weights are
+ * rounded up to 64 passages), and 8 bytes for every 64 of the weights (rows rounded up to 256 passages: at
+ * most 0.4 GiB).  More beyond 3 * 2^20 passages (fp32: 2^18): never fewer than 256 queries to a strip.
+ * GC_OP_BUILD_STORED adds 2 B N bytes for its weight matrix.  Returns 0 for invalid arguments. */
 size_t gc_workspace_bytes(int op, int64_t B, int64_t N, int d, int dtype);
 
 /* Name of the kernel plan the library will use for these sizes:

@@ -1651,13 +1651,13 @@ StripLayout strip_layout(int64_t B, int64_t N, int d, int dtype, bool fwd_only =
     // 65536 passages, and of 1.5-2 GB: 16384 x 32768 x 768 2.38 / 2.33, 40000 x 80000 x 512 11.1 / 10.7,
     // 65536 x 131072 x 768 38.3 / 37.0, loss and gradients of 40000 x 120000 x 256 11.5 / 11.0; 4 GB would
     // give 10.5, 37.8 and 10.5); fp32 holds 8 bytes a pair and does four times the arithmetic: 64 M pairs.
-    int64_t r = ((int64_t)(f32 ? 64 : 768) << 20) / N / 256 * 256;
+    l.ldw = ceil_div(N, 64) * 64;
+    int64_t r = ((int64_t)(f32 ? 64 : 768) << 20) / l.ldw / 256 * 256;
     if (r < 256) r = 256;
     const int64_t n = ceil_div(B, r);
     r = ceil_div(ceil_div(B, n), 256) * 256;
     l.strips = (int)ceil_div(B, r);
     l.rows = B < r ? B : r;
-    l.ldw = ceil_div(N, 64) * 64;
     l.slot_pitch = (int)(ceil_div(N, 256) * 4);
     const int64_t tiles = ceil_div(l.rows, 256) * ceil_div(d, 128) + ceil_div(N, 256) * ceil_div(d, 128);
     size_t off = 0;

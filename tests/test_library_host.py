@@ -55,6 +55,17 @@ def test_workspace_is_linear_in_rows_not_quadratic(binding):
     assert b.gc_workspace_bytes(b.GC_OP_FWD, 8, 8, 8, 5) == 0
 
 
+@pytest.mark.parametrize("N,d", [(65, 8), (1, 8), (64, 8), (129, 16), (1000, 8)])
+def test_a_strip_of_fp32_rows_stays_within_its_bound(binding, N, d):
+    """Many queries: a strip's logits and weights take 512 MiB together however far N is from a multiple of
+    64; beside them the three terms of every input, and what is linear in the queries."""
+    b = binding
+    B = 8000000 if N < 200 else 1 << 22
+    assert b.gc_plan_name(b.GC_OP_BUILD, B, N, d, b.GC_F32) == "tcgen05-tiles"
+    need = b.gc_workspace_bytes(b.GC_OP_BUILD, B, N, d, b.GC_F32)
+    assert need <= (512 << 20) + 6 * d * (B + N) + 16 * B + (128 << 20)
+
+
 def test_plan_names(binding):
     b = binding
     # one tile: fp32 up to 128 x 128, bf16 up to 128 x 256, d a multiple of 8 up to 1024
