@@ -1609,8 +1609,9 @@ GradDeal deal_grads(int64_t rows, int64_t N, int d, bool f32, bool dq, bool dp) 
         } else {
             for (int w = tq ? 1 : 0; w <= (tp ? pairs - 1 : pairs); ++w) {
                 if (!tq && w) break;
-                const double a = tq ? (double)(ceil_div(tq, w) * kq) : 0, b = tp ? (double)(ceil_div(tp, pairs - w) * kp) : 0;
-                offer((a > b ? a : b) * unit, w, pairs);
+                const double a = tq ? tiles_cost(ceil_div(tq, w), kq, epi_q) : 0;
+                const double b = tp ? tiles_cost(ceil_div(tp, pairs - w), kp, epi_p) : 0;
+                offer(a > b ? a : b, w, pairs);
             }
         }
         // equal runs of contraction blocks, at least four to a pair: as many as cost least
@@ -1620,7 +1621,11 @@ GradDeal deal_grads(int64_t rows, int64_t N, int d, bool f32, bool dq, bool dp) 
         if (groups > pairs / tn) groups = pairs / tn;
         if (groups > units / 4) groups = (int)(units / 4);
         if (groups < 1) groups = 1;
-        offer(units / groups * unit + cut + part * longest * groups / units, -1, groups * tn);
+        const double run = units / groups;
+        double cost = run * unit;
+        if (tq && run > kq && run / kq * epi_q > cost) cost = run / kq * epi_q;
+        if (tp && run > kp && run / kp * epi_p > cost) cost = run / kp * epi_p;
+        offer(cost + cut + part * longest * groups / units, -1, groups * tn);
     }
     return best;
 }
@@ -1663,11 +1668,18 @@ StripLayout strip_layout(int64_t B, int64_t N, int d, int dtype, bool fwd_only =
     size_t off = 0;
     const size_t counters = fwd_only ? 0 : (size_t)tiles * 16;
     l.zero = off;  off += up256(sizeof(int) * (64 + counters));
+        // A pair's next tile takes at least the epilogue of this one (dQ's adds what the positives' weights lost):
+        // tiles of few contraction blocks are bound by it.  4671 x 30 x 128, both gradients: 18 dQ tiles of one
+        // block to a pair 71 us, 19 pairs for them 14; 7 x 9470 x 128: 26 dP tiles of one block to a pair 44 us.
+        const double epi_q = width == 256 ? 12000 : 6000, epi_p = width == 256 ? 6400 : 3200;
     l.pos = off;   off += up256(sizeof(float) * (size_t)l.rows);
     l.red = off;   off += up256(sizeof(float) * (size_t)(B + 8 * sm_count()));
     if (!f32) {
         const int64_t pitch = fwd_only ? 2 * ceil_div(N, 128) : l.slot_pitch;
         l.slots = off;  off += up256(sizeof(float2) * (size_t)l.rows * (size_t)pitch);
+        auto tiles_cost = [&](int64_t n, int64_t k, double epilogue) {
+            return (double)(n - 1) * (k * unit > epilogue ? k * unit : epilogue) + k * unit;
+        };
     } else {
         const size_t dp = (size_t)((d + 7) / 8 * 8);
         l.s = off;   off += up256(4 * (size_t)l.rows * (size_t)l.ldw);
