@@ -26,6 +26,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "tc_common.cuh"
@@ -762,14 +763,18 @@ struct RowParams {
     float* col_neg;               // where LOGIT_W2's column factors go
 };
 
-// Shares of the loss are added in a fixed order: a block's rows in row order, then the blocks in a fixed
-// pattern by the block that draws the last ticket.
+// Shares of the loss, EACH per block (of its first threads), are added in a fixed order: a share's rows in row
+// order, then the shares in a fixed pattern by the block that draws the last ticket.
+template <int EACH = 1>
 __device__ __forceinline__ void loss_share(const RowParams& p, float mine) {
     __shared__ int last_s;
     __shared__ float warp_s[8];
-    if (threadIdx.x == 0) {
-        p.red[p.block0 + blockIdx.x] = mine;
+    if (threadIdx.x < EACH) {
+        p.red[(p.block0 + blockIdx.x) * EACH + threadIdx.x] = mine;
         __threadfence();
+    }
+    if (EACH > 1) __syncthreads();
+    if (threadIdx.x == 0) {
         last_s = atomicAdd(p.ticket, 1) == p.blocks_total - 1;
     }
     __syncthreads();
@@ -777,7 +782,7 @@ __device__ __forceinline__ void loss_share(const RowParams& p, float mine) {
     __threadfence();
     float v = 0.f;
 #pragma unroll 4
-    for (int b = threadIdx.x; b < p.blocks_total; b += blockDim.x) v += __ldcg(p.red + b);
+    for (int b = threadIdx.x; b < p.blocks_total * EACH; b += blockDim.x) v += __ldcg(p.red + b);
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     if ((threadIdx.x & 31) == 0) warp_s[threadIdx.x >> 5] = v;
     __syncthreads();
@@ -809,6 +814,7 @@ __device__ __forceinline__ int row_pos(const RowParams& p, int i, int* flags) {
 // RESIDENT, the blocks an SM is to hold: seven (72 registers a thread), six where the grid then fits in
 // one go (1531 x 3062: 5.1 us with seven, 4.7 with six; 4096 x 8192: 20.3 and 22.0).
 constexpr int row_warps(bool write) { return write ? 4 : 8; }      // rows per block
+constexpr int MOST_THREAD_SLOTS = 8;                // strip_lse_kernel
 constexpr int ROW_PIECES = 8;                       // of 8 columns, per lane and round
 constexpr int ROW_ROUND = 32 * ROW_PIECES;          // pieces per warp and round: 32 groups of 64 columns
 template <bool WRITE, int RESIDENT>
@@ -960,31 +966,81 @@ strip_row_kernel(uint4* __restrict__ W, const RowParams p) {
     }
 }
 
-// fp32 inputs: one block per row of raw logits.  Maximum, sum and weights are three passes over the
-// row (from the first level cache after the first); the weights leave as two bf16 terms, planes
-// [2][rows][ldw].  With lse_given (gc_loss_bwd) only the last pass runs.
+// The loss alone where a row has few slots and there are many rows: a thread per row (strip_row_kernel<false>
+// gives a warp to the two slots of 256 passages: 64000 x 128, 32.7 us a launch, 6.3 here; 8000 rows are even).
+__global__ void __launch_bounds__(256)
+strip_lse_kernel(const RowParams p) {
+    __shared__ float sums[8];
+    dep_release();
+    dep_wait();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int i = blockIdx.x * 256 + (int)threadIdx.x;
+    float term = 0.f;
+    if (i < p.rows) {
+        const float2* sl = p.slots + (int64_t)i * p.slot_pitch;
+        float2 v[MOST_THREAD_SLOTS];
+        float m = -INFINITY, l = 0.f;
+#pragma unroll
+        for (int s = 0; s < MOST_THREAD_SLOTS; ++s) {
+            v[s] = s < p.nslots ? __ldcg(sl + s) : make_float2(-INFINITY, 0.f);
+            m = fmaxf(m, v[s].x);
+        }
+        int flags;
+        const int pos = row_pos(p, i, &flags);
+        const float ref = m == -INFINITY ? 0.f : m;
+#pragma unroll
+        for (int s = 0; s < MOST_THREAD_SLOTS; ++s) l = fmaf(v[s].y, ex2((v[s].x - ref) * p.c1), l);
+        const float lse = m * p.inv_tau + log2f(l) * LN2;
+        const float pl = pos < 0 ? 0.f : __ldcg(p.pos_ws + i) * p.inv_tau;
+        p.row_lse[i] = lse;
+        if (p.pos_logit) p.pos_logit[i] = pl;
+        if (flags && p.dev_status) atomicOr(p.dev_status, flags);
+        if (p.count && pos >= 0) atomicAdd(p.count + pos, 1);
+        if (p.col_neg) {
+            const int n = p.mult[i];
+            p.col_neg[i] = n > 0 ? log2f((float)n) - lse * LOG2E : -INFINITY;
+        }
+        term = lse - pl;
+    }
+    for (int o = 16; o > 0; o >>= 1) term += __shfl_xor_sync(0xffffffffu, term, o);
+    if (lane == 0) sums[warp] = term;
+    __syncthreads();
+    float share = 0.f;
+    if (threadIdx.x == 0)
+        for (int w = 0; w < 8; ++w) share += sums[w];
+    loss_share(p, share);
+}
+
+// fp32 inputs: one block (BLOCK = true), or a warp of it, per row of raw logits.  Maximum, sum and weights
+// are three passes over the row (from the first level cache after the first; a warp from 101776 rows of 34: 49 us,
+// a block 269); the weights leave as two
+// bf16 terms, planes [2][rows][ldw].  With lse_given (gc_loss_bwd) only the last pass runs.
+template <bool BLOCK>
 __global__ void __launch_bounds__(256)
 strip_row_f32_kernel(uint2* __restrict__ W, const RowParams p) {
     __shared__ float sm[8];
     dep_release();
     dep_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int T = BLOCK ? 256 : 32;                  // threads of a row
+    const int t = BLOCK ? (int)threadIdx.x : lane;
     const int n4 = (p.N + 3) / 4;
     float share = 0.f;
-    for (int i = blockIdx.x; i < p.rows; i += (int)gridDim.x) {
+    for (int i = BLOCK ? blockIdx.x : blockIdx.x * 8 + warp; i < p.rows; i += (int)gridDim.x * (BLOCK ? 1 : 8)) {
         const float4* row = reinterpret_cast<const float4*>(p.S + (int64_t)i * p.lds);
         const int masked = p.mask_on ? i + p.mask_shift : -1;
         int flags;
         const int pos = row_pos(p, i, &flags);
-        if (threadIdx.x == 0 && flags && p.dev_status) atomicOr(p.dev_status, flags);
+        if (t == 0 && flags && p.dev_status) atomicOr(p.dev_status, flags);
         auto load = [&](int k, float (&s)[4]) {
             const float4 v = row[k];
             s[0] = v.x; s[1] = v.y; s[2] = v.z; s[3] = v.w;
 #pragma unroll
             for (int e = 0; e < 4; ++e) if (4 * k + e == masked || 4 * k + e >= p.N) s[e] = -INFINITY;
         };
-        auto block_max = [&](float v) {
+        auto row_max = [&](float v) {
             for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+            if (!BLOCK) return v;
             if (lane == 0) sm[warp] = v;
             __syncthreads();
             v = sm[0];
@@ -992,8 +1048,9 @@ strip_row_f32_kernel(uint2* __restrict__ W, const RowParams p) {
             __syncthreads();
             return v;
         };
-        auto block_sum = [&](float v) {
+        auto row_sum = [&](float v) {
             for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (!BLOCK) return v;
             if (lane == 0) sm[warp] = v;
             __syncthreads();
             v = sm[0];
@@ -1008,32 +1065,32 @@ strip_row_f32_kernel(uint2* __restrict__ W, const RowParams p) {
         } else {
             float m = -INFINITY;
 #pragma unroll 4
-            for (int k = threadIdx.x; k < n4; k += 256) {
+            for (int k = t; k < n4; k += T) {
                 float s[4];
                 load(k, s);
                 m = fmaxf(m, fmaxf(fmaxf(s[0], s[1]), fmaxf(s[2], s[3])));
             }
-            m = block_max(m);
+            m = row_max(m);
             const float ref = m == -INFINITY ? 0.f : m;
             float l = 0.f;
 #pragma unroll 4
-            for (int k = threadIdx.x; k < n4; k += 256) {
+            for (int k = t; k < n4; k += T) {
                 float s[4];
                 load(k, s);
 #pragma unroll
                 for (int e = 0; e < 4; ++e) l += ex2((s[e] - ref) * p.c1);
             }
-            l = block_sum(l);
+            l = row_sum(l);
             // the row's logsumexp and its positive logit come out of the same product with 1/tau: their
             // difference is exactly 0 when the positive is the only column
             lse = m * p.inv_tau + log2f(l) * LN2;
             const float pl = raw_pos * p.inv_tau;
-            if (threadIdx.x == 0) {
+            if (t == 0) {
                 p.row_lse[i] = lse;
                 if (p.pos_logit) p.pos_logit[i] = pl;
             }
             share += lse - pl;
-            if (p.want_w && threadIdx.x == 0) p.red[p.row0 + i] = lse - pl;
+            if (p.want_w && t == 0) p.red[p.row0 + i] = lse - pl;
         }
         if (p.want_w) {
             const float lse2 = lse * LOG2E;
@@ -1041,7 +1098,7 @@ strip_row_f32_kernel(uint2* __restrict__ W, const RowParams p) {
             uint2* w2 = w1 + (int64_t)p.rows * (p.ldw / 4);
             const int wpos = pos;
 #pragma unroll 4
-            for (int k = threadIdx.x; k < n4; k += 256) {
+            for (int k = t; k < n4; k += T) {
                 float s[4];
                 load(k, s);
 #pragma unroll
@@ -1056,7 +1113,16 @@ strip_row_f32_kernel(uint2* __restrict__ W, const RowParams p) {
             }
         }
     }
-    if (!p.lse_given && !p.want_w) loss_share(p, share);
+    if (!p.lse_given && !p.want_w) {
+        // (a build adds the terms row by row in the same pattern: up to 8 rows per SM and warp, the same bits)
+        if (!BLOCK) {
+            if (lane == 0) sm[warp] = share;
+            __syncthreads();
+            loss_share<8>(p, threadIdx.x < 8 ? sm[threadIdx.x] : 0.f);
+        } else {
+            loss_share(p, share);
+        }
+    }
 }
 
 // ---------------------------------------------------------------------------------------------------
@@ -1598,10 +1664,17 @@ GradDeal deal_grads(int64_t rows, int64_t N, int d, bool f32, bool dq, bool dp) 
         const double unit = f32 ? 1320 : width == 256 ? 560 : 364;
         const double cut = f32 ? 6300 : width == 256 ? 18000 : 8800;
         const double part = f32 ? 970 : width == 256 ? 3080 : 1580;
+        // A pair's next tile takes at least the epilogue of this one (dQ's adds what the positives' weights lost):
+        // tiles of few contraction blocks are bound by it.  4671 x 30 x 128, both gradients: 18 dQ tiles of one
+        // block to a pair 71 us, 19 pairs for them 14; 7 x 9470 x 128: 26 dP tiles of one block to a pair 44 us.
+        const double epi_q = width == 256 ? 12000 : 6000, epi_p = width == 256 ? 6400 : 3200;
         const int64_t kq = ceil_div(N, KB), kp = ceil_div(rows, KB);
         const int64_t tq = dq ? ceil_div(rows, 256) * tn : 0, tp = dp ? ceil_div(N, 256) * tn : 0;
         auto offer = [&](double cost, int whole, int used) {
             if (best.pairs == 0 || cost < best_cost) { best = {width, whole, used}; best_cost = cost; }
+        };
+        auto tiles_cost = [&](int64_t n, int64_t k, double epilogue) {
+            return (double)(n - 1) * (k * unit > epilogue ? k * unit : epilogue) + k * unit;
         };
         // whole tiles, every split of the pairs between the two products
         if (tq + tp <= pairs) {
@@ -1668,18 +1741,11 @@ StripLayout strip_layout(int64_t B, int64_t N, int d, int dtype, bool fwd_only =
     size_t off = 0;
     const size_t counters = fwd_only ? 0 : (size_t)tiles * 16;
     l.zero = off;  off += up256(sizeof(int) * (64 + counters));
-        // A pair's next tile takes at least the epilogue of this one (dQ's adds what the positives' weights lost):
-        // tiles of few contraction blocks are bound by it.  4671 x 30 x 128, both gradients: 18 dQ tiles of one
-        // block to a pair 71 us, 19 pairs for them 14; 7 x 9470 x 128: 26 dP tiles of one block to a pair 44 us.
-        const double epi_q = width == 256 ? 12000 : 6000, epi_p = width == 256 ? 6400 : 3200;
     l.pos = off;   off += up256(sizeof(float) * (size_t)l.rows);
     l.red = off;   off += up256(sizeof(float) * (size_t)(B + 8 * sm_count()));
     if (!f32) {
         const int64_t pitch = fwd_only ? 2 * ceil_div(N, 128) : l.slot_pitch;
         l.slots = off;  off += up256(sizeof(float2) * (size_t)l.rows * (size_t)pitch);
-        auto tiles_cost = [&](int64_t n, int64_t k, double epilogue) {
-            return (double)(n - 1) * (k * unit > epilogue ? k * unit : epilogue) + k * unit;
-        };
     } else {
         const size_t dp = (size_t)((d + 7) / 8 * 8);
         l.s = off;   off += up256(4 * (size_t)l.rows * (size_t)l.ldw);
@@ -1788,9 +1854,14 @@ struct StripRun {
         return go(strip_logit_kernel<LOGIT_W, 256>, strip_logit_kernel<LOGIT_W, 128>);
     }
 
-    // rows per block of the row kernel: a row of few passages takes a warp's worth of threads
+    // fp32: a warp to a row of logits
+    bool short_rows() const { return p.N <= 512; }
+    // the loss alone: a thread to a row
+    int forward_slots(int s) const { return (int)(2 * ceil_div(p.N, logit_width(rows_of(s), p.N))); }
+    bool row_threads(int s) const { return forward_slots(s) <= MOST_THREAD_SLOTS && rows_of(s) >= 8192; }
     int row_blocks(int s, bool write) const {
-        if (!f32) return (int)ceil_div(rows_of(s), row_warps(write));
+        if (!f32) return (int)ceil_div(rows_of(s), write ? row_warps(true) : row_threads(s) ? 256 : row_warps(false));
+        if (short_rows()) return (int)std::min<int64_t>(ceil_div(rows_of(s), 8), 8 * (int64_t)sm_count());
         const int64_t n = rows_of(s), most = 8 * (int64_t)sm_count();
         return (int)(n < most ? n : most);
     }
@@ -1809,8 +1880,7 @@ struct StripRun {
             rp.slot_pitch = l.slot_pitch;
             rp.nslots = (int)ceil_div(p.N, 64);
         } else {
-            const int bn = logit_width(rows, p.N);
-            rp.nslots = rp.slot_pitch = (int)(2 * ceil_div(p.N, bn));
+            rp.nslots = rp.slot_pitch = forward_slots(s);
         }
         rp.pos_ws = at<float>(l.pos);
         rp.res = at<float>(l.res);
@@ -1834,7 +1904,10 @@ struct StripRun {
             else              rp.count = two->mult;
         }
         const unsigned grid = (unsigned)row_blocks(s, write);
-        if (f32) return launch_chained(strip_row_f32_kernel, grid, 256, 0, 1, st, at<uint2>(l.w), rp);
+        if (f32)
+            return short_rows() ? launch_chained(strip_row_f32_kernel<false>, grid, 256, 0, 1, st, at<uint2>(l.w), rp)
+                                : launch_chained(strip_row_f32_kernel<true>, grid, 256, 0, 1, st, at<uint2>(l.w), rp);
+        if (!write && row_threads(s)) return launch_chained(strip_lse_kernel, grid, 256, 0, 1, st, rp);
         const int64_t rounds = ceil_div(p.N, 8 * ROW_ROUND);
         // four warps to a row from three rounds on; a second segment where they would have more than two
         // rounds each (6144 x 24000: 132 us with it, 134 without; 4096 x 131072: 472 and 481), more

@@ -215,3 +215,36 @@ def test_chained_calls_of_pairs_with_one_to_four_tiles(binding, oracle, B, N, d,
     assert int(b.dev_status.item()) == 0
     for name in ("loss", "row_lse", "pos_logit", "dQ", "dP"):
         assert torch.equal(getattr(a, name), getattr(b, name)), name
+
+
+@pytest.mark.parametrize("B,N,d,dtype", [
+    (8191, 200, 64, "bf16"), (8192, 1, 64, "bf16"), (9001, 512, 128, "bf16"), (8500, 1024, 64, "bf16"),
+    (8500, 1025, 64, "bf16"), (1, 512, 24, "f32"), (1300, 511, 24, "f32"), (9600, 5, 16, "f32"),
+    (700, 513, 24, "f32"),
+])
+def test_short_rows_of_the_row_pass(binding, oracle, B, N, d, dtype):
+    """A thread per row of the loss (at most eight slots, many rows), a warp per row of fp32 logits: both
+    sides of each limit, last blocks and warps that are not full, unusable positives."""
+    prob = inputs.random_problem(B, N, d, dtype, seed=B + N, tau=0.5, scale=d ** -0.5)
+    Q, P, pos = to_device(prob)
+    b = binding.Outputs(B, N, d, binding._dtype_code(Q))
+    args = (Q, P, pos, prob.tau, prob.mask_mode)
+    binding.gc_loss_fwd(*args, b.loss, b.row_lse, b.pos_logit, b.ws, b.dev_status)
+    binding.gc_loss_bwd(*args, b.row_lse, b.dQ, b.dP, b.ws, b.dev_status)
+    torch.cuda.synchronize()
+    ref = _oracle_full(oracle, prob)
+    check_against_oracle(prob, b, ref)
+    check_against_oracle(prob, run_build(prob), ref)
+    bad = pos.clone()
+    bad[0], bad[B // 2] = N, -1
+    binding.gc_loss_fwd(Q, P, bad, *args[3:], b.loss, b.row_lse, b.pos_logit, b.ws, b.dev_status)
+    torch.cuda.synchronize()
+    assert int(b.dev_status.item()) == binding.GC_DEV_POS_RANGE
+    assert b.pos_logit[0].item() == 0 and b.pos_logit[B // 2].item() == 0
+
+
+@pytest.mark.parametrize("B,N,d", [(4671, 30, 128), (4000, 64, 512), (7, 9470, 128), (2000, 100, 2048)])
+def test_one_side_far_longer_than_the_other(binding, oracle, B, N, d):
+    """Gradient tiles of one or two contraction blocks beside tiles of very many."""
+    prob = inputs.random_problem(B, N, d, "bf16", seed=B + N, tau=0.5, scale=d ** -0.5)
+    check_against_oracle(prob, run_build(prob), _oracle_full(oracle, prob))
