@@ -10,8 +10,7 @@
 //                        cache rows against the rows they belong to, in a fixed order.
 //
 // All three are bound by HBM traffic, or by launch and load latency for small batches: one warp per row,
-// which holds its pieces in registers (a second read of the row only beyond 1024
-// columns), fp32 arithmetic, launched early (programmatic dependent launch).
+// which may hold its pieces in registers, fp32 arithmetic, launched early (programmatic dependent launch).
 #include <cuda_bf16.h>
 #include <math.h>
 
@@ -49,10 +48,12 @@ __device__ __forceinline__ void store4(void* row, int k, float4 v) {
 }
 
 // A lane's pieces of a row: 4 columns at 4 lane + 128 x, x < ROW_KEEP, held in registers; the rest is
-// loaded each time it is asked for.  ROW_KEEP is 4 up to 512 columns (more warps per SM), else 8.
+// loaded each time it is asked for.  What is held saves the second read of a row and the wait for it, and costs
+// warps per SM: see keep_normalize, keep_cosine; row_dot_kernel:
+// none for bf16 and beyond 1024 columns, else 4 up to 512, 8.
 template <int ROW_KEEP, typename Load>
 struct RowPieces {
-    float4 v[ROW_KEEP];
+    float4 v[ROW_KEEP > 0 ? ROW_KEEP : 1];
     Load load;
     int d, k0;
     __device__ __forceinline__ RowPieces(Load l, int d_, int lane) : load(l), d(d_), k0(4 * lane) {
@@ -173,6 +174,28 @@ ordered_sum_kernel(const float* v, int64_t n, float scale, float* __restrict__ o
     }
 }
 
+// Pieces to hold.  Measured, us per launch with none / 4 / 8 held (before they were: with none and not chained):
+//   cosine_bwd  bf16  65536 x 128    13 / 17 / 41      4096 x 512     5.5 / 5.4 / 5.5    4096 x 1024  7.9 / 7.4 / 6.1
+//                     32768 x 640    37 / 36 / 49      65536 x 2048   285 / 230 / 304
+//               fp32  16384 x 256   6.4 / 5.7 / 11     32768 x 1024    59 / 56 / 53 and more for narrower, 1536 even
+//   normalize   bf16  65536 x 768    35 / 39 / 38      32768 x 512    9.8 / 8.6 / 11     65536 x 2048 110 / 99 / 92
+//               fp32  65536 x 512    49 / 44 / 44      65536 x 768     77 / 66 / 64
+//   row_dot     bf16  32768 x 640    25 / 26 / 30      65536 x 2048   127 / 136 / 197    (one read of a row: nothing
+//               fp32  65536 x 512    50 / 46 / 47      65536 x 1024    95 / 85 / 83       to save but the wait)
+//                     32768 x 4096  169 / 176 / 230
+int keep_cosine(int64_t rows, int d, int dtype) {
+    if (dtype == GC_F32) return d <= 512 ? 4 : 8;
+    return d <= 256 ? 0 : d > 768 && d <= 1536 && rows <= 4096 ? 8 : 4;
+}
+int keep_normalize(int64_t rows, int d, int dtype) {
+    if (dtype == GC_BF16 && d <= 768 && rows * d > 20000000) return 0;      // neither rows nor unit rows stay in the L2
+    return d <= 512 ? 4 : 8;
+}
+// go(kernel<BF16, KEEP>)
+#define GC_KEEP_CALL(kernel, keep)                                                                               \
+    (dtype == GC_F32 ? ((keep) == 4 ? go(kernel<false, 4>) : go(kernel<false, 8>))                               \
+                     : ((keep) == 0 ? go(kernel<true, 0>) : (keep) == 4 ? go(kernel<true, 4>) : go(kernel<true, 8>)))
+
 int grid_for(int64_t rows) {
     int64_t blocks = (rows + 7) / 8;
     const int cap = sm_count() * 8;
@@ -216,8 +239,8 @@ int gc_row_normalize(const void* X, int64_t ldx, int64_t rows, int d, int dtype,
         return launch_chained(kernel, dim3(grid_for(rows)), 256, 0, 1, st, X, ldx, rows, d, Xn, ldxn,
                               inv_norm);
     };
-    if (dtype == GC_BF16) e = d <= 512 ? go(row_normalize_kernel<true, 4>) : go(row_normalize_kernel<true, 8>);
-    else                  e = d <= 512 ? go(row_normalize_kernel<false, 4>) : go(row_normalize_kernel<false, 8>);
+    const int keep = keep_normalize(rows, d, dtype);
+    e = GC_KEEP_CALL(row_normalize_kernel, keep);
     return e == cudaSuccess ? GC_OK : GC_ERR_CUDA;
 }
 
@@ -234,8 +257,8 @@ int gc_cosine_bwd(const void* X, int64_t ldx, int64_t rows, int d, int dtype, co
         return launch_chained(kernel, dim3(grid_for(rows)), 256, 0, 1, st, X, ldx, inv_norm, dXn, lddxn,
                               rows, d, dX, lddx);
     };
-    if (dtype == GC_BF16) e = d <= 512 ? go(cosine_bwd_kernel<true, 4>) : go(cosine_bwd_kernel<true, 8>);
-    else                  e = d <= 512 ? go(cosine_bwd_kernel<false, 4>) : go(cosine_bwd_kernel<false, 8>);
+    const int keep = keep_cosine(rows, d, dtype);
+    e = GC_KEEP_CALL(cosine_bwd_kernel, keep);
     return e == cudaSuccess ? GC_OK : GC_ERR_CUDA;
 }
 
@@ -257,8 +280,8 @@ int gc_dtau(const void* Q, int64_t ldq, const float* dQ, int64_t lddq, int64_t B
     auto go = [&](auto kernel) {
         return launch_chained(kernel, dim3(grid_for(B)), 256, 0, 1, st, Q, ldq, dQ, lddq, B, d, row_dot);
     };
-    if (dtype == GC_BF16) e = d <= 512 ? go(row_dot_kernel<true, 4>) : go(row_dot_kernel<true, 8>);
-    else                  e = d <= 512 ? go(row_dot_kernel<false, 4>) : go(row_dot_kernel<false, 8>);
+    if (dtype == GC_BF16) e = go(row_dot_kernel<true, 0>);
+    else e = d > 1024 ? go(row_dot_kernel<false, 0>) : d <= 512 ? go(row_dot_kernel<false, 4>) : go(row_dot_kernel<false, 8>);
     if (e != cudaSuccess) return GC_ERR_CUDA;
     e = launch_chained(ordered_sum_kernel, dim3(1), 1024, 0, 1, st, row_dot, B, -1.f / tau, dtau);
     return e == cudaSuccess ? GC_OK : GC_ERR_CUDA;

@@ -207,3 +207,34 @@ def test_two_direction_loss(binding, oracle, B, N, d, dtype, tau):
     assert grad_err(dQ.cpu().numpy(), ref["dQ"], floor) <= tol["grad"]
     assert grad_err(dP.cpu().numpy(), ref["dP"], floor) <= tol["grad"]
     assert torch.equal(dQ, outs[1][1]) and torch.equal(dP, outs[1][2])
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("rows,d", [(7, 8), (300, 256), (300, 264), (4096, 520), (1001, 776), (4096, 1024),
+                                    (4097, 1024), (130, 1536), (130, 1544), (9, 4104), (27000, 744)])
+def test_row_kernels_at_every_width(rows, d, dtype):
+    """Unit rows, the gradient through the normalisation and dL/dtau where the number of pieces that a lane
+    holds changes, against 64-bit arithmetic on the same values: bounded by the roundings of the results."""
+    from paper_2101_06983_b200 import binding as b
+    g = torch.Generator(device="cuda").manual_seed(rows + d)
+    dt = torch.float32 if dtype == "f32" else torch.bfloat16
+    X = torch.randn(rows, d, generator=g, device="cuda").to(dt)
+    G = torch.randn(rows, d, generator=g, device="cuda")
+    X[rows // 2] = 0
+    Xn, inv = torch.empty_like(X), torch.empty(rows, device="cuda")
+    b.gc_row_normalize(X, Xn, inv)
+    dX, dtau = torch.empty_like(G), torch.empty(1, device="cuda")
+    b.gc_cosine_bwd(X, inv, G, dX)
+    b.gc_dtau(X, G, 0.5, dtau)
+    x, gg = X.double(), G.double()
+    norm = x.norm(dim=1, keepdim=True)
+    i64 = torch.where(norm > 0, 1 / norm, torch.zeros_like(norm))
+    n = x * i64
+    eps = 2.0 ** -21                       # a few fp32 roundings: sums over a warp's pieces, sqrt, products
+    unit = eps if dtype == "f32" else 2.0 ** -8 + eps
+    assert bool(((Xn.double() - n).abs() <= unit * n.abs() + 1e-30).all())
+    want = i64 * (gg - n * (n * gg).sum(1, keepdim=True))
+    scale = i64 * (gg.abs() + n.abs() * (n * gg).abs().sum(1, keepdim=True))
+    assert bool(((dX.double() - want).abs() <= eps * scale + 1e-30).all())
+    ref, terms = -2.0 * (x * gg).sum(), 2.0 * (x * gg).abs().sum()
+    assert abs(dtau.double() - ref).item() <= eps * terms.item()
