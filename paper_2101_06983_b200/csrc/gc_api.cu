@@ -721,7 +721,7 @@ int gc_loss_bwd(const void* Q, int64_t ldq, const void* P, int64_t ldp, const in
     if (small_applicable(B, N, d, dtype) && (dQ || dP))
         return run_small(GC_OP_BWD, p, row_lse, nullptr, nullptr, nullptr, dQ, lddq, dP, lddp,
                          dev_status, st);
-    if ((dQ || dP) && pl.strips >> (dQ && dP ? STRIP_BWD : STRIP_BWD_ONE) & 1) {
+    if ((dQ || dP) && pl.strips >> (dQ && dP ? STRIP_BWD : dQ ? STRIP_BWD_DQ : STRIP_BWD_DP) & 1) {
         KernelTimer t(1, st);
         return strip_backward(p, ws, row_lse, dQ, lddq, dP, lddp, dev_status, st) == cudaSuccess
                    ? GC_OK : GC_ERR_CUDA;
@@ -837,7 +837,7 @@ int gc_shard_dp(const void* Q, int64_t ldq, const void* P, int64_t ldp, const in
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     char* w = static_cast<char*>(ws);
     const char* p_first = static_cast<const char*>(P) + (size_t)p0 * (size_t)ldp * elem_size(dtype);
-    if (pl.strips >> STRIP_BWD_ONE & 1) {
+    if (pl.strips >> STRIP_SHARD_DP & 1) {
         Problem p = make_problem(Q, ldq, p_first, ldp, pos_idx, B, p_count, d, tau, mask_mode, dtype);
         p.mask_shift = -p0;
         p.pos_base = p0;

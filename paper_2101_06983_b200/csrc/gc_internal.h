@@ -242,8 +242,9 @@ cudaError_t launch_small_tiled_fwd(const Problem& pr, float* part_m, float* part
 
 // gc_strip.cu
 // What a call wants of the strip plan: the loss alone; both gradients with the loss, or given row_lse; dQ
-// with the loss; one gradient given row_lse; the two-direction loss.
-enum StripUse { STRIP_FWD, STRIP_BUILD, STRIP_BWD, STRIP_BUILD_DQ, STRIP_BWD_ONE, STRIP_TWO_DIR, STRIP_USES };
+// with the loss; dQ or dP alone given row_lse; dP of a rank's passages; the two-direction loss.
+enum StripUse { STRIP_FWD, STRIP_BUILD, STRIP_BWD, STRIP_BUILD_DQ, STRIP_BWD_DQ, STRIP_BWD_DP, STRIP_SHARD_DP,
+                STRIP_TWO_DIR, STRIP_USES };
 bool strip_applicable(StripUse use, int64_t B, int64_t N, int d, int dtype);
 size_t strip_workspace_bytes(int64_t B, int64_t N, int d, int dtype);
 size_t strip_forward_bytes(int64_t B, int64_t N, int d, int dtype);     // strip_forward's share of it

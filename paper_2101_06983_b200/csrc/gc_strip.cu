@@ -1969,26 +1969,72 @@ struct StripRun {
 
 }  // namespace
 
+// Calls with rows of at most 384 values that the sweeps (gc_narrow.cu, gc_tc.cu) serve better: they keep the
+// weights on the chip and form the logits again, where strips write and read (in a build, also convert) the
+// weights in memory.  They gain with the pairs; and where one side is far longer than the other, since the
+// strip plan has few long gradient tiles there and few CTA pairs to take them.  us, sweeps / strips:
+//   build     d =  64  2900 x 5800 57 / 56     4500 x 4500 58 / 63    d = 128  4000 x 4000 58 / 53   4500 x 4500 61 / 63
+//             d = 256  6000 x 6000 101 / 101, 8192 x 8192 to the sweeps by the older sweep of sizes
+//             d <= 128 6500 x 128 40 / 39      10000 x 128 42 / 53    12500 x 384 46 / 44
+//                      64 x 6500 43 / 38       64 x 10000 47 / 53     100 x 12500 51 / 44
+//             d = 256  64 x 10000 56 / 54      64 x 12500 60 / 63     64 x 16000 65 / 76    64 x 64000 10 : 8
+//   backward  d =  64  2000 x 2000 28 / 24     2048 x 4096 31 / 34    d = 128  3000 x 1500 33 / 27   2048 x 4096 32 / 35
+//             d <= 128 4000 x 64 about even    5000 x 64 27 / 30      5000 x 256 33 / 30     6500 x 256 35 / 36
+//                      64 x 4000 about even    64 x 5000 25 / 29      100 x 32000 52 / 54    180 x 16000 even
+//             d = 256  64 x 5000 31 / 30       64 x 6500 33 / 35      64 x 32000 79 / 89     64 x 64000 9 : 10
+//   dQ alone  d <= 128 600 x 600 16 / 15       1000 x 1000 15 / 17    64 x 4000 10 : 13      16 x 16000 10 : 12
+//             d = 256  1000 x 1000 18 / 18     1500 x 1500 20 / 21    64 x 12500 33 / 31     16000 x 256 10 : 17
+//             d = 384  2000 x 2000 26 / 26     2000 x 4000 32 / 36    1024 x 16384 60 / 47   16000 x 180 10 : 13
+//   dP alone  d <= 128 1000 x 1000 16 / 15     2000 x 1000 16 / 19    4000 x 64 10 : 15
+//             d = 256  1500 x 1500 20 / 19     2000 x 2000 20 / 24    4000 x 256 10 : 9      128 x 16000 10 : 13
+//             d = 384  2000 x 2000 27 / 25     4000 x 2000 32 / 36    6000 x 12000 159 / 123
+//   dQ, loss  d <= 128 3500 x 3500 43 / 43     4000 x 4000 40 / 50    1000 x 12000 48 / 48   64000 x 128 10 : 14
+//             d = 256  4000 x 4000 53 / 54     4000 x 8000 even
+//             d = 384  4000 x 4000 54 / 54     4000 x 8000 77 / 87    1024 x 32768 122 / 93
+//   dP of a rank (of eight; the sweeps launch two kernels more)   d = 128  3000 x 750 23 / 23   4096 x 1024 23 / 27
+//             d = 256  6000 x 1500 37 / 34     8192 x 2048 44 / 44, 16384 x 2048 65 / 71
+//   both directions  d = 128  12000 x 12000 431 / 366   16384 x 16384 585 / 646   7 x 9470 60 / 76
+static bool sweeps_serve(StripUse use, int64_t B, int64_t N, int d) {
+    constexpr int64_t M = 1 << 20;
+    const int64_t pairs = B * N;
+    const bool narrow = d <= 128, middle = !narrow && d <= 256;       // else up to 384
+    if (use == STRIP_FWD) return false;
+    if (use == STRIP_BUILD) {
+        if (narrow && ((B >= 7168 && N <= 256) || (N >= 7168 && B <= 64))) return true;
+        if (middle && B <= 64 && N >= 11264 && N < 49152) return true;
+        return pairs > (d <= 64 ? 17 * M : narrow ? 18 * M : middle ? 56 * M : pairs);
+    }
+    if (use == STRIP_BWD) {
+        if (narrow && ((B >= 4608 && N <= 128) || (B >= 6144 && N <= 384))) return true;
+        if (narrow && N >= 4608 && (B <= 64 || (B <= 128 && N < 24576))) return true;
+        if (middle && N >= 6144 && N < 49152 && B <= 64) return true;
+        return narrow && pairs > (d <= 64 ? 6 * M : 7 * M);
+    }
+    if (use == STRIP_BUILD_DQ) {
+        if (narrow) return B >= 32768 || pairs > (B <= 1024 ? 20 * M : 12 * M);
+        return pairs > (middle ? 28 * M : B <= 1500 ? 44 * M : 15 * M);
+    }
+    if (use == STRIP_BWD_DQ) {
+        if (narrow) return pairs > 3 * M / 4 || B > 2560 || N > 2560;
+        if (middle) return B <= 256 ? N > 1280 && N < 8192 : pairs > M || B >= 8192;
+        return B > 1024 && (pairs > 4 * M || B >= 8192);
+    }
+    if (use == STRIP_BWD_DP) {
+        if (narrow) return pairs > 3 * M / 4 || B > 2560 || N > 8192;
+        if (middle) return N > 256 && (pairs > 9 * M / 4 || N >= 8192);
+        return N > 512 && pairs > 4 * M && (N < B + B / 2 || N > 8 * B);
+    }
+    if (use == STRIP_SHARD_DP) return pairs > (narrow ? 2 * M : middle ? 14 * M : pairs);
+    if (!narrow && !middle) return false;
+    return (narrow && pairs > 160 * M) || (B <= 64 && N >= 4096);       // STRIP_TWO_DIR
+}
+
 // Which calls take the strip plan.  fp32 and bf16 widths that are no multiple of 64: the problems of
-// small_tiled_applicable (up to 2 GiB of tile-pair planes, 64 tile pairs).  bf16 rows in whole 64s, in one
-// strip or up to N = 2^18 (a strip's weights are bounded, so more passages mean fewer queries per strip
-// and more passes over dP): the loss alone always; with gradients, narrow rows only up to a number of pairs, beyond which
-// the weights, written and read (and, in a build, converted) in memory, cost more than the sweeps of
-// gc_narrow.cu and gc_tc.cu, which keep them on the chip and form the logits again.  Measured, us, sweeps
-// / strips, on both sides of each limit (in units of 2^20 pairs):
-//   build      d =  64  5000 x 5000 61 / 61      4096 x 8192 66 / 68
-//              d = 128  4096 x 8192 72 / 70      6000 x 6000 76 / 78
-//              d = 256  5000 x 10000 140 / 137   6000 x 12000 158 / 165
-//              d = 384  8192 x 16384 421 / 375   16384 x 32768 1812 / 1661
-//   backward   d =  64  4096 x 4096 39 / 37      3000 x 6000 37 / 40     (d = 128: 5000 x 5000 53 / 49,
-//              4096 x 8192 57 / 61; d = 256: 8192 x 16384 262 / 201)
-//   dQ only    d = 128  1024 x 16384 58 / 50     2048 x 16384 60 / 68
-//   (of eight) d = 256  1500 x 24000 88 / 86     2048 x 16384 82 / 87
-//              d = 384  1500 x 24000 109 / 96    2048 x 32768 154 / 182  (d = 512: 247 / 217)
-//   dP only    d = 128  3000 x 750 23 / 23       4096 x 1024 23 / 27
-//   (of eight) d = 256  6000 x 1500 37 / 34      8192 x 2048 44 / 44, 16384 x 2048 65 / 71
-//   both directions, d = 128: 12000 x 12000 431 / 366, 16384 x 16384 585 / 646
-//   loss alone d =  64  16384 x 32768 283 / 238  30000 x 60000 994 / 801
+// small_tiled_applicable.  (Both its bounds come from an earlier plan, which kept planes of partial sums per tile
+// pair; strips would not need them.)  bf16 rows in whole 64s: all calls but those of sweeps_serve, and but more
+// than 2^18 passages with more than 256 M pairs.  That limit dates from strips of as many pairs and is not where
+// the routes cross now (us, sweeps / strips, 1024 x 300000 x 768: loss 514 / 322, backward 2394 / 1154, build 2572 /
+// 1451, dQ with the loss 853 / 1084; 2048 x 524288 x 768: 1595 / 1098, 6409 / 4078, 6539 / 6681, 2911 / 3705).
 // GRADCACHE_PLAN=sweeps: as in gc_small.cu.
 bool strip_applicable(StripUse use, int64_t B, int64_t N, int d, int dtype) {
     const char* e = getenv("GRADCACHE_PLAN");
@@ -1997,17 +2043,7 @@ bool strip_applicable(StripUse use, int64_t B, int64_t N, int d, int dtype) {
     if (N > (1 << 24) || B > (1 << 24)) return false;
     if (dtype == GC_F32 || d % 64 != 0) return small_tiled_applicable(B, N, d, dtype);
     if (N > 1 << 18 && B * N > (int64_t)256 << 20) return false;
-    if (use == STRIP_FWD || d > 384) return true;
-    constexpr int ANY = 0;
-    static const int most[][4] = {      // d <= 64, 128, 256, 384
-        {24, 32, 56, ANY},              // STRIP_BUILD
-        {16, 24, ANY, ANY},             // STRIP_BWD
-        {20, 20, 28, 44},               // STRIP_BUILD_DQ
-        {2, 2, 14, ANY},                // STRIP_BWD_ONE
-        {160, 160, ANY, ANY},           // STRIP_TWO_DIR
-    };
-    const int limit = most[use - STRIP_BUILD][d <= 64 ? 0 : d <= 128 ? 1 : d <= 256 ? 2 : 3];
-    return limit == ANY || B * N <= (int64_t)limit << 20;
+    return d > 384 || !sweeps_serve(use, B, N, d);
 }
 
 // A build that forms the logits twice, for the logsumexp and then for the weights, and has no row pass:

@@ -79,3 +79,28 @@ def test_twice_is_bit_identical(binding):
         assert torch.equal(getattr(a, name), getattr(b, name)), name
     assert grad_err(a.dQ.cpu().numpy(), b.dQ.cpu().numpy()) == 0.0
     assert TOL["bf16"]["grad"] > 0
+
+
+@pytest.mark.parametrize("B,N,d", [(8000, 100, 64), (50, 9000, 128), (60, 12500, 256), (4500, 4400, 128),
+                                   (8500, 300, 384)])
+def test_batches_that_the_sweeps_serve(binding, oracle, B, N, d):
+    """Narrow rows with many pairs, or with one side far longer than the other: every call, whichever route
+    each of them takes, against the oracle; the dispatch keeps at least one of them on the sweeps."""
+    prob = inputs.random_problem(B, N, d, "bf16", seed=B + N, tau=0.5, scale=d ** -0.5)
+    ref = _oracle_full(oracle, prob)
+    check_against_oracle(prob, run_build(prob), ref)
+    Q, P, pos = to_device(prob)
+    o = binding.Outputs(B, N, d, binding.GC_BF16)
+    args = (Q, P, pos, prob.tau, prob.mask_mode)
+    binding.gc_loss_fwd(*args, o.loss, o.row_lse, o.pos_logit, o.ws, o.dev_status)
+    binding.gc_loss_bwd(*args, o.row_lse, o.dQ, o.dP, o.ws, o.dev_status)
+    torch.cuda.synchronize()
+    check_against_oracle(prob, o, ref)
+    o.dQ.fill_(float("nan"))
+    o.dP.fill_(float("nan"))
+    binding.gc_loss_bwd(*args, o.row_lse, o.dQ, None, o.ws, o.dev_status)
+    binding.gc_loss_bwd(*args, o.row_lse, None, o.dP, o.ws, o.dev_status)
+    torch.cuda.synchronize()
+    check_against_oracle(prob, o, ref)
+    if d <= 256:
+        assert binding.gc_kernel_launches(binding.GC_OP_BUILD, B, N, d, binding.GC_BF16) > 3
