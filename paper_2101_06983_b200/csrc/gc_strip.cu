@@ -499,7 +499,7 @@ strip_logit_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
                     const float4* cn = reinterpret_cast<const float4*>(p.col_neg + jg);
 #pragma unroll
                     for (int e = 0; e < 64; e += 4) {
-                        const float4 n4 = jg + e < p.N ? __ldcg(cn + (e >> 2)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        const float4 n4 = jg + e < p.N ? cn[e >> 2] : make_float4(0.f, 0.f, 0.f, 0.f);
                         const float nn[4] = {n4.x, n4.y, n4.z, n4.w};
 #pragma unroll
                         for (int x = 0; x < 4; ++x)
@@ -1442,7 +1442,7 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
                         if (col + 8 * j >= sd.cols) break;
-                        const uint4 x = __ldcg(pr + j);
+                        const uint4 x = pr[j];
                         const uint32_t w[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
