@@ -88,9 +88,10 @@ size_t gc_workspace_bytes(int op, int64_t B, int64_t N, int d, int dtype);
  *                       4096; at most two CTAs' worth of 64-column slices per SM)
  *   "tcgen05"           bf16, d a multiple of 64 up to 4096, TMA + tcgen05 MMA.  The strip plan: three
  *                       products over strips of query rows whose weights are held in the workspace;
- *                       or, for gradients of narrow rows (at most 256 values; 384 for one rank's dQ)
- *                       with many pairs and for more than 2^18 passages, sweeps that keep every
- *                       logit on the chip (one CTA, a CTA pair or a cluster of four per tile)
+ *                       or sweeps that keep every logit on the chip (one CTA, a CTA pair or a cluster
+ *                       of four per tile): for gradients of narrow rows (at most 256 values; 384 for one
+ *                       gradient alone) with many pairs or with one side far longer than the other, and
+ *                       for more than 2^18 passages with more than 256 M pairs
  *   "simt"              fp32 FMA tiles: every other case (other widths, fp32 batches beyond that)
  * "invalid" for an unknown op, non-positive sizes, or a problem GC_OP_BUILD_STORED refuses.
  * Static string.  With GRADCACHE_PLAN=sweeps in the environment (read at every call; a
@@ -353,6 +354,9 @@ int gc_loss_fwd_static(const void* Q, int64_t ldq, const void* P, int64_t ldp,
  * gc_profile_read_call(c, ...) waits for that call's events and returns each kernel's duration
  * in milliseconds (0 for a kernel the call did not launch; GC_ERR_LIMIT when call c was never
  * made or its set has been reused); gc_profile_read does the same for the most recent call.
+ * Those are the kernels of the sweeps.  The strip plan and the one-tile plan form all of a call in
+ * launches that are not told apart: their time, from the first to the last, comes as the forward's
+ * (gc_loss_fwd of the strip plan), the dP sweep's (gc_shard_dp) or else the dQ sweep's, the rest 0.
  * Host pointers.  One series of event sets per process: use it for single-stream measurement
  * runs only.  While it is on, the event between the anchor kernel and the fused sweep keeps
  * the sweep from starting early (see gc_build_cache).
