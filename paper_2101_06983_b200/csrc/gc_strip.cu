@@ -27,7 +27,6 @@
 #include <string.h>
 
 #include <algorithm>
-#include <type_traits>
 
 #include "tc_common.cuh"
 
@@ -929,31 +928,47 @@ strip_row_kernel(uint4* __restrict__ W, const RowParams p) {
                 const float2 now = next;
                 if (kr + stride < k1) next = slot_of(kr + stride);
                 const float fg = now.x > -INFINITY ? ex2(fmaf(now.x, p.c1, neg)) : 0.f;
-                auto round = [&](auto small) {
+                auto weights = [&](int k, const float2 (&v)[4]) {
+                    float w[8];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) { w[2 * e] = v[e].x; w[2 * e + 1] = v[e].y; }
+                    if (wk == k) {
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) if (e == (pos & 7)) w[e] = pw;
+                    }
+                    row[k] = make_uint4(pack_b2(w[0], w[1]), pack_b2(w[2], w[3]),
+                                        pack_b2(w[4], w[5]), pack_b2(w[6], w[7]));
+                };
+                if (!__any_sync(0xffffffffu, now.y < 0.f)) {
 #pragma unroll
                     for (int x = 0; x < ROW_PIECES; ++x) {
                         const float f = __shfl_sync(0xffffffffu, fg, 4 * x + (lane >> 3));
                         const int k = kr + lane + 32 * x;
                         if (k >= k1) continue;
-                        const uint32_t h[4] = {raw[x].x, raw[x].y, raw[x].z, raw[x].w};
-                        float w[8];
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const float2 v = decltype(small)::value ? stash_times_small(h[e], f) : stash_times(h[e], f);
-                            w[2 * e] = v.x;
-                            w[2 * e + 1] = v.y;
-                        }
-                        if (wk == k) {
-#pragma unroll
-                            for (int e = 0; e < 8; ++e) if (e == (pos & 7)) w[e] = pw;
-                        }
-                        row[k] = make_uint4(pack_b2(w[0], w[1]), pack_b2(w[2], w[3]),
-                                            pack_b2(w[4], w[5]), pack_b2(w[6], w[7]));
+                        const float2 v[4] = {stash_times(raw[x].x, f), stash_times(raw[x].y, f),
+                                             stash_times(raw[x].z, f), stash_times(raw[x].w, f)};
+                        weights(k, v);
                         if (k + stride < k1) raw[x] = __ldcg(row + k + stride);
                     }
-                };
-                if (__any_sync(0xffffffffu, now.y < 0.f)) round(std::true_type{});
-                else                                      round(std::false_type{});
+                } else {
+                    // both forms: one piece after the other, read again (code kept short: unrolled like the other it
+                    // cost every launch, 872 x 872 x 768 22.2 us a build against 21.7)
+#pragma unroll 1
+                    for (int x = 0; x < ROW_PIECES; ++x) {
+                        const float f = __shfl_sync(0xffffffffu, fg, 4 * x + (lane >> 3));
+                        const int k = kr + lane + 32 * x;
+                        if (k >= k1) continue;
+                        const uint4 h = __ldcg(row + k);
+                        const float2 v[4] = {stash_times_small(h.x, f), stash_times_small(h.y, f),
+                                             stash_times_small(h.z, f), stash_times_small(h.w, f)};
+                        weights(k, v);
+                    }
+#pragma unroll
+                    for (int x = 0; x < ROW_PIECES; ++x) {
+                        const int k = kr + lane + 32 * x + stride;
+                        if (k < k1) raw[x] = __ldcg(row + k);
+                    }
+                }
             }
         }
     }
