@@ -2,7 +2,7 @@
 side-stream work is forked from and joined back into that stream, and nothing in it touches the
 host allocator or synchronises, so one call can be captured once and replayed.  The replay must
 give the eager call's results bit for bit (and those are checked against the oracle), for every
-plan."""
+plan: on the route that the library chooses, and on the sweeps, whose side stream is captured with them."""
 import pytest
 import torch
 
@@ -22,8 +22,8 @@ def binding():
 
 
 CASES = [
-    # B, N, d, dtype, mask: one launch, tile pairs, four-CTA sweeps, narrow-row sweeps, paired wide
-    # rows, FMA tiles
+    # B, N, d, dtype, mask: one launch in both dtypes, strips of a few tiles and of many, with the self mask,
+    # of an odd width; FMA tiles.  On the sweeps: four-CTA (640, 768), narrow-row (128) and paired (320) ones
     (128, 256, 768, "bf16", 0), (64, 128, 768, "f32", 0), (300, 520, 640, "bf16", 0),
     (1030, 1300, 768, "bf16", 0), (2100, 2100, 128, "bf16", 1), (700, 1400, 320, "bf16", 0),
     (150, 140, 36, "f32", 0),
@@ -31,7 +31,7 @@ CASES = [
 
 
 @pytest.mark.parametrize("B,N,d,dtype,mask", CASES)
-def test_graph_replay_equals_the_eager_call(binding, oracle, B, N, d, dtype, mask):
+def test_graph_replay_equals_the_eager_call(binding, oracle, B, N, d, dtype, mask, plan_mode):
     prob = inputs.random_problem(B, N, d, dtype, seed=B + d, tau=0.5, scale=d ** -0.5,
                                  mask_mode=mask, shared=bool(mask))
     Q, P, pos = binding.problem_tensors(prob)

@@ -86,8 +86,8 @@ def test_four_cta_cluster_sweeps_self_mask(binding, oracle, plan_mode):
 
 
 @pytest.mark.parametrize("B,N", [(300, 45000), (45000, 300)])
-def test_streamed_matrix_larger_than_l2_uses_cta_pairs(binding, oracle, B, N):
-    """When the streamed matrix (P for the forward/dQ sweeps, Q for the dP sweep) exceeds 64 MB
+def test_streamed_matrix_larger_than_l2_uses_cta_pairs(binding, oracle, B, N, plan_mode):
+    """On the sweeps: when the streamed matrix (P for the forward/dQ sweeps, Q for the dP sweep) exceeds 64 MB
     the wide-row kernels run as CTA pairs that share every streamed chunk.  Both orientations,
     with an odd number of 128-row tiles on the stationary side (3), against the full oracle."""
     prob = inputs.random_problem(B, N, 768, "bf16", seed=B + N, tau=0.5, scale=768 ** -0.5)

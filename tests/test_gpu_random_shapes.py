@@ -1,7 +1,8 @@
 """Seeded random problem shapes through gc_build_cache against the CPU oracle, element by element:
-sizes drawn so that every plan is met (one-tile batches in bf16 and fp32, narrow and wide bf16
-rows with ragged tiles and split ranges, the four-CTA sweeps, fp32 batches of a few tiles, the
-FMA-tile plan for widths that are not a multiple of 8), both mask modes, several temperatures.
+sizes drawn so that every plan is met (one-tile batches in bf16 and fp32; bf16 batches of several tiles
+on strips and, a second time, on the sweeps: narrow, wide and four-CTA ones with ragged tiles and split
+ranges; fp32 strips; the FMA tiles for widths that are not a multiple of 8), both mask modes, several
+temperatures.
 The shapes are fixed by the seed: the same forty-odd cases every run."""
 import numpy as np
 import pytest
@@ -51,8 +52,7 @@ def binding():
     return b
 
 
-@pytest.mark.parametrize("kind,dtype,B,N,d,mask,tau,seed", _cases())
-def test_random_shape(binding, oracle, kind, dtype, B, N, d, mask, tau, seed):
+def _problem(dtype, B, N, d, mask, tau, seed):
     if dtype == "bf16" and d % 8:
         d = (d + 7) // 8 * 8
     if mask:
@@ -61,12 +61,26 @@ def test_random_shape(binding, oracle, kind, dtype, B, N, d, mask, tau, seed):
                                      mask_mode=inputs.MASK_SELF, shared=True)
     else:
         prob = inputs.random_problem(B, N, d, dtype, seed=seed, tau=tau, scale=d ** -0.5)
+    return prob
+
+
+@pytest.mark.parametrize("kind,dtype,B,N,d,mask,tau,seed", _cases())
+def test_random_shape(binding, oracle, kind, dtype, B, N, d, mask, tau, seed):
+    prob = _problem(dtype, B, N, d, mask, tau, seed)
     code = binding.GC_BF16 if dtype == "bf16" else binding.GC_F32
     plan = binding.gc_plan_name(binding.GC_OP_BUILD, prob.B, prob.N, prob.d, code)
     if kind == "one-tile":
         assert plan == "tcgen05-one-tile"
     if kind == "fma":            # fp32 beyond one tile: tcgen05 per tile pair, or FMA tiles
         assert plan == ("tcgen05-tiles" if prob.d % 8 == 0 else "simt")
+    out = run_build(prob)
+    ref = oracle.build_cache(prob.Q, prob.P, prob.pos_idx, prob.tau, prob.mask_mode)
+    check_against_oracle(prob, out, ref)
+
+
+@pytest.mark.parametrize("kind,dtype,B,N,d,mask,tau,seed", [c for c in _cases() if c[0] in ("narrow", "wide", "quad")])
+def test_random_shape_on_the_sweeps(binding, oracle, kind, dtype, B, N, d, mask, tau, seed, sweeps_only):
+    prob = _problem(dtype, B, N, d, mask, tau, seed)
     out = run_build(prob)
     ref = oracle.build_cache(prob.Q, prob.P, prob.pos_idx, prob.tau, prob.mask_mode)
     check_against_oracle(prob, out, ref)

@@ -23,15 +23,16 @@ def binding():
 CASES = [
     # B, N, d, dtype, world
     (50, 90, 40, "f32", 3),        # FMA-tile plan
+    # strips, and on the sweeps:
     (300, 610, 128, "bf16", 2),    # narrow rows, fixed row scale
     (700, 1300, 768, "bf16", 3),   # four-CTA sweeps per rank
     (250, 520, 768, "bf16", 2),    # 125 queries per rank: one x tile, online-maximum sweep
-    (130, 260, 1024, "bf16", 4),
+    (130, 260, 1024, "bf16", 4),   # paired wide rows
 ]
 
 
 @pytest.mark.parametrize("B,N,d,dtype,world", CASES)
-def test_ranks_together_reproduce_the_full_batch(binding, oracle, B, N, d, dtype, world):
+def test_ranks_together_reproduce_the_full_batch(binding, oracle, B, N, d, dtype, world, plan_mode):
     prob = inputs.random_problem(B, N, d, dtype, seed=B + N, tau=0.5, scale=d ** -0.5)
     ref = oracle.build_cache(prob.Q, prob.P, prob.pos_idx, prob.tau, prob.mask_mode)
     Q, P, pos = to_device(prob)
@@ -70,7 +71,7 @@ MASKED = [
 
 
 @pytest.mark.parametrize("n,d,dtype,world", MASKED)
-def test_self_mask_follows_the_rank_ranges(binding, oracle, n, d, dtype, world):
+def test_self_mask_follows_the_rank_ranges(binding, oracle, n, d, dtype, world, plan_mode):
     prob = inputs.random_problem(n, n, d, dtype, seed=n + d, tau=0.2, mask_mode=inputs.MASK_SELF,
                                  scale=d ** -0.5, shared=True)
     ref = oracle.build_cache(prob.Q, prob.P, prob.pos_idx, prob.tau, prob.mask_mode)
@@ -116,8 +117,8 @@ def test_sharded_step_object_on_one_gpu(binding, oracle):
 
 
 def test_one_rank_is_the_whole_batch(binding, sweeps_only):
-    """world = 1: the two calls together are gc_loss_fwd + gc_loss_bwd on the same kernels (the
-    rank-local calls always run the sweeps, so the whole-batch call is kept on them too)."""
+    """world = 1: the two calls together give the whole batch's results, bit for bit on the sweeps, where the
+    loss and dQ come from the same kernels."""
     prob = inputs.random_problem(140, 270, 64, "bf16", seed=5, tau=0.7, scale=0.125)
     Q, P, pos = to_device(prob)
     a = binding.build_cache(Q, P, pos, prob.tau, prob.mask_mode)

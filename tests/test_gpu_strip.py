@@ -168,7 +168,8 @@ def _hard_negatives(B, N, d, seed):
 
 
 @pytest.mark.parametrize("B,N,d,tau", [(512, 2048, 512, 0.05), (512, 2048, 512, 0.02), (300, 1000, 448, 0.012),
-                                       (300, 1111, 512, 0.2), (130, 900, 64, 0.03)])
+                                       (300, 1111, 512, 0.2), (130, 900, 64, 0.03), (200, 5000, 64, 0.03),
+                                       (150, 17001, 512, 0.05)])
 def test_rows_of_small_weights_keep_their_precision(binding, B, N, d, tau):
     """dP row by row, for passages whose every weight lies up to a hundred powers of two below their row's
     largest.  A weight is rounded at most twice, to 8 bits of mantissa (2^-9 of it) in between and to bf16
@@ -248,3 +249,64 @@ def test_one_side_far_longer_than_the_other(binding, oracle, B, N, d):
     """Gradient tiles of one or two contraction blocks beside tiles of very many."""
     prob = inputs.random_problem(B, N, d, "bf16", seed=B + N, tau=0.5, scale=d ** -0.5)
     check_against_oracle(prob, run_build(prob), _oracle_full(oracle, prob))
+
+
+def test_several_strips_given_row_lse(binding, oracle):
+    """gc_loss_fwd, then gc_loss_bwd over two strips with the self mask: row_lse, the masked diagonal, the
+    counters and the sums into dP of the second strip."""
+    n, d = 33000, 448
+    prob = inputs.random_problem(n, n, d, "bf16", seed=16, tau=0.5, mask_mode=inputs.MASK_SELF, scale=d ** -0.5)
+    assert binding.gc_kernel_launches(binding.GC_OP_BWD, n, n, d, binding.GC_BF16) == 2 * 2
+    Q, P, pos = to_device(prob)
+    o = binding.Outputs(n, n, d, binding.GC_BF16)
+    args = (Q, P, pos, prob.tau, prob.mask_mode)
+    binding.gc_loss_fwd(*args, o.loss, o.row_lse, o.pos_logit, o.ws, o.dev_status)
+    binding.gc_loss_bwd(*args, o.row_lse, o.dQ, o.dP, o.ws, o.dev_status)
+    torch.cuda.synchronize()
+    assert int(o.dev_status.item()) == 0
+    _check_sampled(oracle, prob, o, 48, 24, full_lse=o.row_lse.cpu().numpy().astype(np.float64))
+    _check_properties(prob, o, Q, P)
+
+
+def test_logits_formed_twice_over_several_strips(binding, oracle):
+    n, d = 28800, 320
+    prob = inputs.random_problem(n, n, d, "bf16", seed=17, tau=0.5, scale=d ** -0.5)
+    assert binding.gc_kernel_launches(binding.GC_OP_BUILD, n, n, d, binding.GC_BF16) == 2 * 4
+    out = run_build(prob)
+    assert int(out.dev_status.item()) == 0
+    _check_sampled(oracle, prob, out, 48, 24, full_lse=out.row_lse.cpu().numpy().astype(np.float64))
+    Q, P, _ = to_device(prob)
+    _check_properties(prob, out, Q, P)
+
+
+def test_two_directions_over_several_strips(binding):
+    """Both directions in one set of weights over two strips, against 64-bit sums in blocks of rows."""
+    n, d, tau = 28800, 192, 0.5
+    g = torch.Generator(device="cuda").manual_seed(18)
+    Q = (torch.randn(n, d, generator=g, device="cuda") * d ** -0.5).bfloat16()
+    P = (torch.randn(n, d, generator=g, device="cuda") * d ** -0.5).bfloat16()
+    pos = torch.randint(0, n, (n,), generator=g, device="cuda")
+    f = dict(dtype=torch.float32, device="cuda")
+    loss, lse, dQ, dP = torch.zeros(1, **f), torch.empty(n, **f), torch.empty(n, d, **f), torch.empty(n, d, **f)
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    binding.gc_build_cache_two_direction(Q, P, pos.int(), tau, loss, lse, dQ, dP, dev_status=st)
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0
+    q, p = Q.double(), P.double()
+    rows = [slice(a, min(a + 3200, n)) for a in range(0, n, 3200)]
+    row_lse = torch.cat([torch.logsumexp(q[r] @ p.T / tau, 1) for r in rows])
+    col_lse = torch.cat([torch.logsumexp(p[r] @ q.T / tau, 1) for r in rows])
+    mult = torch.bincount(pos, minlength=n).double()
+    pl = (q * p[pos]).sum(1) / tau
+    want = 0.5 * ((row_lse - pl) + (col_lse[pos] - pl)).mean().item()
+    rQ, rP = torch.empty_like(q), torch.zeros_like(p)
+    for r in rows:
+        S = q[r] @ p.T / tau
+        W = torch.exp(S - row_lse[r, None]) + mult * torch.exp(S - col_lse)
+        W[torch.arange(W.shape[0], device="cuda"), pos[r]] -= 2.0
+        rQ[r] = W @ p / (2 * n * tau)
+        rP += W.T @ q[r] / (2 * n * tau)
+    tol = TOL["bf16"]
+    assert abs(loss.item() - want) <= tol["loss"] * abs(want)
+    assert grad_err(dQ.cpu().numpy(), rQ.cpu().numpy()) <= tol["grad"]
+    assert grad_err(dP.cpu().numpy(), rP.cpu().numpy()) <= tol["grad"]
