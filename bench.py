@@ -43,9 +43,9 @@ NOMINAL_BF16_TFLOPS = 2250.0      # public dense bf16 figure for B200, context o
 STRIP_SOURCES = ['gc_strip.cu', 'tc_common.cuh']
 ONE_TILE_SOURCES = ['gc_small.cu', 'gc_small_f32.cu', 'tc_common.cuh']
 NCU_STEP_TRAFFIC = {
-    "cfg2_": (276.7e6, STRIP_SOURCES, "ac64f880ab2dd210781007168b2e9357cfe4489f"),
-    "cfg1_": (0.627e6, ONE_TILE_SOURCES, "0cd4e6330cdbe269ff964a2ca75e1035488fc56c"),
-    "cfg0_": (0.634e6, ONE_TILE_SOURCES, "0cd4e6330cdbe269ff964a2ca75e1035488fc56c"),
+    "cfg2_": (272.8e6, STRIP_SOURCES, "01077da8e666c6915687c74dc79e2a9dc4a5d43d"),
+    "cfg1_": (0.627e6, ONE_TILE_SOURCES, "43562d0a6d23d54a678b682771c6a3f376388009"),
+    "cfg0_": (0.634e6, ONE_TILE_SOURCES, "43562d0a6d23d54a678b682771c6a3f376388009"),
 }
 FP32_LANES_PER_SM = 128           # fp32 FMA lanes of one SM (2 FLOP per lane and clock)
 
@@ -626,7 +626,7 @@ def run_apply(args):
     # profiles/apply_kernel_rows4096_d768_din768.txt; reported while gc_apply.cu is unchanged
     import hashlib
     with open(os.path.join(ROOT, "paper_2101_06983_b200", "csrc", "gc_apply.cu"), "rb") as fh:
-        same = hashlib.sha1(fh.read()).hexdigest() == "ee38bebd7446ec94ae01602901763dce147fab0f"
+        same = hashlib.sha1(fh.read()).hexdigest() == "eaf2e4acea8752d9943868df4cb693e7d390c902"
     traffic = 37.8e6 if same and rows == 4096 else None
     import oracle
     t0 = time.perf_counter()
