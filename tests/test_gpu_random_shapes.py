@@ -71,7 +71,7 @@ def test_random_shape(binding, oracle, kind, dtype, B, N, d, mask, tau, seed):
     plan = binding.gc_plan_name(binding.GC_OP_BUILD, prob.B, prob.N, prob.d, code)
     if kind == "one-tile":
         assert plan == "tcgen05-one-tile"
-    if kind == "fma":            # fp32 beyond one tile: tcgen05 per tile pair, or FMA tiles
+    if kind == "fma":            # fp32 beyond one tile: strips, or FMA tiles
         assert plan == ("tcgen05-tiles" if prob.d % 8 == 0 else "simt")
     out = run_build(prob)
     ref = oracle.build_cache(prob.Q, prob.P, prob.pos_idx, prob.tau, prob.mask_mode)

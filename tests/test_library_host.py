@@ -72,7 +72,7 @@ def test_plan_names(binding):
     assert b.gc_plan_name(b.GC_OP_BUILD, 64, 128, 768, b.GC_F32) == "tcgen05-one-tile"
     assert b.gc_plan_name(b.GC_OP_BUILD, 128, 256, 768, b.GC_BF16) == "tcgen05-one-tile"
     assert b.gc_kernel_launches(b.GC_OP_BUILD, 64, 128, 768, b.GC_F32) == 1
-    # fp32 batches of a few tiles: the same kernel per tile pair, plus combine and reduces
+    # fp32 batches of a few tiles: strips, after a pass that splits the inputs into terms
     assert b.gc_plan_name(b.GC_OP_BUILD, 64, 129, 768, b.GC_F32) == "tcgen05-tiles"
     assert b.gc_kernel_launches(b.GC_OP_BUILD, 64, 129, 768, b.GC_F32) == 4
     assert b.gc_plan_name(b.GC_OP_BUILD, 300, 200, 320, b.GC_F32) == "tcgen05-tiles"
