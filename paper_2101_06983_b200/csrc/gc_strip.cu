@@ -37,6 +37,7 @@ namespace {
 constexpr int ST_THREADS = 32 * (NPROD + 1 + NSOFT);
 constexpr int KB = 64;                               // contraction depth of a ring stage
 constexpr int MAX_ST = 6;
+constexpr int MAX_ACC = 4;                           // accumulators in tensor memory: two of 256 columns, four of 128
 constexpr uint32_t HALF_CHUNK = 8192;                // 64 rows x 128 bytes
 constexpr float LOG2E = 1.4426950408889634f;
 constexpr float LN2 = 0.6931471805599453f;
@@ -46,9 +47,9 @@ enum LogitMode { LOGIT_FWD = 0, LOGIT_STASH = 1, LOGIT_W = 2, LOGIT_W2 = 3 };
 struct StripBars {
     uint64_t full[MAX_ST];
     uint64_t empty[MAX_ST];
-    uint64_t acc_full[2];
-    uint64_t acc_free[2];        // this CTA's epilogue warps have read the buffer
-    uint64_t acc_free_peer[2];   // leader: the same, forwarded from the second CTA
+    uint64_t acc_full[MAX_ACC];
+    uint64_t acc_free[MAX_ACC];        // this CTA's epilogue warps have read the buffer
+    uint64_t acc_free_peer[MAX_ACC];   // leader: the same, forwarded from the second CTA
 };
 
 __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap* map, int c0, int c1,
@@ -146,7 +147,7 @@ __device__ __forceinline__ PairCtx pair_setup(uint8_t* raw, StripBars& bars, uin
             mbar_init(smem_u32(&bars.full[s]), 2);        // the leader's two producer warps
             mbar_init(smem_u32(&bars.empty[s]), 1);
         }
-        for (int b = 0; b < 2; ++b) {
+        for (int b = 0; b < MAX_ACC; ++b) {
             mbar_init(smem_u32(&bars.acc_full[b]), 1);
             mbar_init(smem_u32(&bars.acc_free[b]), NSOFT);
             mbar_init(smem_u32(&bars.acc_free_peer[b]), 1);
@@ -189,18 +190,20 @@ __device__ __forceinline__ void pair_teardown(const PairCtx& c, volatile int* ab
 
 // The second CTA's idle issuing warp passes "buffer read" on to the leader: one remote arrival per
 // use instead of eight (a remote arrival stalls the arriving warp for more than a thousand cycles).  Only
-// what the leader waits for (wait_acc_free, of use n + 2): an arrival that nobody waits for could reach the
+// what the leader waits for (wait_acc_free, of use n + NB): an arrival that nobody waits for could reach the
 // leader's shared memory after it has left.
+template <int NB = 2>
 __device__ __forceinline__ void forward_acc_free(StripBars& bars, int uses, volatile int* abort_flag) {
-    for (int n = 0; n < uses - 2; ++n) {
-        const int b = n & 1;
-        if (!mbar_wait(smem_u32(&bars.acc_free[b]), (uint32_t)(n >> 1) & 1u, abort_flag)) return;
+    for (int n = 0; n < uses - NB; ++n) {
+        const int b = n % NB;
+        if (!mbar_wait(smem_u32(&bars.acc_free[b]), (uint32_t)(n / NB) & 1u, abort_flag)) return;
         if (elect_one()) mbar_arrive_cluster(mapa_u32(smem_u32(&bars.acc_free_peer[b]), 0));
     }
 }
+template <int NB = 2>
 __device__ __forceinline__ bool wait_acc_free(StripBars& bars, int n, volatile int* abort_flag) {
-    const int b = n & 1;
-    const uint32_t par = ((uint32_t)(n >> 1) & 1u) ^ 1u;
+    const int b = n % NB;
+    const uint32_t par = ((uint32_t)(n / NB) & 1u) ^ 1u;
     return mbar_wait(smem_u32(&bars.acc_free[b]), par, abort_flag) &&
            mbar_wait(smem_u32(&bars.acc_free_peer[b]), par, abort_flag);
 }
@@ -1269,6 +1272,7 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
     constexpr int NST = F32 ? 3 : 6;
     constexpr int CHUNK_KB = 2;                           // F32: blocks per accumulator read-out
     constexpr int HW = WIDTH / 2;                         // columns of an epilogue warp
+    constexpr int NACC = F32 ? 4 : 2;                     // accumulators in tensor memory
     const int pair = blockIdx.x >> 1;
     dep_release();
     dep_wait();
@@ -1339,10 +1343,10 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
                 for (int k = 0; k < sg.n; ++k) {
                     const bool fresh = F32 ? k % CHUNK_KB == 0 : k == 0;
                     if (fresh) {
-                        ok = wait_acc_free(bars, use, abort_flag);
+                        ok = wait_acc_free<NACC>(bars, use, abort_flag);
                         if (!ok) break;
                         tc_fence_after();
-                        acc = c.tmem + (use & 1) * 256;
+                        acc = c.tmem + (use % NACC) * (TMEM_COLS / NACC);
                     }
                     ok = mbar_wait(smem_u32(&bars.full[stage]), phase, abort_flag);
                     if (!ok) break;
@@ -1366,7 +1370,7 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
                             }
                         }
                         tc_commit_pair(smem_u32(&bars.empty[stage]));
-                        if (last) tc_commit_pair(smem_u32(&bars.acc_full[use & 1]));
+                        if (last) tc_commit_pair(smem_u32(&bars.acc_full[use % NACC]));
                     }
                     if (last) ++use;
                     if (++stage == NST) { stage = 0; phase ^= 1u; }
@@ -1377,7 +1381,7 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
             SegmentWalk walk(p, pair);
             Segment sg;
             while (walk.next(p, sg)) uses += F32 ? (sg.n + CHUNK_KB - 1) / CHUNK_KB : 1;
-            forward_acc_free(bars, uses, abort_flag);
+            forward_acc_free<NACC>(bars, uses, abort_flag);
         }
     } else {
         const int ew = c.warp - (NPROD + 1);
@@ -1422,11 +1426,14 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
             float acc[F32 ? HW : 1];
             if (F32) {
                 const int chunks = (sg.n + CHUNK_KB - 1) / CHUNK_KB;
+#pragma unroll
+                for (int e = 0; e < (F32 ? HW : 1); ++e) acc[e] = -0.f;       // adds nothing, not even a sign
+#pragma unroll 1
                 for (int ch = 0; ch < chunks && ok; ++ch, ++use) {
-                    ok = mbar_wait(smem_u32(&bars.acc_full[use & 1]), (uint32_t)(use >> 1) & 1u, abort_flag);
+                    ok = mbar_wait(smem_u32(&bars.acc_full[use % NACC]), (uint32_t)(use / NACC) & 1u, abort_flag);
                     if (!ok) break;
                     tc_fence_after();
-                    const uint32_t src = c.tmem + (use & 1) * 256 + lanes + half * HW;
+                    const uint32_t src = c.tmem + (use % NACC) * (TMEM_COLS / NACC) + lanes + half * HW;
 #pragma unroll
                     for (int g = 0; g < HW / 32; ++g) {
                         uint32_t v[32];
@@ -1435,20 +1442,20 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
 #pragma unroll
                         for (int e = 0; e < 32; ++e) {
                             const float x = __uint_as_float(v[e]);
-                            acc[32 * g + e] = ch == 0 ? x : acc[32 * g + e] + x;
+                            acc[32 * g + e] += x;
                         }
                     }
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(smem_u32(&bars.acc_free[use & 1]));
+                    if (lane == 0) mbar_arrive(smem_u32(&bars.acc_free[use % NACC]));
                 }
                 if (!ok) break;
             } else {
-                ok = mbar_wait(smem_u32(&bars.acc_full[use & 1]), (uint32_t)(use >> 1) & 1u, abort_flag);
+                ok = mbar_wait(smem_u32(&bars.acc_full[use % NACC]), (uint32_t)(use / NACC) & 1u, abort_flag);
                 if (!ok) break;
                 tc_fence_after();
             }
-            const uint32_t src = c.tmem + (use & 1) * 256 + lanes + half * hw;
+            const uint32_t src = c.tmem + (use % NACC) * (TMEM_COLS / NACC) + lanes + half * hw;
             // one block of 32 columns to the output: scale, the positives' remainder, staging, store
             auto finish = [&](uint32_t (&v)[32], int cb) {
                 const int col = col0 + 32 * cb;
@@ -1496,7 +1503,7 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
                         if (32 * (cb + 1) >= hw) {
                             tc_fence_before();
                             __syncwarp();
-                            if (lane == 0) mbar_arrive(smem_u32(&bars.acc_free[use & 1]));
+                            if (lane == 0) mbar_arrive(smem_u32(&bars.acc_free[use % NACC]));
                         }
                     }
                     finish(v, cb);
@@ -1528,16 +1535,18 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
                     if (F32) return;
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(smem_u32(&bars.acc_free[use & 1]));
+                    if (lane == 0) mbar_arrive(smem_u32(&bars.acc_free[use % NACC]));
                 };
                 // Where all other shares are in memory already (as a rule: a group meets the front part
                 // of its first tile long before the neighbour meets the back part of its last), this
-                // share goes into the sum straight from tensor memory.
+                // share goes into the sum straight from tensor memory.  (Not from the registers of the fp32 sums: the
+                // two sums at once do not fit, and with the running one in local memory a read-out took 4 K cycles
+                // where its products take 2.6 K: 2048 x 4096 x 768, 239 us a build against 199.)
                 int published = 0;
-                if (lane == 0)
+                if (!F32 && lane == 0)
                     asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(published) : "l"(counter) : "memory");
                 published = __shfl_sync(0xffffffffu, published, 0);
-                const bool direct = published == gl - gf;
+                const bool direct = !F32 && published == gl - gf;
                 if (!direct) {
                     float4* mine = part_of(group, sg.kb == 0 ? 1 : 0);
 #pragma unroll
