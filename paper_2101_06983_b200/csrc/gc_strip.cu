@@ -27,6 +27,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "tc_common.cuh"
 
@@ -1173,8 +1174,11 @@ struct GradParams {
     int n_terms;
     float inv_mean;
     float* loss;
+    float* out[2];                // dQ, dP, and their pitches
+    int64_t ldo[2];
     float* part;                  // [pairs][2 slots][2 CTAs][8 warps][32 x hw] partial tiles
-    int* count;                   // [tiles of both sides][2 CTAs][8 warps]
+    int* count;                   // [tiles of both sides][2 CTAs][8 warps]: shares in memory, and pieces of
+                                  // their sum drawn << 16
     int* dev_status;
 };
 
@@ -1184,8 +1188,9 @@ struct Segment {
     int t0;                       // whole < 0: first unit of the row tile
 };
 
+// units * groups stays below 2^32: rows x passages of a strip are at most 768 M, or 256 x 2^24
 __device__ __forceinline__ int unit_start(const GradParams& p, int g) {
-    return (int)((int64_t)p.units * g / p.groups);
+    return (int)((unsigned)p.units * (unsigned)g / (unsigned)p.groups);
 }
 // Iterates over a pair's segments.  In a cut run the two cut tiles come first (their partial sums meet
 // under the products of the tiles that follow), the whole ones after them.
@@ -1247,9 +1252,14 @@ struct SegmentWalk {
     }
 };
 
-// A tile cut between groups is summed from partial tiles in contraction order by whichever of its
-// warps finishes last (the order of the sum, not of the arrivals, decides the bits), so no pair ever
-// waits for another.
+// A tile cut between groups is summed from partial tiles in contraction order (the order of the sum, not of the
+// arrivals, decides the bits).  The last warp to finish a share sees that all are in memory and sums them; warps
+// that finished theirs before, and have no other work, are still there as a rule and draw pieces of the sum as well.
+// Nobody depends on them: a warp that has waited SUM_WAIT_NS leaves, and what has not been drawn is left to the last.
+// (One rank's dQ of 512 x 8192 x 768, 10 shares to a tile: the last warp alone spent up to 15 K cycles on its 32 x 64
+// sums, the warps together 6-8 K; one rank of eight of 4096 x 8192 x 768 71.7 -> 67.5 us.)
+constexpr uint64_t SUM_WAIT_NS = 20000;
+constexpr int SUM_TAKEN = 0x8000;             // the last warp sums from tensor memory
 //
 // F32: weights as two terms, rows of the other side as three; products w1 (t1 + t2 + t3) +
 // w2 (t1 + t2), 256 x 128 tiles.  The tensor core's additions truncate: every 128 of the contraction
@@ -1275,7 +1285,6 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
     constexpr int NACC = F32 ? 4 : 2;                     // accumulators in tensor memory
     const int pair = blockIdx.x >> 1;
     dep_release();
-    dep_wait();
     // columns of a tile that exist, in whole 128s: a last tile of at most 128 columns runs at half width
     auto tile_width = [&](const GradSide& sd, int n0) { return WIDTH == 256 && sd.cols - n0 <= 128 ? 128 : WIDTH; };
 
@@ -1284,9 +1293,14 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
         int stage = 0;
         uint32_t phase = 0;
         bool ok = true;
+        // (The divisions of the first segment run under the kernel before.  Every role has a walk of its own: one made
+        // before the roles part takes the operands of loads and products out of the uniform registers, 4096 x 8192 x
+        // 768 5 us a build.)
         SegmentWalk walk(p, pair);
         Segment sg;
-        while (ok && walk.next(p, sg)) {
+        bool more = walk.next(p, sg);
+        dep_wait();
+        for (; ok && more; more = walk.next(p, sg)) {
             const GradSide& sd = p.side[sg.side];
             const int m0 = sg.tile_m * 256 + (int)c.rank * 128;
             const int n0t = sg.tile_n * WIDTH;
@@ -1392,6 +1406,10 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
         constexpr size_t PART_FLOATS = 32 * HW;
         int use = 0, nstore = 0;
         bool ok = true;
+        SegmentWalk walk(p, pair);
+        Segment sg, nx;
+        bool more = walk.next(p, nx);
+        dep_wait();
         if (p.terms && blockIdx.x == 0) {
             // the loss: a fixed order of sums, under the first products
             __shared__ float sums[NSOFT];
@@ -1407,9 +1425,9 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
                 *p.loss = v * p.inv_mean;
             }
         }
-        SegmentWalk walk(p, pair);
-        Segment sg;
-        while (ok && walk.next(p, sg)) {
+        for (bool any = more; ok && any; any = more) {
+            sg = nx;
+            more = walk.next(p, nx);                      // false: sg is the pair's last
             const GradSide& sd = p.side[sg.side];
             const int row0 = sg.tile_m * 256 + (int)c.rank * 128 + 32 * q;
             const int n0 = sg.tile_n * WIDTH;
@@ -1417,11 +1435,38 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
             const int col0 = n0 + half * hw;
             const bool whole = sg.n == sd.kblocks;
             const uint32_t lanes = (uint32_t)(32 * q) << 16;
+            // What the positives' weights lost is r_i times the positive's passage.  A lane reads 8 columns of row
+            // 8 k + lane / 4 of those (a lane per row, 32 cache lines to a load, held up a tile's epilogue by
+            // 7 K cycles), two blocks ahead of their use and the first two before the products are waited for.
             float r_i = 0.f;
-            const __nv_bfloat16* p_row = nullptr;
+            int pos_i = -1;
             if (!F32 && sg.side == 0 && p.res && row0 + lane < sd.rows) {
                 r_i = p.res[row0 + lane];
-                if (r_i != 0.f) p_row = p.P + (int64_t)p.pos_idx[row0 + lane] * p.ldp;
+                if (r_i != 0.f) pos_i = p.pos_idx[row0 + lane];
+            }
+            const bool fix = !F32 && __any_sync(0xffffffffu, pos_i >= 0);
+            uint4 px[F32 ? 1 : 8];
+            auto fetch_p = [&](int cb) {
+                if (F32 || !fix) return;
+                const int col = col0 + 32 * cb + 8 * (lane & 3);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int pos = __shfl_sync(0xffffffffu, pos_i, 8 * k + (lane >> 2));
+                    px[F32 ? 0 : 4 * (cb & 1) + k] = pos >= 0 && col < sd.cols
+                        ? *reinterpret_cast<const uint4*>(p.P + (int64_t)pos * p.ldp + col) : make_uint4(0, 0, 0, 0);
+                }
+            };
+            // first and last group with a share of this tile, and the tile's counter
+            const int group = walk.group, tn = sd.tiles_n;
+            int gf = group, gl = group, published = 0;
+            int* counter = p.count + ((sg.side ? p.side[0].tiles : 0) + sg.tile_m * tn + sg.tile_n) * 16 + cw;
+            if (!whole) {
+                const int t1 = sg.t0 + sd.kblocks;
+                while (unit_start(p, gf) > sg.t0) --gf;
+                while (unit_start(p, gl + 1) < t1) ++gl;
+            } else {
+                fetch_p(0);
+                fetch_p(1);                               // (a tile has at least two blocks of 32 columns per warp)
             }
             float acc[F32 ? HW : 1];
             if (F32) {
@@ -1456,98 +1501,164 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
                 tc_fence_after();
             }
             const uint32_t src = c.tmem + (use % NACC) * (TMEM_COLS / NACC) + lanes + half * hw;
-            // one block of 32 columns to the output: scale, the positives' remainder, staging, store
-            auto finish = [&](uint32_t (&v)[32], int cb) {
-                const int col = col0 + 32 * cb;
-                if (!F32 && p_row) {
-                    const uint4* pr = reinterpret_cast<const uint4*>(p_row + col);
+            auto own_block = [&](int cb, uint32_t (&v)[32]) {
+                if (F32) {
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        if (col + 8 * j >= sd.cols) break;
-                        const uint4 x = pr[j];
-                        const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+                    for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(acc[F32 ? 32 * cb + e : 0]);
+                } else {
+                    tmem_ld32(src + 32 * cb, v);
+                    tmem_ld_wait();
+                }
+            };
+            auto release_acc = [&]() {
+                if (F32) return;
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&bars.acc_free[use % NACC]));
+            };
+            // The passages from there to lane = row, through 2 KB of shared memory: 64 bytes to a row, 16-byte chunks
+            // swizzled against conflicts.
+            auto spread_p = [&](uint32_t box, int cb) {
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            v[8 * j + 2 * e] = __float_as_uint(fmaf(
-                                r_i, __uint_as_float(w[e] << 16), __uint_as_float(v[8 * j + 2 * e])));
-                            v[8 * j + 2 * e + 1] = __float_as_uint(fmaf(
-                                r_i, __uint_as_float(w[e] & 0xffff0000u), __uint_as_float(v[8 * j + 2 * e + 1])));
-                        }
+                for (int k = 0; k < 4; ++k) {
+                    const int r = 8 * k + (lane >> 2);
+                    const uint4 x = px[F32 ? 0 : 4 * (cb & 1) + k];
+                    sts_v4(box + r * 64 + (((lane & 3) ^ (r >> 1 & 3)) << 4), x.x, x.y, x.z, x.w);
+                }
+            };
+            auto add_p = [&](uint32_t box, uint32_t (&v)[32]) {
+                if (pos_i < 0) return;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    uint32_t w[4];
+                    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3])
+                                 : "r"(box + lane * 64 + ((j ^ (lane >> 1 & 3)) << 4)) : "memory");
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        v[8 * j + 2 * e] = __float_as_uint(fmaf(
+                            r_i, __uint_as_float(w[e] << 16), __uint_as_float(v[8 * j + 2 * e])));
+                        v[8 * j + 2 * e + 1] = __float_as_uint(fmaf(
+                            r_i, __uint_as_float(w[e] & 0xffff0000u), __uint_as_float(v[8 * j + 2 * e + 1])));
                     }
                 }
+            };
+            auto store = [&](uint32_t buf, int cb) {     // (an empty group when nothing is stored)
+                const int col = col0 + 32 * cb;
+                const CUtensorMap* map = sg.side == 0 ? &mapDQ : &mapDP;
+                if (row0 >= sd.rows || col >= sd.cols)
+                    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                else if (sd.add) tma_add_3d(map, buf, col, row0, 0);
+                else             tma_store_3d(map, buf, col, row0, 0);
+            };
+            // one block of 32 columns to the output: the positives' remainder, scale, staging, store
+            auto finish = [&](uint32_t (&v)[32], int cb) {
                 if (lane == 0) asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(SB - 1) : "memory");
                 __syncwarp();
                 const uint32_t buf = stage_buf + (uint32_t)(nstore & (SB - 1)) * 4096u;
+                ++nstore;
+                if (!F32 && fix) {
+                    spread_p(buf, cb);
+                    __syncwarp();
+                    add_p(buf, v);
+                    __syncwarp();
+                }
                 stage_block(buf, v, p.scale, lane);
                 __syncwarp();
-                if (lane == 0) {                         // (an empty group when nothing is stored)
-                    const CUtensorMap* map = sg.side == 0 ? &mapDQ : &mapDP;
-                    if (row0 >= sd.rows || col >= sd.cols)
-                        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-                    else if (sd.add) tma_add_3d(map, buf, col, row0, 0);
-                    else             tma_store_3d(map, buf, col, row0, 0);
-                }
-                ++nstore;
+                if (lane == 0) store(buf, cb);
             };
-            if (whole) {
+            // group g's share of the tile: slot 0 when its run starts inside the tile, else 1
+            auto part_of = [&](int g, int slot) {
+                return reinterpret_cast<float4*>(
+                    p.part + (((size_t)(g * tn + sg.tile_n) * 2 + slot) * 16 + cw) * PART_FLOATS);
+            };
+            if (whole && !more) {
+                // The pair's last tile: nothing uses the ring any more, so that every block has a buffer of its own there.
+                // (4096 x 4096 x 512, both gradients, one tile to a pair: from the last product to the last store 7.8 K
+                // cycles for dQ, 6.5 K for dP, as long as 16 MB take into the L2; block after block through one buffer,
+                // with a lane per row of the passages, 12 K and 5-7 K.)
+                const uint32_t buf = c.smem + (uint32_t)ew * (HW / 32 * 4096u);
+                const uint32_t box = c.smem + NSOFT * (HW / 32 * 4096u) + (uint32_t)ew * (HW / 32 * 2048u);
+                if (!F32 && fix) {
+#pragma unroll
+                    for (int cb = 0; cb < HW / 32; ++cb) {
+                        if (32 * cb >= hw) break;
+                        spread_p(box + cb * 2048u, cb);
+                        if (cb + 2 < HW / 32 && 32 * (cb + 2) < hw) fetch_p(cb + 2);
+                    }
+                    __syncwarp();
+                }
 #pragma unroll
                 for (int cb = 0; cb < HW / 32; ++cb) {
                     if (32 * cb >= hw) break;
                     uint32_t v[32];
-                    if (F32) {
+                    own_block(cb, v);
+                    if (!F32 && fix) add_p(box + cb * 2048u, v);
+                    stage_block_unfenced(buf + cb * 4096u, v, p.scale, lane);
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0)
+                    for (int cb = 0; 32 * cb < hw; ++cb) store(buf + cb * 4096u, cb);
+            } else if (whole) {
 #pragma unroll
-                        for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(acc[F32 ? 32 * cb + e : 0]);
-                    } else {
-                        tmem_ld32(src + 32 * cb, v);
-                        tmem_ld_wait();
-                        if (32 * (cb + 1) >= hw) {
-                            tc_fence_before();
-                            __syncwarp();
-                            if (lane == 0) mbar_arrive(smem_u32(&bars.acc_free[use % NACC]));
-                        }
-                    }
+                for (int cb = 0; cb < HW / 32; ++cb) {
+                    if (32 * cb >= hw) break;
+                    uint32_t v[32];
+                    own_block(cb, v);
+                    if (32 * (cb + 1) >= hw) release_acc();
                     finish(v, cb);
+                    if (cb + 2 < HW / 32 && 32 * (cb + 2) < hw) fetch_p(cb + 2);
                 }
             } else {
-                // this group's share of the tile: slot 0 when it starts inside the tile, else 1
-                const int group = walk.group, tn = sd.tiles_n;
-                auto part_of = [&](int g, int slot) {
-                    return reinterpret_cast<float4*>(
-                        p.part + (((size_t)(g * tn + sg.tile_n) * 2 + slot) * 16 + cw) * PART_FLOATS);
-                };
-                // first and last group with a share of this tile
-                const int t1 = sg.t0 + sd.kblocks;
-                int gf = group, gl = group;
-                while (unit_start(p, gf) > sg.t0) --gf;
-                while (unit_start(p, gl + 1) < t1) ++gl;
-                const int tile_id = (sg.side ? p.side[0].tiles : 0) + sg.tile_m * tn + sg.tile_n;
-                int* counter = p.count + tile_id * 16 + cw;
-                auto own_block = [&](int cb, uint32_t (&v)[32]) {
-                    if (F32) {
-#pragma unroll
-                        for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(acc[F32 ? 32 * cb + e : 0]);
-                    } else {
-                        tmem_ld32(src + 32 * cb, v);
-                        tmem_ld_wait();
-                    }
-                };
-                auto release_acc = [&]() {
-                    if (F32) return;
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(smem_u32(&bars.acc_free[use % NACC]));
-                };
-                // Where all other shares are in memory already (as a rule: a group meets the front part
+                // Where all other shares (of a few) are in memory already (as a rule: a group meets the front part
                 // of its first tile long before the neighbour meets the back part of its last), this
-                // share goes into the sum straight from tensor memory.  (Not from the registers of the fp32 sums: the
-                // two sums at once do not fit, and with the running one in local memory a read-out took 4 K cycles
-                // where its products take 2.6 K: 2048 x 4096 x 768, 239 us a build against 199.)
-                int published = 0;
-                if (!F32 && lane == 0)
-                    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(published) : "l"(counter) : "memory");
-                published = __shfl_sync(0xffffffffu, published, 0);
-                const bool direct = !F32 && published == gl - gf;
-                if (!direct) {
+                // share goes into the sum straight from tensor memory, and whoever waits need not.  (Not from the
+                // registers of the fp32 sums: the two sums at once do not fit, and with the running one in local memory a
+                // read-out took 4 K cycles where its products take 2.6 K: 2048 x 4096 x 768, 239 us a build against 199.)
+                bool direct = false;
+                if (!F32 && gl - gf < 3) {
+                    if (lane == 0) {
+                        asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(published) : "l"(counter) : "memory");
+                        if (published == gl - gf) atomicAdd(counter, SUM_TAKEN);
+                    }
+                    direct = __shfl_sync(0xffffffffu, published, 0) == gl - gf;
+                }
+                if (direct) {
+                    __threadfence();
+#pragma unroll
+                    for (int cb = 0; cb < HW / 32; ++cb) {
+                        if (32 * cb >= hw) break;
+                        uint32_t v[32];
+                        own_block(cb, v);
+                        float s[32];
+                        for (int g = gf; g <= gl; ++g) {
+                            if (g == group) {
+#pragma unroll
+                                for (int e = 0; e < 32; ++e)
+                                    s[e] = g == gf ? __uint_as_float(v[e]) : s[e] + __uint_as_float(v[e]);
+                                continue;
+                            }
+                            const float4* o = part_of(g, g == gf ? 1 : 0);
+#pragma unroll
+                            for (int j0 = 0; j0 < 8; j0 += 4) {
+                                float4 x[4];
+#pragma unroll
+                                for (int j = 0; j < 4; ++j) x[j] = __ldcg(o + (cb * 8 + j0 + j) * 32 + lane);
+#pragma unroll
+                                for (int j = 0; j < 4; ++j) {
+                                    float* t = s + 4 * (j0 + j);
+                                    if (g == gf) { t[0] = x[j].x; t[1] = x[j].y; t[2] = x[j].z; t[3] = x[j].w; }
+                                    else         { t[0] += x[j].x; t[1] += x[j].y; t[2] += x[j].z; t[3] += x[j].w; }
+                                }
+                            }
+                        }
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(s[e]);
+                        fetch_p(cb);
+                        finish(v, cb);
+                    }
+                    release_acc();
+                } else {
                     float4* mine = part_of(group, sg.kb == 0 ? 1 : 0);
 #pragma unroll
                     for (int cb = 0; cb < HW / 32; ++cb) {
@@ -1563,44 +1674,87 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
                     release_acc();
                     __threadfence();
                     __syncwarp();
-                    if (lane == 0) published = atomicAdd(counter, 1);
-                    published = __shfl_sync(0xffffffffu, published, 0);
-                }
-                if (published == gl - gf) {
-                    __threadfence();
+                    // A share is in memory: one more in the counter's lower half.  A warp with nothing left to do waits
+                    // a little for the others, so that they sum the tile together; it need not (see SUM_WAIT_NS).
+                    int complete = 0;
+                    if (lane == 0) {
+                        complete = (atomicAdd(counter, 1) & 0xffff) == gl - gf;
+                        if (!complete && !more) {
+                            const uint64_t t0 = global_ns();
+                            do {
+                                asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(published) : "l"(counter) : "memory");
+                                complete = (published & 0xffff) == gl - gf + 1;
+                            } while (!complete && !(published & SUM_TAKEN) && global_ns() - t0 < SUM_WAIT_NS);
+                        }
+                    }
+                    if (__shfl_sync(0xffffffffu, complete, 0)) {
+                        __threadfence();
+                        const int row = row0 + lane;
+                        float* out_row = p.out[sg.side] + (int64_t)row * p.ldo[sg.side];
+                        // pieces of 4 NJ columns, drawn from the counter's upper half; PB shares' loads in flight
+                        auto sum_pieces = [&](auto nj) {
+                            constexpr int NJ = decltype(nj)::value, PB = (F32 ? 8 : 12) / NJ;
+                            auto draw = [&]() { return lane == 0 ? atomicAdd(counter, 0x10000) >> 16 : 0; };
+                            const int pieces = hw / (4 * NJ);
+                            int drawn = draw();
+                            for (;;) {
+                                const int piece = __shfl_sync(0xffffffffu, drawn, 0);
+                                if (piece >= pieces) break;
+                                float4 s[NJ];
+                                uint2 pw[NJ];            // the positive's passage
 #pragma unroll
-                    for (int cb = 0; cb < HW / 32; ++cb) {
-                        if (32 * cb >= hw) break;
-                        uint32_t v[32];
-                        if (direct) own_block(cb, v);
-                        float s[32];
-                        for (int g = gf; g <= gl; ++g) {
-                            if (direct && g == group) {
+                                for (int j = 0; j < NJ; ++j) {
+                                    const int col = col0 + 4 * (piece * NJ + j);
+                                    if (!F32 && pos_i >= 0 && col < sd.cols)
+                                        pw[j] = *reinterpret_cast<const uint2*>(p.P + (int64_t)pos_i * p.ldp + col);
+                                    s[j] = make_float4(-0.f, -0.f, -0.f, -0.f);
+                                }
+#pragma unroll 1
+                                for (int g0 = gf; g0 <= gl; g0 += PB) {
+                                    float4 x[PB][NJ];
 #pragma unroll
-                                for (int e = 0; e < 32; ++e)
-                                    s[e] = g == gf ? __uint_as_float(v[e]) : s[e] + __uint_as_float(v[e]);
-                                continue;
-                            }
-                            const float4* o = part_of(g, g == gf ? 1 : 0);
-                            float4 x[8];
+                                    for (int b = 0; b < PB; ++b) {
+                                        const int g = min(g0 + b, gl);
+                                        const float4* o = part_of(g, g == gf ? 1 : 0) + piece * NJ * 32 + lane;
 #pragma unroll
-                            for (int j = 0; j < 8; ++j) x[j] = __ldcg(o + (cb * 8 + j) * 32 + lane);
+                                        for (int j = 0; j < NJ; ++j) x[b][j] = __ldcg(o + j * 32);
+                                    }
+                                    if (g0 == gf) drawn = draw();
 #pragma unroll
-                            for (int j = 0; j < 8; ++j) {
-                                if (g == gf) {
-                                    s[4 * j] = x[j].x; s[4 * j + 1] = x[j].y;
-                                    s[4 * j + 2] = x[j].z; s[4 * j + 3] = x[j].w;
-                                } else {
-                                    s[4 * j] += x[j].x; s[4 * j + 1] += x[j].y;
-                                    s[4 * j + 2] += x[j].z; s[4 * j + 3] += x[j].w;
+                                    for (int b = 0; b < PB; ++b) {
+                                        if (g0 + b <= gl) {
+#pragma unroll
+                                            for (int j = 0; j < NJ; ++j) {
+                                                s[j].x += x[b][j].x; s[j].y += x[b][j].y;
+                                                s[j].z += x[b][j].z; s[j].w += x[b][j].w;
+                                            }
+                                        }
+                                    }
+                                }
+#pragma unroll
+                                for (int j = 0; j < NJ; ++j) {
+                                    const int col = col0 + 4 * (piece * NJ + j);
+                                    if (row >= sd.rows || col >= sd.cols) continue;
+                                    if (!F32 && pos_i >= 0) {
+                                        s[j].x = fmaf(r_i, __uint_as_float(pw[j].x << 16), s[j].x);
+                                        s[j].y = fmaf(r_i, __uint_as_float(pw[j].x & 0xffff0000u), s[j].y);
+                                        s[j].z = fmaf(r_i, __uint_as_float(pw[j].y << 16), s[j].z);
+                                        s[j].w = fmaf(r_i, __uint_as_float(pw[j].y & 0xffff0000u), s[j].w);
+                                    }
+                                    float4 r = make_float4(s[j].x * p.scale, s[j].y * p.scale, s[j].z * p.scale, s[j].w * p.scale);
+                                    float4* dst = reinterpret_cast<float4*>(out_row + col);
+                                    if (sd.add) {
+                                        const float4 o = *dst;
+                                        r = make_float4(__fadd_rn(o.x, r.x), __fadd_rn(o.y, r.y), __fadd_rn(o.z, r.z),
+                                                        __fadd_rn(o.w, r.w));
+                                    }
+                                    *dst = r;
                                 }
                             }
-                        }
-#pragma unroll
-                        for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(s[e]);
-                        finish(v, cb);
+                        };
+                        if (gl - gf < 7) sum_pieces(std::integral_constant<int, 4>{});
+                        else             sum_pieces(std::integral_constant<int, 2>{});
                     }
-                    if (direct) release_acc();
                 }
             }
             if (!F32) ++use;
@@ -1970,6 +2124,8 @@ struct StripRun {
             gp.loss = loss;
             gp.inv_mean = 1.f / (float)(p.b_total > 0 ? p.b_total : p.B);
         }
+        gp.out[0] = dQ ? dQ + row0 * lddq : nullptr; gp.ldo[0] = lddq;
+        gp.out[1] = dP; gp.ldo[1] = lddp;
         gp.part = at<float>(l.part);
         gp.count = at<int>(l.zero) + 64;
         gp.dev_status = dev_status;

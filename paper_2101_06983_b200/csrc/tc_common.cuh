@@ -275,8 +275,7 @@ __device__ __forceinline__ void tmem_st_wait() {
 // swizzle the tensor map expects (16-byte chunk j of row r at chunk j ^ (r & 7)), which also
 // makes the float4 stores conflict-free, and then leaves with one bulk tensor store; rows past
 // the end of the matrix are clipped by the tensor map.
-__device__ __forceinline__ void stage_block(uint32_t buf, const uint32_t (&v)[32], float sc,
-                                            int lane) {
+__device__ __forceinline__ void stage_block_unfenced(uint32_t buf, const uint32_t (&v)[32], float sc, int lane) {
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
         const uint32_t addr = buf + lane * 128 + ((j ^ (lane & 7)) << 4);
@@ -287,6 +286,10 @@ __device__ __forceinline__ void stage_block(uint32_t buf, const uint32_t (&v)[32
                        "f"(__uint_as_float(v[4 * j + 3]) * sc)
                      : "memory");
     }
+}
+__device__ __forceinline__ void stage_block(uint32_t buf, const uint32_t (&v)[32], float sc,
+                                            int lane) {
+    stage_block_unfenced(buf, v, sc, lane);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // visible to the bulk store
 }
 __device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, uint32_t src, int c0, int c1,

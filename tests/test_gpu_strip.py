@@ -310,3 +310,26 @@ def test_two_directions_over_several_strips(binding):
     assert abs(loss.item() - want) <= tol["loss"] * abs(want)
     assert grad_err(dQ.cpu().numpy(), rQ.cpu().numpy()) <= tol["grad"]
     assert grad_err(dP.cpu().numpy(), rP.cpu().numpy()) <= tol["grad"]
+
+
+@pytest.mark.parametrize("B,N,d,dtype", [(512, 8192, 768, "bf16"), (300, 9000, 200, "bf16"), (40, 16500, 72, "f32"),
+                                         (2100, 260, 136, "f32")])
+def test_sums_of_cut_gradient_tiles(binding, oracle, B, N, d, dtype):
+    """One gradient alone over a long contraction: tiles in up to dozens of shares, summed in pieces by whoever is
+    there; ragged last rows and columns; the same bits in every run."""
+    prob = inputs.random_problem(B, N, d, dtype, seed=B + N + d, tau=0.5, scale=d ** -0.5)
+    ref = _oracle_full(oracle, prob)
+    Q, P, pos = to_device(prob)
+    b = binding.Outputs(B, N, d, binding._dtype_code(Q))
+    args = (Q, P, pos, prob.tau, prob.mask_mode)
+    binding.gc_loss_fwd(*args, b.loss, b.row_lse, b.pos_logit, b.ws, b.dev_status)
+    binding.gc_loss_bwd(*args, b.row_lse, b.dQ, None, b.ws, b.dev_status)
+    binding.gc_loss_bwd(*args, b.row_lse, None, b.dP, b.ws, b.dev_status)
+    torch.cuda.synchronize()
+    check_against_oracle(prob, b, ref)
+    first = b.dQ.clone(), b.dP.clone()
+    for _ in range(20):
+        b.dQ.fill_(float("nan")), b.dP.fill_(float("nan"))
+        binding.gc_loss_bwd(*args, b.row_lse, b.dQ, None, b.ws, b.dev_status)
+        binding.gc_loss_bwd(*args, b.row_lse, None, b.dP, b.ws, b.dev_status)
+        assert torch.equal(b.dQ, first[0]) and torch.equal(b.dP, first[1])
