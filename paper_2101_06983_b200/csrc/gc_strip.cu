@@ -1836,12 +1836,16 @@ GradDeal deal_grads(int64_t rows, int64_t N, int d, bool f32, bool dq, bool dp) 
     for (int width = f32 ? 128 : 256; width >= 128; width -= 128) {
         const int tn = (int)ceil_div(d, width);
         // Cycles per contraction block; what cutting tiles costs by itself; and per part of a tile, whose
-        // sums its last pair adds up one after the other (dQ alone of 512 x 8192 x 64: 64 runs 49 us, 12 runs
-        // 28).  Fitted to 258 shapes (150 to 16384 queries, 64 to 1024 columns, one gradient or both) with
-        // every choice forced: the choice this makes is within 7 % of the best at each, 0.3 % on average.
-        const double unit = f32 ? 1320 : width == 256 ? 560 : 364;
-        const double cut = f32 ? 6300 : width == 256 ? 18000 : 8800;
-        const double part = f32 ? 970 : width == 256 ? 3080 : 1580;
+        // sums are added up one after the other.  Fitted to 54 shapes (34 to 12000 queries, 256 to 1024 columns, one
+        // gradient or both) with 4 to 16 choices forced at each: the choice this makes is within 8 % of the best at
+        // each, 0.4 % on average (us, longer runs before / now: dQ of 2048 x 16384 x 768 106 / 93, dP of 8192 x 2048 x
+        // 768 60.5 / 57.0, of 2632 x 658 x 640 29.4 / 25.8).
+        const double unit = f32 ? 1390 : width == 256 ? 560 : 370;
+        const double cut = width == 256 ? 7800 : 8000;
+        const double part = width == 256 ? 820 : 580;
+        // the shares' traffic under long runs: both gradients of 4096 x 8192 x 1024, whole tiles (192 to 256 blocks to a
+        // pair) 243.6 us with the loss, equal runs (228) 248.7
+        const double along = f32 ? 0 : 0.1;
         // A pair's next tile takes at least the epilogue of this one (dQ's adds what the positives' weights lost):
         // tiles of few contraction blocks are bound by it.  4671 x 30 x 128, both gradients: 18 dQ tiles of one
         // block to a pair 71 us, 19 pairs for them 14; 7 x 9470 x 128: 26 dP tiles of one block to a pair 44 us.
@@ -1876,7 +1880,7 @@ GradDeal deal_grads(int64_t rows, int64_t N, int d, bool f32, bool dq, bool dp) 
         double cost = run * unit;
         if (tq && run > kq && run / kq * epi_q > cost) cost = run / kq * epi_q;
         if (tp && run > kp && run / kp * epi_p > cost) cost = run / kp * epi_p;
-        offer(cost + cut + part * longest * groups / units, -1, groups * tn);
+        offer(cost + cut + along * run * unit + part * longest * groups / units, -1, groups * tn);
     }
     return best;
 }
