@@ -1743,7 +1743,7 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
                                     }
                                     float4 r = make_float4(s[j].x * p.scale, s[j].y * p.scale, s[j].z * p.scale, s[j].w * p.scale);
                                     float4* dst = reinterpret_cast<float4*>(out_row + col);
-                                    if (sd.add) {
+                                    if (sd.add) {         // rounds as bulk reductions do: neither flushes subnormals
                                         const float4 o = *dst;
                                         r = make_float4(__fadd_rn(o.x, r.x), __fadd_rn(o.y, r.y), __fadd_rn(o.z, r.z),
                                                         __fadd_rn(o.w, r.w));

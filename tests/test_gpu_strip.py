@@ -333,3 +333,29 @@ def test_sums_of_cut_gradient_tiles(binding, oracle, B, N, d, dtype):
         binding.gc_loss_bwd(*args, b.row_lse, b.dQ, None, b.ws, b.dev_status)
         binding.gc_loss_bwd(*args, b.row_lse, None, b.dP, b.ws, b.dev_status)
         assert torch.equal(b.dQ, first[0]) and torch.equal(b.dP, first[1])
+
+
+@pytest.mark.parametrize("B,N,d,dtype,lse2,tau2", [(32768, 25000, 448, "bf16", 15, 112), (32768, 25000, 1024, "bf16", 15, 112),
+                                                   (8192, 8250, 136, "f32", 13, 114)])
+def test_subnormal_gradients_of_a_second_strip(binding, B, N, d, dtype, lse2, tau2):
+    """Weights of 2^-lse2 (2^-lse2 - 1 at the positives, in bf16 rounded to -1), rows of +-2^-6 and a temperature of
+    2^tau2: every entry of dP is a sum of subnormal numbers, exact but for that rounding.  The second strip adds to
+    the first through a bulk reduction or, where a cut tile is summed in pieces, in registers: the same sums."""
+    g = torch.Generator(device="cuda").manual_seed(B + d)
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    Q, P = ((torch.randint(0, 2, (n, d), generator=g, device="cuda") * 2.0 ** -5 - 2.0 ** -6).to(dt) for n in (B, N))
+    pos = torch.randint(0, N, (B,), generator=g, device="cuda").int()
+    code = binding._dtype_code(Q)
+    assert binding.gc_kernel_launches(binding.GC_OP_BWD, B, N, d, code) == (4 if dtype == "bf16" else 1 + 2 * 3)
+    o = binding.Outputs(B, N, d, code)
+    o.row_lse.fill_(lse2 * float(np.log(2.0)))
+    want = Q.double().sum(0).mul(2.0 ** -lse2).repeat(N, 1).index_add_(0, pos.long(), Q.double(), alpha=-1.0)
+    want = want * 2.0 ** -tau2 / B
+    assert float(want.abs().max()) < 2.0 ** -127
+    for dQ in (o.dQ, None):
+        for _ in range(5):
+            o.dP.fill_(float("nan"))
+            binding.gc_loss_bwd(Q, P, pos, 2.0 ** tau2, 0, o.row_lse, dQ, o.dP, o.ws, o.dev_status)
+            err = (o.dP.double() - want).abs().max()      # up to 15 positives to a passage, 2^-149 per strip's sum
+            assert float(err) <= 2.0 ** -lse2 * float(want.abs().max()) + 2 * 2.0 ** -149
+    assert int(o.dev_status.item()) == 0
