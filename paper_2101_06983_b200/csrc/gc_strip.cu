@@ -1179,6 +1179,8 @@ struct GradParams {
     float* part;                  // [pairs][2 slots][2 CTAs][8 warps][32 x hw] partial tiles
     int* count;                   // [tiles of both sides][2 CTAs][8 warps]: shares in memory, and pieces of
                                   // their sum drawn << 16
+    int* started;                 // pairs that have started, over the strips of the call, and how many of them when
+    int all_started;              // all of this launch have (cut runs only)
     int* dev_status;
 };
 
@@ -1252,18 +1254,24 @@ struct SegmentWalk {
     }
 };
 
+// A warp that has nothing left to do waits so long for the other shares of its last tile, if every pair of the launch
+// has started.  Measured on an idle device, over 19 shapes: nearly all waits end within 3 us, the longest after 6.
+constexpr uint64_t SUM_WAIT_NS = 10000;
+constexpr int SUM_TAKEN = 0x8000;             // the last warp sums from tensor memory
+
 // A tile cut between groups is summed from partial tiles in contraction order (the order of the sum, not of the
 // arrivals, decides the bits).  The last warp to finish a share sees that all are in memory and sums them; warps
 // that finished theirs before, and have no other work, are still there as a rule and draw pieces of the sum as well.
-// Nobody depends on them: a warp that has waited SUM_WAIT_NS leaves, and what has not been drawn is left to the last.
+// Nobody depends on them: they leave after SUM_WAIT_NS, and at once while pairs of this launch have yet to start, which
+// may need the room they hold; what has not been drawn is left to the last.
 // (One rank's dQ of 512 x 8192 x 768, 10 shares to a tile: the last warp alone spent up to 15 K cycles on its 32 x 64
-// sums, the warps together 6-8 K; one rank of eight of 4096 x 8192 x 768 71.7 -> 67.5 us.)
-constexpr uint64_t SUM_WAIT_NS = 20000;
-constexpr int SUM_TAKEN = 0x8000;             // the last warp sums from tensor memory
+// sums, the warps together 6-8 K; one rank of eight of 4096 x 8192 x 768 71.7 -> 67.5 us.  dQ of 256 x 16384 x 768 with
+// 20 SMs held by another stream: 76 us with waits of up to 20 us for pairs that could not start, 56 without them; 28
+// on a free device; two streams of it at once 53 and 50 a pair of calls.)
 //
 // F32: weights as two terms, rows of the other side as three; products w1 (t1 + t2 + t3) +
 // w2 (t1 + t2), 256 x 128 tiles.  The tensor core's additions truncate: every 128 of the contraction
-// the accumulator is read out and added in fp32 registers, the other buffer taking over meanwhile.
+// the accumulator is read out and added in fp32 registers, the next of the four taking over meanwhile.
 template <bool F32, int WIDTH>
 __global__ void __launch_bounds__(ST_THREADS, 1)
 strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_constant__ CUtensorMap mapWm,
@@ -1410,6 +1418,7 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
         Segment sg, nx;
         bool more = walk.next(p, nx);
         dep_wait();
+        if (p.whole < 0 && ew == 0 && c.rank == 0 && lane == 0) atomicAdd(p.started, 1);
         if (p.terms && blockIdx.x == 0) {
             // the loss: a fixed order of sums, under the first products
             __shared__ float sums[NSOFT];
@@ -1675,11 +1684,11 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
                     __threadfence();
                     __syncwarp();
                     // A share is in memory: one more in the counter's lower half.  A warp with nothing left to do waits
-                    // a little for the others, so that they sum the tile together; it need not (see SUM_WAIT_NS).
+                    // for the others if they are all at work, so that they sum the tile together (see SUM_WAIT_NS).
                     int complete = 0;
                     if (lane == 0) {
                         complete = (atomicAdd(counter, 1) & 0xffff) == gl - gf;
-                        if (!complete && !more) {
+                        if (!complete && !more && *reinterpret_cast<volatile int*>(p.started) == p.all_started) {
                             const uint64_t t0 = global_ns();
                             do {
                                 asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(published) : "l"(counter) : "memory");
@@ -1922,7 +1931,7 @@ StripLayout strip_layout(int64_t B, int64_t N, int d, int dtype, bool fwd_only =
     const int64_t tiles = ceil_div(l.rows, 256) * ceil_div(d, 128) + ceil_div(N, 256) * ceil_div(d, 128);
     size_t off = 0;
     const size_t counters = fwd_only ? 0 : (size_t)tiles * 16;
-    l.zero = off;  off += up256(sizeof(int) * (64 + counters));
+    l.zero = off;  off += up256(sizeof(int) * (64 + counters));     // word 0: ticket of the loss, 32: pairs started
     l.pos = off;   off += up256(sizeof(float) * (size_t)l.rows);
     l.red = off;   off += up256(sizeof(float) * (size_t)(B + 8 * sm_count()));
     if (!f32) {
@@ -1953,6 +1962,7 @@ struct StripRun {
     const float* col_neg = nullptr;
     const TwoDirection* two = nullptr;
     float grad_scale = 1.f;
+    int started = 0;              // CTA pairs of the gradient launches with cut runs so far
 
     StripRun(const Problem& pr, void* w, int* status, cudaStream_t s, bool fwd_only = false)
         : p(pr), l(strip_layout(pr.B, pr.N, pr.d, pr.dtype, fwd_only)), ws(static_cast<char*>(w)), st(s),
@@ -2132,6 +2142,9 @@ struct StripRun {
         gp.out[1] = dP; gp.ldo[1] = lddp;
         gp.part = at<float>(l.part);
         gp.count = at<int>(l.zero) + 64;
+        if (gp.whole < 0) started += gp.pairs;
+        gp.started = at<int>(l.zero) + 32;
+        gp.all_started = started;
         gp.dev_status = dev_status;
         CUtensorMap wk, wm, mp, mq, mdq, mdp;
         if (!map3(&wk, false, ws + l.w, rows, p.N, l.ldw, planes, rows * l.ldw, 128) ||

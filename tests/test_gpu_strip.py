@@ -359,3 +359,34 @@ def test_subnormal_gradients_of_a_second_strip(binding, B, N, d, dtype, lse2, ta
             err = (o.dP.double() - want).abs().max()      # up to 15 positives to a passage, 2^-149 per strip's sum
             assert float(err) <= 2.0 ** -lse2 * float(want.abs().max()) + 2 * 2.0 ** -149
     assert int(o.dev_status.item()) == 0
+
+
+@pytest.mark.parametrize("B,N,d,side", [(256, 16384, 768, "dQ"), (16384, 256, 768, "dP"), (512, 8192, 448, "dQ")])
+def test_cut_tiles_on_a_busy_device(binding, B, N, d, side):
+    """Two streams with an output and a workspace each: pairs of one launch start when pairs of the other have left.
+    The same bits as alone, and no share that waits for a pair which cannot start."""
+    prob = inputs.random_problem(B, N, d, "bf16", seed=B + N, tau=0.5, scale=d ** -0.5)
+    Q, P, pos = to_device(prob)
+    args = (Q, P, pos, prob.tau, prob.mask_mode)
+    outs = [binding.Outputs(B, N, d, binding.GC_BF16) for _ in range(2)]
+    want = run_build(prob)
+
+    def grad(o):
+        grads = (o.dQ, None) if side == "dQ" else (None, o.dP)
+        binding.gc_loss_bwd(*args, want.row_lse, *grads, o.ws, o.dev_status)
+
+    grad(outs[0])
+    alone = getattr(outs[0], side).clone()
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in outs]
+    for _ in range(5):
+        for o in outs:
+            getattr(o, side).fill_(float("nan"))
+        torch.cuda.synchronize()
+        for _ in range(10):
+            for o, st in zip(outs, streams):
+                with torch.cuda.stream(st):
+                    grad(o)
+        torch.cuda.synchronize()
+        for o in outs:
+            assert torch.equal(getattr(o, side), alone) and int(o.dev_status.item()) == 0
