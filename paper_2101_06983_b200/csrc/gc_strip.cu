@@ -1467,7 +1467,7 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
             };
             // first and last group with a share of this tile, and the tile's counter
             const int group = walk.group, tn = sd.tiles_n;
-            int gf = group, gl = group, published = 0;
+            int gf = group, gl = group;
             int* counter = p.count + ((sg.side ? p.side[0].tiles : 0) + sg.tile_m * tn + sg.tile_n) * 16 + cw;
             if (!whole) {
                 const int t1 = sg.t0 + sd.kblocks;
@@ -1625,6 +1625,7 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
                 // registers of the fp32 sums: the two sums at once do not fit, and with the running one in local memory a
                 // read-out took 4 K cycles where its products take 2.6 K: 2048 x 4096 x 768, 239 us a build against 199.)
                 bool direct = false;
+                int published = 0;
                 if (!F32 && gl - gf < 3) {
                     if (lane == 0) {
                         asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(published) : "l"(counter) : "memory");
@@ -1637,14 +1638,15 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
 #pragma unroll
                     for (int cb = 0; cb < HW / 32; ++cb) {
                         if (32 * cb >= hw) break;
-                        uint32_t v[32];
-                        own_block(cb, v);
                         float s[32];
-                        for (int g = gf; g <= gl; ++g) {
-                            if (g == group) {
 #pragma unroll
-                                for (int e = 0; e < 32; ++e)
-                                    s[e] = g == gf ? __uint_as_float(v[e]) : s[e] + __uint_as_float(v[e]);
+                        for (int e = 0; e < 32; ++e) s[e] = -0.f;
+                        for (int g = gf; g <= gl; ++g) {
+                            if (g == group) {             // (read here: held beside the sums, 300 bytes a thread spilled)
+                                uint32_t v[32];
+                                own_block(cb, v);
+#pragma unroll
+                                for (int e = 0; e < 32; ++e) s[e] += __uint_as_float(v[e]);
                                 continue;
                             }
                             const float4* o = part_of(g, g == gf ? 1 : 0);
@@ -1656,11 +1658,11 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
 #pragma unroll
                                 for (int j = 0; j < 4; ++j) {
                                     float* t = s + 4 * (j0 + j);
-                                    if (g == gf) { t[0] = x[j].x; t[1] = x[j].y; t[2] = x[j].z; t[3] = x[j].w; }
-                                    else         { t[0] += x[j].x; t[1] += x[j].y; t[2] += x[j].z; t[3] += x[j].w; }
+                                    t[0] += x[j].x; t[1] += x[j].y; t[2] += x[j].z; t[3] += x[j].w;
                                 }
                             }
                         }
+                        uint32_t v[32];
 #pragma unroll
                         for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(s[e]);
                         fetch_p(cb);
@@ -1685,7 +1687,7 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
                     __syncwarp();
                     // A share is in memory: one more in the counter's lower half.  A warp with nothing left to do waits
                     // for the others if they are all at work, so that they sum the tile together (see SUM_WAIT_NS).
-                    int complete = 0;
+                    int complete = 0, published = 0;
                     if (lane == 0) {
                         complete = (atomicAdd(counter, 1) & 0xffff) == gl - gf;
                         if (!complete && !more && *reinterpret_cast<volatile int*>(p.started) == p.all_started) {
@@ -1698,8 +1700,6 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
                     }
                     if (__shfl_sync(0xffffffffu, complete, 0)) {
                         __threadfence();
-                        const int row = row0 + lane;
-                        float* out_row = p.out[sg.side] + (int64_t)row * p.ldo[sg.side];
                         // pieces of 4 NJ columns, drawn from the counter's upper half; PB shares' loads in flight
                         auto sum_pieces = [&](auto nj) {
                             constexpr int NJ = decltype(nj)::value, PB = (F32 ? 8 : 12) / NJ;
@@ -1743,7 +1743,7 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
 #pragma unroll
                                 for (int j = 0; j < NJ; ++j) {
                                     const int col = col0 + 4 * (piece * NJ + j);
-                                    if (row >= sd.rows || col >= sd.cols) continue;
+                                    if (row0 + lane >= sd.rows || col >= sd.cols) continue;
                                     if (!F32 && pos_i >= 0) {
                                         s[j].x = fmaf(r_i, __uint_as_float(pw[j].x << 16), s[j].x);
                                         s[j].y = fmaf(r_i, __uint_as_float(pw[j].x & 0xffff0000u), s[j].y);
@@ -1751,7 +1751,8 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
                                         s[j].w = fmaf(r_i, __uint_as_float(pw[j].y & 0xffff0000u), s[j].w);
                                     }
                                     float4 r = make_float4(s[j].x * p.scale, s[j].y * p.scale, s[j].z * p.scale, s[j].w * p.scale);
-                                    float4* dst = reinterpret_cast<float4*>(out_row + col);
+                                    float4* dst = reinterpret_cast<float4*>(
+                                        p.out[sg.side] + (int64_t)(row0 + lane) * p.ldo[sg.side] + col);
                                     if (sd.add) {         // rounds as bulk reductions do: neither flushes subnormals
                                         const float4 o = *dst;
                                         r = make_float4(__fadd_rn(o.x, r.x), __fadd_rn(o.y, r.y), __fadd_rn(o.z, r.z),
