@@ -1846,20 +1846,26 @@ GradDeal deal_grads(int64_t rows, int64_t N, int d, bool f32, bool dq, bool dp) 
     for (int width = f32 ? 128 : 256; width >= 128; width -= 128) {
         const int tn = (int)ceil_div(d, width);
         // Cycles per contraction block; what cutting tiles costs by itself; and per part of a tile, whose
-        // sums are added up one after the other.  Fitted to 54 shapes (34 to 12000 queries, 256 to 1024 columns, one
-        // gradient or both) with 4 to 16 choices forced at each: the choice this makes is within 8 % of the best at
-        // each, 0.4 % on average (us, longer runs before / now: dQ of 2048 x 16384 x 768 106 / 93, dP of 8192 x 2048 x
-        // 768 60.5 / 57.0, of 2632 x 658 x 640 29.4 / 25.8).
-        const double unit = f32 ? 1390 : width == 256 ? 560 : 370;
-        const double cut = width == 256 ? 7800 : 8000;
-        const double part = width == 256 ? 820 : 580;
-        // the shares' traffic under long runs: both gradients of 4096 x 8192 x 1024, whole tiles (192 to 256 blocks to a
-        // pair) 243.6 us with the loss, equal runs (228) 248.7
-        const double along = f32 ? 0 : 0.1;
+        // sums are added up one after the other.  Fitted to 443 bf16 shapes (20 to 24000 queries, 64 to 2048 columns,
+        // one gradient or both) and 129 fp32 shapes (34 to 4096 queries, 64 to 768 columns), with 4 to 25 choices
+        // forced at each.  How much slower the choice this makes is than the best, on average / at worst: ordinary bf16
+        // shapes 0.3 / 6 %, those beyond 4096 x 8192 x 768 0.9 / 14 %, one rank's share of a batch 0.8 / 10 %, one side of
+        // at most 260 rows 3 / 31 %, fp32 0.3 / 6 %.  (us, tiles cut / whole: both gradients of 2952 x 2214 x 512 47.6 /
+        // 35.6, of 4160 x 4160 x 768 87.9 / 77.8, of 12525 x 37575 x 1024 1980 / 2500; dQ of 2048 x 16384 x 768 90 / 109,
+        // of 779 x 3118 x 384 23.8 / 27.2; fp32, 1024 x 2048 x 768 62.0 / 54.9)
+        const bool both = dq && dp;
+        const double unit = f32 ? 1400 : width == 256 ? 560 : 400;
+        const double cut = f32 ? (both ? 14500 : 8500) : width == 256 ? 19000 : both ? 15500 : 11000;
+        const double part = f32 ? 450 : width == 256 ? 2500 : 160;
+        // A block of a cut run takes 5 % more, on average over 92 shapes beyond 4096 x 8192 x 768 in short runs and 55 under
+        // the power cap (both gradients, cut / whole: 6532 x 19596 x 640 413 / 394 us with 4 % more blocks on the longest
+        // pair of whole tiles; under the power cap 20969 x 62907 x 640 5043 / 4879 with 17 % more.  Not everywhere:
+        // 20450 x 20450 x 896 1695 / 1952 with 9 % more).  fp32: none seen.
+        const double along = f32 ? 0 : 0.05;
         // A pair's next tile takes at least the epilogue of this one (dQ's adds what the positives' weights lost):
         // tiles of few contraction blocks are bound by it.  4671 x 30 x 128, both gradients: 18 dQ tiles of one
         // block to a pair 71 us, 19 pairs for them 14; 7 x 9470 x 128: 26 dP tiles of one block to a pair 44 us.
-        const double epi_q = width == 256 ? 12000 : 6000, epi_p = width == 256 ? 6400 : 3200;
+        const double epi_q = width == 256 ? 12000 : 6000, epi_p = width == 256 ? 11000 : 3200;
         const int64_t kq = ceil_div(N, KB), kp = ceil_div(rows, KB);
         const int64_t tq = dq ? ceil_div(rows, 256) * tn : 0, tp = dp ? ceil_div(N, 256) * tn : 0;
         auto offer = [&](double cost, int whole, int used) {
