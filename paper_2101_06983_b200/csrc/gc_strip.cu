@@ -20,8 +20,8 @@
 // logit kernel without its stores; gc_loss_bwd's logit kernel is given row_lse and writes W itself.
 //
 // All matrix work runs in CTA pairs (cta_group::2, M = 256): two producer warps, one issuing warp
-// (the leader's), eight epilogue warps; accumulators are double-buffered in tensor memory, so the
-// epilogue of a tile runs under the next tile's products.  Every wait is bounded.
+// (the leader's), eight epilogue warps; tensor memory holds two accumulators (fp32 gradients: four of half the
+// width), so the epilogue of a tile runs under the next tile's products.  Every wait is bounded.
 #include <cuda_fp16.h>
 #include <stdlib.h>
 #include <string.h>
@@ -1291,6 +1291,7 @@ strip_grad_kernel(const __grid_constant__ CUtensorMap mapWk, const __grid_consta
     constexpr int CHUNK_KB = 2;                           // F32: blocks per accumulator read-out
     constexpr int HW = WIDTH / 2;                         // columns of an epilogue warp
     constexpr int NACC = F32 ? 4 : 2;                     // accumulators in tensor memory
+    static_assert(NSOFT * (HW / 32) * (F32 ? 4096 : 6144) <= NST * STAGE, "the last tile is staged in the ring");
     const int pair = blockIdx.x >> 1;
     dep_release();
     // columns of a tile that exist, in whole 128s: a last tile of at most 128 columns runs at half width

@@ -312,27 +312,53 @@ def test_two_directions_over_several_strips(binding):
     assert grad_err(dP.cpu().numpy(), rP.cpu().numpy()) <= tol["grad"]
 
 
-@pytest.mark.parametrize("B,N,d,dtype", [(512, 8192, 768, "bf16"), (300, 9000, 200, "bf16"), (40, 16500, 72, "f32"),
-                                         (2100, 260, 136, "f32")])
+@pytest.mark.parametrize("B,N,d,dtype", [
+    (512, 8192, 768, "bf16"),                           # dQ in up to 12 shares a tile
+    (300, 4000, 200, "bf16"), (4001, 300, 200, "bf16"), # 200: the last column tile holds 72 of 128; ragged rows
+    (777, 3130, 320, "bf16"), (9001, 700, 640, "bf16"), # tiles of 128, the last of 320 half filled; dQ, dP
+    (1300, 16500, 640, "bf16"),                         # both: tiles of 256 columns, the last one at half width
+    (40, 16500, 72, "f32"), (2100, 260, 136, "f32"), (260, 2100, 136, "f32"),
+])
 def test_sums_of_cut_gradient_tiles(binding, oracle, B, N, d, dtype):
-    """One gradient alone over a long contraction: tiles in up to dozens of shares, summed in pieces by whoever is
-    there; ragged last rows and columns; the same bits in every run."""
+    """Each gradient alone and both, over long contractions: tiles in up to dozens of shares, summed in pieces by
+    whoever is there.  Ragged last rows and columns; outputs inside wider and longer buffers, of which nothing else
+    is written; the same bits in every run."""
     prob = inputs.random_problem(B, N, d, dtype, seed=B + N + d, tau=0.5, scale=d ** -0.5)
-    ref = _oracle_full(oracle, prob)
     Q, P, pos = to_device(prob)
-    b = binding.Outputs(B, N, d, binding._dtype_code(Q))
+    code = binding._dtype_code(Q)
+    assert binding.gc_kernel_launches(binding.GC_OP_BWD, B, N, d, code) == (2 if dtype == "bf16" else 4)   # one strip
+    b = binding.Outputs(B, N, d, code)
     args = (Q, P, pos, prob.tau, prob.mask_mode)
     binding.gc_loss_fwd(*args, b.loss, b.row_lse, b.pos_logit, b.ws, b.dev_status)
-    binding.gc_loss_bwd(*args, b.row_lse, b.dQ, None, b.ws, b.dev_status)
-    binding.gc_loss_bwd(*args, b.row_lse, None, b.dP, b.ws, b.dev_status)
-    torch.cuda.synchronize()
-    check_against_oracle(prob, b, ref)
-    first = b.dQ.clone(), b.dP.clone()
+    wide = {k: torch.full((n + 3, d + 8), float("nan"), device="cuda") for k, n in (("dQ", B), ("dP", N))}
+    b.dQ, b.dP = wide["dQ"][:B, :d], wide["dP"][:N, :d]
+
+    def grads(*which):
+        for w in wide.values():
+            w.fill_(float("nan"))
+        binding.gc_loss_bwd(*args, b.row_lse, *(getattr(b, k) if k in which else None for k in ("dQ", "dP")), b.ws,
+                            b.dev_status)
+        for k, w in wide.items():
+            g = getattr(b, k)
+            assert bool(torch.isfinite(g).all() if k in which else torch.isnan(g).all())
+            assert bool(torch.isnan(w[:, d:]).all()) and bool(torch.isnan(w[g.shape[0]:]).all())
+        return [getattr(b, k).clone() for k in which]
+
+    large = B * N * d > 1 << 33
+    ref = None if large else _oracle_full(oracle, prob)
+    alone = grads("dQ") + grads("dP")
+    both = grads("dQ", "dP")
+    for b.dQ, b.dP in (alone, both):
+        torch.cuda.synchronize()
+        if large:
+            _check_sampled(oracle, prob, b, 48, 24, full_lse=b.row_lse.cpu().numpy().astype(np.float64))
+        else:
+            check_against_oracle(prob, b, ref)
+    b.dQ, b.dP = wide["dQ"][:B, :d], wide["dP"][:N, :d]
     for _ in range(20):
-        b.dQ.fill_(float("nan")), b.dP.fill_(float("nan"))
-        binding.gc_loss_bwd(*args, b.row_lse, b.dQ, None, b.ws, b.dev_status)
-        binding.gc_loss_bwd(*args, b.row_lse, None, b.dP, b.ws, b.dev_status)
-        assert torch.equal(b.dQ, first[0]) and torch.equal(b.dP, first[1])
+        again = grads("dQ") + grads("dP"), grads("dQ", "dP")
+        assert all(torch.equal(x, y) for got, want in zip(again, (alone, both)) for x, y in zip(got, want))
+    assert int(b.dev_status.item()) == 0
 
 
 @pytest.mark.parametrize("B,N,d,dtype,lse2,tau2", [(32768, 25000, 448, "bf16", 15, 112), (32768, 25000, 1024, "bf16", 15, 112),
