@@ -43,9 +43,9 @@ NOMINAL_BF16_TFLOPS = 2250.0      # public dense bf16 figure for B200, context o
 STRIP_SOURCES = ['gc_strip.cu', 'tc_common.cuh']
 ONE_TILE_SOURCES = ['gc_small.cu', 'gc_small_f32.cu', 'tc_common.cuh']
 NCU_STEP_TRAFFIC = {
-    "cfg2_": (272.8e6, STRIP_SOURCES, "01077da8e666c6915687c74dc79e2a9dc4a5d43d"),
-    "cfg1_": (0.627e6, ONE_TILE_SOURCES, "43562d0a6d23d54a678b682771c6a3f376388009"),
-    "cfg0_": (0.634e6, ONE_TILE_SOURCES, "43562d0a6d23d54a678b682771c6a3f376388009"),
+    "cfg2_": (273.1e6, STRIP_SOURCES, "ea0ab94fa351497d351a6c946d74ead4636b8dab"),
+    "cfg1_": (0.627e6, ONE_TILE_SOURCES, "788ca7c65aa3671d925411bad1d574d1f77b345e"),
+    "cfg0_": (0.634e6, ONE_TILE_SOURCES, "788ca7c65aa3671d925411bad1d574d1f77b345e"),
 }
 FP32_LANES_PER_SM = 128           # fp32 FMA lanes of one SM (2 FLOP per lane and clock)
 
